@@ -39,6 +39,7 @@
 // GQA: query head h reads KV head h / G.  The ViT case is G = 1.
 #include <algorithm>
 #include <atomic>
+#include <climits>
 #include <cmath>
 #include <mutex>
 #include <vector>
@@ -83,6 +84,7 @@ struct Cfg {
   using B = TileFmt<D, kStream>;    // streamed tile
   static constexpr int STAGES = (D == 128) ? 2 : (D == 80) ? 4 : 5;
   static constexpr uint32_t IDESC = idesc_bf16_f32(kTile, kStream);
+  static constexpr uint32_t IDESC_HALF = idesc_bf16_f32(kTile, kTile);
 };
 
 // Extra K slice of pass 2 (16 bf16 columns, 32 bytes per row).  Query row i carries the
@@ -132,6 +134,8 @@ struct AttnTable {
   int H;        // query heads
   int G;        // query heads per KV head
   int splits;   // key splits of pass 1
+  int splits2;  // stream splits of pass 2
+  int qrows;    // rows of Q (the rows past them read as zeros)
   int prows;    // padded L rows per head
   int ktot;     // total key rows (part map row count)
 };
@@ -158,22 +162,27 @@ __device__ __forceinline__ bool aborted(const SmemCtl* ctl) {
   return *reinterpret_cast<const volatile int*>(&ctl->abort) != 0;
 }
 
-// TMA of ROWS rows (y .. y + ROWS - 1, columns x0 .. x0 + D) into dst in 128-row boxes;
-// completion is counted on the barrier `bar`.
+// TMA of the q-th 128-row box of a tile of ROWS rows (y .. y + ROWS - 1, columns x0 .. x0 + D) at
+// dst; completion is counted on the barrier `bar`.
+template <int D, int ROWS>
+__device__ __forceinline__ void load_box(uint8_t* dst, const CUtensorMap* m128, const CUtensorMap* m32, int x0, int y,
+                                         int q, uint32_t bar) {
+  using F = TileFmt<D, ROWS>;
+#pragma unroll
+  for (int i = 0; i < F::NB; ++i)
+    tma_load_2d(smem_u32(dst + i * F::BLOCK + q * kTile * 128), m128, x0 + 64 * i, y + q * kTile, bar);
+#pragma unroll
+  for (int r = 0; r < F::R; ++r)
+    tma_load_2d(smem_u32(dst + F::NB * F::BLOCK + r * F::SLICE + q * kTile * 32), m32, x0 + 64 * F::NB + 16 * r,
+                y + q * kTile, bar);
+}
+
+// All boxes of a tile.
 template <int D, int ROWS>
 __device__ __forceinline__ void load_tile(uint8_t* dst, const CUtensorMap* m128, const CUtensorMap* m32, int x0,
                                           int y, uint32_t bar) {
-  using F = TileFmt<D, ROWS>;
 #pragma unroll
-  for (int q = 0; q < ROWS / kTile; ++q) {
-#pragma unroll
-    for (int i = 0; i < F::NB; ++i)
-      tma_load_2d(smem_u32(dst + i * F::BLOCK + q * kTile * 128), m128, x0 + 64 * i, y + q * kTile, bar);
-#pragma unroll
-    for (int r = 0; r < F::R; ++r)
-      tma_load_2d(smem_u32(dst + F::NB * F::BLOCK + r * F::SLICE + q * kTile * 32), m32, x0 + 64 * F::NB + 16 * r,
-                  y + q * kTile, bar);
-  }
+  for (int q = 0; q < ROWS / kTile; ++q) load_box<D, ROWS>(dst, m128, m32, x0, y, q, bar);
 }
 
 // Shared-memory descriptors of a tile: [0] for its 128-byte-swizzled blocks, [1] for its
@@ -184,10 +193,11 @@ __device__ __forceinline__ void tile_desc(const uint8_t* tile, uint64_t& d128, u
   d32 = smem_desc_kmajor_sw32(smem_u32(tile + TileFmt<D, ROWS>::NB * TileFmt<D, ROWS>::BLOCK));
 }
 
-// MMA D[tmem] = A B^T (128 x 256) over the whole head dimension: 4 K-steps per 128-byte
-// block, 1 per 32-byte slice.
+// MMA D[tmem] = A B^T (128 x 256, or 128 x 128 with that instruction descriptor) over the whole
+// head dimension: 4 K-steps per 128-byte block, 1 per 32-byte slice.
 template <int D>
-__device__ __forceinline__ void mma_tile(uint32_t d, uint64_t a128, uint64_t a32, uint64_t b128, uint64_t b32) {
+__device__ __forceinline__ void mma_tile(uint32_t d, uint64_t a128, uint64_t a32, uint64_t b128, uint64_t b32,
+                                         uint32_t idesc = Cfg<D>::IDESC) {
   using FA = typename Cfg<D>::A;
   using FB = typename Cfg<D>::B;
 #pragma unroll
@@ -196,12 +206,12 @@ __device__ __forceinline__ void mma_tile(uint32_t d, uint64_t a128, uint64_t a32
     for (int k = 0; k < 4; ++k) {
       const uint64_t oa = static_cast<uint64_t>(i * (FA::BLOCK >> 4) + k * 2);
       const uint64_t ob = static_cast<uint64_t>(i * (FB::BLOCK >> 4) + k * 2);
-      mma_bf16_ss(d, a128 + oa, b128 + ob, Cfg<D>::IDESC, (i | k) != 0);
+      mma_bf16_ss(d, a128 + oa, b128 + ob, idesc, (i | k) != 0);
     }
 #pragma unroll
   for (int r = 0; r < FA::R; ++r)
     mma_bf16_ss(d, a32 + static_cast<uint64_t>(r * (FA::SLICE >> 4)), b32 + static_cast<uint64_t>(r * (FB::SLICE >> 4)),
-                Cfg<D>::IDESC, (FA::NB | r) != 0);
+                idesc, (FA::NB | r) != 0);
 }
 
 // 64 TMEM columns of this warp's 32 lanes -> v[0..63] (fp32 bit patterns), ready to use.
@@ -340,17 +350,17 @@ __device__ __forceinline__ void colsum64_from(const uint32_t (&v)[64], int lo, f
   colsum64(w, c, a0, a1);
 }
 
-// Overwrites query rows rows .. kStream - 1 of a staged pass-2 tile with zeros: the 128-byte rows
+// Overwrites query rows rows .. end - 1 of a staged pass-2 tile with zeros: the 128-byte rows
 // of its 64-column blocks and the 32-byte rows of its 16-column slices (a swizzle only moves
 // 16-byte pieces within their own row), by the 32 lanes of a warp.  The shift slice keeps the
 // padded rows' -2^100, so these rows add exactly 0 to every key's sum.
 template <int D>
-__device__ __forceinline__ void zero_stage_rows(uint8_t* st, int rows) {
+__device__ __forceinline__ void zero_stage_rows(uint8_t* st, int rows, int end) {
   using F = TileFmt<D, kStream>;
   constexpr int PIECES = F::NB * 8 + F::R * 2;   // 16-byte pieces per row
   const int lane = threadIdx.x & 31;
   const uint4 z = make_uint4(0u, 0u, 0u, 0u);
-  for (int i = lane; i < (kStream - rows) * PIECES; i += 32) {
+  for (int i = lane; i < (end - rows) * PIECES; i += 32) {
     const int row = rows + i / PIECES, pc = i % PIECES;
     uint8_t* dst = pc < F::NB * 8 ? st + (pc >> 3) * F::BLOCK + row * 128 + (pc & 7) * 16
                                   : st + F::NB * F::BLOCK + ((pc - F::NB * 8) >> 1) * F::SLICE + row * 32 +
@@ -418,11 +428,13 @@ __global__ void __launch_bounds__(kThreads, 1) attn_row_lse(const __grid_constan
   r /= t.splits;
   const int npair = t.pair_n[b];
   const int diag = t.diag[b];
-  // causal images: the last query rows see the most keys, so they are scheduled first
-  const int pair = t.pair_lo[b] + (CAUSAL ? npair - 1 - r % npair : r % npair);
-  const int h = r / npair;
+  // causal images: the last query rows see the most keys, so those of every head are scheduled
+  // first; otherwise the query tiles of a head follow one another (they stream the same keys)
+  const int h = CAUSAL ? r % t.H : r / npair;
+  const int pair = t.pair_lo[b] + (CAUSAL ? npair - 1 - r / t.H : r % npair);
   const int g = h / t.G;
   const int qrow0 = pair * kPair + kTile * static_cast<int>(rank);     // this CTA's first local query row
+  if (qrow0 >= t.nq[b]) return;   // the item's second half lies past the image: pass 2 does not read its shift rows
   const int nkt_all = (t.nk[b] + kStream - 1) / kStream;
   const int kt0 = static_cast<int>((static_cast<int64_t>(split) * nkt_all) / t.splits);
   // causal: key tiles past the one holding key qrow0 + 127 + diag are masked for every row (diag >= 0)
@@ -667,35 +679,73 @@ __global__ void __launch_bounds__(kThreads, 1) attn_colsum(const __grid_constant
   auto b_qempty = [&](int s) { return smem_u32(&ctl->bars[2 + ST + s]); };
   auto b_sfull = [&](int p) { return smem_u32(&ctl->bars[2 + 2 * ST + p]); };
   auto b_sfree = [&](int p) { return smem_u32(&ctl->bars[4 + 2 * ST + p]); };
-  // stage s holds an image's ragged last query tile with the rows past the image zeroed: one
-  // arrival per ragged use of the stage (the other tiles need only their copy)
+  // stage s holds an image's last query tile with the next image's rows zeroed: one arrival per
+  // such use of the stage (the other tiles need only their copy)
   auto b_fixed = [&](int s) { return smem_u32(&ctl->bars[6 + 2 * ST + s]); };
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = blockIdx.x & 1u;       // which 128-row half of the item
   const int item = blockIdx.x >> 1;
   const int b = find_image(t, item);
-  const int r = item - t.item_prefix[b];
+  int r = item - t.item_prefix[b];
+  const int sp = r % t.splits2;
+  r /= t.splits2;
   const int nkp = (t.nk[b] + kPair - 1) / kPair;
-  const int kp = r % nkp;
-  const int g = r / nkp;
+  // causal images: the first keys are seen by the most queries, so those of every KV head are
+  // scheduled first; otherwise the key tiles of a head follow one another
+  const int nkv = t.H / t.G;
+  const int g = CAUSAL ? r % nkv : r / nkp;
+  const int kp = CAUSAL ? r / nkv : r % nkp;
   const int krow0 = kp * kPair + kTile * static_cast<int>(rank);     // this CTA's first local key row
+  if (krow0 >= t.nk[b]) return;   // the item's second half lies past the image
   const int diag = t.diag[b];
   const int nqt = (t.nq[b] + kStream - 1) / kStream;
   // causal images: query tiles that end before row krow0 - diag see none of this CTA's keys
   const int qt_min = CAUSAL && krow0 > diag ? (krow0 - diag) / kStream : 0;
   const int nspan = max(nqt - qt_min, 0);
-  const int nj = t.G * nspan;                                         // stream: (head in group, query tile)
-  // query rows of stream tile j that lie inside the image (kStream unless it is the image's last
-  // tile and the image ends inside it)
-  auto ragged_rows = [&](int j) { return min(kStream, t.nq[b] - (qt_min + j % nspan) * kStream); };
-  // the ragged tiles are j = nspan - 1, 2 nspan - 1, .. (when the image ends inside its last query
-  // tile); the phase of b_fixed(j % ST) that ragged tile j completes = how many earlier ragged tiles
-  // used the same stage
-  auto ragged_phase = [&](int j) {
-    int k = 0;
-    for (int j2 = nspan - 1; j2 < j; j2 += nspan) k += (j2 % ST) == (j % ST);
-    return k & 1;
+  // the stream: (head in group, query tile), of which this CTA takes items j0 .. j0 + nj - 1
+  const int nj_all = t.G * nspan;
+  const int each = nj_all / t.splits2, extra = nj_all - each * t.splits2;
+  const int j0 = sp * each + min(sp, extra);
+  const int nj = each + (sp < extra ? 1 : 0);
+  // A last query tile that ends inside the stream tile:
+  //  - its rows past the image are zeros when the image is the last of Q (they lie outside the
+  //    tensor), else the next image's rows, which warp 0 overwrites with zeros (`fix`).  It then
+  //    trades places with an early tile (position `swap`), whose copy is issued in the prologue, so
+  //    that the overwriting runs while the tiles before it are worked on;
+  //  - with at most 128 query rows it takes half the copy, half the MMA and half the epilogue.
+  const int last_rows = t.nq[b] - (nqt - 1) * kStream;   // query rows of the last tile
+  const bool fix = last_rows < kStream && t.q0[b] + t.nq[b] < t.qrows;
+  const bool half = last_rows <= kTile;
+  const int swap = min(ST - 1, nspan - 1);
+  const int special = fix ? swap : nspan - 1;   // the last tile's position in each head's tiles
+  // first local stream item that is such a tile (the next ones follow every nspan items)
+  auto first_special = [&]() {
+    if (!(fix || half) || nj <= 0) return INT_MAX;
+    const int d = special - j0 % nspan;
+    return d < 0 ? d + nspan : d;
+  };
+  struct Pos {   // a stream item: head in group hq, position i in its query tiles
+    int hq, i;
+  };
+  auto pos_at = [&](int j) {
+    Pos q{0, 0};
+    if (nj > 0) {
+      q.hq = (j0 + j) / nspan;
+      q.i = j0 + j - q.hq * nspan;
+    }
+    return q;
+  };
+  auto advance = [&](Pos& q, int n) {
+    q.i += n;
+    while (q.i >= nspan) {
+      q.i -= nspan;
+      ++q.hq;
+    }
+  };
+  auto tile_at = [&](const Pos& q) {   // its query tile
+    const int i = !fix ? q.i : q.i == swap ? nspan - 1 : q.i == nspan - 1 ? swap : q.i;
+    return qt_min + i;
   };
 
   if (threadIdx.x == 0) {
@@ -713,19 +763,21 @@ __global__ void __launch_bounds__(kThreads, 1) attn_colsum(const __grid_constant
     ctl->abort = 0;
     fence_mbar_init();
   }
-  // stage s of stream item j: query tile (head in group, query tile) plus its shift slice
-  auto issue_stage = [&](int j, int s) {
-    const int hq = j / nspan, qt = qt_min + j - hq * nspan;
-    const int h = g * t.G + hq;
+  // stage s: query tile qt of head hq in the group plus its shift slice
+  auto issue_stage = [&](const Pos& q, int s) {
+    const int h = g * t.G + q.hq, qt = tile_at(q);
     uint8_t* st = sQ + s * B2;
-    mbar_arrive_expect_tx(b_qfull(s), B2);
-    load_tile<D, kStream>(st, &tmq, &tmq32, h * D, t.q0[b] + qt * kStream, b_qfull(s));
     const int srow = h * t.prows + t.lpad[b] + qt * kStream;
-#pragma unroll
-    for (int q = 0; q < kStream / kTile; ++q)
-      tma_load_2d(smem_u32(st + C::B::BYTES + q * kTile * kShiftCols * 2), &tmshift, 0, srow + q * kTile,
-                  b_qfull(s));
+    auto box = [&](int x) {
+      load_box<D, kStream>(st, &tmq, &tmq32, h * D, t.q0[b] + qt * kStream, x, b_qfull(s));
+      tma_load_2d(smem_u32(st + C::B::BYTES + x * kTile * kShiftCols * 2), &tmshift, 0, srow + x * kTile, b_qfull(s));
+    };
+    const bool one = half && qt == nqt - 1;
+    mbar_arrive_expect_tx(b_qfull(s), one ? B2 / 2 : B2);
+    box(0);
+    if (!one) box(1);
   };
+  static_assert(kStream == 2 * kTile, "a stream tile is two boxes");
   const int pre = min(nj, ST);   // query stages issued in the prologue (first use of each stage)
   if (threadIdx.x == 0) {
     // the resident key tile and the first query stages are requested before the CTA-wide
@@ -740,7 +792,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_colsum(const __grid_constant
     mbar_arrive_expect_tx(b_afull, A2);
     load_tile<D, kTile>(sA, &tmk, &tmk32, g * D, t.k0[b] + krow0, b_afull);
     tma_load_2d(smem_u32(sA + C::A::BYTES), &tmones, 0, 0, b_afull);
-    for (int j = 0; j < pre; ++j) issue_stage(j, j);
+    Pos q = pos_at(0);
+    for (int j = 0; j < pre; ++j, advance(q, 1)) issue_stage(q, j);
   }
   if (warp == 1) {
     tmem_alloc(smem_u32(&ctl->tmem_base), kTmemCols);
@@ -753,10 +806,11 @@ __global__ void __launch_bounds__(kThreads, 1) attn_colsum(const __grid_constant
 
   if (warp == 0) {
     // The whole warp walks the stream: lane 0 issues the copies; on an image's last query tile,
-    // when it holds rows past the image, all lanes overwrite those rows with zeros once the copy
-    // has landed (they belong to the next image and may hold inf or NaN, which the -2^100 shift of
-    // a padded row would not cancel), and then release the tile to the MMA.
-    for (int j = 0; j < nj; ++j) {
+    // when it holds rows of the next image, all lanes overwrite those rows with zeros once the copy
+    // has landed (they may hold inf or NaN, which the -2^100 shift of a padded row would not
+    // cancel), and then release the tile to the MMA.
+    Pos q = pos_at(0);
+    for (int j = 0; j < nj; ++j, advance(q, 1)) {
       const int s = j % ST, u = j / ST;
       int ok = 1;
       if (j >= pre && lane == 0) {
@@ -766,17 +820,16 @@ __global__ void __launch_bounds__(kThreads, 1) attn_colsum(const __grid_constant
         } else if (aborted(ctl)) {
           ok = 0;
         } else {
-          issue_stage(j, s);
+          issue_stage(q, s);
         }
       }
-      const int rows = ragged_rows(j);
-      if (rows < kStream) {
+      if (fix && q.i == swap) {
         if (lane == 0 && ok && !mbar_wait(b_qfull(s), u & 1, kWaitLimitNs)) {
           set_abort(ctl, status, K_ATTN_COLSUM);
           ok = 0;
         }
         if (__shfl_sync(0xffffffffu, ok, 0)) {
-          zero_stage_rows<D>(sQ + s * B2, rows);
+          zero_stage_rows<D>(sQ + s * B2, last_rows, half ? kTile : kStream);
           fence_proxy_async_shared();
           __syncwarp();
           if (lane == 0) mbar_arrive(b_fixed(s));
@@ -793,6 +846,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_colsum(const __grid_constant
       const uint64_t bshift = smem_desc_kmajor_sw32(smem_u32(sQ + C::B::BYTES));
       bool ok = mbar_wait(b_afull, 0, kWaitLimitNs);
       if (!ok) set_abort(ctl, status, K_ATTN_COLSUM);
+      int next = first_special();
+      uint32_t fixed = 0u;   // bit s: phase of b_fixed(s) that its next use completes
       for (int j = 0; ok && j < nj; ++j) {
         const int s = j % ST, u = j / ST;
         const int p = j & 1, v = j >> 1;
@@ -801,14 +856,22 @@ __global__ void __launch_bounds__(kThreads, 1) attn_colsum(const __grid_constant
           set_abort(ctl, status, K_ATTN_COLSUM);
           break;
         }
-        if (ragged_rows(j) < kStream && !mbar_wait(b_fixed(s), ragged_phase(j), kWaitLimitNs)) {
-          set_abort(ctl, status, K_ATTN_COLSUM);
-          break;
+        uint32_t idesc = C::IDESC;
+        if (j == next) {
+          next += nspan;
+          if (half) idesc = C::IDESC_HALF;
+          if (fix) {
+            if (!mbar_wait(b_fixed(s), (fixed >> s) & 1u, kWaitLimitNs)) {
+              set_abort(ctl, status, K_ATTN_COLSUM);
+              break;
+            }
+            fixed ^= 1u << s;
+          }
         }
         tc_fence_after_sync();
         const uint64_t so = static_cast<uint64_t>(s * (B2 >> 4));
-        mma_tile<D>(tmem + p * 256, ak128, ak32, bq128 + so, bq32 + so);
-        mma_bf16_ss(tmem + p * 256, aone, bshift + so, C::IDESC, 1);   // + (-L_i / c)
+        mma_tile<D>(tmem + p * 256, ak128, ak32, bq128 + so, bq32 + so, idesc);
+        mma_bf16_ss(tmem + p * 256, aone, bshift + so, idesc, 1);   // + (-L_i / c)
         mma_commit(b_sfull(p));
         mma_commit(b_qempty(s));
       }
@@ -824,6 +887,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_colsum(const __grid_constant
     float2 acc = make_float2(0.f, 0.f), acc1 = acc;
     const uint32_t tbuf = tmem + (static_cast<uint32_t>(quad * 32) << 16) + p * 256 + hh * 128;
     const int key = krow0 + rr;
+    int next = hh == 1 && half ? first_special() : INT_MAX;   // next tile without columns for this warp
+    Pos q = CAUSAL ? pos_at(p) : Pos{0, 0};
     for (int j = p; j < nj; j += 2) {
       const int v = j >> 1;
       const bool ok = __all_sync(0xffffffffu, mbar_wait(b_sfull(p), v & 1, kWaitLimitNs));
@@ -832,11 +897,20 @@ __global__ void __launch_bounds__(kThreads, 1) attn_colsum(const __grid_constant
         break;
       }
       tc_fence_after_sync();
+      const int qt = CAUSAL ? tile_at(q) : 0;
+      if (CAUSAL) advance(q, 2);
+      if (j >= next) {   // warp-uniform
+        while (next < j) next += nspan;
+        if (j == next) {
+          if (lane == 0) mbar_arrive(b_sfree(p));
+          continue;
+        }
+      }
       // causal mask: query columns before `lo` do not see this thread's key
       int lo = 0;
       bool masked = false;
       if (CAUSAL) {
-        lo = key - diag - ((qt_min + j % nspan) * kStream + hh * 128);
+        lo = key - diag - (qt * kStream + hh * 128);
         masked = __any_sync(0xffffffffu, lo > 0);
       }
       uint32_t sv[64];
@@ -856,7 +930,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_colsum(const __grid_constant
     named_barrier_sync(1, 32 * kEpiWarps);
     if (e == 0) {
       if (key < t.nk[b])
-        part[static_cast<int64_t>(g) * t.ktot + t.out0[b] + key] =
+        part[(static_cast<int64_t>(g) * t.splits2 + sp) * t.ktot + t.out0[b] + key] =
             (a + ctl->xchg[0][0][rr]) + (ctl->xchg[1][0][rr] + ctl->xchg[2][0][rr]);
     }
   }
@@ -937,7 +1011,7 @@ struct Seg {
 };
 
 struct AttnLayout {
-  int splits;
+  int splits, splits2;
   int64_t prows, ktot;
   size_t L_off, part_off, ml_off, total;
 };
@@ -970,9 +1044,47 @@ int choose_splits(const std::vector<Seg>& segs, int H) {
   return best;
 }
 
+// Stream splits of pass 2 (query heads of a group and query tiles over several CTAs, each with
+// its own row of the part map).  Non-causal images are planned in whole rounds like pass 1; with a
+// causal mask the CTAs' streams differ and the longest start first, so the time is about the
+// average load plus half the longest CTA.
+int choose_splits2(const std::vector<Seg>& segs, int Hq, int groups) {
+  const int G = Hq / groups;
+  int64_t ctas = 0, tiles = 0;
+  int longest = 1;
+  bool causal = false;
+  for (const Seg& sg : segs) {
+    const int nkt = (sg.nv + kTile - 1) / kTile, nqt = (sg.nq + kStream - 1) / kStream;
+    ctas += static_cast<int64_t>(groups) * nkt;
+    longest = std::max(longest, G * nqt);
+    causal |= sg.vdiag != kNoMask;
+    if (sg.vdiag == kNoMask) {
+      tiles += static_cast<int64_t>(groups) * nkt * G * nqt;
+    } else {
+      for (int k = 0; k < nkt; ++k)
+        tiles += static_cast<int64_t>(groups) * G * std::max(nqt - std::max(k * kTile - sg.vdiag, 0) / kStream, 0);
+    }
+  }
+  int best = 1;
+  double best_cost = 0.0;
+  for (int s = 1; s <= std::min(longest, 16); ++s) {
+    const double per = causal ? (static_cast<double>(longest) / s + kSplitOverheadTiles) * 0.5 +
+                                    (static_cast<double>(tiles) + static_cast<double>(ctas) * s * kSplitOverheadTiles) /
+                                        kPlanSms
+                              : static_cast<double>((ctas * s + kPlanSms - 1) / kPlanSms) *
+                                    ((longest + s - 1) / s + kSplitOverheadTiles);
+    if (s == 1 || per < best_cost) {
+      best = s;
+      best_cost = per;
+    }
+  }
+  return best;
+}
+
 AttnLayout attn_layout(const std::vector<Seg>& segs, int H, int groups) {
   AttnLayout L{};
   L.splits = choose_splits(segs, H);
+  L.splits2 = choose_splits2(segs, H, groups);
   int64_t pr = 0, kt = 0;
   for (const Seg& sg : segs) {
     pr += static_cast<int64_t>((sg.nq + kPair - 1) / kPair) * kPair;
@@ -982,7 +1094,7 @@ AttnLayout attn_layout(const std::vector<Seg>& segs, int H, int groups) {
   L.ktot = kt;
   L.L_off = 0;
   L.part_off = align_up(static_cast<size_t>(H) * L.prows * kShiftCols * 2, 256);
-  L.ml_off = L.part_off + align_up(static_cast<size_t>(groups) * L.ktot * sizeof(float), 256);
+  L.ml_off = L.part_off + align_up(static_cast<size_t>(groups) * L.splits2 * L.ktot * sizeof(float), 256);
   L.total = L.ml_off;
   if (L.splits > 1) L.total += align_up(static_cast<size_t>(L.splits) * H * L.prows * sizeof(float2), 256);
   return L;
@@ -1094,29 +1206,39 @@ pace_status_t run_importance(const void* Q, const void* K, int64_t qrows, int64_
     t.H = Hq;
     t.G = G;
     t.splits = Lay.splits;
+    t.splits2 = Lay.splits2;
+    t.qrows = static_cast<int>(qrows);
     t.prows = static_cast<int>(Lay.prows);
     t.ktot = static_cast<int>(Lay.ktot);
-    int items1 = 0, ctiles = 0;
-    t.item_prefix[0] = 0;
+    // Table order: the images whose CTAs stream the longest first (keys in pass 1, queries in pass
+    // 2), so that a ragged batch ends on its shortest CTAs.
+    int lpads[kAttnMaxB], order[kAttnMaxB], ctiles = 0;
     for (int i = 0; i < nb; ++i) {
-      const Seg& sg = segs[c0 + i];
+      const int rows = (segs[c0 + i].nq + kPair - 1) / kPair * kPair;
+      lpads[i] = lpad;
+      lpad += rows;
+      order[i] = c0 + i;
+      ctiles += rows / kTile;
+    }
+    auto by_length = [&](int Seg::* len) {
+      if (nb > 1) std::stable_sort(order, order + nb, [&](int x, int y) { return segs[x].*len > segs[y].*len; });
+    };
+    by_length(&Seg::nk);
+    for (int i = 0; i < nb; ++i) {
+      const Seg& sg = segs[order[i]];
       t.q0[i] = sg.q0;
       t.nq[i] = sg.nq;
       t.k0[i] = sg.k0;
       t.nk[i] = sg.nk;
       t.diag[i] = sg.diag;
-      t.lpad[i] = lpad;
-      lpad += (sg.nq + kPair - 1) / kPair * kPair;
-      items1 += Hq * ((sg.nq + kPair - 1) / kPair) * Lay.splits;
-      t.item_prefix[i + 1] = items1;
-      ctiles += (sg.nq + kPair - 1) / kPair * 2;
+      t.lpad[i] = lpads[order[i] - c0];
     }
     const int pieces = chunks.n > 0 ? chunks.n : 1;
     for (int pc = 0; pc < pieces; ++pc) {
       int items_pc = 0;
       t.item_prefix[0] = 0;
       for (int i = 0; i < nb; ++i) {
-        const Seg& sg = segs[c0 + i];
+        const Seg& sg = segs[order[i]];
         const int npair = (sg.nq + kPair - 1) / kPair;
         int lo = 0, hi = npair;
         if (chunks.n > 0) {   // pairs whose last row falls in [end_row[pc - 1], end_row[pc])
@@ -1134,20 +1256,24 @@ pace_status_t run_importance(const void* Q, const void* K, int64_t qrows, int64_
       if (chunks.n > 0) PACE_CUDA(cudaStreamWaitEvent(stream, chunks.ready[pc], 0));
       PACE_CHECK(launch_pairs(attn_row_lse<D, CAUSAL>, items_pc, s1, stream, mq, mq32, mk, mk32, t, c, Lw, ml, status));
     }
-    (void)items1;
     if (Lay.splits > 1 && ctiles > 0) {
       attn_lse_combine<<<dim3(ctiles, Hq), kTile, 0, stream>>>(t, c, ml, Lw);
       PACE_CHECK(check_launch());
     }
     // pass 2 streams the same query rows (and L rows) against the scored keys
     int items2 = 0;
+    t.item_prefix[0] = 0;
+    by_length(&Seg::nq);
     for (int i = 0; i < nb; ++i) {
-      const Seg& sg = segs[c0 + i];
+      const Seg& sg = segs[order[i]];
+      t.q0[i] = sg.q0;
+      t.nq[i] = sg.nq;
       t.k0[i] = sg.v0;
       t.nk[i] = sg.nv;
       t.diag[i] = sg.vdiag;
+      t.lpad[i] = lpads[order[i] - c0];
       t.out0[i] = sg.out0;
-      items2 += Hkv * ((sg.nv + kPair - 1) / kPair);
+      items2 += Hkv * ((sg.nv + kPair - 1) / kPair) * Lay.splits2;
       t.item_prefix[i + 1] = items2;
     }
     PACE_CHECK(launch_pairs(attn_colsum<D, CAUSAL>, items2, s2, stream, mq, mq32, mk, mk32, mshift, mones, t, c, part,
@@ -1155,8 +1281,8 @@ pace_status_t run_importance(const void* Q, const void* K, int64_t qrows, int64_
   }
   const int nout = static_cast<int>(Lay.ktot / merge);
   if (nout > 0) {
-    attn_reduce<<<(nout * kReduceLanes + 255) / 256, 256, 0, stream>>>(part, Hkv, static_cast<int>(Lay.ktot), merge,
-                                                                         out);
+    attn_reduce<<<(nout * kReduceLanes + 255) / 256, 256, 0, stream>>>(part, Hkv * Lay.splits2,
+                                                                        static_cast<int>(Lay.ktot), merge, out);
     PACE_CHECK(check_launch());
   }
   return PACE_OK;
