@@ -412,6 +412,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_row_lse(const __grid_constan
   uint8_t* sQ = smem;                                // this CTA's resident query tile
   uint8_t* sK = sQ + C::A::BYTES;                    // ST stages of a key tile
   SmemCtl* ctl = reinterpret_cast<SmemCtl*>(sK + ST * C::B::BYTES);
+  launch_dependents();   // the next kernel's blocks take the SMs that the last wave leaves idle
   const uint32_t b_qfull = smem_u32(&ctl->bars[0]);     // query tile landed
   const uint32_t b_done = smem_u32(&ctl->bars[1]);      // all MMAs of a round finished
   auto b_kfull = [&](int s) { return smem_u32(&ctl->bars[2 + s]); };
@@ -626,6 +627,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_row_lse(const __grid_constan
 // image get the padded-row shift.
 __global__ void __launch_bounds__(128) attn_lse_combine(const __grid_constant__ AttnTable t, float c,
                                                         const float2* __restrict__ ml, uint16_t* __restrict__ shift_out) {
+  launch_dependents();
+  grid_dependency_wait();   // pass 1's partial pairs
   // blockIdx.x = (image, 128-row tile of its padded rows) flattened
   int rem = blockIdx.x;
   const int h = blockIdx.y;
@@ -673,6 +676,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_colsum(const __grid_constant
   constexpr int B2 = C::B::BYTES + kStream * kShiftCols * 2;      // query tile + shift slice
   uint8_t* sQ = sA + A2;                               // ST stages of a query tile
   SmemCtl* ctl = reinterpret_cast<SmemCtl*>(sQ + ST * B2);
+  launch_dependents();
   const uint32_t b_afull = smem_u32(&ctl->bars[0]);
   const uint32_t b_done = smem_u32(&ctl->bars[1]);
   auto b_qfull = [&](int s) { return smem_u32(&ctl->bars[2 + s]); };
@@ -781,7 +785,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_colsum(const __grid_constant
   const int pre = min(nj, ST);   // query stages issued in the prologue (first use of each stage)
   if (threadIdx.x == 0) {
     // the resident key tile and the first query stages are requested before the CTA-wide
-    // barrier, so their latency overlaps the TMEM allocation
+    // barrier, so their latency overlaps the TMEM allocation; the key tile does not depend on pass
+    // 1, the stages carry its shift rows
     prefetch_tensormap(&tmq);
     prefetch_tensormap(&tmk);
     if (C::A::R > 0) {
@@ -792,6 +797,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_colsum(const __grid_constant
     mbar_arrive_expect_tx(b_afull, A2);
     load_tile<D, kTile>(sA, &tmk, &tmk32, g * D, t.k0[b] + krow0, b_afull);
     tma_load_2d(smem_u32(sA + C::A::BYTES), &tmones, 0, 0, b_afull);
+    grid_dependency_wait();
     Pos q = pos_at(0);
     for (int j = 0; j < pre; ++j, advance(q, 1)) issue_stage(q, j);
   }
@@ -945,6 +951,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_colsum(const __grid_constant
 constexpr int kReduceLanes = 4;
 __global__ void __launch_bounds__(256) attn_reduce(const float* __restrict__ part, int groups, int ktot, int merge,
                                                    float* __restrict__ out) {
+  grid_dependency_wait();
   const int tid = blockIdx.x * blockDim.x + threadIdx.x;
   const int m = tid / kReduceLanes, j = tid % kReduceLanes;
   const int nout = ktot / merge;
@@ -954,7 +961,7 @@ __global__ void __launch_bounds__(256) attn_reduce(const float* __restrict__ par
       const float* p = part + static_cast<int64_t>(g) * ktot + static_cast<int64_t>(m) * merge;
       float gs;
       if (merge == 4 && (ktot & 3) == 0) {   // 16-byte aligned rows of four
-        const float4 v = __ldg(reinterpret_cast<const float4*>(p));
+        const float4 v = __ldcg(reinterpret_cast<const float4*>(p));
         gs = (v.x + v.y) + (v.z + v.w);
       } else {
         gs = 0.f;
@@ -1155,14 +1162,6 @@ pace_status_t set_smem_attrs(size_t* s1, size_t* s2) {
   return PACE_OK;
 }
 
-// Launches `items` work items of two independent CTAs each.
-template <typename... Params, typename... Args>
-pace_status_t launch_pairs(void (*kernel)(Params...), int items, size_t smem, cudaStream_t stream, Args... args) {
-  if (items <= 0) return PACE_OK;
-  kernel<<<dim3(2 * static_cast<unsigned>(items)), dim3(kThreads), smem, stream>>>(args...);
-  return check_launch();
-}
-
 // Pass 1 in pieces: piece c waits for event ready[c] and takes the query pairs whose last row
 // (a global row of Q) is below end_row[c] (and not below end_row[c - 1]).
 struct QueryChunks {
@@ -1254,11 +1253,15 @@ pace_status_t run_importance(const void* Q, const void* K, int64_t qrows, int64_
         t.item_prefix[i + 1] = items_pc;
       }
       if (chunks.n > 0) PACE_CUDA(cudaStreamWaitEvent(stream, chunks.ready[pc], 0));
-      PACE_CHECK(launch_pairs(attn_row_lse<D, CAUSAL>, items_pc, s1, stream, mq, mq32, mk, mk32, t, c, Lw, ml, status));
+      if (items_pc > 0) {   // two CTAs per work item
+        attn_row_lse<D, CAUSAL><<<2 * static_cast<unsigned>(items_pc), kThreads, s1, stream>>>(mq, mq32, mk, mk32, t, c, Lw,
+                                                                                               ml, status);
+        PACE_CHECK(check_launch());
+      }
     }
     if (Lay.splits > 1 && ctiles > 0) {
-      attn_lse_combine<<<dim3(ctiles, Hq), kTile, 0, stream>>>(t, c, ml, Lw);
-      PACE_CHECK(check_launch());
+      PACE_CHECK(launch_dependent(attn_lse_combine, dim3(ctiles, Hq), kTile, 0, 1, stream, t, c,
+                                  static_cast<const float2*>(ml), Lw));
     }
     // pass 2 streams the same query rows (and L rows) against the scored keys
     int items2 = 0;
@@ -1276,14 +1279,14 @@ pace_status_t run_importance(const void* Q, const void* K, int64_t qrows, int64_
       items2 += Hkv * ((sg.nv + kPair - 1) / kPair) * Lay.splits2;
       t.item_prefix[i + 1] = items2;
     }
-    PACE_CHECK(launch_pairs(attn_colsum<D, CAUSAL>, items2, s2, stream, mq, mq32, mk, mk32, mshift, mones, t, c, part,
-                            status));
+    if (items2 > 0)
+      PACE_CHECK(launch_dependent(attn_colsum<D, CAUSAL>, 2 * static_cast<unsigned>(items2), kThreads, s2, 1, stream, mq,
+                                  mq32, mk, mk32, mshift, mones, t, c, part, status));
   }
   const int nout = static_cast<int>(Lay.ktot / merge);
   if (nout > 0) {
-    attn_reduce<<<(nout * kReduceLanes + 255) / 256, 256, 0, stream>>>(part, Hkv * Lay.splits2,
-                                                                        static_cast<int>(Lay.ktot), merge, out);
-    PACE_CHECK(check_launch());
+    PACE_CHECK(launch_dependent(attn_reduce, (nout * kReduceLanes + 255) / 256, 256, 0, 1, stream,
+                                static_cast<const float*>(part), Hkv * Lay.splits2, static_cast<int>(Lay.ktot), merge, out));
   }
   return PACE_OK;
 }

@@ -80,6 +80,19 @@ pace_status_t check_launch() {
   return PACE_OK;
 }
 
+pace_status_t sm_count(int* sms) {
+  static std::atomic<int> count[kMaxDevices];
+  int dev = 0;
+  PACE_CUDA(cudaGetDevice(&dev));
+  int n = dev >= 0 && dev < kMaxDevices ? count[dev].load(std::memory_order_relaxed) : 0;
+  if (n == 0) {
+    PACE_CUDA(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
+    if (dev >= 0 && dev < kMaxDevices) count[dev].store(n, std::memory_order_relaxed);
+  }
+  *sms = n;
+  return PACE_OK;
+}
+
 // One CTA waits on an mbarrier that nothing ever arrives at: the bounded wait must give up
 // after limit_ns and record PACE_ERR_TIMEOUT, leaving the context usable.
 __global__ void selftest_wait_kernel(uint64_t limit_ns, int* status) {

@@ -41,6 +41,7 @@ pace_status_t set_cuda_error(cudaError_t e);
 pace_status_t check_device();              // current device is sm_103 and initialised
 int* device_status_word();                 // status word of the current device
 pace_status_t check_launch();              // cudaGetLastError -> status
+pace_status_t sm_count(int* sms);          // SMs of the current device
 
 // Generation of the library's per-device set-up.  pace_init(dev) advances it, so every cache
 // built on DeviceOnce below (function attributes, symbol addresses) is filled again on the next
@@ -63,6 +64,45 @@ class DeviceOnce {
  private:
   std::atomic<uint32_t> flag_[kMaxDevices];
 };
+
+// Launch with `cluster` blocks along x per cluster and, if `dependent`, programmatic dependent launch.
+template <typename... Params, typename... Args>
+pace_status_t launch_ex(bool dependent, void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem,
+                        unsigned cluster, cudaStream_t stream, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute at[2] = {};
+  cfg.attrs = at;
+  if (dependent) {
+    at[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[cfg.numAttrs].val.programmaticStreamSerializationAllowed = 1;
+    ++cfg.numAttrs;
+  }
+  if (cluster > 1) {
+    at[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+    at[cfg.numAttrs].val.clusterDim.x = cluster;
+    at[cfg.numAttrs].val.clusterDim.y = at[cfg.numAttrs].val.clusterDim.z = 1;
+    ++cfg.numAttrs;
+  }
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+  if (e != cudaSuccess) return set_cuda_error(e);
+  return check_launch();
+}
+// A kernel that may start while the stream's previous kernel is still running: it calls
+// ptx::grid_dependency_wait() before it reads or writes anything that other work touches.
+template <typename... Params, typename... Args>
+pace_status_t launch_dependent(void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem, unsigned cluster,
+                               cudaStream_t stream, Args... args) {
+  return launch_ex(true, kernel, grid, threads, smem, cluster, stream, args...);
+}
+template <typename... Params, typename... Args>
+pace_status_t launch_cluster(void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem, unsigned cluster,
+                             cudaStream_t stream, Args... args) {
+  return launch_ex(false, kernel, grid, threads, smem, cluster, stream, args...);
+}
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
