@@ -61,6 +61,7 @@ class HotPath:
         k_tot = int(self.cu_keep[-1])
         self.kept = torch.empty(max(k_tot, 1), dtype=i32, device=dev)
         self.rows = torch.empty((max(k_tot, 1), self.d["embed"].shape[1]), dtype=torch.bfloat16, device=dev)
+        self.kept_all = self.kept[:k_tot]
         self.ws_density = torch.empty(max(P.pace_apc_density_workspace_size(self.H, self.W), 16), dtype=u8,
                                       device=dev)
         self.ws_vit = torch.empty(max(P.pace_vit_attn_importance_workspace_size(self.cu_patches, synth.VIT_HEADS),
@@ -96,7 +97,7 @@ class HotPath:
 
     def gather(self, d=None):
         d = d or self.d
-        P.pace_gather(d["embed"], self.kept[: int(self.cu_keep[-1])], dst=self.rows)
+        P.pace_gather(d["embed"], self.kept_all, dst=self.rows)
 
     def step(self):
         for _, f in self.parts:

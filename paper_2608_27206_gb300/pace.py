@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+from array import array
 from typing import Optional, Sequence
 
 import numpy as np
@@ -57,53 +58,51 @@ class GatherTensor(ctypes.Structure):
 GATHER_MAX_TENSORS = 16
 
 
-_P = ctypes.c_void_p
-_I32P = ctypes.POINTER(ctypes.c_int32)
-_I64P = ctypes.POINTER(ctypes.c_int64)
+_P = ctypes.c_void_p   # device addresses and host index arrays alike
 _SIGS = {
     "pace_status_string": (ctypes.c_char_p, [ctypes.c_int]),
     "pace_last_cuda_error": (ctypes.c_int, []),
     "pace_kernel_launch_count": (ctypes.c_uint64, []),
     "pace_selftest_wait_timeout": (ctypes.c_int, [ctypes.c_uint32, _P]),
     "pace_init": (ctypes.c_int, [ctypes.c_int]),
-    "pace_device_status": (ctypes.c_int, [_I32P, _I32P, ctypes.c_int]),
+    "pace_device_status": (ctypes.c_int, [_P, _P, ctypes.c_int]),
     "pace_apc_params_default": (None, [ctypes.POINTER(ApcParams)]),
-    "pace_apc_density_workspace_size": (ctypes.c_size_t, [ctypes.c_int, _I32P, _I32P]),
+    "pace_apc_density_workspace_size": (ctypes.c_size_t, [ctypes.c_int, _P, _P]),
     "pace_budget_vanilla": (ctypes.c_int32, [ctypes.c_int32, ctypes.c_int32, ctypes.c_double]),
-    "pace_prune_index": (ctypes.c_int, [ctypes.c_int, _I32P, _I32P, _I32P, _I32P, _P, _P, _P]),
+    "pace_prune_index": (ctypes.c_int, [ctypes.c_int, _P, _P, _P, _P, _P, _P, _P]),
     "pace_gather_multi": (ctypes.c_int, [ctypes.POINTER(GatherTensor), ctypes.c_int, _P, ctypes.c_int64, _P]),
-    "pace_apc_density_tokens_workspace_size": (ctypes.c_size_t, [ctypes.c_int, _I32P, ctypes.c_int]),
-    "pace_apc_density_tokens": (ctypes.c_int, [_P, _I32P, ctypes.c_int, ctypes.c_int, _I32P, _I32P,
+    "pace_apc_density_tokens_workspace_size": (ctypes.c_size_t, [ctypes.c_int, _P, ctypes.c_int]),
+    "pace_apc_density_tokens": (ctypes.c_int, [_P, _P, ctypes.c_int, ctypes.c_int, _P, _P,
                                                ctypes.POINTER(ApcParams), _P, _P, _P, ctypes.c_size_t, _P]),
-    "pace_apc_density": (ctypes.c_int, [_P, _I64P, _I32P, _I32P, ctypes.c_int, ctypes.POINTER(ApcParams), _P, _P,
+    "pace_apc_density": (ctypes.c_int, [_P, _P, _P, _P, ctypes.c_int, ctypes.POINTER(ApcParams), _P, _P,
                                         _P, ctypes.c_size_t, _P]),
-    "pace_apc_pixel_features": (ctypes.c_int, [_P, _I64P, _I32P, _I32P, ctypes.c_int, ctypes.c_int, _P, _P]),
-    "pace_apc_density_pixel_workspace_size": (ctypes.c_size_t, [ctypes.c_int, _I32P, _I32P]),
-    "pace_apc_density_pixel": (ctypes.c_int, [_P, _I64P, _I32P, _I32P, ctypes.c_int, ctypes.c_int,
+    "pace_apc_pixel_features": (ctypes.c_int, [_P, _P, _P, _P, ctypes.c_int, ctypes.c_int, _P, _P]),
+    "pace_apc_density_pixel_workspace_size": (ctypes.c_size_t, [ctypes.c_int, _P, _P]),
+    "pace_apc_density_pixel": (ctypes.c_int, [_P, _P, _P, _P, ctypes.c_int, ctypes.c_int,
                                               ctypes.POINTER(ApcParams), _P, _P, _P, ctypes.c_size_t, _P]),
-    "pace_apc_density_static": (ctypes.c_int, [_P, _I64P, _I32P, _I32P, ctypes.c_int, ctypes.POINTER(ApcParams),
+    "pace_apc_density_static": (ctypes.c_int, [_P, _P, _P, _P, ctypes.c_int, ctypes.POINTER(ApcParams),
                                                _P, _P, _P]),
-    "pace_apc_resample": (ctypes.c_int, [_P, _I64P, _I32P, _I32P, _P, _P, _I64P, ctypes.c_int, _P]),
-    "pace_apc_resample_to": (ctypes.c_int, [_P, _I64P, _I32P, _I32P, _I32P, _I32P, _P, _I64P, ctypes.c_int, _P]),
-    "pace_vit_attn_importance_workspace_size": (ctypes.c_size_t, [ctypes.c_int, _I32P, ctypes.c_int]),
-    "pace_vit_attn_importance": (ctypes.c_int, [_P, _P, _I32P, ctypes.c_int, ctypes.c_int, ctypes.c_int,
+    "pace_apc_resample": (ctypes.c_int, [_P, _P, _P, _P, _P, _P, _P, ctypes.c_int, _P]),
+    "pace_apc_resample_to": (ctypes.c_int, [_P, _P, _P, _P, _P, _P, _P, _P, ctypes.c_int, _P]),
+    "pace_vit_attn_importance_workspace_size": (ctypes.c_size_t, [ctypes.c_int, _P, ctypes.c_int]),
+    "pace_vit_attn_importance": (ctypes.c_int, [_P, _P, _P, ctypes.c_int, ctypes.c_int, ctypes.c_int,
                                                 ctypes.c_float, ctypes.c_int, _P, _P, ctypes.c_size_t, _P]),
-    "pace_vit_attn_importance_chunked": (ctypes.c_int, [_P, _P, _I32P, ctypes.c_int, ctypes.c_int, ctypes.c_int,
+    "pace_vit_attn_importance_chunked": (ctypes.c_int, [_P, _P, _P, ctypes.c_int, ctypes.c_int, ctypes.c_int,
                                                         ctypes.c_float, ctypes.c_int, _P, _P, ctypes.c_size_t,
-                                                        ctypes.c_int, _I64P, ctypes.POINTER(ctypes.c_void_p), _P]),
-    "pace_llm_text_visual_importance_workspace_size": (ctypes.c_size_t, [ctypes.c_int, _I32P, _I32P, ctypes.c_int,
+                                                        ctypes.c_int, _P, ctypes.POINTER(ctypes.c_void_p), _P]),
+    "pace_llm_text_visual_importance_workspace_size": (ctypes.c_size_t, [ctypes.c_int, _P, _P, ctypes.c_int,
                                                                          ctypes.c_int]),
-    "pace_llm_text_visual_importance": (ctypes.c_int, [_P, _P, _I32P, _I32P, ctypes.c_int, ctypes.c_int,
+    "pace_llm_text_visual_importance": (ctypes.c_int, [_P, _P, _P, _P, ctypes.c_int, ctypes.c_int,
                                                        ctypes.c_int, ctypes.c_int, ctypes.c_float, _P, _P,
                                                        ctypes.c_size_t, _P]),
-    "pace_llm_sequence_importance_workspace_size": (ctypes.c_size_t, [ctypes.c_int, _I32P, _I32P, _I32P,
+    "pace_llm_sequence_importance_workspace_size": (ctypes.c_size_t, [ctypes.c_int, _P, _P, _P,
                                                                       ctypes.c_int, ctypes.c_int, ctypes.c_int]),
-    "pace_llm_sequence_importance": (ctypes.c_int, [_P, _P, _I32P, _I32P, _I32P, ctypes.c_int, ctypes.c_int,
+    "pace_llm_sequence_importance": (ctypes.c_int, [_P, _P, _P, _P, _P, ctypes.c_int, ctypes.c_int,
                                                     ctypes.c_int, ctypes.c_int, ctypes.c_float, ctypes.c_int, _P,
                                                     _P, ctypes.c_size_t, _P]),
     "pace_ddae_params_default": (None, [ctypes.POINTER(DdaeParams)]),
     "pace_budget": (ctypes.c_int32, [ctypes.c_int32, ctypes.c_double]),
-    "pace_ddae_select": (ctypes.c_int, [_P, _P, _I32P, _I32P, ctypes.c_int, ctypes.POINTER(DdaeParams), _P, _P,
+    "pace_ddae_select": (ctypes.c_int, [_P, _P, _P, _P, ctypes.c_int, ctypes.POINTER(DdaeParams), _P, _P,
                                         _P, _P]),
     "pace_gather": (ctypes.c_int, [_P, ctypes.c_int64, ctypes.c_int64, _P, ctypes.c_int64, _P, _P]),
 }
@@ -137,20 +136,45 @@ def _check(fn: str, status: int):
         raise PaceError(fn, status, detail)
 
 
-def _i32(a) -> np.ndarray:
-    return np.ascontiguousarray(np.asarray(a, dtype=np.int32))
+# Host index arrays.  A call costs the GPU as little as 15 us, so what happens per argument counts:
+# a list becomes an array.array (0.3 us; a numpy conversion with its ctypes pointer 3 us), a numpy
+# array of the right type is passed as it is.  Each helper returns (owner, address, length); the
+# owner has to outlive the call.
+def _ints(a, code: str, dtype):
+    if type(a) is list or type(a) is tuple:
+        try:
+            x = array(code, a)
+            return x, x.buffer_info()[0], len(x)
+        except (TypeError, OverflowError):
+            pass    # nested, or not whole numbers: numpy decides
+    elif type(a) is np.ndarray and a.dtype == dtype and a.flags.c_contiguous:
+        return a, a.__array_interface__["data"][0], len(a)
+    x = np.ascontiguousarray(np.asarray(a, dtype=dtype))
+    return x, x.__array_interface__["data"][0], len(x)
 
 
-def _i64(a) -> np.ndarray:
-    return np.ascontiguousarray(np.asarray(a, dtype=np.int64))
+_I32, _I64 = np.dtype(np.int32), np.dtype(np.int64)
 
 
-def _pi32(a: np.ndarray):
-    return a.ctypes.data_as(_I32P)
+def _i32(a):
+    return _ints(a, "i", _I32)
 
 
-def _pi64(a: np.ndarray):
-    return a.ctypes.data_as(_I64P)
+def _i64(a):
+    return _ints(a, "q", _I64)
+
+
+def _n_patches(h, w) -> int:
+    """Patches of the images whose sides the owners h and w hold."""
+    if len(h) != len(w):
+        raise ValueError("H and W differ in length")
+    if len(h) == 1:
+        return int(h[0]) // 14 * (int(w[0]) // 14)
+    return sum(x // 14 * (y // 14) for x, y in zip(h.tolist(), w.tolist()))
+
+
+def _first(t: torch.Tensor, n: int) -> torch.Tensor:
+    return t if t.shape[0] == n else t[:n]
 
 
 def _dev(t: Optional[torch.Tensor]):
@@ -160,21 +184,32 @@ def _dev(t: Optional[torch.Tensor]):
         raise ValueError("expected a CUDA tensor")
     if not t.is_contiguous():
         raise ValueError("expected a contiguous tensor")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
+
+
+# The current stream's handle without a Stream object around it (0.1 us against 2.9), where torch has it.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream(stream):
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is not None:
+        return _raw_stream(torch.cuda.current_device())
+    return torch.cuda.current_stream().cuda_stream
 
 
-def _workspace(nbytes: int, ws: Optional[torch.Tensor], device) -> torch.Tensor:
-    if ws is not None:
-        if ws.numel() * ws.element_size() < nbytes:
-            raise PaceError("workspace", PACE_ERR_WORKSPACE)
-        return ws
-    return torch.empty(max(int(nbytes), 16), dtype=torch.uint8, device=device)
+def _workspace(size, args, ws: Optional[torch.Tensor], device):
+    """The workspace tensor and its bytes: the caller's, or a new one of size(*args) bytes."""
+    if ws is None:
+        ws = torch.empty(max(int(size(*args)), 16), dtype=torch.uint8, device=device)
+    return ws, ws.numel() * ws.element_size()
+
+
+def _check_ws(fn: str, status: int, given):
+    """_check; a caller's workspace that is too small is named as such."""
+    if status != PACE_OK:
+        _check("workspace" if status == PACE_ERR_WORKSPACE and given is not None else fn, status)
 
 
 # ----------------------------------------------------------------------------------------------
@@ -225,29 +260,34 @@ def ddae_params(**kw) -> DdaeParams:
 # Condense
 # ----------------------------------------------------------------------------------------------
 def pace_apc_density_workspace_size(H: Sequence[int], W: Sequence[int]) -> int:
-    h, w = _i32(H), _i32(W)
-    return int(lib().pace_apc_density_workspace_size(len(h), _pi32(h), _pi32(w)))
+    (_h, hp, B), (_w, wp, _) = _i32(H), _i32(W)
+    return int(lib().pace_apc_density_workspace_size(B, hp, wp))
+
+
+def _density_outputs(n: int, B: int, dev, d_out, stats):
+    if d_out is None:
+        d_out = torch.empty(max(n, 1), dtype=torch.float32, device=dev)
+    if stats is None:
+        stats = torch.zeros((max(B, 1), 10), dtype=torch.int32, device=dev)
+    return d_out, stats
+
+
+def _params(params):
+    return ctypes.byref(params) if params is not None else None
 
 
 def pace_apc_density(img: torch.Tensor, img_off, H, W, params: Optional[ApcParams] = None,
                      d_out: Optional[torch.Tensor] = None, stats: Optional[torch.Tensor] = None,
                      ws: Optional[torch.Tensor] = None, stream=None):
     """APC density of B packed uint8 images.  Returns (d [sum N] float32, stats [B, 10] int32 view)."""
-    off, h, w = _i64(img_off), _i32(H), _i32(W)
-    B = len(h)
-    n = int(((h // 14).astype(np.int64) * (w // 14)).sum())
-    dev = img.device
-    if d_out is None:
-        d_out = torch.empty(max(n, 1), dtype=torch.float32, device=dev)
-    if stats is None:
-        stats = torch.zeros((max(B, 1), 10), dtype=torch.int32, device=dev)
-    nbytes = pace_apc_density_workspace_size(h, w)
-    ws = _workspace(nbytes, ws, dev)
-    st = lib().pace_apc_density(_dev(img), _pi64(off), _pi32(h), _pi32(w), B,
-                                ctypes.byref(params) if params is not None else None, _dev(d_out), _dev(stats),
-                                _dev(ws), ws.numel() * ws.element_size(), _stream(stream))
-    _check("pace_apc_density", st)
-    return d_out[:n], stats[:B]
+    (_o, op, _), (h, hp, B), (w, wp, _) = _i64(img_off), _i32(H), _i32(W)
+    n = _n_patches(h, w)
+    d_out, stats = _density_outputs(n, B, img.device, d_out, stats)
+    L = lib()
+    buf, nbytes = _workspace(L.pace_apc_density_workspace_size, (B, hp, wp), ws, img.device)
+    _check_ws("pace_apc_density", L.pace_apc_density(_dev(img), op, hp, wp, B, _params(params), _dev(d_out), _dev(stats),
+                                                     _dev(buf), nbytes, _stream(stream)), ws)
+    return _first(d_out, n), _first(stats, B)
 
 
 def _feature(feature) -> int:
@@ -258,40 +298,33 @@ def pace_apc_pixel_features(img: torch.Tensor, img_off, H, W, feature, out: Opti
                             stream=None) -> torch.Tensor:
     """Pixel-statistic feature tokens float32 [sum N, 8] of B packed uint8 images; feature is
     "rgb_stats", "color_entropy", "edge_density", "laplacian" or a FEATURE_* code."""
-    off, h, w = _i64(img_off), _i32(H), _i32(W)
-    B = len(h)
-    n = int(((h // 14).astype(np.int64) * (w // 14)).sum())
+    (_o, op, _), (h, hp, B), (w, wp, _) = _i64(img_off), _i32(H), _i32(W)
+    n = _n_patches(h, w)
     if out is None:
         out = torch.empty((max(n, 1), PIXEL_FEATURE_DIM), dtype=torch.float32, device=img.device)
-    st = lib().pace_apc_pixel_features(_dev(img), _pi64(off), _pi32(h), _pi32(w), B, _feature(feature), _dev(out),
-                                       _stream(stream))
-    _check("pace_apc_pixel_features", st)
-    return out[:n]
+    _check("pace_apc_pixel_features", lib().pace_apc_pixel_features(_dev(img), op, hp, wp, B, _feature(feature), _dev(out),
+                                                                    _stream(stream)))
+    return _first(out, n)
 
 
 def pace_apc_density_pixel_workspace_size(H, W) -> int:
-    h, w = _i32(H), _i32(W)
-    return int(lib().pace_apc_density_pixel_workspace_size(len(h), _pi32(h), _pi32(w)))
+    (_h, hp, B), (_w, wp, _) = _i32(H), _i32(W)
+    return int(lib().pace_apc_density_pixel_workspace_size(B, hp, wp))
 
 
 def pace_apc_density_pixel(img: torch.Tensor, img_off, H, W, feature, params: Optional[ApcParams] = None,
                            d_out: Optional[torch.Tensor] = None, stats: Optional[torch.Tensor] = None,
                            ws: Optional[torch.Tensor] = None, stream=None):
     """APC density with a pixel-statistic preview.  Returns (d [sum N], stats [B, 10])."""
-    off, h, w = _i64(img_off), _i32(H), _i32(W)
-    B = len(h)
-    n = int(((h // 14).astype(np.int64) * (w // 14)).sum())
-    dev = img.device
-    if d_out is None:
-        d_out = torch.empty(max(n, 1), dtype=torch.float32, device=dev)
-    if stats is None:
-        stats = torch.zeros((max(B, 1), 10), dtype=torch.int32, device=dev)
-    ws = _workspace(pace_apc_density_pixel_workspace_size(h, w), ws, dev)
-    st = lib().pace_apc_density_pixel(_dev(img), _pi64(off), _pi32(h), _pi32(w), B, _feature(feature),
-                                      ctypes.byref(params) if params is not None else None, _dev(d_out), _dev(stats),
-                                      _dev(ws), ws.numel() * ws.element_size(), _stream(stream))
-    _check("pace_apc_density_pixel", st)
-    return d_out[:n], stats[:B]
+    (_o, op, _), (h, hp, B), (w, wp, _) = _i64(img_off), _i32(H), _i32(W)
+    n = _n_patches(h, w)
+    d_out, stats = _density_outputs(n, B, img.device, d_out, stats)
+    L = lib()
+    buf, nbytes = _workspace(L.pace_apc_density_pixel_workspace_size, (B, hp, wp), ws, img.device)
+    _check_ws("pace_apc_density_pixel",
+              L.pace_apc_density_pixel(_dev(img), op, hp, wp, B, _feature(feature), _params(params), _dev(d_out), _dev(stats),
+                                       _dev(buf), nbytes, _stream(stream)), ws)
+    return _first(d_out, n), _first(stats, B)
 
 
 PACE_APC_STATIC_MAX_IMAGES = 16
@@ -307,45 +340,33 @@ def pace_apc_density_static(img: torch.Tensor, img_off, H, W, params: Optional[A
     images and PACE_APC_STATIC_MAX_PATCHES patches per call; calls that overlap on the GPU
     share one scratch array and must be serialised.  Returns (d, stats) like pace_apc_density.
     """
-    off, h, w = _i64(img_off), _i32(H), _i32(W)
-    B = len(h)
-    n = int(((h // 14).astype(np.int64) * (w // 14)).sum())
-    dev = img.device
-    if d_out is None:
-        d_out = torch.empty(max(n, 1), dtype=torch.float32, device=dev)
-    if stats is None:
-        stats = torch.zeros((max(B, 1), 10), dtype=torch.int32, device=dev)
-    st = lib().pace_apc_density_static(_dev(img), _pi64(off), _pi32(h), _pi32(w), B,
-                                       ctypes.byref(params) if params is not None else None, _dev(d_out),
-                                       _dev(stats), _stream(stream))
-    _check("pace_apc_density_static", st)
-    return d_out[:n], stats[:B]
+    (_o, op, _), (h, hp, B), (w, wp, _) = _i64(img_off), _i32(H), _i32(W)
+    n = _n_patches(h, w)
+    d_out, stats = _density_outputs(n, B, img.device, d_out, stats)
+    _check("pace_apc_density_static", lib().pace_apc_density_static(_dev(img), op, hp, wp, B, _params(params), _dev(d_out),
+                                                                    _dev(stats), _stream(stream)))
+    return _first(d_out, n), _first(stats, B)
 
 
 def pace_apc_density_tokens_workspace_size(cu_tokens, D: int) -> int:
-    cu = _i32(cu_tokens)
-    return int(lib().pace_apc_density_tokens_workspace_size(len(cu) - 1, _pi32(cu), D))
+    _c, cp, n = _i32(cu_tokens)
+    return int(lib().pace_apc_density_tokens_workspace_size(n - 1, cp, D))
 
 
 def pace_apc_density_tokens(T: torch.Tensor, cu_tokens, H, W, params: Optional[ApcParams] = None,
                             d_out: Optional[torch.Tensor] = None, stats: Optional[torch.Tensor] = None,
                             ws: Optional[torch.Tensor] = None, stream=None):
     """APC density of B images' preview tokens T (bf16 [sum N, D]).  Returns (d [sum N], stats)."""
-    cu, h, w = _i32(cu_tokens), _i32(H), _i32(W)
-    B = len(cu) - 1
+    (cu, cp, B), (_h, hp, _), (_w, wp, _) = _i32(cu_tokens), _i32(H), _i32(W)
+    B -= 1
     n, D = int(cu[-1]), int(T.shape[-1])
-    dev = T.device
-    if d_out is None:
-        d_out = torch.empty(max(n, 1), dtype=torch.float32, device=dev)
-    if stats is None:
-        stats = torch.zeros((max(B, 1), 10), dtype=torch.int32, device=dev)
+    d_out, stats = _density_outputs(n, B, T.device, d_out, stats)
+    L = lib()
     if ws is None:
-        ws = torch.empty(max(pace_apc_density_tokens_workspace_size(cu, D), 16), dtype=torch.uint8, device=dev)
-    st = lib().pace_apc_density_tokens(_dev(T), _pi32(cu), B, D, _pi32(h), _pi32(w),
-                                       ctypes.byref(params) if params is not None else None, _dev(d_out),
-                                       _dev(stats), _dev(ws), ws.numel(), _stream(stream))
-    _check("pace_apc_density_tokens", st)
-    return d_out[:n], stats[:B]
+        ws = torch.empty(max(int(L.pace_apc_density_tokens_workspace_size(B, cp, D)), 16), dtype=torch.uint8, device=T.device)
+    _check("pace_apc_density_tokens", L.pace_apc_density_tokens(_dev(T), cp, B, D, hp, wp, _params(params), _dev(d_out),
+                                                                _dev(stats), _dev(ws), ws.numel(), _stream(stream)))
+    return _first(d_out, n), _first(stats, B)
 
 
 def pace_budget_vanilla(n_vis_vanilla: int, n_vis_condensed: int, frac: float) -> int:
@@ -355,14 +376,13 @@ def pace_budget_vanilla(n_vis_vanilla: int, n_vis_condensed: int, frac: float) -
 def pace_prune_index(cu_seq, vis_start, cu_vis, cu_keep, kept: torch.Tensor, out: Optional[torch.Tensor] = None,
                      stream=None):
     """Row list of the pruned sequences (global pre-prune rows), int32 on kept's device."""
-    sq, vs, v, kp = _i32(cu_seq), _i32(vis_start), _i32(cu_vis), _i32(cu_keep)
-    B = len(sq) - 1
-    n_out = int((sq[1:] - sq[:-1]).sum() - v[-1] + kp[-1]) if B > 0 else 0
+    (sq, sp, B), (_vs, vsp, _), (v, vp, _), (kp, kpp, _) = _i32(cu_seq), _i32(vis_start), _i32(cu_vis), _i32(cu_keep)
+    B -= 1
+    n_out = int(sq[-1]) - int(sq[0]) - int(v[-1]) + int(kp[-1]) if B > 0 else 0
     if out is None:
         out = torch.empty(max(n_out, 1), dtype=torch.int32, device=kept.device)
-    st = lib().pace_prune_index(B, _pi32(sq), _pi32(vs), _pi32(v), _pi32(kp), _dev(kept), _dev(out), _stream(stream))
-    _check("pace_prune_index", st)
-    return out[:n_out]
+    _check("pace_prune_index", lib().pace_prune_index(B, sp, vsp, vp, kpp, _dev(kept), _dev(out), _stream(stream)))
+    return _first(out, n_out)
 
 
 def gather_spec(src: torch.Tensor, dst: torch.Tensor, dim: int) -> GatherTensor:
@@ -400,17 +420,16 @@ def stats_dict(stats: torch.Tensor):
 
 def pace_apc_resample(src: torch.Tensor, src_off, H, W, stats: torch.Tensor, dst: torch.Tensor, dst_off,
                       stream=None) -> None:
-    off, h, w, doff = _i64(src_off), _i32(H), _i32(W), _i64(dst_off)
-    _check("pace_apc_resample", lib().pace_apc_resample(_dev(src), _pi64(off), _pi32(h), _pi32(w), _dev(stats),
-                                                        _dev(dst), _pi64(doff), len(h), _stream(stream)))
+    (_o, op, _), (_h, hp, B), (_w, wp, _), (_d, dp, _) = _i64(src_off), _i32(H), _i32(W), _i64(dst_off)
+    _check("pace_apc_resample", lib().pace_apc_resample(_dev(src), op, hp, wp, _dev(stats), _dev(dst), dp, B,
+                                                        _stream(stream)))
 
 
 def pace_apc_resample_to(src: torch.Tensor, src_off, H, W, H_out, W_out, dst: torch.Tensor, dst_off,
                          stream=None) -> None:
-    off, h, w, doff = _i64(src_off), _i32(H), _i32(W), _i64(dst_off)
-    ho, wo = _i32(H_out), _i32(W_out)
-    _check("pace_apc_resample_to", lib().pace_apc_resample_to(_dev(src), _pi64(off), _pi32(h), _pi32(w), _pi32(ho),
-                                                              _pi32(wo), _dev(dst), _pi64(doff), len(h),
+    (_o, op, _), (_h, hp, B), (_w, wp, _), (_d, dp, _) = _i64(src_off), _i32(H), _i32(W), _i64(dst_off)
+    (_ho, hop, _), (_wo, wop, _) = _i32(H_out), _i32(W_out)
+    _check("pace_apc_resample_to", lib().pace_apc_resample_to(_dev(src), op, hp, wp, hop, wop, _dev(dst), dp, B,
                                                               _stream(stream)))
 
 
@@ -418,32 +437,34 @@ def pace_apc_resample_to(src: torch.Tensor, src_off, H, W, H_out, W_out, dst: to
 # Extract
 # ----------------------------------------------------------------------------------------------
 def pace_vit_attn_importance_workspace_size(cu_seqlens, n_heads: int) -> int:
-    cu = _i32(cu_seqlens)
-    return int(lib().pace_vit_attn_importance_workspace_size(len(cu) - 1, _pi32(cu), int(n_heads)))
+    _c, cp, n = _i32(cu_seqlens)
+    return int(lib().pace_vit_attn_importance_workspace_size(n - 1, cp, int(n_heads)))
 
 
 def pace_vit_attn_importance(Q: torch.Tensor, K: torch.Tensor, cu_seqlens, scale: Optional[float] = None,
                              merge: int = 4, out: Optional[torch.Tensor] = None,
                              ws: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """S_vis_raw [total / merge] from bf16 Q, K [total, heads, head_dim]."""
-    cu = _i32(cu_seqlens)
-    B = len(cu) - 1
+    cu, cp, B = _i32(cu_seqlens)
+    B -= 1
     total, Hh, D = Q.shape
+    n = int(cu[-1]) // merge
     if scale is None:
         scale = float(D) ** -0.5
     if out is None:
-        out = torch.empty(max(int(cu[-1]) // merge, 1), dtype=torch.float32, device=Q.device)
-    ws = _workspace(pace_vit_attn_importance_workspace_size(cu, Hh), ws, Q.device)
-    st = lib().pace_vit_attn_importance(_dev(Q), _dev(K), _pi32(cu), B, Hh, D, float(scale), int(merge), _dev(out),
-                                        _dev(ws), ws.numel() * ws.element_size(), _stream(stream))
-    _check("pace_vit_attn_importance", st)
-    return out[: int(cu[-1]) // merge]
+        out = torch.empty(max(n, 1), dtype=torch.float32, device=Q.device)
+    L = lib()
+    buf, nbytes = _workspace(L.pace_vit_attn_importance_workspace_size, (B, cp, Hh), ws, Q.device)
+    _check_ws("pace_vit_attn_importance",
+              L.pace_vit_attn_importance(_dev(Q), _dev(K), cp, B, Hh, D, float(scale), int(merge), _dev(out), _dev(buf),
+                                         nbytes, _stream(stream)), ws)
+    return _first(out, n)
 
 
 def vit_chunk_rows(cu_seqlens, n_chunks: int, pair: int = 256) -> np.ndarray:
     """End rows of `n_chunks` near-equal pieces of Q, each end moved down to the end of a
     `pair`-row block of its image (or the image's end), so no block waits for a later piece."""
-    cu = _i32(cu_seqlens).astype(np.int64)
+    cu = np.asarray(cu_seqlens, dtype=np.int64)
     total = int(cu[-1])
     ends = []
     for c in range(1, n_chunks):
@@ -462,48 +483,50 @@ def pace_vit_attn_importance_chunked(Q: torch.Tensor, K: torch.Tensor, cu_seqlen
                                      ws: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """pace_vit_attn_importance whose row log-sum-exp pass runs in pieces of query rows, piece c
     after the (already recorded) event chunk_ready[c]; bit-identical results."""
-    cu = _i32(cu_seqlens)
-    B = len(cu) - 1
+    cu, cp, B = _i32(cu_seqlens)
+    B -= 1
     total, Hh, D = Q.shape
+    n = int(cu[-1]) // merge
     if scale is None:
         scale = float(D) ** -0.5
     if out is None:
-        out = torch.empty(max(int(cu[-1]) // merge, 1), dtype=torch.float32, device=Q.device)
-    ends = _i64(chunk_end_rows)
-    if len(chunk_ready) != len(ends):
+        out = torch.empty(max(n, 1), dtype=torch.float32, device=Q.device)
+    _e, ep, n_ends = _i64(chunk_end_rows)
+    if len(chunk_ready) != n_ends:
         raise ValueError("one event per chunk")
-    evs = (ctypes.c_void_p * max(len(ends), 1))(*[int(e.cuda_event) for e in chunk_ready])
-    ws = _workspace(pace_vit_attn_importance_workspace_size(cu, Hh), ws, Q.device)
-    st = lib().pace_vit_attn_importance_chunked(_dev(Q), _dev(K), _pi32(cu), B, Hh, D, float(scale), int(merge),
-                                                _dev(out), _dev(ws), ws.numel() * ws.element_size(), len(ends),
-                                                _pi64(ends), evs, _stream(stream))
-    _check("pace_vit_attn_importance_chunked", st)
-    return out[: int(cu[-1]) // merge]
+    evs = (ctypes.c_void_p * max(n_ends, 1))(*[int(e.cuda_event) for e in chunk_ready])
+    L = lib()
+    buf, nbytes = _workspace(L.pace_vit_attn_importance_workspace_size, (B, cp, Hh), ws, Q.device)
+    _check_ws("pace_vit_attn_importance_chunked",
+              L.pace_vit_attn_importance_chunked(_dev(Q), _dev(K), cp, B, Hh, D, float(scale), int(merge), _dev(out),
+                                                 _dev(buf), nbytes, n_ends, ep, evs, _stream(stream)), ws)
+    return _first(out, n)
 
 
 def pace_llm_text_visual_importance_workspace_size(cu_q, cu_k, n_q_heads: int, n_kv_heads: int) -> int:
-    q, k = _i32(cu_q), _i32(cu_k)
-    return int(lib().pace_llm_text_visual_importance_workspace_size(len(q) - 1, _pi32(q), _pi32(k), int(n_q_heads),
-                                                                    int(n_kv_heads)))
+    (_q, qp, n), (_k, kp, _) = _i32(cu_q), _i32(cu_k)
+    return int(lib().pace_llm_text_visual_importance_workspace_size(n - 1, qp, kp, int(n_q_heads), int(n_kv_heads)))
 
 
 def pace_llm_text_visual_importance(Q: torch.Tensor, K: torch.Tensor, cu_q, cu_k, scale: Optional[float] = None,
                                     out: Optional[torch.Tensor] = None, ws: Optional[torch.Tensor] = None,
                                     stream=None) -> torch.Tensor:
     """S_llm_raw [sum Nv] from bf16 Q [sum Tq, Hq, D] and K [sum Nv, Hkv, D]."""
-    q, k = _i32(cu_q), _i32(cu_k)
-    B = len(q) - 1
+    (_q, qp, B), (k, kp, _) = _i32(cu_q), _i32(cu_k)
+    B -= 1
     _, Hq, D = Q.shape
     Hkv = K.shape[1]
+    n = int(k[-1])
     if scale is None:
         scale = float(D) ** -0.5
     if out is None:
-        out = torch.empty(max(int(k[-1]), 1), dtype=torch.float32, device=Q.device)
-    ws = _workspace(pace_llm_text_visual_importance_workspace_size(q, k, Hq, Hkv), ws, Q.device)
-    st = lib().pace_llm_text_visual_importance(_dev(Q), _dev(K), _pi32(q), _pi32(k), B, Hq, Hkv, D, float(scale),
-                                               _dev(out), _dev(ws), ws.numel() * ws.element_size(), _stream(stream))
-    _check("pace_llm_text_visual_importance", st)
-    return out[: int(k[-1])]
+        out = torch.empty(max(n, 1), dtype=torch.float32, device=Q.device)
+    L = lib()
+    buf, nbytes = _workspace(L.pace_llm_text_visual_importance_workspace_size, (B, qp, kp, Hq, Hkv), ws, Q.device)
+    _check_ws("pace_llm_text_visual_importance",
+              L.pace_llm_text_visual_importance(_dev(Q), _dev(K), qp, kp, B, Hq, Hkv, D, float(scale), _dev(out), _dev(buf),
+                                                nbytes, _stream(stream)), ws)
+    return _first(out, n)
 
 
 def _query_set(query_set) -> int:
@@ -512,9 +535,8 @@ def _query_set(query_set) -> int:
 
 def pace_llm_sequence_importance_workspace_size(cu_seq, vis_start, n_vis, n_q_heads: int, n_kv_heads: int,
                                                 query_set="vision_text") -> int:
-    c, v, n = _i32(cu_seq), _i32(vis_start), _i32(n_vis)
-    return int(lib().pace_llm_sequence_importance_workspace_size(len(c) - 1, _pi32(c), _pi32(v), _pi32(n),
-                                                                 int(n_q_heads), int(n_kv_heads),
+    (_c, cp, B), (_v, vp, _), (_n, np_, _) = _i32(cu_seq), _i32(vis_start), _i32(n_vis)
+    return int(lib().pace_llm_sequence_importance_workspace_size(B - 1, cp, vp, np_, int(n_q_heads), int(n_kv_heads),
                                                                  _query_set(query_set)))
 
 
@@ -524,51 +546,50 @@ def pace_llm_sequence_importance(Q: torch.Tensor, K: torch.Tensor, cu_seq, vis_s
                                  stream=None) -> torch.Tensor:
     """Full-sequence S_llm_raw [sum n_vis] from bf16 Q [sum S, Hq, D] and K [sum S, Hkv, D] of causal
     sequences; query_set is "vision_text", "text" or "last" (or a QUERY_* code)."""
-    c, v, n = _i32(cu_seq), _i32(vis_start), _i32(n_vis)
-    B = len(c) - 1
+    (_c, cp, B), (_v, vp, _), (n, np_, _) = _i32(cu_seq), _i32(vis_start), _i32(n_vis)
+    B -= 1
     _, Hq, D = Q.shape
     Hkv = K.shape[1]
     qs = _query_set(query_set)
     if scale is None:
         scale = float(D) ** -0.5
-    total = int(n.sum()) if B > 0 else 0
+    total = sum(n.tolist()) if B > 0 else 0
     if out is None:
         out = torch.empty(max(total, 1), dtype=torch.float32, device=Q.device)
-    ws = _workspace(pace_llm_sequence_importance_workspace_size(c, v, n, Hq, Hkv, qs), ws, Q.device)
-    st = lib().pace_llm_sequence_importance(_dev(Q), _dev(K), _pi32(c), _pi32(v), _pi32(n), B, Hq, Hkv, D,
-                                            float(scale), qs, _dev(out), _dev(ws), ws.numel() * ws.element_size(),
-                                            _stream(stream))
-    _check("pace_llm_sequence_importance", st)
-    return out[:total]
+    L = lib()
+    buf, nbytes = _workspace(L.pace_llm_sequence_importance_workspace_size, (B, cp, vp, np_, Hq, Hkv, qs), ws, Q.device)
+    _check_ws("pace_llm_sequence_importance",
+              L.pace_llm_sequence_importance(_dev(Q), _dev(K), cp, vp, np_, B, Hq, Hkv, D, float(scale), qs, _dev(out),
+                                             _dev(buf), nbytes, _stream(stream)), ws)
+    return _first(out, total)
 
 
 def pace_ddae_select(s_llm_raw: torch.Tensor, s_vis_raw: torch.Tensor, cu_v, cu_keep,
                      params: Optional[DdaeParams] = None, s_final: Optional[torch.Tensor] = None,
                      weights: Optional[torch.Tensor] = None, kept: Optional[torch.Tensor] = None, stream=None):
     """Returns (s_final [sum Nv], weights [B, 2], kept int32 [sum K])."""
-    v, kp = _i32(cu_v), _i32(cu_keep)
-    B = len(v) - 1
+    (v, vp, B), (kp, kpp, _) = _i32(cu_v), _i32(cu_keep)
+    B -= 1
+    n, k = int(v[-1]), int(kp[-1])
     dev = s_llm_raw.device
     if s_final is None:
-        s_final = torch.empty(max(int(v[-1]), 1), dtype=torch.float32, device=dev)
+        s_final = torch.empty(max(n, 1), dtype=torch.float32, device=dev)
     if weights is None:
         weights = torch.empty((max(B, 1), 2), dtype=torch.float32, device=dev)
     if kept is None:
-        kept = torch.empty(max(int(kp[-1]), 1), dtype=torch.int32, device=dev)
-    st = lib().pace_ddae_select(_dev(s_llm_raw), _dev(s_vis_raw), _pi32(v), _pi32(kp), B,
-                                ctypes.byref(params) if params is not None else None, _dev(s_final),
-                                _dev(weights), _dev(kept), _stream(stream))
-    _check("pace_ddae_select", st)
-    return s_final[: int(v[-1])], weights[:B], kept[: int(kp[-1])]
+        kept = torch.empty(max(k, 1), dtype=torch.int32, device=dev)
+    _check("pace_ddae_select", lib().pace_ddae_select(_dev(s_llm_raw), _dev(s_vis_raw), vp, kpp, B, _params(params),
+                                                      _dev(s_final), _dev(weights), _dev(kept), _stream(stream)))
+    return _first(s_final, n), _first(weights, B), _first(kept, k)
 
 
 def pace_gather(src: torch.Tensor, idx: torch.Tensor, dst: Optional[torch.Tensor] = None, stream=None):
     """dst[r] = src[idx[r]] row by row (byte copy); src is [rows, ...] contiguous."""
     n_src = src.shape[0]
-    row_bytes = src[0].numel() * src.element_size() if n_src else 0
+    row_bytes = src.numel() // n_src * src.element_size() if n_src else 0
     n = idx.numel()
     if dst is None:
         dst = torch.empty((max(n, 1),) + tuple(src.shape[1:]), dtype=src.dtype, device=src.device)
     st = lib().pace_gather(_dev(src), n_src, row_bytes, _dev(idx), n, _dev(dst), _stream(stream))
     _check("pace_gather", st)
-    return dst[:n]
+    return _first(dst, n)
