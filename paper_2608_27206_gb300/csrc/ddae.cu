@@ -592,55 +592,76 @@ __global__ void __launch_bounds__(256) prune_index_kernel(const __grid_constant_
   }
 }
 
-// One launch over several tensors gathered with the same row list (hidden states, KV-cache
-// rows, position ids ...): work item = (tensor, slab, output row), one warp each.
+// One launch over several tensors gathered with the same row list (hidden states, KV-cache rows,
+// position ids ...).  Each tensor's output is one run of 16-, 4- or 1-byte elements in (slab, row,
+// column) order, cut into blocks of kGmBlock elements; a thread takes kGmU of them a block apart,
+// with all its loads in flight, so that rows of any length (7 KB hidden states, 256-byte K and V
+// heads, 4-byte position ids) fill the warps alike.
+constexpr int kGmThreads = 256, kGmU = 4, kGmBlock = kGmThreads * kGmU;
 struct GatherMultiTable {
   pace_gather_tensor g[PACE_GATHER_MAX_TENSORS];
-  int64_t item_prefix[PACE_GATHER_MAX_TENSORS + 1];   // slabs x rows per tensor
-  int width[PACE_GATHER_MAX_TENSORS];                  // copy width in bytes: 16, 4 or 1
+  int64_t block_prefix[PACE_GATHER_MAX_TENSORS + 1];   // blocks of kGmBlock elements
+  int width[PACE_GATHER_MAX_TENSORS];                  // element width in bytes: 16, 4 or 1
   int n;
 };
 
-template <typename V>
-__device__ __forceinline__ void copy_row(const uint8_t* sp, uint8_t* dp, int64_t bytes, int lane) {
-  const V* s = reinterpret_cast<const V*>(sp);
-  V* d = reinterpret_cast<V*>(dp);
-  const int64_t n = bytes / static_cast<int64_t>(sizeof(V));
-  for (int64_t c = lane; c < n; c += 32) d[c] = s[c];
-}
-template <typename V>
-__device__ __forceinline__ void zero_row(uint8_t* dp, int64_t bytes, int lane) {
-  V* d = reinterpret_cast<V*>(dp);
-  const int64_t n = bytes / static_cast<int64_t>(sizeof(V));
-  for (int64_t c = lane; c < n; c += 32) d[c] = V{};
+// INDEX: unsigned when the tensor has fewer than 2^31 elements (a 64-bit division is several times
+// a 32-bit one), else the 64-bit type.
+template <typename V, typename INDEX>
+__device__ __forceinline__ void gather_block(const pace_gather_tensor& g, INDEX first, const int32_t* __restrict__ idx,
+                                             INDEX n_idx, int* status) {
+  const INDEX cols = static_cast<INDEX>(g.row_bytes / static_cast<int64_t>(sizeof(V)));
+  const INDEX total = static_cast<INDEX>(g.n_slabs) * n_idx * cols;
+  INDEX slab[kGmU], row[kGmU], col[kGmU];
+  int32_t src[kGmU];
+  V v[kGmU];
+#pragma unroll
+  for (int u = 0; u < kGmU; ++u) {
+    const INDEX e = first + static_cast<INDEX>(u * kGmThreads + threadIdx.x);
+    const INDEX r = e / cols;
+    col[u] = e - r * cols;
+    slab[u] = r / n_idx;
+    row[u] = r - slab[u] * n_idx;
+    src[u] = e < total ? __ldg(idx + row[u]) : -1;
+  }
+#pragma unroll
+  for (int u = 0; u < kGmU; ++u) {
+    v[u] = V{};
+    if (src[u] >= 0 && src[u] < g.n_src_rows)
+      v[u] = __ldcs(reinterpret_cast<const V*>(static_cast<const uint8_t*>(g.src) + static_cast<int64_t>(slab[u]) * g.src_slab_stride +
+                                               src[u] * g.src_row_stride) + col[u]);
+  }
+#pragma unroll
+  for (int u = 0; u < kGmU; ++u) {
+    if (first + static_cast<INDEX>(u * kGmThreads + threadIdx.x) >= total) continue;
+    if (src[u] < 0 || src[u] >= g.n_src_rows) record_error(status, PACE_ERR_INVALID_ARG, K_GATHER_MULTI);
+    __stcs(reinterpret_cast<V*>(static_cast<uint8_t*>(g.dst) + static_cast<int64_t>(slab[u]) * g.dst_slab_stride +
+                                static_cast<int64_t>(row[u]) * g.dst_row_stride) + col[u],
+           v[u]);
+  }
 }
 
-__global__ void __launch_bounds__(256) gather_multi_kernel(const __grid_constant__ GatherMultiTable t,
-                                                           const int32_t* __restrict__ idx, int64_t n_idx,
-                                                           int* status) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warp0 = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
-  const int64_t total = t.item_prefix[t.n];
-  for (int64_t w = warp0; w < total; w += nwarps) {
+template <typename V>
+__device__ __forceinline__ void gather_block_of(const pace_gather_tensor& g, int64_t block, const int32_t* __restrict__ idx,
+                                                int64_t n_idx, int* status) {
+  const int64_t total = g.n_slabs * n_idx * (g.row_bytes / static_cast<int64_t>(sizeof(V)));
+  if (total < (int64_t{1} << 31))
+    gather_block<V, unsigned>(g, static_cast<unsigned>(block * kGmBlock), idx, static_cast<unsigned>(n_idx), status);
+  else
+    gather_block<V, unsigned long long>(g, static_cast<unsigned long long>(block * kGmBlock), idx,
+                                        static_cast<unsigned long long>(n_idx), status);
+}
+
+__global__ void __launch_bounds__(kGmThreads) gather_multi_kernel(const __grid_constant__ GatherMultiTable t,
+                                                                  const int32_t* __restrict__ idx, int64_t n_idx,
+                                                                  int* status) {
+  for (int64_t w = blockIdx.x; w < t.block_prefix[t.n]; w += gridDim.x) {
     int k = 0;
-    while (k + 1 < t.n && t.item_prefix[k + 1] <= w) ++k;
-    const pace_gather_tensor& g = t.g[k];
-    const int64_t local = w - t.item_prefix[k];
-    const int64_t slab = local / n_idx, r = local - slab * n_idx;
-    const int64_t s = idx[r];
-    uint8_t* dp = static_cast<uint8_t*>(g.dst) + slab * g.dst_slab_stride + r * g.dst_row_stride;
-    if (s < 0 || s >= g.n_src_rows) {
-      if (t.width[k] == 16) zero_row<uint4>(dp, g.row_bytes, lane);
-      else if (t.width[k] == 4) zero_row<uint32_t>(dp, g.row_bytes, lane);
-      else zero_row<uint8_t>(dp, g.row_bytes, lane);
-      if (lane == 0) record_error(status, PACE_ERR_INVALID_ARG, K_GATHER_MULTI);
-      continue;
-    }
-    const uint8_t* sp = static_cast<const uint8_t*>(g.src) + slab * g.src_slab_stride + s * g.src_row_stride;
-    if (t.width[k] == 16) copy_row<uint4>(sp, dp, g.row_bytes, lane);
-    else if (t.width[k] == 4) copy_row<uint32_t>(sp, dp, g.row_bytes, lane);
-    else copy_row<uint8_t>(sp, dp, g.row_bytes, lane);
+    while (k + 1 < t.n && t.block_prefix[k + 1] <= w) ++k;
+    const int64_t block = w - t.block_prefix[k];
+    if (t.width[k] == 16) gather_block_of<uint4>(t.g[k], block, idx, n_idx, status);
+    else if (t.width[k] == 4) gather_block_of<uint32_t>(t.g[k], block, idx, n_idx, status);
+    else gather_block_of<uint8_t>(t.g[k], block, idx, n_idx, status);
   }
 }
 
@@ -789,7 +810,7 @@ extern "C" pace_status_t pace_gather_multi(const pace_gather_tensor* tensors, in
   if (tensors == nullptr || idx == nullptr) return PACE_ERR_INVALID_ARG;
   GatherMultiTable t{};
   t.n = n_tensors;
-  t.item_prefix[0] = 0;
+  t.block_prefix[0] = 0;
   for (int k = 0; k < n_tensors; ++k) {
     const pace_gather_tensor& g = tensors[k];
     if (g.src == nullptr || g.dst == nullptr || g.row_bytes <= 0 || g.n_slabs < 0 || g.n_src_rows < 0 ||
@@ -801,16 +822,13 @@ extern "C" pace_status_t pace_gather_multi(const pace_gather_tensor* tensors, in
                         static_cast<uintptr_t>(g.dst_row_stride) | static_cast<uintptr_t>(g.src_slab_stride) |
                         static_cast<uintptr_t>(g.dst_slab_stride);
     t.width[k] = (a % 16 == 0) ? 16 : (a % 4 == 0) ? 4 : 1;
-    t.item_prefix[k + 1] = t.item_prefix[k] + g.n_slabs * n_idx;
+    t.block_prefix[k + 1] =
+        t.block_prefix[k] + (g.n_slabs * n_idx * (g.row_bytes / t.width[k]) + kGmBlock - 1) / kGmBlock;
   }
-  if (t.item_prefix[n_tensors] == 0) return PACE_OK;
+  if (t.block_prefix[n_tensors] == 0) return PACE_OK;
   PACE_CHECK(check_device());
   int* status = device_status_word();
-  int sms = 152, dev = 0;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  int64_t blocks = (t.item_prefix[n_tensors] + 7) / 8;
-  const int64_t cap = static_cast<int64_t>(sms) * 16;
-  if (blocks > cap) blocks = cap;
-  gather_multi_kernel<<<static_cast<unsigned>(blocks), 256, 0, stream>>>(t, idx, n_idx, status);
+  const unsigned grid = static_cast<unsigned>(std::min<int64_t>(t.block_prefix[n_tensors], 1 << 20));
+  gather_multi_kernel<<<grid, kGmThreads, 0, stream>>>(t, idx, n_idx, status);
   return check_launch();
 }
