@@ -1,23 +1,17 @@
 // Condense: Adaptive Pixel Compressor (Sec. 3.2, Eq. 1-6) and the bicubic resize (App. B.3).
 //
-// Density, three kernels on the caller's stream:
-//   apc_pass1  one CTA per strip of up to 32 patches of one patch row.  The strip's
-//              14 image rows are staged in shared memory with coalesced 2- or 4-byte
-//              loads; each warp reduces |x|^2 of its patches (exact integers) to the
-//              inverse token norm 1/|T_i|; the strip's weighted column sums
-//              sum_i x_ik / (255 |T_i|) (and sum_i 1/|T_i| for the constant coordinate)
-//              are added to a per-image 589-vector as 2^-32 fixed-point integers, so the
-//              reduction is exact and independent of the CTA order.
-//   apc_pass2  same strips: c = sums / N, phi = |c|^2, c_hat = c / |c| (recomputed per
-//              CTA from the 589 integers), then d_i = |t_i - c_hat| computed directly from
-//              the staged pixels (no 2 - 2cos cancellation), counted into the tail's value
-//              buckets (global atomics).
-//   apc_tail_scan  one CTA per 4096 distances of an image: the k_tail-th largest's bucket from
-//              the counts, the distances above it summed (2^-32 fixed point) and the bucket's
-//              members listed; the image's last CTA ranks the members (directly, or by offset
-//              rounds over their fp32 bits) and computes the tail mean, rho_d, rho, r and the
-//              target size.  The token and pixel-statistic densities share it (their pass 2
-//              counts the buckets the same way).
+// Density, four kernels on the caller's stream, each started before the one before it has drained
+// (programmatic dependent launch): apc_zero clears the sums, then
+//   apc_pass1  strips of up to 32 patches of one patch row, their 14 image rows staged in shared
+//              memory: |x|^2 of each patch gives the inverse token norm 1/|T_i|; the weighted column
+//              sums sum_i x_ik / (255 |T_i|) (and sum_i 1/|T_i| for the constant coordinate) are added
+//              to a per-image 589-vector of 64-bit whole numbers, exactly, whatever the order.
+//   apc_pass2  same strips: c = sums / N, phi = |c|^2, c_hat = c / |c| (recomputed per CTA from the
+//              589 integers), then d_i = |t_i - c_hat| from exact dot products (no cancellation),
+//              counted and summed (fixed point) in the tail's value buckets (global atomics).
+//   apc_tail   the k_tail-th largest's bucket from the counts, its members from the distances, the
+//              tail mean, rho_d, rho, r and the target size.  The token and pixel-statistic
+//              densities share it (their pass 2 fills the buckets the same way).
 // Resize: apc_resample, four CTAs per SM walking the 16 x 32 output tiles of the batch; for
 // downscales up to 2.75x per side the input window is staged in shared memory and filtered
 // there with precomputed weights, steeper downscales take a generic path with per-tap weights.
@@ -25,7 +19,10 @@
 #include <atomic>
 #include <cfloat>
 #include <cmath>
+#include <cstddef>
 #include <mutex>
+
+#include <cooperative_groups.h>
 
 #include "pace_common.cuh"
 #include "pace_ptx.cuh"
@@ -34,13 +31,14 @@
 namespace pace {
 namespace {
 
+namespace cg = cooperative_groups;
+
 constexpr int kPatch = 14;
 constexpr int kPatchBytes = kPatch * kPatch * 3;     // 588
 constexpr int kTokDim = kPatchBytes + 1;             // 589: pixels + constant coordinate
 constexpr int kStrip = 32;                           // patches per strip
 constexpr int kStripRowBytes = kStrip * kPatch * 3;  // 1344 bytes of one image row per strip
 constexpr int kApcThreads = 256;
-constexpr int kPairIters = (kPatchBytes / 2 + 31) / 32;   // 10: coordinate pairs per lane
 constexpr int kApcMaxB = 64;
 // Column sums are 2^-32 fixed point in 64-bit integers.  The conversions below use only 32-bit
 // conversions and fp32 (no fp64, which is a slow pipe on this GPU); fix32 rounds exactly like
@@ -75,6 +73,7 @@ struct ApcTable {
   int unit_prefix[kApcMaxB + 1];
   int nb;
   int b_base;               // global index of image 0 of this table
+  int strip_log2[kApcMaxB]; // log2 of the patches per strip of image b
 };
 
 __device__ __forceinline__ int find_image(const ApcTable& t, int unit) {
@@ -126,40 +125,6 @@ __device__ __forceinline__ float warp_sum_f(float v) {
   return v;
 }
 
-// The two bytes of a 16-bit pair as floats: byte permutes build 2^23 + b in each word, one packed
-// subtract removes the 2^23.
-__device__ __forceinline__ float2 bytes2_to_float2(uint32_t v) {
-  const float2 w = make_float2(__uint_as_float(__byte_perm(v, 0x4B000000u, 0x7540)),
-                               __uint_as_float(__byte_perm(v, 0x4B000000u, 0x7541)));
-  return ptx::fadd2(w, make_float2(-8388608.0f, -8388608.0f));
-}
-
-// Shared-memory offset of token coordinates 2j, 2j + 1 of patch 0 in a staged strip (row y of the
-// patch, byte kk within its 42-byte row).
-__device__ __forceinline__ int pair_offset(int j) {
-  const int k = 2 * j, y = k / 42;
-  return y * kStripRowBytes + (k - y * 42);
-}
-
-// Sum of squares of the 42 bytes at s (2-byte aligned): 4-byte words with dp4a, the unaligned
-// ends as 16-bit loads.
-__device__ __forceinline__ uint32_t row_sumsq42(const uint8_t* s) {
-  uint32_t acc = 0u;
-  const int lead = (reinterpret_cast<uintptr_t>(s) & 3u) ? 1 : 0;   // one 16-bit head to reach 4-byte alignment
-  if (lead) {
-    const uint32_t h = *reinterpret_cast<const uint16_t*>(s);
-    acc = __dp4a(h, h, acc);
-  }
-  const uint32_t* w = reinterpret_cast<const uint32_t*>(s + 2 * lead);
-#pragma unroll
-  for (int i = 0; i < 10; ++i) acc = __dp4a(w[i], w[i], acc);
-  if (!lead) {
-    const uint32_t h = *reinterpret_cast<const uint16_t*>(s + 40);
-    acc = __dp4a(h, h, acc);
-  }
-  return acc;
-}
-
 struct Strip {
   int b, u, py, px0, np;
 };
@@ -181,116 +146,360 @@ __device__ __forceinline__ void issue_strip(const uint8_t* __restrict__ img, con
   cp_async_commit();
 }
 
-// Both passes run a grid of resident CTAs over the strips (unit = blockIdx.x, + gridDim.x, ...),
-// loading the next strip asynchronously while the current one is worked on.
-template <bool WIDE>
-__global__ void __launch_bounds__(kApcThreads) apc_pass1(const uint8_t* __restrict__ img,
-                                                         const __grid_constant__ ApcTable t, int units,
-                                                         float* __restrict__ inv_norm,
-                                                         unsigned long long* __restrict__ sums) {
-  __shared__ __align__(16) uint8_t s2[2][kPatch * kStripRowBytes];
-  __shared__ uint32_t ssq[8][kStrip];
-  __shared__ __align__(16) float inv[kStrip];
-  int unit = blockIdx.x;
-  if (unit >= units) return;
-  // weighted column sums: thread slot j (j = tid, tid + 256) owns columns 2j, 2j+1 (a pair never
-  // crosses a 42-byte row); slot 294 owns the constant coordinate.  Each strip's sums are rounded
-  // to 2^-32 fixed point and added exactly; one atomic per column when the image changes.
-  constexpr int kSlots = kPatchBytes / 2 + 1;   // 295
-  unsigned long long acc[2][2] = {{0ull, 0ull}, {0ull, 0ull}};
-  int cur_b = -1;
-  auto flush = [&]() {
-    if (cur_b < 0) return;
-    unsigned long long* sb = sums + static_cast<int64_t>(t.b_base + cur_b) * kTokDim;
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const int j = threadIdx.x + q * kApcThreads;
-      if (j < kPatchBytes / 2) {
-        atomicAdd(sb + 2 * j, acc[q][0]);
-        atomicAdd(sb + 2 * j + 1, acc[q][1]);
-      } else if (j == kPatchBytes / 2) {
-        atomicAdd(sb + kPatchBytes, acc[q][0]);
-      }
-      acc[q][0] = acc[q][1] = 0ull;
+// ------------------------------------------------------------------------------------------------
+// density on raw pixels
+// ------------------------------------------------------------------------------------------------
+// Both passes run one CTA per SM over its share of consecutive strips (so that it meets few images):
+// three groups of 320 threads take the strips of an image in turn, each with its own buffers, the next
+// strip being copied (TMA bulk copies, one per image row) while the current one is worked on.  One CTA
+// per SM, because each ends an image with 589 64-bit atomics, which run at about one in 1.5 ns to a
+// line (four CTAs per SM: 15 us of a 4K image's pass; clusters that add up before the atomics leave
+// SMs idle).  They are bound by instruction issue, not by memory (the image is read once from
+// HBM and once from L2), so both reduce to dot products of bytes that run four to an instruction
+// (dp4a), exactly, in integers:
+//   pass 1  |x|^2 of every patch, and the column sums of x_ik / |T_i|: 1/|T_i| in fp32 is a whole
+//           multiple of 2^-31 (it lies in [2^-5, 1]), so its four bytes are the weights of four dp4a
+//           over four patches at a time and the sums have no rounding at all;
+//   pass 2  the dot products x_i . c_hat with c_hat in 2^-32 fixed point, four dp4a per four
+//           coordinates, and |t_i - c_hat|^2 = |t_i|^2 + |c_hat|^2 - 2 t_i . c_hat in fp64 from those
+//           whole numbers, so that nothing is lost when t_i is close to c_hat.
+// Everything works on the 84 bytes of a patch pair's image row as 21 words: one 4-byte shared load
+// brings four coordinates.  Word 10 holds the last two coordinates of the first patch and the first
+// two of the second; a single last patch has an absent partner with weight 0.  On a 4K image the two
+// passes took 19.9 + 15.8 us with a byte-to-float conversion and a packed fp32 FMA per coordinate.
+constexpr int kDThreads = 320;                       // threads of a group
+constexpr int kDGroups = 3;                          // groups of a CTA
+constexpr int kDAll = kDThreads * kDGroups;
+constexpr int kPairWords = 21;                       // words of a pair's image row
+constexpr int kPairBytes = 4 * kPairWords;
+constexpr int kStageRow = 1472;                      // bytes per staged row: 1344 + 16 slack, = 16 words mod 32
+constexpr int kStageBytes = kPatch * kStageRow;      // so that two rows' pairs take different banks
+constexpr int kWordSlots = kPatch * kPairWords;      // 294: word positions of a pair
+constexpr int kStripLog2 = 5, kMinStripLog2 = 3;     // strips of 32 patches, 16 or 8
+static_assert(kStrip == 1 << kStripLog2, "strip width");
+constexpr int kSumSlots = 4;                         // copies of an image's column sums that the atomics spread over
+constexpr int kGroups = kStrip / 8;                  // groups of four pairs in a full strip
+// A dp4a of pass 1 adds at most 4 * 255^2 and a strip kGroups of them: the 32-bit digit sums are
+// folded into 64 bits before they can overflow.
+constexpr int kFoldStrips = 2048;
+static_assert(static_cast<int64_t>(kFoldStrips) * kGroups * 4 * 255 * 255 < (int64_t{1} << 32), "digit sums");
+// The strips [first, end) of this CTA.
+__device__ __forceinline__ int2 unit_range(int units) {
+  const int each = units / static_cast<int>(gridDim.x), extra = units - each * static_cast<int>(gridDim.x);
+  const int i = static_cast<int>(blockIdx.x), first = i * each + min(i, extra);
+  return make_int2(first, first + each + (i < extra ? 1 : 0));
+}
+
+// Zeroes a call's sums and tail scratch (two ranges of 16-byte words); the first pass of the density
+// starts beside it and waits for it before its first atomic.  A memset in its place is a full stop in
+// the stream: 2.3 us.
+__global__ void __launch_bounds__(256) apc_zero(uint4* __restrict__ a, unsigned na, uint4* __restrict__ b, unsigned nb) {
+  ptx::launch_dependents();
+  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < na + nb; i += gridDim.x * blockDim.x)
+    *(i < na ? a + i : b + (i - na)) = make_uint4(0u, 0u, 0u, 0u);
+}
+
+struct alignas(16) StripRef {
+  int b, py, px0, np;
+  int pairs_log2;   // log2 of the pairs of a full strip
+  uint32_t first;   // byte of the image at which the strip's first row starts (an image is below 2^32 bytes)
+  uint32_t pitch;   // bytes per image row
+};
+__device__ __forceinline__ void strip_place(const ApcTable& t, StripRef& q) {
+  q.np = min(2 << q.pairs_log2, t.gw[q.b] - q.px0);
+  q.first = static_cast<uint32_t>(q.py) * kPatch * q.pitch + static_cast<uint32_t>(q.px0) * (kPatch * 3);
+}
+__device__ __forceinline__ void strip_image(const ApcTable& t, StripRef& q) {
+  q.pairs_log2 = t.strip_log2[q.b] - 1;
+  q.pitch = static_cast<uint32_t>(t.W[q.b]) * 3u;
+}
+__device__ __forceinline__ StripRef strip_ref(const ApcTable& t, int unit) {
+  StripRef q;
+  q.b = find_image(t, unit);
+  const int u = unit - t.unit_prefix[q.b];
+  q.py = u / t.chunks[q.b];
+  strip_image(t, q);
+  q.px0 = (u - q.py * t.chunks[q.b]) << (q.pairs_log2 + 1);
+  strip_place(t, q);
+  return q;
+}
+// The strip n on in the same image.
+__device__ __forceinline__ void strip_advance(const ApcTable& t, StripRef& q, int n) {
+  q.px0 += n << (q.pairs_log2 + 1);
+  while (q.px0 >= t.chunks[q.b] << (q.pairs_log2 + 1)) {
+    q.px0 -= t.chunks[q.b] << (q.pairs_log2 + 1);
+    ++q.py;
+  }
+  strip_place(t, q);
+}
+// Row y of a strip is staged from the 16-byte boundary at or before its first byte: this many bytes on.
+__device__ __forceinline__ uint32_t row_phase(const StripRef& q, int y) {
+  return (q.first + static_cast<uint32_t>(y) * q.pitch) & 15u;
+}
+
+// Called by one whole warp: copies a strip's 14 rows to s (a lane per row), counted on the mbarrier
+// `bar`, and the strip's place to `slot`.  Nothing past the image is read: the last row's last few bytes, which do not fill a 16-byte
+// piece, are stored by the lane itself, before the warp's arrival on the barrier.
+__device__ __forceinline__ void copy_strip(const uint8_t* __restrict__ img, const ApcTable& t, const StripRef& q, uint8_t* s,
+                                           uint32_t bar, StripRef* slot) {
+  const int lane = threadIdx.x & 31;
+  uint32_t bytes = 0u;
+  int64_t a = 0;
+  const uint8_t* base = img + t.off[q.b];
+  if (lane < kPatch) {
+    const uint32_t ph = row_phase(q, lane);
+    a = static_cast<int64_t>(q.first) + static_cast<int64_t>(lane) * q.pitch - ph;
+    bytes = (ph + static_cast<uint32_t>(q.np) * (kPatch * 3) + 15u) & ~15u;
+    const int64_t left = static_cast<int64_t>(t.H[q.b]) * q.pitch - a;
+    if (bytes > left) {
+      bytes = static_cast<uint32_t>(left) & ~15u;
+      for (uint32_t i = bytes; i < left; i += 4u)   // an image holds a multiple of 4 bytes
+        *reinterpret_cast<uint32_t*>(s + lane * kStageRow + i) = __ldg(reinterpret_cast<const uint32_t*>(base + a + i));
+      ptx::fence_proxy_async_shared();
     }
-  };
-  issue_strip<WIDE>(img, t, unit, s2[0]);
-  for (int i = 0; unit < units; ++i, unit += gridDim.x) {
-    const int next = unit + static_cast<int>(gridDim.x);
-    if (next < units) {
-      issue_strip<WIDE>(img, t, next, s2[(i + 1) & 1]);
-      cp_async_wait_group<1>();
+  }
+  const uint32_t total = __reduce_add_sync(0xffffffffu, bytes);
+  __syncwarp();
+  if (lane == 0) {
+    *slot = q;
+    ptx::mbar_arrive_expect_tx(bar, total);
+  }
+  __syncwarp();
+  if (bytes > 0u) ptx::bulk_load(ptx::smem_u32(s + lane * kStageRow), base + a, bytes, bar);
+}
+
+// The words of a pair's row that starts at byte `a` of shared memory.  ALIGNED: a is a multiple of
+// 4 (every image an even number of patches wide); otherwise a is even and each word is put together
+// from two aligned ones.
+template <bool ALIGNED>
+struct RowWords {
+  const uint32_t* w;
+  uint32_t cur, sh;
+  __device__ __forceinline__ explicit RowWords(const uint8_t* a) {
+    if (ALIGNED) {
+      w = reinterpret_cast<const uint32_t*>(a);
     } else {
-      cp_async_wait_group<0>();
+      sh = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(a) & 2u) * 8u;
+      w = reinterpret_cast<const uint32_t*>(a - (sh >> 3));
+      cur = w[0];
     }
-    __syncthreads();
-    const uint8_t* s = s2[i & 1];
-    const Strip q = strip_of(t, unit);
-    if (q.b != cur_b) {
-      flush();
-      cur_b = q.b;
+  }
+  __device__ __forceinline__ uint32_t get(int j) {   // j = 0, 1, 2, .. in order
+    if (ALIGNED) return w[j];
+    const uint32_t nxt = w[j + 1];
+    const uint32_t v = __funnelshift_r(cur, nxt, sh);
+    cur = nxt;
+    return v;
+  }
+};
+// One word at byte `a` (4-byte aligned if ALIGNED, else 2-byte: sh = 8 (a mod 4)).
+template <bool ALIGNED>
+__device__ __forceinline__ uint32_t word_at(const uint8_t* a, uint32_t sh) {
+  if (ALIGNED) return *reinterpret_cast<const uint32_t*>(a);
+  const uint32_t* w = reinterpret_cast<const uint32_t*>(a - (sh >> 3));
+  return __funnelshift_r(w[0], w[1], sh);
+}
+
+// 1/|T_i| of a patch from its |x|^2.
+__device__ __forceinline__ float inv_norm_of(uint32_t ss) {
+  return 1.0f / sqrtf(static_cast<float>(ss) * (1.0f / 65025.0f) + 1.0f);
+}
+
+// A group's strips of one image (first, first + STEP, .. below end), which one of its warps copies into
+// its two buffers.  `used` counts the strips that the group has worked on, i.e. the uses of its buffers.
+template <int STEP>
+struct StripPipe {
+  uint8_t (*s2)[kStageBytes];
+  uint64_t* bars;
+  StripRef* ref;
+  unsigned used;
+  __device__ __forceinline__ void copy(const uint8_t* img, const ApcTable& t, const StripRef& q, unsigned use) {
+    copy_strip(img, t, q, s2[use & 1], ptx::smem_u32(&bars[use & 1]), &ref[use & 1]);
+  }
+  // the image's first two strips (called by the copying warp of a group that is done with its buffers)
+  __device__ __forceinline__ void begin(const uint8_t* img, const ApcTable& t, int first, int end) {
+    if (first >= end) return;
+    StripRef q = strip_ref(t, first);
+    copy(img, t, q, used);
+    if (first + STEP < end) {
+      strip_advance(t, q, STEP);
+      copy(img, t, q, used + 1);
     }
-    // |x|^2 of every patch: thread (p = tid % 32, rows yg and yg + 8)
-    {
-      const int p = threadIdx.x & 31, yg = threadIdx.x >> 5;
-      uint32_t a = 0u;
-      if (p < q.np) {
-        a = row_sumsq42(s + yg * kStripRowBytes + p * 42);
-        if (yg + 8 < kPatch) a += row_sumsq42(s + (yg + 8) * kStripRowBytes + p * 42);
-      }
-      ssq[yg][p] = a;
-    }
-    __syncthreads();
-    if (threadIdx.x < q.np) {
-      const int p = threadIdx.x;
-      uint32_t ss = 0u;
+  }
+  __device__ __forceinline__ bool wait() { return ptx::mbar_wait(ptx::smem_u32(&bars[used & 1]), (used >> 1) & 1u, kWaitLimitNs); }
+  __device__ __forceinline__ const uint8_t* data() const { return s2[used & 1]; }
+  __device__ __forceinline__ const StripRef& place() const { return ref[used & 1]; }
+  // the strip after `cur`, once the group is done with the strip before it (called by the copying warp)
+  __device__ __forceinline__ void next(const uint8_t* img, const ApcTable& t, const StripRef& cur) {
+    StripRef q = cur;
+    strip_advance(t, q, STEP);
+    copy(img, t, q, used + 1);
+  }
+};
+
+struct Pass1Group {
+  uint8_t s2[2][kStageBytes];
+  uint32_t ssq[kPatch][kStrip];
+  // the four bytes of the weights 2^31 / |T_i|: [group of four pairs][first or second patch][byte]
+  uint8_t wdig[kGroups][2][4][4];
+  unsigned long long col[kTokDim + 1];
+  uint64_t bars[2];
+  StripRef ref[2];
+};
+static_assert(kStageBytes % 16 == 0 && offsetof(Pass1Group, wdig) % 16 == 0 && sizeof(Pass1Group) % 16 == 0, "shared layout");
+
+template <bool ALIGNED>
+__global__ void __launch_bounds__(kDAll, 1) apc_pass1(const uint8_t* __restrict__ img, const __grid_constant__ ApcTable t,
+                                                      int units, uint32_t* __restrict__ sumsq,
+                                                      unsigned long long* __restrict__ sums, int* status) {
+  extern __shared__ __align__(16) unsigned char d_smem[];
+  ptx::launch_dependents();
+  const int tid = threadIdx.x, grp = threadIdx.y, warp = tid >> 5;   // thread and warp of the group
+  Pass1Group* all = reinterpret_cast<Pass1Group*>(d_smem);
+  Pass1Group& sh = all[grp];
+  auto group_sync = [&]() { ptx::named_barrier_sync(1 + grp, kDThreads); };
+  const int2 range = unit_range(units);
+  constexpr int kCopyWarp = kDThreads / 32 - 1;
+  if (tid == 0) {
+    ptx::mbar_init(ptx::smem_u32(&sh.bars[0]), 1);
+    ptx::mbar_init(ptx::smem_u32(&sh.bars[1]), 1);
+    ptx::fence_mbar_init();
+  }
+  group_sync();
+  StripPipe<kDGroups> pipe{sh.s2, sh.bars, sh.ref, 0u};
+  // thread j < 294 owns the four columns of word position j (row j / 21): their digit sums; lane 0 of
+  // warp 0 the constant coordinate
+  uint32_t acc[4][4] = {};
+  unsigned long long one = 0ull;
+  const int wy = tid / kPairWords, wj = tid - wy * kPairWords;
+  int strips = 0;   // in the digit sums
+  // moves the digit sums to (or adds them to) the group's 64-bit column sums (a column has two owners:
+  // the first and the second patch of a pair)
+  auto fold = [&](bool add) {
+    auto put = [&](bool second) {
+      if (tid < kWordSlots) {
 #pragma unroll
-      for (int g = 0; g < 8; ++g) ss += ssq[g][p];
-      const float n2 = static_cast<float>(ss) * (1.0f / 65025.0f) + 1.0f;
-      const float iv = 1.0f / sqrtf(n2);
-      inv[p] = iv;
-      inv_norm[t.patch0[q.b] + q.py * t.gw[q.b] + q.px0 + p] = iv;
-    }
-    __syncthreads();
-    float ivr[kStrip];   // full strips: the 32 inverse norms in registers, the patch loop unrolled
-    if (q.np == kStrip) {
-#pragma unroll
-      for (int p = 0; p < kStrip; p += 4) {
-        const float4 v4 = *reinterpret_cast<const float4*>(inv + p);
-        ivr[p] = v4.x;
-        ivr[p + 1] = v4.y;
-        ivr[p + 2] = v4.z;
-        ivr[p + 3] = v4.w;
-      }
-    }
-#pragma unroll
-    for (int qs = 0; qs < 2; ++qs) {
-      const int j = threadIdx.x + qs * kApcThreads;
-      if (j < kPatchBytes / 2) {
-        const uint16_t* col = reinterpret_cast<const uint16_t*>(s + pair_offset(j));
-        float2 a = make_float2(0.f, 0.f);
-        if (q.np == kStrip) {
-#pragma unroll
-          for (int p = 0; p < kStrip; ++p)
-            a = ptx::ffma2(make_float2(ivr[p], ivr[p]), bytes2_to_float2(col[p * 21]), a);
-        } else {
-          for (int p = 0; p < q.np; ++p) {
-            const float iv = inv[p];
-            a = ptx::ffma2(make_float2(iv, iv), bytes2_to_float2(col[p * 21]), a);
+        for (int q = 0; q < 4; ++q) {
+          const int c = 4 * wj + q;   // byte of the pair's row
+          const unsigned long long v = acc[q][0] + (static_cast<unsigned long long>(acc[q][1]) << 8) +
+                                       (static_cast<unsigned long long>(acc[q][2]) << 16) +
+                                       (static_cast<unsigned long long>(acc[q][3]) << 24);
+          if ((c >= 42) == second) {
+            unsigned long long* p = &sh.col[wy * 42 + (second ? c - 42 : c)];
+            *p = (second || add ? *p : 0ull) + v;
           }
         }
-        acc[qs][0] += fix32(a.x * (1.0f / 255.0f));
-        acc[qs][1] += fix32(a.y * (1.0f / 255.0f));
-      } else if (j == kPatchBytes / 2) {
-        float a = 0.f;
-        for (int p = 0; p < q.np; ++p) a += inv[p];
-        acc[qs][0] += fix32(a);
+      }
+      if (tid == 0 && !second) sh.col[kPatchBytes] = (add ? sh.col[kPatchBytes] : 0ull) + one;
+    };
+    put(false);
+    group_sync();
+    put(true);
+    group_sync();
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int d = 0; d < 4; ++d) acc[q][d] = 0u;
+    one = 0ull;
+    strips = 0;
+  };
+  int first = range.x;
+  for (int b = first < range.y ? find_image(t, first) : 0; first < range.y; ++b) {   // the CTA's strips of image b
+    const int end = min(range.y, t.unit_prefix[b + 1]);
+    if (warp == kCopyWarp) pipe.begin(img, t, first + grp, end);
+    bool folded = false;
+    for (int unit = first + grp; unit < end; unit += kDGroups, ++pipe.used) {
+      if (!pipe.wait()) record_error(status, PACE_ERR_TIMEOUT, K_APC_PASS1);
+      const StripRef cur = pipe.place();
+      const uint8_t* s = pipe.data();
+      if (strips == kFoldStrips) {
+        fold(folded);
+        folded = true;
+      }
+      ++strips;
+      const int npair = (cur.np + 1) >> 1;
+      const int iy = tid >> cur.pairs_log2, ip = tid & ((1 << cur.pairs_log2) - 1);
+      if (iy < kPatch && ip < npair) {   // |x|^2 of one image row of a pair
+        RowWords<ALIGNED> w(s + iy * kStageRow + row_phase(cur, iy) + ip * kPairBytes);
+        uint32_t p = 0u, q = 0u;
+#pragma unroll
+        for (int j = 0; j < kPairWords; ++j) {
+          const uint32_t v = w.get(j);
+          if (j < 10) p = __dp4a(v, v, p);
+          else if (j > 10) q = __dp4a(v, v, q);
+          else {
+            p = __dp4a(v & 0xFFFFu, v, p);
+            q = __dp4a(v & 0xFFFF0000u, v, q);
+          }
+        }
+        *reinterpret_cast<uint2*>(&sh.ssq[iy][2 * ip]) = make_uint2(p, q);
+      }
+      group_sync();   // (the group is also done with its other buffer)
+      // (the image's first two strips were requested at its start)
+      if (warp == kCopyWarp && unit >= first + kDGroups && unit + kDGroups < end) pipe.next(img, t, cur);
+      if (warp == 0) {   // lane p: patch p of the strip
+        uint32_t weight = 0u;
+        if (tid < cur.np) {
+          uint32_t ss = 0u;
+#pragma unroll
+          for (int y = 0; y < kPatch; ++y) ss += sh.ssq[y][tid];
+          sumsq[t.patch0[b] + cur.py * t.gw[b] + cur.px0 + tid] = ss;
+          weight = __float2uint_rn(inv_norm_of(ss) * 2147483648.0f);   // exact
+        }
+#pragma unroll
+        for (int d = 0; d < 4; ++d) sh.wdig[tid >> 3][tid & 1][d][(tid >> 1) & 3] = static_cast<uint8_t>(weight >> (8 * d));
+        const uint32_t lo = __reduce_add_sync(0xffffffffu, weight & 0xFFFFu), hi = __reduce_add_sync(0xffffffffu, weight >> 16);
+        if (tid == 0) one += lo + (static_cast<unsigned long long>(hi) << 16);
+      }
+      group_sync();
+      if (tid < kWordSlots) {
+        const uint32_t off = row_phase(cur, wy) + 4u * wj;
+        const uint8_t* wp = s + wy * kStageRow + off;
+        const uint32_t shf = (off & 2u) * 8u;
+        const uint4* wl = reinterpret_cast<const uint4*>(sh.wdig) + (wj <= 10 ? 0 : 1);   // patch of the word's first two bytes
+        const uint4* wh = reinterpret_cast<const uint4*>(sh.wdig) + (wj < 10 ? 0 : 1);    // and of its last two
+        auto take = [&](int g) {   // four pairs: their bytes column by column, against the weights' digits
+          uint32_t w[4];
+#pragma unroll
+          for (int r = 0; r < 4; ++r) w[r] = word_at<ALIGNED>(wp + (4 * g + r) * kPairBytes, shf);
+          const uint32_t a0 = __byte_perm(w[0], w[1], 0x5140), a1 = __byte_perm(w[0], w[1], 0x7362);
+          const uint32_t b0 = __byte_perm(w[2], w[3], 0x5140), b1 = __byte_perm(w[2], w[3], 0x7362);
+          const uint32_t c[4] = {__byte_perm(a0, b0, 0x5410), __byte_perm(a0, b0, 0x7632), __byte_perm(a1, b1, 0x5410),
+                                 __byte_perm(a1, b1, 0x7632)};
+          const uint4 l = wl[2 * g], h = wh[2 * g];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const uint4 d = k < 2 ? l : h;
+            acc[k][0] = __dp4a(c[k], d.x, acc[k][0]);
+            acc[k][1] = __dp4a(c[k], d.y, acc[k][1]);
+            acc[k][2] = __dp4a(c[k], d.z, acc[k][2]);
+            acc[k][3] = __dp4a(c[k], d.w, acc[k][3]);
+          }
+        };
+        if (npair > 4 * (kGroups - 1)) {
+#pragma unroll
+          for (int g = 0; g < kGroups; ++g) take(g);
+        } else {
+          for (int g = 0; 4 * g < npair; ++g) take(g);
+        }
       }
     }
-    __syncthreads();   // this buffer is refilled two strips on
+    // the image's sums: the groups' added up, one atomic per column
+    fold(folded);
+    ptx::grid_dependency_wait();   // the zeroed sums
+    __syncthreads();
+    const int k = grp * kDThreads + tid;
+    if (k < kTokDim) {
+      unsigned long long x = 0ull;
+#pragma unroll
+      for (int g = 0; g < kDGroups; ++g) x += all[g].col[k];
+      atomicAdd(sums + (static_cast<int64_t>(t.b_base + b) * kSumSlots + blockIdx.x % kSumSlots) * kTokDim + k, x);
+    }
+    first = end;
+    if (first < range.y) __syncthreads();   // the column sums are rewritten
   }
-  flush();
-  static_assert(kSlots <= 2 * kApcThreads, "column slots");
+  static_assert(kWordSlots <= kDThreads - 32 + 6 && kPatch * (kStrip / 2) <= kDThreads && kStrip == 32 && kTokDim <= kDAll,
+                "thread roles");
 }
 
 struct TailParams {
@@ -309,114 +518,166 @@ __device__ __forceinline__ int tail_bucket(float v) {
   return __float_as_int(__fadd_rz(x, 8388608.0f)) - 0x4B000000;
 }
 
-// Scratch of the density tail over several CTAs per image (apc_tail_scan): the counts of the
-// distances per bucket (pass 2 adds them), then the sum and count of the distances above the
-// k-th largest's bucket, the members of that bucket, and how many of the image's CTAs are done.
-constexpr int kTailChunk = 4096;   // distances per CTA of apc_tail_scan
-constexpr int kTailList = 4096;    // members of the selected bucket kept for the last CTA's rank
+// Scratch of the density tail, filled by pass 2 with atomics (exact, so in any order): the count
+// and the 2^-32 fixed-point sum of the distances of each bucket.
 struct TailWork {
-  unsigned long long above_fix;    // distances above the bucket, 2^-32 fixed point
-  unsigned above_cnt;
-  unsigned list_n;
-  unsigned done;
-  unsigned pad;
+  unsigned long long sum[kTailBins];
   unsigned hist[kTailBins];
-  unsigned list[kTailList];
 };
+__device__ __forceinline__ void tail_count(TailWork* w, float d) {
+  const int b = tail_bucket(d);
+  atomicAdd(&w->hist[b], 1u);
+  atomicAdd(&w->sum[b], fix32(d));
+}
 
-template <bool WIDE>
-__global__ void __launch_bounds__(kApcThreads, 4) apc_pass2(const uint8_t* __restrict__ img,
-                                                         const __grid_constant__ ApcTable t, int units,
-                                                         const float* __restrict__ inv_norm,
-                                                         const unsigned long long* __restrict__ sums,
-                                                         float* __restrict__ d_out,
-                                                         pace_apc_stats* __restrict__ stats,
-                                                         TailWork* __restrict__ work) {
-  __shared__ __align__(16) uint8_t s2[2][kPatch * kStripRowBytes];
-  __shared__ __align__(8) float chat[kTokDim + 3];
-  __shared__ float red[kApcThreads / 32];
-  int unit = blockIdx.x;
-  if (unit >= units) return;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int off[kPairIters];   // this lane's coordinate pairs j = lane + 32 it
+struct Pass2Group {
+  uint8_t s2[2][kStageBytes];
+  unsigned long long part[2][kPatch][kStrip];   // x . c_hat of one image row of a patch
+  uint64_t bars[2];
+  StripRef ref[2];
+};
+struct Pass2Smem {
+  Pass2Group g[kDGroups];
+  // the four bytes of c_hat (2^-32 fixed point) of a pair's words, the two patches one after the
+  // other: [image row][word][byte][coordinate of the word]
+  uint8_t cdig[kPatch][kPairWords][4][4];
+  float craw[kTokDim + 3];
+  float red[kDAll / 32];
+  unsigned long long redq[kDAll / 32];
+};
+static_assert(sizeof(Pass2Group) % 16 == 0 && offsetof(Pass2Smem, cdig) % 16 == 0, "shared layout");
+
+template <bool ALIGNED>
+__global__ void __launch_bounds__(kDAll, 1) apc_pass2(const uint8_t* __restrict__ img, const __grid_constant__ ApcTable t,
+                                                      int units, const uint32_t* __restrict__ sumsq,
+                                                      const unsigned long long* __restrict__ sums, float* __restrict__ d_out,
+                                                      pace_apc_stats* __restrict__ stats, TailWork* __restrict__ work,
+                                                      int* status) {
+  extern __shared__ __align__(16) unsigned char d_smem[];
+  Pass2Smem& sh = *reinterpret_cast<Pass2Smem*>(d_smem);
+  ptx::launch_dependents();
+  const int tid = threadIdx.x, grp = threadIdx.y, warp = tid >> 5, lane = tid & 31;   // thread and warp of the group
+  const int ct = grp * kDThreads + tid;                                               // thread of the CTA
+  Pass2Group& my = sh.g[grp];
+  auto group_sync = [&]() { ptx::named_barrier_sync(1 + grp, kDThreads); };
+  constexpr int kCopyWarp = kDThreads / 32 - 1;
+  const int2 range = unit_range(units);
+  if (tid == 0) {
+    ptx::mbar_init(ptx::smem_u32(&my.bars[0]), 1);
+    ptx::mbar_init(ptx::smem_u32(&my.bars[1]), 1);
+    ptx::fence_mbar_init();
+  }
+  group_sync();
+  StripPipe<kDGroups> pipe{my.s2, my.bars, my.ref, 0u};
+  int first = range.x;
+  for (int b = first < range.y ? find_image(t, first) : 0; first < range.y; ++b) {   // the CTA's strips of image b
+    const int end = min(range.y, t.unit_prefix[b + 1]);
+    if (warp == kCopyWarp) pipe.begin(img, t, first + grp, end);   // (the image does not depend on pass 1)
+    ptx::grid_dependency_wait();
+    // c = sums / N, |c|^2 (fixed summation order), c_hat = c / |c|
+    const int N = t.n[b];
+    const float inv_n = 1.0f / static_cast<float>(N);
+    const unsigned long long* sb = sums + static_cast<int64_t>(t.b_base + b) * (kSumSlots * kTokDim);
+    float c = 0.f;
+    if (ct < kTokDim) {   // a thread per coordinate
+      unsigned long long x = 0ull;
 #pragma unroll
-  for (int it = 0; it < kPairIters; ++it) off[it] = pair_offset(min(lane + 32 * it, kPatchBytes / 2 - 1));
-  int cur_b = -1;
-  bool reload = false;
-  float2 chr[kPairIters];   // c_hat of this lane's coordinate pairs, in registers
-  unsigned* hist = nullptr; // the current image's tail bucket counts
-  issue_strip<WIDE>(img, t, unit, s2[0]);
-  for (int i = 0; unit < units; ++i, unit += gridDim.x) {
-    const int next = unit + static_cast<int>(gridDim.x);
-    const Strip q = strip_of(t, unit);
-    if (q.b != cur_b) {   // c = sums / N, |c|^2 (fixed summation order), c_hat = c / |c|
-      cur_b = q.b;
-      reload = true;
-      hist = work[t.b_base + q.b].hist;
-      const int N = (t.H[q.b] / kPatch) * t.gw[q.b];
-      const float inv_n = 1.0f / static_cast<float>(N);
-      const unsigned long long* sb = sums + static_cast<int64_t>(t.b_base + q.b) * kTokDim;
-      float part = 0.f;
-      for (int k = threadIdx.x; k < kTokDim; k += kApcThreads) {
-        const float c = unfix32<false>(sb[k], inv_n);
-        chat[k] = c;
-        part = fmaf(c, c, part);
-      }
-      part = warp_sum_f(part);
-      if (lane == 0) red[warp] = part;
-      __syncthreads();
-      float phi = 0.f;
-#pragma unroll
-      for (int w = 0; w < kApcThreads / 32; ++w) phi += red[w];
-      const float inv_c = 1.0f / sqrtf(phi);
-      __syncthreads();
-      for (int k = threadIdx.x; k < kTokDim; k += kApcThreads) chat[k] *= inv_c;
-      if (q.u == 0 && threadIdx.x == 0) {
-        stats[t.b_base + q.b].phi = phi;
-        stats[t.b_base + q.b].rho_g = 1.0f - phi;
-        stats[t.b_base + q.b].n_patches = N;
-        stats[t.b_base + q.b].k_tail = t.ktail[q.b];
-      }
+      for (int r = 0; r < kSumSlots; ++r) x += __ldcg(sb + r * kTokDim + ct);
+      // sums are multiples of 2^-31 (and, but for the constant coordinate, of 1/255)
+      c = unfix32<false>(x, inv_n) * (ct < kPatchBytes ? 2.0f / 255.0f : 2.0f);
+      if (ct == kPatchBytes) sh.craw[0] = c;
     }
-    if (next < units) {
-      issue_strip<WIDE>(img, t, next, s2[(i + 1) & 1]);
-      cp_async_wait_group<1>();
-    } else {
-      cp_async_wait_group<0>();
-    }
+    const float p2 = warp_sum_f(c * c);
+    if (lane == 0) sh.red[ct >> 5] = p2;
     __syncthreads();
-    const uint8_t* s = s2[i & 1];
-    // d_i = |t_i - c_hat| computed directly: warp per patch, lanes over column pairs
-    const float* pinv = inv_norm + t.patch0[q.b] + q.py * t.gw[q.b] + q.px0;
-    const float2* chat2 = reinterpret_cast<const float2*>(chat);
-    if (reload) {
+    float phi = 0.f;
 #pragma unroll
-      for (int it = 0; it < kPairIters; ++it) chr[it] = chat2[min(lane + 32 * it, kPatchBytes / 2 - 1)];
-      reload = false;
+    for (int w = 0; w < (kTokDim + 31) / 32; ++w) phi += sh.red[w];
+    const float inv_c = 1.0f / sqrtf(phi);
+    unsigned long long sq = 0ull;   // square, 2^-56 fixed point
+    if (ct < kPatchBytes) {
+      const int y = ct / 42, x = ct - y * 42;
+      const uint32_t v = __float2uint_rn(fminf(c * inv_c, 0.99999994f) * 4294967296.0f);
+      sq = static_cast<unsigned long long>(v) * v >> 8;
+#pragma unroll
+      for (int d = 0; d < 4; ++d) {
+        const uint8_t byte = static_cast<uint8_t>(v >> (8 * d));
+        sh.cdig[y][x >> 2][d][x & 3] = byte;
+        sh.cdig[y][(x + 42) >> 2][d][(x + 42) & 3] = byte;
+      }
     }
-    for (int p = warp; p < q.np; p += kApcThreads / 32) {
-      const float sc = pinv[p] * (1.0f / 255.0f);
-      const float2 sc2 = make_float2(sc, sc);
-      float2 acc2 = make_float2(0.f, 0.f);
 #pragma unroll
-      for (int it = 0; it < kPairIters; ++it) {   // lanes over the 294 coordinate pairs
-        const int j = lane + 32 * it;
-        if (it < kPairIters - 1 || j < kPatchBytes / 2) {
-          const uint32_t v = *reinterpret_cast<const uint16_t*>(s + off[it] + p * 42);
-          const float2 e = ptx::ffma2(bytes2_to_float2(v), sc2, make_float2(-chr[it].x, -chr[it].y));
-          acc2 = ptx::ffma2(e, e, acc2);
+    for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+    if (lane == 0) sh.redq[ct >> 5] = sq;
+    __syncthreads();
+    double cc = 0.0, c1 = 0.0;   // a group's warp 0: |c_hat|^2 and the constant coordinate of c_hat
+    if (warp == 0) {             // (fp64 is slow on this GPU: one warp's worth per group and strip)
+      sq = 0ull;
+#pragma unroll
+      for (int w = 0; w < (kPatchBytes + 31) / 32; ++w) sq += sh.redq[w];
+      c1 = static_cast<double>(sh.craw[0] * inv_c);
+      cc = fma(static_cast<double>(sq), 0x1p-56, c1 * c1);
+    }
+    if (first == t.unit_prefix[b] && ct == 0) {
+      stats[t.b_base + b].phi = phi;
+      stats[t.b_base + b].rho_g = 1.0f - phi;
+      stats[t.b_base + b].n_patches = N;
+      stats[t.b_base + b].k_tail = t.ktail[b];
+    }
+    for (int unit = first + grp; unit < end; unit += kDGroups, ++pipe.used) {
+      if (!pipe.wait()) record_error(status, PACE_ERR_TIMEOUT, K_APC_PASS2);
+      const StripRef cur = pipe.place();
+      const uint8_t* s = pipe.data();
+      auto& part = my.part[pipe.used & 1];
+      const int p0 = t.patch0[b] + cur.py * t.gw[b] + cur.px0;   // the strip's first patch
+      const int npair = (cur.np + 1) >> 1;
+      const int iy = tid >> cur.pairs_log2, ip = tid & ((1 << cur.pairs_log2) - 1);   // this thread's (row, pair)
+      uint32_t ss = 0u;
+      if (warp == 0 && lane < cur.np) ss = __ldcg(sumsq + p0 + lane);
+      // x . c_hat over one image row of a pair
+      if (iy < kPatch && ip < npair) {
+        RowWords<ALIGNED> w(s + iy * kStageRow + row_phase(cur, iy) + ip * kPairBytes);
+        const uint4* cd = reinterpret_cast<const uint4*>(sh.cdig[iy]);
+        uint32_t p[4] = {}, q[4] = {};
+        auto dot = [](uint32_t v, const uint4& d, uint32_t (&x)[4]) {
+          x[0] = __dp4a(v, d.x, x[0]);
+          x[1] = __dp4a(v, d.y, x[1]);
+          x[2] = __dp4a(v, d.z, x[2]);
+          x[3] = __dp4a(v, d.w, x[3]);
+        };
+#pragma unroll
+        for (int j = 0; j < kPairWords; ++j) {
+          const uint32_t v = w.get(j);
+          const uint4 d = cd[j];
+          if (j < 10) dot(v, d, p);
+          else if (j > 10) dot(v, d, q);
+          else {
+            dot(v & 0xFFFFu, d, p);
+            dot(v & 0xFFFF0000u, d, q);
+          }
         }
+        auto join = [](const uint32_t (&x)[4]) {
+          return x[0] + (static_cast<unsigned long long>(x[1]) << 8) + (static_cast<unsigned long long>(x[2]) << 16) +
+                 (static_cast<unsigned long long>(x[3]) << 24);
+        };
+        *reinterpret_cast<ulonglong2*>(&part[iy][2 * ip]) = make_ulonglong2(join(p), join(q));
       }
-      const float iv = pinv[p];
-      float acc = warp_sum_f(acc2.x + acc2.y);
-      if (lane == 0) {
-        const float v = iv - chat[kPatchBytes];
-        const float dv = sqrtf(fmaf(v, v, acc));
-        d_out[t.patch0[q.b] + q.py * t.gw[q.b] + q.px0 + p] = dv;
-        atomicAdd(hist + tail_bucket(dv), 1u);   // the tail's bucket counts
+      group_sync();   // (the group is also done with its other buffer)
+      if (warp == kCopyWarp && unit >= first + kDGroups && unit + kDGroups < end) pipe.next(img, t, cur);
+      if (warp == 0 && lane < cur.np) {
+        unsigned long long x = 0ull;
+#pragma unroll
+        for (int y = 0; y < kPatch; ++y) x += part[y][lane];
+        const double iv = static_cast<double>(inv_norm_of(ss));
+        const double dot = iv * fma(static_cast<double>(x), 0x1p-32 / 255.0, c1);                  // t . c_hat
+        const double tt = iv * iv * fma(static_cast<double>(ss), 1.0 / 65025.0, 1.0);              // |t|^2
+        const float dv = sqrtf(fmaxf(static_cast<float>(tt + cc - 2.0 * dot), 0.f));
+        d_out[p0 + lane] = dv;
+        tail_count(work + t.b_base + b, dv);
       }
     }
-    __syncthreads();   // this buffer is refilled two strips on; chat may be rewritten
+    first = end;
+    if (first < range.y) __syncthreads();   // c_hat is rewritten, and every group is done with its buffers
   }
 }
 
@@ -610,26 +871,23 @@ __global__ void __launch_bounds__(kApcThreads) apc_tok_pass2(const uint32_t* __r
     if (lane == 0) {
       const float dv = sqrtf(acc);
       d_out[t.tok0[b] + c0 + p] = dv;
-      atomicAdd(&work[t.b_base + b].hist[tail_bucket(dv)], 1u);   // the tail's bucket counts
+      tail_count(work + t.b_base + b, dv);
     }
   }
 }
 
-// Called by all 1024 threads: the bin holding the r-th largest entry, counting from bin NBINS - 1
-// down (1 <= r <= total): sel[0] = that bin, sel[1] = entries in the bins above it.  wsum: 32 words.
-template <int NBINS>
-__device__ __forceinline__ void select_from_top(const unsigned* bins, unsigned r, unsigned* sel, unsigned* wsum) {
-  constexpr int PER = NBINS / 1024;   // bins per thread
-  static_assert(PER >= 1 && PER * 1024 == NBINS, "bins");
+// Called by all 1024 threads, thread t holding the counts of bins top .. top - PER + 1 (top =
+// PER * 1024 - 1 - PER * t): the bin holding the r-th largest entry, counting from the last bin down
+// (1 <= r <= total): sel[0] = that bin, sel[1] = entries in the bins above it, *count = entries in it.
+// wsum: 32 words.
+template <int PER>
+__device__ __forceinline__ void select_from_counts(const unsigned (&c)[PER], int top, unsigned r, unsigned* sel,
+                                                   unsigned* wsum, unsigned* count) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int top = NBINS - 1 - PER * static_cast<int>(threadIdx.x);   // this thread: bins top .. top - PER + 1
-  unsigned c4[PER], s4 = 0u;
+  unsigned own = 0u;
 #pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    c4[q] = bins[top - q];
-    s4 += c4[q];
-  }
-  unsigned incl = s4;
+  for (int q = 0; q < PER; ++q) own += c[q];
+  unsigned incl = own;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const unsigned n = __shfl_up_sync(0xffffffffu, incl, o);
@@ -637,31 +895,39 @@ __device__ __forceinline__ void select_from_top(const unsigned* bins, unsigned r
   }
   if (lane == 31) wsum[warp] = incl;
   __syncthreads();
-  if (warp == 0) {
-    unsigned w = wsum[lane];
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned n = __shfl_up_sync(0xffffffffu, w, o);
-      if (lane >= o) w += n;
-    }
-    wsum[lane] = w;   // entries in warps 0 .. lane
-  }
-  __syncthreads();
-  incl += warp > 0 ? wsum[warp - 1] : 0u;
-  const unsigned excl = incl - s4;
+  incl += __reduce_add_sync(0xffffffffu, lane < warp ? wsum[lane] : 0u);   // entries in the warps before
+  const unsigned excl = incl - own;
   if (excl < r && incl >= r) {   // exactly one thread
     unsigned above = excl;
     int q = 0;
 #pragma unroll
     for (int qq = 0; qq < PER - 1; ++qq)
-      if (q == qq && above + c4[qq] < r) {
-        above += c4[qq];
+      if (q == qq && above + c[qq] < r) {
+        above += c[qq];
         q = qq + 1;
       }
+    unsigned n = c[0];
+#pragma unroll
+    for (int qq = 1; qq < PER; ++qq)
+      if (q == qq) n = c[qq];
     sel[0] = static_cast<unsigned>(top - q);
     sel[1] = above;
+    *count = n;
   }
   __syncthreads();
+}
+
+// The same for NBINS counts in shared memory.
+template <int NBINS>
+__device__ __forceinline__ void select_from_top(const unsigned* bins, unsigned r, unsigned* sel, unsigned* wsum) {
+  constexpr int PER = NBINS / 1024;   // bins per thread
+  static_assert(PER >= 1 && PER * 1024 == NBINS, "bins");
+  __shared__ unsigned count;
+  const int top = NBINS - 1 - PER * static_cast<int>(threadIdx.x);
+  unsigned c[PER];
+#pragma unroll
+  for (int q = 0; q < PER; ++q) c[q] = bins[top - q];
+  select_from_counts<PER>(c, top, r, sel, wsum, &count);
 }
 
 // Eq. 5-6 and R3-R4 from the tail mean d_top of image b: rho_d, rho, r and the target size.
@@ -686,154 +952,170 @@ __device__ __forceinline__ void tail_finish(const ApcTable& t, int b, const Tail
   st.w_out = wo;
 }
 
-// The density tail (Eq. 5: the mean of the k_tail largest d_i, then Eq. 6 and R3-R4), several
-// CTAs per image; pass 2 has counted the distances into 4096 value buckets of width 1/2048 (the
-// top one also takes anything above).  CTA c of image b takes distances c kTailChunk .. : it
-// selects the k-th largest's bucket from the counts (level 1), adds the distances above that
-// bucket to the image's total in 2^-32 fixed point (exact, so the order of the CTAs does not
-// matter) and lists the bucket's members.  The image's last CTA to finish narrows the members to
-// the k-th largest distance T (level 2: each member ranked against the others when there are at
-// most 1024, else rounds of 1024 bins over the key offsets from the bucket's first fp32 key) and
-// writes the statistics; a bucket too crowded for the list is narrowed over the whole array by
-// rounds of 4096 bins.
-__global__ void __launch_bounds__(1024) apc_tail_scan(const __grid_constant__ ApcTable t, const float* __restrict__ d,
-                                                      TailParams prm, pace_apc_stats* __restrict__ stats,
-                                                      TailWork* __restrict__ work) {
-  __shared__ unsigned bins[kTailBins];
-  __shared__ unsigned hist2[kTailBins2];
-  __shared__ unsigned sel[2];
+// The density tail (Eq. 5: the mean of the k_tail largest d_i, then Eq. 6 and R3-R4).  Pass 2 has
+// counted and summed the distances in 4096 value buckets of width 1/2048 (the top one also takes
+// anything above), so the k-th largest's bucket and the sum of everything above it follow from the
+// counts alone, and only that bucket's members are looked for in the distances.  A cluster of
+// CTAs per image: every CTA selects the bucket for itself, scans its share of the distances
+// (loaded before the selection, so that the two latencies overlap) and appends the members to the
+// first CTA's shared list; after one cluster barrier the first CTA narrows the members to the k-th
+// largest distance T (members all equal: at once; at most 1024: each ranked against the others;
+// else rounds of 1024 bins over the key offsets from the bucket's first fp32 key) and writes the
+// statistics.  A bucket with too many different members for the list is narrowed over the whole
+// array by rounds of 4096 bins.  Everything is latency: a chain of L2 reads and block barriers.
+constexpr int kTailList = 4096;    // members listed
+constexpr int kTailAhead = 8;      // distances per thread loaded ahead of the selection
+constexpr int kTailCluster = 8;    // CTAs per image above kTailAhead * 1024 distances
+
+__global__ void __launch_bounds__(1024) apc_tail(const __grid_constant__ ApcTable t, const float* __restrict__ d,
+                                                 TailParams prm, pace_apc_stats* __restrict__ stats,
+                                                 const TailWork* __restrict__ work) {
+  __shared__ unsigned list[kTailList];
+  __shared__ unsigned bins[kTailBins];   // bins of the narrowing rounds
+  __shared__ unsigned sel[2], selb[2];
   __shared__ unsigned cred[32];
   __shared__ unsigned long long fred[32];
-  __shared__ int last;
+  __shared__ unsigned list_n, key_min, key_max;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int rank = static_cast<int>(blockIdx.x), ncta = static_cast<int>(gridDim.x);
+  if (tid == 0) {
+    list_n = 0u;
+    key_min = 0xFFFFFFFFu;
+    key_max = 0u;
+  }
+  if (ncta > 1) ptx::cluster_arrive();   // the first CTA's list is ready: waited for before the first append
+  ptx::launch_dependents();
+  ptx::grid_dependency_wait();
   const int b = blockIdx.y;
   const int N = t.n[b];
-  const int nchunk = (N + kTailChunk - 1) / kTailChunk;
-  if (static_cast<int>(blockIdx.x) >= nchunk) return;
-  TailWork* w = work + (t.b_base + b);
+  const TailWork* w = work + (t.b_base + b);
   const float* db = d + t.patch0[b];
   const unsigned k = static_cast<unsigned>(t.ktail[b]);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // level 1 on the counts (written by the previous kernel: read through L2)
-  for (int i = threadIdx.x; i < kTailBins; i += blockDim.x) bins[i] = __ldcg(&w->hist[i]);
-  __syncthreads();
-  select_from_top<kTailBins>(bins, k, sel, cred);
-  const int tb = static_cast<int>(sel[0]);
-  const unsigned cb = bins[tb];         // entries in the k-th largest's bucket
-  const unsigned above_n = sel[1];      // entries in the buckets above it
-  const bool listed = cb <= kTailList;
-  // this CTA's chunk
+  // this CTA's distances rank * 1024 + tid, + 1024 ncta, ..
+  const int i0 = rank * 1024 + tid, step = ncta * 1024;
+  float ahead[kTailAhead];
+#pragma unroll
+  for (int q = 0; q < kTailAhead; ++q) {
+    const int i = i0 + q * step;
+    ahead[q] = i < N ? __ldcg(db + i) : 0.f;
+  }
+  // level 1: thread t holds buckets 4095 - 4t .. 4092 - 4t
+  const int top = kTailBins - 1 - 4 * tid;
+  const uint4 cv = __ldcg(reinterpret_cast<const uint4*>(w->hist + top - 3));
+  const unsigned c4[4] = {cv.w, cv.z, cv.y, cv.x};
   unsigned long long s_fix = 0ull;
-  unsigned cnt = 0u;
-  bool wrote = false;   // this thread listed a member
-  const int i0 = static_cast<int>(blockIdx.x) * kTailChunk, i1 = min(N, i0 + kTailChunk);
-  for (int base = i0; base < i1; base += blockDim.x) {   // uniform trip count: the ballot below
-    const int i = base + static_cast<int>(threadIdx.x);
-    const float v = i < i1 ? db[i] : 0.f;
-    const int bk = i < i1 ? tail_bucket(v) : -1;
-    if (bk > tb) {
-      s_fix += fix32(v);
-      ++cnt;
-    }
-    const bool member = listed && bk == tb;
-    const unsigned ball = __ballot_sync(0xffffffffu, member);
-    if (ball != 0u) {   // one slot reservation per warp
-      unsigned slot = 0u;
-      if (lane == 0) slot = atomicAdd(&w->list_n, static_cast<unsigned>(__popc(ball)));
-      slot = __shfl_sync(0xffffffffu, slot, 0);
-      if (member) {
-        w->list[slot + __popc(ball & ((1u << lane) - 1u))] = __float_as_uint(v);
-        wrote = true;
-      }
-    }
-  }
-  for (int o = 16; o > 0; o >>= 1) {
-    cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-    s_fix += __shfl_xor_sync(0xffffffffu, s_fix, o);
-  }
-  if (lane == 0) {
-    cred[warp] = cnt;
-    fred[warp] = s_fix;
-  }
-  if (wrote) __threadfence();   // this thread's list entries, before the CTA reports its chunk done
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    unsigned c = 0u;
-    unsigned long long f = 0ull;
-    for (int i = 0; i < static_cast<int>(blockDim.x >> 5); ++i) {
-      c += cred[i];
-      f += fred[i];
-    }
-    atomicAdd(&w->above_fix, f);
-    atomicAdd(&w->above_cnt, c);
-    __threadfence();
-    last = atomicAdd(&w->done, 1u) == static_cast<unsigned>(nchunk - 1);
-  }
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  // the image's totals and rho_g, read now so that their latency overlaps level 2
-  unsigned tot_cnt = 0u;
-  unsigned long long tot_fix = 0ull;
+  ulonglong2 s01, s23;
   float rho_g = 0.f;
-  if (threadIdx.x == 0) {
-    tot_cnt = __ldcg(&w->above_cnt);
-    tot_fix = __ldcg(&w->above_fix);
-    rho_g = stats[t.b_base + b].rho_g;
+  if (rank == 0) {
+    s23 = __ldcg(reinterpret_cast<const ulonglong2*>(w->sum + top - 3));
+    s01 = __ldcg(reinterpret_cast<const ulonglong2*>(w->sum + top - 1));
+    if (tid == 0) rho_g = __ldcg(&stats[t.b_base + b].rho_g);
   }
-  // level 2 (the image's last CTA): T = the k-th largest distance; the members of the bucket
-  // above T are summed in fixed point (c counts every distance above T)
-  unsigned remaining = k - above_n;
+  select_from_counts<4>(c4, top, k, sel, cred, selb);
+  const int tb = static_cast<int>(sel[0]);
+  const unsigned above_n = sel[1];     // entries in the buckets above it
+  const unsigned cb = selb[0];         // entries in the k-th largest's bucket
+  if (rank == 0) {                     // the sum of the distances in the buckets above it
+    if (top > tb) s_fix += s01.y;
+    if (top - 1 > tb) s_fix += s01.x;
+    if (top - 2 > tb) s_fix += s23.y;
+    if (top - 3 > tb) s_fix += s23.x;
+  }
+  const bool listed = cb <= kTailList, spread = cb > 1024u;
+  unsigned* list0 = list;
+  unsigned *n0 = &list_n, *min0 = &key_min, *max0 = &key_max;
+  if (ncta > 1) {
+    ptx::cluster_wait();
+    list0 = cluster.map_shared_rank(list, 0);
+    n0 = cluster.map_shared_rank(&list_n, 0);
+    min0 = cluster.map_shared_rank(&key_min, 0);
+    max0 = cluster.map_shared_rank(&key_max, 0);
+  }
+  // this CTA's members of the bucket
+  unsigned kmin = 0xFFFFFFFFu, kmax = 0u;
+  auto scan = [&](float v, bool live) {
+    const bool member = live && tail_bucket(v) == tb;
+    const unsigned ball = __ballot_sync(0xffffffffu, member);
+    if (ball == 0u) return;
+    const unsigned key = __float_as_uint(v);
+    if (member) {
+      kmin = min(kmin, key);
+      kmax = max(kmax, key);
+    }
+    if (!listed) return;
+    unsigned slot = 0u;   // one slot reservation per warp
+    if (lane == 0) slot = atomicAdd(n0, static_cast<unsigned>(__popc(ball)));
+    slot = __shfl_sync(0xffffffffu, slot, 0) + __popc(ball & ((1u << lane) - 1u));
+    if (member) list0[slot] = key;
+  };
+#pragma unroll
+  for (int q = 0; q < kTailAhead; ++q) scan(ahead[q], i0 + q * step < N);
+  for (int base = rank * 1024 + kTailAhead * step; base < N; base += step) {   // uniform trip count per CTA
+    const int i = base + tid;
+    scan(i < N ? __ldcg(db + i) : 0.f, i < N);
+  }
+  if (spread) {
+    kmin = __reduce_min_sync(0xffffffffu, kmin);
+    kmax = __reduce_max_sync(0xffffffffu, kmax);
+    if (lane == 0 && kmax >= kmin) {
+      atomicMin(min0, kmin);
+      atomicMax(max0, kmax);
+    }
+  }
+  if (ncta > 1) cluster.sync();
+  else __syncthreads();
+  if (rank != 0) return;
+  // level 2: T = the k-th largest distance; the members of the bucket above T are summed in fixed
+  // point (c counts every distance above T)
+  unsigned remaining = k - above_n, cnt = 0u;
   unsigned lo = __float_as_uint(static_cast<float>(tb) * (1.0f / 2048.0f));
   unsigned span = (tb == kTailBins - 1 ? 0x7F800001u : __float_as_uint(static_cast<float>(tb + 1) * (1.0f / 2048.0f))) - lo;
   const unsigned bucket_lo = lo, bucket_span = span;
-  s_fix = 0ull;
-  cnt = 0u;
   unsigned prefix;
-  __syncthreads();   // everyone has read sel and bins[tb]
-  if (listed) {
-    for (int i = threadIdx.x; i < static_cast<int>(cb); i += blockDim.x) bins[i] = __ldcg(&w->list[i]);
+  if (!spread) {
+    // one member per thread, ranked against the whole list: a member with fewer than `remaining`
+    // members at or above it lies above the k-th largest (and is summed); with fewer than
+    // `remaining` above it but at least that many at or above it, it is the k-th largest
+    int mi;
+    unsigned gt, ge;
+    if (rank_in_list(list, cb, mi, gt, ge)) {
+      const unsigned mine = list[mi];
+      if (ge < remaining) {
+        s_fix += fix32(__uint_as_float(mine));
+        ++cnt;
+      } else if (gt < remaining) {
+        selb[1] = mine;   // the same key from every member equal to it
+      }
+    }
     __syncthreads();
-    if (cb <= blockDim.x) {
-      // one member per thread, ranked against the whole list: a member with fewer than
-      // `remaining` members at or above it lies above the k-th largest (and is summed); with fewer
-      // than `remaining` above it but at least that many at or above it, it is the k-th largest
-      int mi;
-      unsigned gt, ge;
-      if (rank_in_list(bins, cb, mi, gt, ge)) {
-        const unsigned mine = bins[mi];
-        if (ge < remaining) {
-          s_fix += fix32(__uint_as_float(mine));
-          ++cnt;
-        } else if (gt < remaining) {
-          sel[0] = mine;   // the same key from every member equal to it
-        }
+    prefix = selb[1];
+  } else if (key_min == key_max) {   // every member is the same distance
+    prefix = key_min;
+  } else if (listed) {
+    while (true) {
+      const int bits = 32 - __clz(span - 1u);
+      const int shift = bits > 10 ? bits - 10 : 0;
+      for (int i = tid; i < kTailBins2; i += blockDim.x) bins[i] = 0u;
+      __syncthreads();
+      for (int i = tid; i < static_cast<int>(cb); i += blockDim.x) {
+        const unsigned off = list[i] - lo;   // wraps for keys below lo
+        if (off < span) atomicAdd(&bins[off >> shift], 1u);
       }
       __syncthreads();
-      prefix = sel[0];
-    } else {
-      while (true) {
-        const int bits = 32 - __clz(span - 1u);
-        const int shift = bits > 10 ? bits - 10 : 0;
-        for (int i = threadIdx.x; i < kTailBins2; i += blockDim.x) hist2[i] = 0u;
-        __syncthreads();
-        for (int i = threadIdx.x; i < static_cast<int>(cb); i += blockDim.x) {
-          const unsigned off = bins[i] - lo;   // wraps for keys below lo
-          if (off < span) atomicAdd(&hist2[off >> shift], 1u);
-        }
-        __syncthreads();
-        select_from_top<kTailBins2>(hist2, remaining, sel, cred);
-        lo += sel[0] << shift;
-        remaining -= sel[1];
-        if (shift == 0) break;
-        span = min(span - (sel[0] << shift), 1u << shift);
-      }
-      prefix = lo;
-      for (int i = threadIdx.x; i < static_cast<int>(cb); i += blockDim.x) {
-        const unsigned key = bins[i];
-        if (key > prefix) {
-          s_fix += fix32(__uint_as_float(key));
-          ++cnt;
-        }
+      select_from_top<kTailBins2>(bins, remaining, sel, cred);
+      lo += sel[0] << shift;
+      remaining -= sel[1];
+      if (shift == 0) break;
+      span = min(span - (sel[0] << shift), 1u << shift);
+      __syncthreads();   // everyone has read sel and the bins
+    }
+    prefix = lo;
+    for (int i = tid; i < static_cast<int>(cb); i += blockDim.x) {
+      const unsigned key = list[i];
+      if (key > prefix) {
+        s_fix += fix32(__uint_as_float(key));
+        ++cnt;
       }
     }
   } else {
@@ -843,10 +1125,10 @@ __global__ void __launch_bounds__(1024) apc_tail_scan(const __grid_constant__ Ap
       const int bits = 32 - __clz(span - 1u);
       const int shift = bits > 12 ? bits - 12 : 0;
       __syncthreads();                               // everyone has read sel and the bins
-      for (int i = threadIdx.x; i < kTailBins; i += blockDim.x) bins[i] = 0u;
+      for (int i = tid; i < kTailBins; i += blockDim.x) bins[i] = 0u;
       __syncthreads();
       for (int base = 0; base < N; base += blockDim.x) {   // uniform trip count: __match_any_sync below
-        const int i = base + static_cast<int>(threadIdx.x);
+        const int i = base + tid;
         const unsigned off = i < N ? __float_as_uint(db[i]) - lo : span;   // wraps for keys below lo
         const bool in = off < span;
         const unsigned digit = in ? off >> shift : kTailBins;
@@ -866,7 +1148,7 @@ __global__ void __launch_bounds__(1024) apc_tail_scan(const __grid_constant__ Ap
       span = min(span - (sel[0] << shift), 1u << shift);
     }
     prefix = lo;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {   // the bucket's members above T
+    for (int i = tid; i < N; i += blockDim.x) {   // the bucket's members above T
       const unsigned key = __float_as_uint(db[i]);
       if (key > prefix && key - bucket_lo < bucket_span) {
         s_fix += fix32(__uint_as_float(key));
@@ -874,29 +1156,25 @@ __global__ void __launch_bounds__(1024) apc_tail_scan(const __grid_constant__ Ap
       }
     }
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-    s_fix += __shfl_xor_sync(0xffffffffu, s_fix, o);
-  }
-  __syncthreads();   // the level-2 reads of cred and sel are done
+  cnt = __reduce_add_sync(0xffffffffu, cnt);
+  for (int o = 16; o > 0; o >>= 1) s_fix += __shfl_xor_sync(0xffffffffu, s_fix, o);
+  __syncthreads();   // the earlier reads of cred are done
   if (lane == 0) {
     cred[warp] = cnt;
     fred[warp] = s_fix;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    unsigned c = tot_cnt;
-    unsigned long long f = tot_fix;
-    for (int i = 0; i < static_cast<int>(blockDim.x >> 5); ++i) {
-      c += cred[i];
-      f += fred[i];
+  if (warp == 0) {
+    const unsigned c = above_n + __reduce_add_sync(0xffffffffu, cred[lane]);
+    unsigned long long f = fred[lane];
+    for (int o = 16; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
+    if (lane == 0) {
+      const float T = __uint_as_float(prefix);   // k-th largest d
+      const float tot = unfix32<false>(f, 1.0f) + static_cast<float>(k - c) * T;   // the rest equal T
+      tail_finish(t, b, prm, stats, rho_g, tot / static_cast<float>(k));
     }
-    const float T = __uint_as_float(prefix);   // k-th largest d
-    const float tot = unfix32<false>(f, 1.0f) + static_cast<float>(k - c) * T;   // the rest equal T
-    tail_finish(t, b, prm, stats, rho_g, tot / static_cast<float>(k));
   }
 }
-
 
 // ------------------------------------------------------------------------------------------------
 // pixel-statistic previews (App. "Shallow Feature Preview Ablation"): one small token per patch,
@@ -1134,7 +1412,7 @@ __global__ void __launch_bounds__(kApcThreads) apc_pix_pass2(const __grid_consta
   }
   const float dv = sqrtf(acc);
   d_out[t.tok0[b] + i] = dv;
-  atomicAdd(&work[t.b_base + b].hist[tail_bucket(dv)], 1u);   // the tail's bucket counts
+  tail_count(work + t.b_base + b, dv);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1464,7 +1742,7 @@ __global__ void __launch_bounds__(kRsThreads) apc_resample(const uint8_t* __rest
 // host side
 // ------------------------------------------------------------------------------------------------
 struct DensityLayout {
-  size_t sums_off, work_off, zero_bytes, inv_off, d_off, total;   // [0, zero_bytes) is zeroed per call
+  size_t sums_off, work_off, zero_bytes, sumsq_off, d_off, total;   // [0, zero_bytes) is zeroed per call
   int64_t n_total;
 };
 
@@ -1474,15 +1752,15 @@ DensityLayout density_layout(int B, const int32_t* H, const int32_t* W) {
   for (int b = 0; b < B; ++b) n += static_cast<int64_t>(H[b] / kPatch) * (W[b] / kPatch);
   L.n_total = n;
   L.sums_off = 0;
-  L.work_off = align_up(static_cast<size_t>(B) * kTokDim * sizeof(unsigned long long), 256);
+  L.work_off = align_up(static_cast<size_t>(B) * kSumSlots * kTokDim * sizeof(unsigned long long), 256);
   L.zero_bytes = L.work_off + static_cast<size_t>(B) * sizeof(TailWork);
-  L.inv_off = align_up(L.zero_bytes, 256);
-  L.d_off = L.inv_off + align_up(static_cast<size_t>(n) * sizeof(float), 256);
+  L.sumsq_off = align_up(L.zero_bytes, 256);
+  L.d_off = L.sumsq_off + align_up(static_cast<size_t>(n) * sizeof(float), 256);
   L.total = L.d_off + align_up(static_cast<size_t>(n) * sizeof(float), 256);
   return L;
 }
 
-// Grid of the strip passes: the CTAs that are resident at once (capped by the strips).
+// Grid of the strip walks: the CTAs that are resident at once (capped by the strips).
 unsigned strip_grid(int units) {
   static std::atomic<int> cap[64];
   int dev = 0;
@@ -1491,23 +1769,115 @@ unsigned strip_grid(int units) {
   if (c == 0) {
     int nsm = 0, per = 0;
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, apc_pass2<true>, kApcThreads, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, apc_pix_features<true>, kApcThreads, 0);
     c = std::max(1, nsm * std::max(per, 1));
     cap[dev & 63].store(c, std::memory_order_relaxed);
   }
   return static_cast<unsigned>(std::max(1, std::min(units, c)));
 }
 
-// Launches apc_tail_scan on one ApcTable: kTailChunk distances per CTA, the largest image's
-// chunks per row of the grid (CTAs past a smaller image's chunks return at once).
-void launch_tail_scan(const ApcTable& t, const float* d, TailParams tp, pace_apc_stats* stats, TailWork* work,
-                      cudaStream_t stream) {
-  int chunks = 1;
-  for (int i = 0; i < t.nb; ++i) chunks = std::max(chunks, (t.n[i] + kTailChunk - 1) / kTailChunk);
-  apc_tail_scan<<<dim3(static_cast<unsigned>(chunks), static_cast<unsigned>(t.nb)), 1024, 0, stream>>>(t, d, tp, stats,
-                                                                                                     work);
+// Launches apc_tail on one ApcTable: a cluster of CTAs per image, one CTA when every image's
+// distances fit its first loads.
+pace_status_t launch_tail(const ApcTable& t, const float* d, TailParams tp, pace_apc_stats* stats, TailWork* work,
+                          cudaStream_t stream) {
+  int most = 0;
+  for (int i = 0; i < t.nb; ++i) most = std::max(most, t.n[i]);
+  const unsigned ctas = most <= kTailAhead * 1024 ? 1u : kTailCluster;
+  return launch_dependent(apc_tail, dim3(ctas, static_cast<unsigned>(t.nb)), 1024, 0, ctas, stream, t, d, tp, stats,
+                          static_cast<const TailWork*>(work));
 }
 
+pace_status_t launch_zero(void* a, size_t a_bytes, void* b, size_t b_bytes, cudaStream_t stream) {
+  const size_t na = a_bytes / 16, nb = b_bytes / 16;
+  apc_zero<<<static_cast<unsigned>(std::min<size_t>((na + nb + 1023) / 1024, 2048)), 256, 0, stream>>>(
+      static_cast<uint4*>(a), static_cast<unsigned>(na), static_cast<uint4*>(b), static_cast<unsigned>(nb));
+  return check_launch();
+}
+
+// Strip table of images c0 .. c0 + nb - 1; patch0 runs on over the calls.  Each image has the widest
+// strips of which it has at least `enough` (else the narrowest): a small image is all latency
+// (448 x 448: 32 strips of 32 patches, 128 of 8), a large one all issue, and wide strips spend
+// least of it on barriers.  The width goes by the image alone, not by the batch, so that its column
+// sums (rounded once per strip) are the same bits in any batch.
+void fill_strip_table(ApcTable& t, int c0, int nb, const int64_t* img_off, const int32_t* H, const int32_t* W,
+                      float tail_frac, int enough, int& patch0) {
+  t = ApcTable{};
+  t.nb = nb;
+  t.b_base = c0;
+  t.unit_prefix[0] = 0;
+  for (int i = 0; i < nb; ++i) {
+    const int b = c0 + i;
+    t.off[i] = img_off[b];
+    t.H[i] = H[b];
+    t.W[i] = W[b];
+    t.gw[i] = W[b] / kPatch;
+    int lg = kStripLog2;
+    while (lg > kMinStripLog2 && ((t.gw[i] + (1 << lg) - 1) >> lg) * (H[b] / kPatch) < enough) --lg;
+    t.strip_log2[i] = lg;
+    t.chunks[i] = (t.gw[i] + (1 << lg) - 1) >> lg;
+    t.patch0[i] = patch0;
+    const int N = (H[b] / kPatch) * t.gw[i];
+    t.n[i] = N;
+    double kt = std::floor(static_cast<double>(tail_frac) * N + 0.5);
+    if (kt < 1) kt = 1;
+    if (kt > N) kt = N;
+    t.ktail[i] = static_cast<int>(kt);
+    patch0 += N;
+    t.unit_prefix[i + 1] = t.unit_prefix[i] + (H[b] / kPatch) * t.chunks[i];
+  }
+}
+
+// Whether every image row of the table starts on a 4-byte boundary (an even number of patches wide).
+bool rows_aligned(const ApcTable& t) {
+  bool all = true;
+  for (int i = 0; i < t.nb; ++i) all = all && t.gw[i] % 2 == 0;
+  return all;
+}
+
+pace_status_t check_params(const pace_apc_params* params, pace_apc_params& p) {
+  if (params) p = *params;
+  else pace_apc_params_default(&p);
+  if (!(p.tail_frac > 0.f && p.tail_frac <= 1.f) || !(p.gamma > 0.f) || !(p.alpha >= 0.f && p.alpha <= 1.f) ||
+      !(p.r_min <= p.r_max) || p.align < 1)
+    return PACE_ERR_INVALID_ARG;
+  return PACE_OK;
+}
+
+// The three density kernels, after the kernel that zeroes their sums and tail scratch.
+pace_status_t run_density(const uint8_t* img, const int64_t* img_off, const int32_t* H, const int32_t* W, int B,
+                          const pace_apc_params& p, float* d, pace_apc_stats* stats, unsigned long long* sums,
+                          TailWork* work, uint32_t* sumsq, cudaStream_t stream) {
+  int sms = 0, dev = 0;
+  PACE_CHECK(sm_count(&sms));
+  PACE_CUDA(cudaGetDevice(&dev));
+  static DeviceOnce once;   // opt in to the passes' shared memory
+  if (!once.done(dev)) {
+    for (auto* k : {apc_pass1<true>, apc_pass1<false>})
+      PACE_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kDGroups * sizeof(Pass1Group)));
+    for (auto* k : {apc_pass2<true>, apc_pass2<false>})
+      PACE_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(Pass2Smem)));
+    once.mark(dev);
+  }
+  int* status = device_status_word();
+  int patch0 = 0;
+  for (int c0 = 0; c0 < B; c0 += kApcMaxB) {
+    const int nb = std::min(kApcMaxB, B - c0);
+    ApcTable t;
+    fill_strip_table(t, c0, nb, img_off, H, W, p.tail_frac, 2 * sms, patch0);
+    const int units = t.unit_prefix[nb];
+    const unsigned grid = static_cast<unsigned>(std::min(units, sms));
+    const dim3 block(kDThreads, kDGroups);
+    const bool aligned = rows_aligned(t);
+    PACE_CHECK(launch_dependent(aligned ? apc_pass1<true> : apc_pass1<false>, grid, block, kDGroups * sizeof(Pass1Group), 1,
+                                stream, img, t, units, sumsq, sums, status));
+    PACE_CHECK(launch_dependent(aligned ? apc_pass2<true> : apc_pass2<false>, grid, block, sizeof(Pass2Smem), 1, stream, img,
+                                t, units, static_cast<const uint32_t*>(sumsq), static_cast<const unsigned long long*>(sums), d,
+                                stats, work, status));
+    const TailParams tp{p.alpha, p.gamma, p.r_min, p.r_max, p.align};
+    PACE_CHECK(launch_tail(t, d, tp, stats, work, stream));
+  }
+  return PACE_OK;
+}
 
 pace_status_t check_images(const uint8_t* img, const int64_t* off, const int32_t* H, const int32_t* W, int B) {
   if (B < 0) return PACE_ERR_INVALID_ARG;
@@ -1541,57 +1911,15 @@ extern "C" pace_status_t pace_apc_density(const uint8_t* img, const int64_t* img
   if (B == 0) return PACE_OK;
   if (stats == nullptr) return PACE_ERR_INVALID_ARG;
   pace_apc_params p;
-  if (params) p = *params; else pace_apc_params_default(&p);
-  if (!(p.tail_frac > 0.f && p.tail_frac <= 1.f) || !(p.gamma > 0.f) || !(p.alpha >= 0.f && p.alpha <= 1.f) ||
-      !(p.r_min <= p.r_max) || p.align < 1)
-    return PACE_ERR_INVALID_ARG;
+  PACE_CHECK(check_params(params, p));
   const DensityLayout L = density_layout(B, H, W);
   if (ws == nullptr || ws_bytes < L.total || reinterpret_cast<uintptr_t>(ws) % 16) return PACE_ERR_WORKSPACE;
   PACE_CHECK(check_device());
   uint8_t* w8 = static_cast<uint8_t*>(ws);
-  auto* sums = reinterpret_cast<unsigned long long*>(w8 + L.sums_off);
-  auto* work = reinterpret_cast<TailWork*>(w8 + L.work_off);
-  auto* inv = reinterpret_cast<float*>(w8 + L.inv_off);
   float* d = d_out ? d_out : reinterpret_cast<float*>(w8 + L.d_off);
-  PACE_CUDA(cudaMemsetAsync(w8, 0, L.zero_bytes, stream));   // column sums and tail scratch
-  int patch0 = 0;
-  for (int c0 = 0; c0 < B; c0 += kApcMaxB) {
-    const int nb = (B - c0) < kApcMaxB ? (B - c0) : kApcMaxB;
-    ApcTable t{};
-    t.nb = nb;
-    t.b_base = c0;
-    t.unit_prefix[0] = 0;
-    bool wide = true;
-    for (int i = 0; i < nb; ++i) {
-      const int b = c0 + i;
-      t.off[i] = img_off[b];
-      t.H[i] = H[b];
-      t.W[i] = W[b];
-      t.gw[i] = W[b] / kPatch;
-      t.chunks[i] = (t.gw[i] + kStrip - 1) / kStrip;
-      t.patch0[i] = patch0;
-      const int N = (H[b] / kPatch) * t.gw[i];
-      t.n[i] = N;
-      double kt = std::floor(static_cast<double>(p.tail_frac) * N + 0.5);
-      if (kt < 1) kt = 1;
-      if (kt > N) kt = N;
-      t.ktail[i] = static_cast<int>(kt);
-      patch0 += N;
-      t.unit_prefix[i + 1] = t.unit_prefix[i] + (H[b] / kPatch) * t.chunks[i];
-      if ((static_cast<int64_t>(W[b]) * 3) % 4 != 0 || (t.gw[i] % 2) != 0 || (img_off[b] % 4) != 0) wide = false;
-    }
-    const int units = t.unit_prefix[nb];
-    if (wide) apc_pass1<true><<<strip_grid(units), kApcThreads, 0, stream>>>(img, t, units, inv, sums);
-    else apc_pass1<false><<<strip_grid(units), kApcThreads, 0, stream>>>(img, t, units, inv, sums);
-    PACE_CHECK(check_launch());
-    if (wide) apc_pass2<true><<<strip_grid(units), kApcThreads, 0, stream>>>(img, t, units, inv, sums, d, stats, work);
-    else apc_pass2<false><<<strip_grid(units), kApcThreads, 0, stream>>>(img, t, units, inv, sums, d, stats, work);
-    PACE_CHECK(check_launch());
-    TailParams tp{p.alpha, p.gamma, p.r_min, p.r_max, p.align};
-    launch_tail_scan(t, d, tp, stats, work, stream);
-    PACE_CHECK(check_launch());
-  }
-  return PACE_OK;
+  PACE_CHECK(launch_zero(w8, L.zero_bytes, nullptr, 0, stream));   // column sums and tail scratch
+  return run_density(img, img_off, H, W, B, p, d, stats, reinterpret_cast<unsigned long long*>(w8 + L.sums_off),
+                     reinterpret_cast<TailWork*>(w8 + L.work_off), reinterpret_cast<uint32_t*>(w8 + L.sumsq_off), stream);
 }
 
 static pace_status_t resample_impl(const uint8_t* src, const int64_t* src_off, const int32_t* H, const int32_t* W,
@@ -1667,16 +1995,16 @@ extern "C" pace_status_t pace_apc_resample_to(const uint8_t* src, const int64_t*
 // pace_apc_density_static: the same density computation with library-owned scratch
 // ------------------------------------------------------------------------------------------------
 // Scratch of pace_apc_density_static, in a file-scope device array instead of caller memory:
-// the per-image 589-entry fixed-point column sums, then the per-patch inverse token norms.
+// the per-image 589-entry fixed-point column sums (kSumSlots copies), the tail's buckets, then |x|^2 per patch.
 // Every GPU that loads the library holds this array until the process exits.
 namespace pace {
 namespace {
 constexpr size_t kStaticSumsBytes =
-    static_cast<size_t>(PACE_APC_STATIC_MAX_IMAGES) * kTokDim * sizeof(unsigned long long);
+    static_cast<size_t>(PACE_APC_STATIC_MAX_IMAGES) * kSumSlots * kTokDim * sizeof(unsigned long long);
 constexpr size_t kStaticWorkOff = (kStaticSumsBytes + 255) / 256 * 256;
 constexpr size_t kStaticZeroBytes = kStaticWorkOff + static_cast<size_t>(PACE_APC_STATIC_MAX_IMAGES) * sizeof(TailWork);
-constexpr size_t kStaticInvOff = (kStaticZeroBytes + 255) / 256 * 256;
-constexpr size_t kStaticBytes = kStaticInvOff + static_cast<size_t>(PACE_APC_STATIC_MAX_PATCHES) * sizeof(float);
+constexpr size_t kStaticSumsqOff = (kStaticZeroBytes + 255) / 256 * 256;
+constexpr size_t kStaticBytes = kStaticSumsqOff + static_cast<size_t>(PACE_APC_STATIC_MAX_PATCHES) * sizeof(uint32_t);
 
 static __device__ __align__(256) unsigned char g_apc_static_scratch[kStaticBytes];
 
@@ -1716,53 +2044,18 @@ extern "C" pace_status_t pace_apc_density_static(const uint8_t* img, const int64
   for (int b = 0; b < B; ++b) n_total += static_cast<int64_t>(H[b] / kPatch) * (W[b] / kPatch);
   if (n_total > PACE_APC_STATIC_MAX_PATCHES) return PACE_ERR_INVALID_ARG;
   pace_apc_params p;
-  if (params) p = *params; else pace_apc_params_default(&p);
-  if (!(p.tail_frac > 0.f && p.tail_frac <= 1.f) || !(p.gamma > 0.f) || !(p.alpha >= 0.f && p.alpha <= 1.f) ||
-      !(p.r_min <= p.r_max) || p.align < 1)
-    return PACE_ERR_INVALID_ARG;
+  PACE_CHECK(check_params(params, p));
   PACE_CHECK(check_device());
   unsigned char* scratch = nullptr;
   PACE_CHECK(static_scratch(&scratch));
   auto* sums = reinterpret_cast<unsigned long long*>(scratch);
   auto* work = reinterpret_cast<TailWork*>(scratch + kStaticWorkOff);
-  auto* inv = reinterpret_cast<float*>(scratch + kStaticInvOff);
   // the array keeps the previous call's contents: the column sums and the tail scratch of the
   // call's images must start from zero
-  PACE_CUDA(cudaMemsetAsync(sums, 0, static_cast<size_t>(B) * kTokDim * sizeof(unsigned long long), stream));
-  PACE_CUDA(cudaMemsetAsync(work, 0, static_cast<size_t>(B) * sizeof(TailWork), stream));
-  ApcTable t{};
-  t.nb = B;
-  t.b_base = 0;
-  t.unit_prefix[0] = 0;
-  bool wide = true;
-  int patch0 = 0;
-  for (int b = 0; b < B; ++b) {
-    t.off[b] = img_off[b];
-    t.H[b] = H[b];
-    t.W[b] = W[b];
-    t.gw[b] = W[b] / kPatch;
-    t.chunks[b] = (t.gw[b] + kStrip - 1) / kStrip;
-    t.patch0[b] = patch0;
-    const int N = (H[b] / kPatch) * t.gw[b];
-    t.n[b] = N;
-    double kt = std::floor(static_cast<double>(p.tail_frac) * N + 0.5);
-    if (kt < 1) kt = 1;
-    if (kt > N) kt = N;
-    t.ktail[b] = static_cast<int>(kt);
-    patch0 += N;
-    t.unit_prefix[b + 1] = t.unit_prefix[b] + (H[b] / kPatch) * t.chunks[b];
-    if ((static_cast<int64_t>(W[b]) * 3) % 4 != 0 || (t.gw[b] % 2) != 0 || (img_off[b] % 4) != 0) wide = false;
-  }
-  const int units = t.unit_prefix[B];
-  if (wide) apc_pass1<true><<<strip_grid(units), kApcThreads, 0, stream>>>(img, t, units, inv, sums);
-  else apc_pass1<false><<<strip_grid(units), kApcThreads, 0, stream>>>(img, t, units, inv, sums);
-  PACE_CHECK(check_launch());
-  if (wide) apc_pass2<true><<<strip_grid(units), kApcThreads, 0, stream>>>(img, t, units, inv, sums, d_out, stats, work);
-  else apc_pass2<false><<<strip_grid(units), kApcThreads, 0, stream>>>(img, t, units, inv, sums, d_out, stats, work);
-  PACE_CHECK(check_launch());
-  TailParams tp{p.alpha, p.gamma, p.r_min, p.r_max, p.align};
-  launch_tail_scan(t, d_out, tp, stats, work, stream);
-  return check_launch();
+  PACE_CHECK(launch_zero(sums, static_cast<size_t>(B) * kSumSlots * kTokDim * sizeof(unsigned long long), work,
+                         static_cast<size_t>(B) * sizeof(TailWork), stream));
+  return run_density(img, img_off, H, W, B, p, d_out, stats, sums, work,
+                     reinterpret_cast<uint32_t*>(scratch + kStaticSumsqOff), stream);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1831,10 +2124,7 @@ extern "C" pace_status_t pace_apc_density_tokens(const void* T, const int32_t* c
   for (int b = 0; b < B; ++b)
     if (cu_tokens[b + 1] - cu_tokens[b] < 1 || H[b] < 1 || W[b] < 1) return PACE_ERR_INVALID_ARG;
   pace_apc_params p;
-  if (params) p = *params; else pace_apc_params_default(&p);
-  if (!(p.tail_frac > 0.f && p.tail_frac <= 1.f) || !(p.gamma > 0.f) || !(p.alpha >= 0.f && p.alpha <= 1.f) ||
-      !(p.r_min <= p.r_max) || p.align < 1)
-    return PACE_ERR_INVALID_ARG;
+  PACE_CHECK(check_params(params, p));
   const TokLayout L = tok_layout(B, cu_tokens, D);
   if (ws == nullptr || ws_bytes < L.total || reinterpret_cast<uintptr_t>(ws) % 16) return PACE_ERR_WORKSPACE;
   PACE_CHECK(check_device());
@@ -1878,8 +2168,7 @@ extern "C" pace_status_t pace_apc_density_tokens(const void* T, const int32_t* c
     apc_tok_pass2<<<units, kApcThreads, 0, stream>>>(T32, tt, inv, sums, d_out, stats, work);
     PACE_CHECK(check_launch());
     TailParams tp{p.alpha, p.gamma, p.r_min, p.r_max, p.align};
-    launch_tail_scan(at, d_out, tp, stats, work, stream);
-    PACE_CHECK(check_launch());
+    PACE_CHECK(launch_tail(at, d_out, tp, stats, work, stream));
   }
   return PACE_OK;
 }
@@ -1890,39 +2179,10 @@ extern "C" pace_status_t pace_apc_density_tokens(const void* T, const int32_t* c
 namespace pace {
 namespace {
 
-// Strip table of images c0 .. c0 + nb - 1 (as the density passes build it); false if an image
-// is not laid out for 4-byte copies (then the narrow loader is used).
-bool fill_strip_table(ApcTable& t, int c0, int nb, const int64_t* img_off, const int32_t* H, const int32_t* W,
-                      float tail_frac, int& patch0) {
-  bool wide = true;
-  t = ApcTable{};
-  t.nb = nb;
-  t.b_base = c0;
-  t.unit_prefix[0] = 0;
-  for (int i = 0; i < nb; ++i) {
-    const int b = c0 + i;
-    t.off[i] = img_off[b];
-    t.H[i] = H[b];
-    t.W[i] = W[b];
-    t.gw[i] = W[b] / kPatch;
-    t.chunks[i] = (t.gw[i] + kStrip - 1) / kStrip;
-    t.patch0[i] = patch0;
-    const int N = (H[b] / kPatch) * t.gw[i];
-    t.n[i] = N;
-    double kt = std::floor(static_cast<double>(tail_frac) * N + 0.5);
-    if (kt < 1) kt = 1;
-    if (kt > N) kt = N;
-    t.ktail[i] = static_cast<int>(kt);
-    patch0 += N;
-    t.unit_prefix[i + 1] = t.unit_prefix[i] + (H[b] / kPatch) * t.chunks[i];
-    if ((static_cast<int64_t>(W[b]) * 3) % 4 != 0 || (t.gw[i] % 2) != 0 || (img_off[b] % 4) != 0) wide = false;
-  }
-  return wide;
-}
-
-pace_status_t launch_pix_features(const uint8_t* img, const ApcTable& t, bool wide, int feature, float* tokens,
+pace_status_t launch_pix_features(const uint8_t* img, const ApcTable& t, int feature, float* tokens,
                                   cudaStream_t stream) {
   const int units = t.unit_prefix[t.nb];
+  const bool wide = rows_aligned(t);
   if (wide) apc_pix_features<true><<<strip_grid(units), kApcThreads, 0, stream>>>(img, t, units, feature, tokens);
   else apc_pix_features<false><<<strip_grid(units), kApcThreads, 0, stream>>>(img, t, units, feature, tokens);
   return check_launch();
@@ -1948,8 +2208,8 @@ extern "C" pace_status_t pace_apc_pixel_features(const uint8_t* img, const int64
   int patch0 = 0;
   for (int c0 = 0; c0 < B; c0 += kApcMaxB) {
     ApcTable t;
-    const bool wide = fill_strip_table(t, c0, std::min(kApcMaxB, B - c0), img_off, H, W, 0.1f, patch0);
-    PACE_CHECK(launch_pix_features(img, t, wide, feature, tokens, stream));
+    fill_strip_table(t, c0, std::min(kApcMaxB, B - c0), img_off, H, W, 0.1f, 0, patch0);
+    PACE_CHECK(launch_pix_features(img, t, feature, tokens, stream));
   }
   return PACE_OK;
 }
@@ -1972,10 +2232,7 @@ extern "C" pace_status_t pace_apc_density_pixel(const uint8_t* img, const int64_
   if (feature < kFeatRgb || feature > kFeatLaplacian || d_out == nullptr || stats == nullptr)
     return PACE_ERR_INVALID_ARG;
   pace_apc_params p;
-  if (params) p = *params; else pace_apc_params_default(&p);
-  if (!(p.tail_frac > 0.f && p.tail_frac <= 1.f) || !(p.gamma > 0.f) || !(p.alpha >= 0.f && p.alpha <= 1.f) ||
-      !(p.r_min <= p.r_max) || p.align < 1)
-    return PACE_ERR_INVALID_ARG;
+  PACE_CHECK(check_params(params, p));
   const size_t tok_bytes = align_up(static_cast<size_t>(total_patches(B, H, W)) * kPixDim * sizeof(float), 256);
   if (ws == nullptr || ws_bytes < pace_apc_density_pixel_workspace_size(B, H, W) ||
       reinterpret_cast<uintptr_t>(ws) % 16)
@@ -1990,8 +2247,8 @@ extern "C" pace_status_t pace_apc_density_pixel(const uint8_t* img, const int64_
   for (int c0 = 0; c0 < B; c0 += kApcMaxB) {
     const int nb = std::min(kApcMaxB, B - c0);
     ApcTable at;
-    const bool wide = fill_strip_table(at, c0, nb, img_off, H, W, p.tail_frac, patch0);
-    PACE_CHECK(launch_pix_features(img, at, wide, feature, tokens, stream));
+    fill_strip_table(at, c0, nb, img_off, H, W, p.tail_frac, 0, patch0);
+    PACE_CHECK(launch_pix_features(img, at, feature, tokens, stream));
     PixTable pt{};
     pt.nb = nb;
     pt.b_base = c0;
@@ -2008,8 +2265,7 @@ extern "C" pace_status_t pace_apc_density_pixel(const uint8_t* img, const int64_
     apc_pix_pass2<<<units, kApcThreads, 0, stream>>>(pt, tokens, sums, d_out, stats, work);
     PACE_CHECK(check_launch());
     TailParams tp{p.alpha, p.gamma, p.r_min, p.r_max, p.align};
-    launch_tail_scan(at, d_out, tp, stats, work, stream);
-    PACE_CHECK(check_launch());
+    PACE_CHECK(launch_tail(at, d_out, tp, stats, work, stream));
   }
   return PACE_OK;
 }

@@ -67,11 +67,11 @@ class DeviceOnce {
 
 // Launch with `cluster` blocks along x per cluster and, if `dependent`, programmatic dependent launch.
 template <typename... Params, typename... Args>
-pace_status_t launch_ex(bool dependent, void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem,
+pace_status_t launch_ex(bool dependent, void (*kernel)(Params...), dim3 grid, dim3 threads, size_t smem,
                         unsigned cluster, cudaStream_t stream, Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
-  cfg.blockDim = dim3(threads);
+  cfg.blockDim = threads;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cudaLaunchAttribute at[2] = {};
@@ -94,12 +94,12 @@ pace_status_t launch_ex(bool dependent, void (*kernel)(Params...), dim3 grid, un
 // A kernel that may start while the stream's previous kernel is still running: it calls
 // ptx::grid_dependency_wait() before it reads or writes anything that other work touches.
 template <typename... Params, typename... Args>
-pace_status_t launch_dependent(void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem, unsigned cluster,
+pace_status_t launch_dependent(void (*kernel)(Params...), dim3 grid, dim3 threads, size_t smem, unsigned cluster,
                                cudaStream_t stream, Args... args) {
   return launch_ex(true, kernel, grid, threads, smem, cluster, stream, args...);
 }
 template <typename... Params, typename... Args>
-pace_status_t launch_cluster(void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem, unsigned cluster,
+pace_status_t launch_cluster(void (*kernel)(Params...), dim3 grid, dim3 threads, size_t smem, unsigned cluster,
                              cudaStream_t stream, Args... args) {
   return launch_ex(false, kernel, grid, threads, smem, cluster, stream, args...);
 }

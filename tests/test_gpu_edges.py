@@ -77,3 +77,57 @@ def test_gather_multi_blocks(pace, n_idx):
     assert pace.pace_device_status(clear=True) == (pace.PACE_ERR_INVALID_ARG, 13)
     for b, (_, d) in zip(dst, shapes):
         assert not b.select(d, 0).any()
+
+
+# strips of 8, 16 and 32 patches, full and partial, single last patches (odd widths: image rows on
+# 2-byte boundaries), the last image row's odd end, several images per CTA
+@pytest.mark.parametrize("shapes", [[(14, 14)], [(28, 42)], [(14, 14 * 33)], [(14 * 3, 14 * 31), (14, 14 * 8), (28, 14 * 9)],
+                                    [(14 * 20, 14 * 17)], [(14 * 60, 14 * 35)], [(14 * 100, 14 * 97), (14, 28)]])
+def test_density_strips(pace, shapes):
+    rng = np.random.default_rng(len(shapes) + shapes[0][1])
+    imgs = [synth.make_image(rng, h, w, max(1, w // 90), max(1, h // 90), 0.4) for h, w in shapes]
+    imgs[0][-1, -1] = 255   # the image's very last bytes count
+    buf, off = synth.pack_images(imgs)
+    d, st = pace.pace_apc_density(torch.from_numpy(buf).cuda(), off, [s[0] for s in shapes], [s[1] for s in shapes])
+    d, p0 = d.cpu().numpy(), 0
+    for im, s in zip(imgs, pace.stats_dict(st)):
+        ref = O.apc_density(im)
+        assert_distances_close(d[p0:p0 + ref["N"]], ref["d"])
+        assert abs(s["phi"] - ref["phi"]) <= 1e-5 and abs(s["d_top"] - ref["d_top"]) <= 1e-5
+        p0 += ref["N"]
+
+
+# the black patch's weight is exactly 2^31, the white one's the smallest; identical patches have d = 0
+# up to the rounding of 1/|t| (2^-24 of a unit vector, twice)
+@pytest.mark.parametrize("value", [0, 255])
+def test_density_extreme_values(pace, value):
+    img = np.full((14 * 6, 14 * 40, 3), value, np.uint8)
+    d, st = pace.pace_apc_density(torch.from_numpy(img.reshape(-1)).cuda(), [0], [84], [560])
+    assert d.abs().max().item() <= 4 * 2.0 ** -24 and abs(pace.stats_dict(st)[0]["phi"] - 1) <= 1e-6
+    img[:14, :14] = 255 - value
+    d, _ = pace.pace_apc_density(torch.from_numpy(img.reshape(-1)).cuda(), [0], [84], [560])
+    assert_distances_close(d.cpu().numpy(), O.apc_density(img)["d"])
+
+
+# the tail over a cluster (more than 8192 distances): a bucket of equal distances too many for the
+# list, a list ranked in rounds (quantised values: many equal, several different), a direct ranking
+@pytest.mark.parametrize("kind", ["equal", "steps", "natural"])
+def test_density_tail_cluster(pace, kind):
+    rng = np.random.default_rng(9)
+    side = 14 * 104
+    img = synth.make_image(rng, side, side, 9, 9, 0.3) if kind == "natural" else np.full((side, side, 3), 120, np.uint8)
+    n = 104 * 104
+    for q in (rng.choice(n, size=n // 2 if kind == "steps" else n // 20, replace=False) if kind != "natural" else ()):
+        y, x = divmod(int(q), 104)
+        p = img[14 * y:14 * y + 14, 14 * x:14 * x + 14]
+        if kind == "equal":
+            p[:] = rng.integers(0, 256, p.shape, dtype=np.uint8)
+        else:
+            p[:7] = 120 + (q % 5)   # a few nearby values: thousands of distances in one bucket, five of them different
+    d, st = pace.pace_apc_density(torch.from_numpy(img.reshape(-1)).cuda(), [0], [side], [side])
+    ref = O.apc_density(img)
+    assert_distances_close(d.cpu().numpy(), ref["d"])
+    # the tail of the GPU's own distances, exactly up to fp32 rounding of the mean
+    k = pace.stats_dict(st)[0]["k_tail"]
+    top = np.sort(d.cpu().numpy().astype(np.float64))[::-1][:k].mean()
+    assert abs(pace.stats_dict(st)[0]["d_top"] - top) <= 4e-7 * top + 1e-9
