@@ -700,6 +700,7 @@ struct TokTable {
   int b_base;
   int D;
   int rows1;                     // tokens per pass-1 chunk (a chunk fits a 40 KB stage)
+  int run_prefix[kApcMaxB + 1];  // runs of kTokRun tokens (the register kernels)
 };
 
 constexpr int kTok1StageBytes = 40960;   // one pass-1 stage: rows1 token rows
@@ -748,7 +749,7 @@ __global__ void __launch_bounds__(kApcThreads) apc_tok_pass1(const uint32_t* __r
   int cur_b = -1;
   auto flush = [&]() {
     if (cur_b < 0) return;
-    unsigned long long* sb = sums + static_cast<int64_t>(t.b_base + cur_b) * t.D;
+    unsigned long long* sb = sums + static_cast<int64_t>(t.b_base + cur_b) * kSumSlots * t.D;   // the first copy
 #pragma unroll
     for (int q = 0; q < kTok1MaxSlots; ++q) {
       const int w = threadIdx.x + q * kApcThreads;
@@ -832,7 +833,7 @@ __global__ void __launch_bounds__(kApcThreads) apc_tok_pass2(const uint32_t* __r
   const int N = t.n[b], D = t.D, words = D >> 1;
   const float inv_n = 1.0f / static_cast<float>(N);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const unsigned long long* sb = sums + static_cast<int64_t>(t.b_base + b) * D;
+  const unsigned long long* sb = sums + static_cast<int64_t>(t.b_base + b) * kSumSlots * D;
   float part = 0.f;
   for (int k = threadIdx.x; k < D; k += kApcThreads) {
     const float cv = unfix32<true>(sb[k], inv_n);
@@ -873,6 +874,255 @@ __global__ void __launch_bounds__(kApcThreads) apc_tok_pass2(const uint32_t* __r
       d_out[t.tok0[b] + c0 + p] = dv;
       tail_count(work + t.b_base + b, dv);
     }
+  }
+}
+
+// Token widths of up to 1536 in whole 16-byte vectors (the ViT widths): a warp per token, lane l
+// holding vectors l, l + 32, .. in registers, so a token is read once per pass straight into the
+// norm, the column sums and the distance, with no staging and no block barrier (bound by HBM in
+// pass 1).  Other widths take the staged kernels below.
+constexpr int kTokVecMax = 6;            // 16-byte vectors per lane
+constexpr int kTokThreads = 384;         // of pass 1: one CTA per SM, since each ends an image with D atomics
+constexpr int kTokAhead = 2;             // tokens a warp of pass 1 has in flight
+constexpr int kTokRun = 8;               // tokens (from a multiple of it on) whose column sums stay in fp32
+                                         // before they are rounded, whatever the batch and the grid
+static_assert(kTokRun % kTokAhead == 0, "a run's tokens keep to their buffers");
+
+// 2^-32 fixed point without conversions: v + 1.5 2^11 leaves v rounded to 2^-12 in the low mantissa
+// bits, the exact remainder times 2^32 plus 1.5 2^23 the rest, so acc collects
+// bits(hi) 2^20 + bits(lo), i.e. round(v 2^32) (ties to even, |v| < 2^9) plus the constant kFixBias,
+// which the caller takes off again once per addition.
+constexpr unsigned long long kFixBias = (0x45400000ull << 20) + 0x4B400000ull;
+__device__ __forceinline__ void fix_add(unsigned long long& acc, float v) {
+  const float m = v + 3072.0f;
+  const float l = fmaf(v - (m - 3072.0f), 4294967296.0f, 12582912.0f);
+  acc += static_cast<unsigned long long>(__float_as_uint(m)) * 1048576ull;
+  acc += __float_as_uint(l);
+}
+
+template <int V>
+struct TokRow {
+  uint4 v[V];
+};
+template <int V>
+__device__ __forceinline__ void tok_load(TokRow<V>& r, const uint4* __restrict__ T, int64_t token, int vecs) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int i = 0; i < V; ++i) {
+    const int c = lane + 32 * i;
+    r.v[i] = i < V - 1 || c < vecs ? __ldg(T + token * vecs + c) : make_uint4(0u, 0u, 0u, 0u);
+  }
+}
+__device__ __forceinline__ float2 bf16_pair(uint32_t v) { return make_float2(bf16_lo(v), bf16_hi(v)); }
+__device__ __forceinline__ uint32_t word_of(const uint4& v, int q) { return q == 0 ? v.x : q == 1 ? v.y : q == 2 ? v.z : v.w; }
+
+// CTA c's share [a0, a1) of the table's runs of kTokRun tokens, counted over the images.
+__device__ __forceinline__ void tok_share(const TokTable& t, int& a0, int& a1) {
+  const int64_t runs = t.run_prefix[t.nb];
+  a0 = static_cast<int>(runs * blockIdx.x / gridDim.x);
+  a1 = static_cast<int>(runs * (blockIdx.x + 1) / gridDim.x);
+}
+
+// Pass 1: the warps take the runs of their CTA's share in turn.
+template <int V>
+__global__ void __launch_bounds__(kTokThreads, 1) apc_tok_vec1(const uint4* __restrict__ T,
+                                                               const __grid_constant__ TokTable t,
+                                                               float* __restrict__ inv_norm,
+                                                               unsigned long long* __restrict__ sums) {
+  // [warps][kRow]: a warp's totals, lane-contiguous (no bank conflicts): entry 2 (32 (4 i + e) + lane)
+  // + u is column 8 (lane + 32 i) + 2 e + u
+  extern __shared__ __align__(16) unsigned long long tok_acc[];
+  ptx::launch_dependents();
+  constexpr int kWarps = kTokThreads / 32;
+  const int D = t.D, vecs = D >> 3;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  constexpr int kRow = V * 256;
+  unsigned long long* own = tok_acc + warp * kRow;
+  auto clear_own = [&]() {
+#pragma unroll
+    for (int i = 0; i < 4 * V; ++i) reinterpret_cast<ulonglong2*>(own)[32 * i + lane] = make_ulonglong2(0ull, 0ull);
+  };
+  int a0, a1, cur_b = -1, runs = 0;
+  // adds the CTA's totals of image cur_b (`runs` additions to each column) to the image's sums
+  auto finish = [&]() {
+    ptx::grid_dependency_wait();   // the zeroed sums
+    __syncthreads();
+    if (cur_b < 0) return;
+    const unsigned long long bias = kFixBias * static_cast<unsigned>(runs);
+    unsigned long long* sb = sums + (static_cast<int64_t>(t.b_base + cur_b) * kSumSlots + blockIdx.x % kSumSlots) * D;
+    for (int k = threadIdx.x; k < kRow; k += kTokThreads) {
+      const int c = ((k >> 1) & 31) + 32 * (k >> 8), e = (k >> 6) & 3;   // entry k's vector and word
+      if (c >= vecs) continue;
+      unsigned long long x = 0ull;
+#pragma unroll
+      for (int w = 0; w < kWarps; ++w) x += tok_acc[w * kRow + k];
+      atomicAdd(sb + 8 * c + 2 * e + (k & 1), x - bias);
+    }
+  };
+  tok_share(t, a0, a1);
+  clear_own();
+  for (int b = 0; b < t.nb; ++b) {
+    const int lo = max(a0, t.run_prefix[b]), hi = min(a1, t.run_prefix[b + 1]);
+    if (lo >= hi) continue;
+    if (cur_b >= 0) {   // the CTA moves to the next image
+      finish();
+      __syncthreads();
+      clear_own();
+    }
+    cur_b = b;
+    runs = hi - lo;
+    const int64_t end = t.tok0[b] + t.n[b];
+    auto token = [&](int run, int q) { return t.tok0[b] + static_cast<int64_t>(run - t.run_prefix[b]) * kTokRun + q; };
+    TokRow<V> buf[kTokAhead];
+    auto fetch = [&](TokRow<V>& r, int run, int q) {
+      const int64_t tok = token(run, q);
+      if (run < hi && tok < end) tok_load<V>(r, T, tok, vecs);
+    };
+#pragma unroll
+    for (int r = 0; r < kTokAhead; ++r) fetch(buf[r], lo + warp, r);
+    for (int run = lo + warp; run < hi; run += kWarps) {
+      float2 col[V][4];
+#pragma unroll
+      for (int i = 0; i < V; ++i)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) col[i][e] = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int r = 0; r < kTokRun; ++r) {
+        TokRow<V>& row = buf[r % kTokAhead];
+        if (token(run, r) < end) {   // warp-uniform
+          float2 x[V][4];
+          float2 ss2 = make_float2(0.f, 0.f), ss3 = ss2;
+#pragma unroll
+          for (int i = 0; i < V; ++i)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              x[i][e] = bf16_pair(word_of(row.v[i], e));
+              if (e & 1) ss3 = ptx::ffma2(x[i][e], x[i][e], ss3);
+              else ss2 = ptx::ffma2(x[i][e], x[i][e], ss2);
+            }
+          if (r + kTokAhead < kTokRun) fetch(row, run, r + kTokAhead);
+          else fetch(row, run + kWarps, r + kTokAhead - kTokRun);
+          ss2 = ptx::fadd2(ss2, ss3);
+          const float ss = warp_sum_f(ss2.x + ss2.y);
+          const float iv = ss > 0.f ? 1.0f / sqrtf(ss) : 0.f;
+          if (lane == 0) inv_norm[token(run, r)] = iv;
+          const float2 iv2 = make_float2(iv, iv);
+#pragma unroll
+          for (int i = 0; i < V; ++i)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) col[i][e] = ptx::ffma2(iv2, x[i][e], col[i][e]);
+        }
+      }
+      // the run's sums, rounded to fixed point, into this warp's totals
+#pragma unroll
+      for (int i = 0; i < V; ++i) {
+        const int c = lane + 32 * i;
+        if (i < V - 1 || c < vecs) {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            ulonglong2* p = reinterpret_cast<ulonglong2*>(own) + 32 * (4 * i + e) + lane;
+            ulonglong2 x = *p;
+            fix_add(x.x, fabsf(col[i][e].x) <= kTokRun ? col[i][e].x : 0.f);   // (a NaN counts as 0)
+            fix_add(x.y, fabsf(col[i][e].y) <= kTokRun ? col[i][e].y : 0.f);
+            *p = x;
+          }
+        }
+      }
+    }
+  }
+  finish();
+}
+
+// Pass 2: c = sums / N, phi = |c|^2, c_hat = c / |c| in registers, then d_i = |t_hat_i - c_hat|
+// directly.  The tokens are taken from the last to the first: the last ones read by pass 1 are the
+// ones still in L2.
+template <int V>
+__global__ void __launch_bounds__(kApcThreads, 2) apc_tok_vec2(const uint4* __restrict__ T,
+                                                               const __grid_constant__ TokTable t,
+                                                               const float* __restrict__ inv_norm,
+                                                               const unsigned long long* __restrict__ sums,
+                                                               float* __restrict__ d_out,
+                                                               pace_apc_stats* __restrict__ stats,
+                                                               TailWork* __restrict__ work) {
+  __shared__ __align__(16) float chat[kTokVecMax * 256];
+  __shared__ float red[kApcThreads / 32];
+  ptx::launch_dependents();
+  ptx::grid_dependency_wait();
+  constexpr int kWarps = kApcThreads / 32;
+  const int D = t.D, vecs = D >> 3;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t first = t.tok0[0], total = t.tok0[t.nb - 1] + t.n[t.nb - 1] - first;
+  const int64_t a0 = first + total * blockIdx.x / gridDim.x, a1 = first + total * (blockIdx.x + 1) / gridDim.x;
+  for (int b = t.nb - 1; b >= 0; --b) {
+    const int64_t lo = max(a0, t.tok0[b]), hi = min(a1, t.tok0[b] + t.n[b]);
+    if (lo >= hi) continue;
+    int64_t tok = hi - 1 - warp;
+    TokRow<V> buf[2];
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+      if (tok - r * kWarps >= lo) tok_load<V>(buf[r], T, tok - r * kWarps, vecs);
+    const int N = t.n[b];
+    const float inv_n = 1.0f / static_cast<float>(N);
+    const unsigned long long* sb = sums + static_cast<int64_t>(t.b_base + b) * kSumSlots * D;
+    float part = 0.f;
+    for (int k = threadIdx.x; k < D; k += kApcThreads) {
+      unsigned long long x = 0ull;
+#pragma unroll
+      for (int r = 0; r < kSumSlots; ++r) x += __ldcg(sb + r * D + k);
+      const float cv = unfix32<true>(x, inv_n);
+      chat[k] = cv;
+      part = fmaf(cv, cv, part);
+    }
+    part = warp_sum_f(part);
+    if (lane == 0) red[warp] = part;
+    __syncthreads();
+    float phi = 0.f;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) phi += red[w];
+    const float inv_c = phi > 0.f ? 1.0f / sqrtf(phi) : 0.f;
+    float2 nch[V][4];   // -c_hat of this lane's columns
+#pragma unroll
+    for (int i = 0; i < V; ++i) {
+      const int c = lane + 32 * i;
+      const bool has = i < V - 1 || c < vecs;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float2 x = has ? *reinterpret_cast<const float2*>(chat + 8 * c + 2 * q) : make_float2(0.f, 0.f);
+        nch[i][q] = make_float2(-x.x * inv_c, -x.y * inv_c);
+      }
+    }
+    if (lo == t.tok0[b] && threadIdx.x == 0) {
+      stats[t.b_base + b].phi = phi;
+      stats[t.b_base + b].rho_g = 1.0f - phi;
+      stats[t.b_base + b].n_patches = N;
+      stats[t.b_base + b].k_tail = t.ktail[b];
+    }
+    while (tok >= lo) {
+#pragma unroll
+      for (int r = 0; r < 2; ++r, tok -= kWarps) {
+        if (tok < lo) break;
+        const float iv = __ldcg(inv_norm + tok);
+        const float2 iv2 = make_float2(iv, iv);
+        float2 acc = make_float2(0.f, 0.f), acc1 = acc;
+#pragma unroll
+        for (int i = 0; i < V; ++i)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const float2 e = ptx::ffma2(bf16_pair(word_of(buf[r].v[i], q)), iv2, nch[i][q]);
+            if (q & 1) acc1 = ptx::ffma2(e, e, acc1);
+            else acc = ptx::ffma2(e, e, acc);
+          }
+        if (tok - 2 * kWarps >= lo) tok_load<V>(buf[r], T, tok - 2 * kWarps, vecs);
+        acc = ptx::fadd2(acc, acc1);
+        const float d2 = warp_sum_f(acc.x + acc.y);
+        if (lane == 0) {
+          const float dv = sqrtf(d2);
+          d_out[tok] = dv;
+          tail_count(work + t.b_base + b, dv);
+        }
+      }
+    }
+    __syncthreads();   // chat and red are rewritten for the next image
   }
 }
 
@@ -2090,13 +2340,48 @@ unsigned tok_pass1_grid(int units) {
   return static_cast<unsigned>(std::max(1, std::min(units, c)));
 }
 
+// The two register kernels for V 16-byte vectors per lane.
+template <int V>
+pace_status_t launch_tok_vec_n(const uint4* T, const TokTable& t, unsigned grid, float* d, pace_apc_stats* stats, float* inv,
+                               unsigned long long* sums, TailWork* work, cudaStream_t stream) {
+  constexpr size_t kWarps = kTokThreads / 32;
+  int dev = 0;
+  PACE_CUDA(cudaGetDevice(&dev));
+  static DeviceOnce once;
+  if (!once.done(dev)) {
+    PACE_CUDA(cudaFuncSetAttribute(apc_tok_vec1<V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   static_cast<int>(kWarps * V * 256 * sizeof(unsigned long long))));
+    once.mark(dev);
+  }
+  PACE_CHECK(launch_dependent(apc_tok_vec1<V>, grid, kTokThreads, kWarps * V * 256 * sizeof(unsigned long long), 1, stream, T,
+                              t, inv, sums));
+  return launch_dependent(apc_tok_vec2<V>, 2 * grid, kApcThreads, 0, 1, stream, T, t, static_cast<const float*>(inv),
+                          static_cast<const unsigned long long*>(sums), d, stats, work);
+}
+
+pace_status_t launch_tok_vec(const void* T, const TokTable& t, int64_t tokens, float* d, pace_apc_stats* stats, float* inv,
+                             unsigned long long* sums, TailWork* work, cudaStream_t stream) {
+  int sms = 0;
+  PACE_CHECK(sm_count(&sms));
+  const unsigned grid = static_cast<unsigned>(std::min<int64_t>(sms, (tokens + 7) / 8));
+  const uint4* T4 = static_cast<const uint4*>(T);
+  switch ((t.D + 255) / 256) {
+    case 1: return launch_tok_vec_n<1>(T4, t, grid, d, stats, inv, sums, work, stream);
+    case 2: return launch_tok_vec_n<2>(T4, t, grid, d, stats, inv, sums, work, stream);
+    case 3: return launch_tok_vec_n<3>(T4, t, grid, d, stats, inv, sums, work, stream);
+    case 4: return launch_tok_vec_n<4>(T4, t, grid, d, stats, inv, sums, work, stream);
+    case 5: return launch_tok_vec_n<5>(T4, t, grid, d, stats, inv, sums, work, stream);
+    default: return launch_tok_vec_n<6>(T4, t, grid, d, stats, inv, sums, work, stream);
+  }
+}
+
 struct TokLayout {
   size_t sums_off, work_off, zero_bytes, inv_off, total;   // [0, zero_bytes) is zeroed per call
 };
 TokLayout tok_layout(int B, const int32_t* cu, int D) {
   TokLayout L{};
   L.sums_off = 0;
-  L.work_off = align_up(static_cast<size_t>(B) * D * sizeof(unsigned long long), 256);
+  L.work_off = align_up(static_cast<size_t>(B) * kSumSlots * D * sizeof(unsigned long long), 256);
   L.zero_bytes = L.work_off + static_cast<size_t>(B) * sizeof(TailWork);
   L.inv_off = align_up(L.zero_bytes, 256);
   L.total = L.inv_off + align_up(static_cast<size_t>(cu[B]) * sizeof(float), 256);
@@ -2132,7 +2417,7 @@ extern "C" pace_status_t pace_apc_density_tokens(const void* T, const int32_t* c
   auto* sums = reinterpret_cast<unsigned long long*>(w8 + L.sums_off);
   auto* work = reinterpret_cast<TailWork*>(w8 + L.work_off);
   auto* inv = reinterpret_cast<float*>(w8 + L.inv_off);
-  PACE_CUDA(cudaMemsetAsync(w8, 0, L.zero_bytes, stream));   // column sums and tail scratch
+  PACE_CHECK(launch_zero(w8, L.zero_bytes, nullptr, 0, stream));   // column sums and tail scratch
   const uint32_t* T32 = static_cast<const uint32_t*>(T);
   for (int c0 = 0; c0 < B; c0 += kApcMaxB) {
     const int nb = (B - c0) < kApcMaxB ? (B - c0) : kApcMaxB;
@@ -2144,6 +2429,7 @@ extern "C" pace_status_t pace_apc_density_tokens(const void* T, const int32_t* c
     tt.rows1 = std::max(1, std::min(32, kTok1StageBytes / (D * 2)));
     tt.unit_prefix[0] = 0;
     tt.unit_prefix1[0] = 0;
+    tt.run_prefix[0] = 0;
     for (int i = 0; i < nb; ++i) {
       const int b = c0 + i;
       const int N = cu_tokens[b + 1] - cu_tokens[b];
@@ -2155,9 +2441,18 @@ extern "C" pace_status_t pace_apc_density_tokens(const void* T, const int32_t* c
       tt.ktail[i] = at.ktail[i] = static_cast<int>(kt);
       tt.unit_prefix[i + 1] = tt.unit_prefix[i] + (N + kTokChunk - 1) / kTokChunk;
       tt.unit_prefix1[i + 1] = tt.unit_prefix1[i] + (N + tt.rows1 - 1) / tt.rows1;
+      tt.run_prefix[i + 1] = tt.run_prefix[i] + (N + kTokRun - 1) / kTokRun;
       at.H[i] = H[b];
       at.W[i] = W[b];
       at.patch0[i] = cu_tokens[b];
+    }
+    const TailParams tp{p.alpha, p.gamma, p.r_min, p.r_max, p.align};
+    // whole 16-byte vectors and at most kTokVecMax of them per lane: the register kernels
+    if (D % 8 == 0 && D <= kTokVecMax * 256 && reinterpret_cast<uintptr_t>(T) % 16 == 0) {
+      PACE_CHECK(launch_tok_vec(T, tt, static_cast<int64_t>(cu_tokens[c0 + nb]) - cu_tokens[c0], d_out, stats, inv, sums,
+                                work, stream));
+      PACE_CHECK(launch_tail(at, d_out, tp, stats, work, stream));
+      continue;
     }
     const int units = tt.unit_prefix[nb];
     const int units1 = tt.unit_prefix1[nb];
@@ -2167,7 +2462,6 @@ extern "C" pace_status_t pace_apc_density_tokens(const void* T, const int32_t* c
     PACE_CHECK(check_launch());
     apc_tok_pass2<<<units, kApcThreads, 0, stream>>>(T32, tt, inv, sums, d_out, stats, work);
     PACE_CHECK(check_launch());
-    TailParams tp{p.alpha, p.gamma, p.r_min, p.r_max, p.align};
     PACE_CHECK(launch_tail(at, d_out, tp, stats, work, stream));
   }
   return PACE_OK;

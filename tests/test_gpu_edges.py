@@ -131,3 +131,36 @@ def test_density_tail_cluster(pace, kind):
     k = pace.stats_dict(st)[0]["k_tail"]
     top = np.sort(d.cpu().numpy().astype(np.float64))[::-1][:k].mean()
     assert abs(pace.stats_dict(st)[0]["d_top"] - top) <= 4e-7 * top + 1e-9
+
+
+# register kernels (whole 16-byte vectors, up to 1536) and the staged ones (other widths), runs of 8
+# tokens with remainders, several images per CTA
+@pytest.mark.parametrize("D", [8, 248, 256, 264, 1152, 1536, 1544, 1284, 6])
+@pytest.mark.parametrize("lens", [(1,), (7, 8, 9), (300, 1, 2500)])
+def test_token_widths(pace, D, lens):
+    rng = np.random.default_rng(D)
+    cu = _cu(lens)
+    T = rng.normal(size=D)[None] * rng.uniform(0.5, 2, (int(cu[-1]), 1)) + rng.normal(size=(int(cu[-1]), D))
+    T[0] = 0
+    bits = synth.f32_to_bf16_bits(T.astype(np.float32))
+    sides = [28 * 9] * len(lens)
+    d, st = pace.pace_apc_density_tokens(bf16_tensor(bits), cu, sides, sides)
+    d = d.cpu().numpy()
+    for b, s in enumerate(pace.stats_dict(st)):
+        ref = O.apc_density_preview(f64(bits)[cu[b]:cu[b + 1]], 252, 252)
+        assert_distances_close(d[cu[b]:cu[b + 1]], ref["d"])
+        assert abs(s["phi"] - ref["phi"]) <= 1e-5 and abs(s["d_top"] - ref["d_top"]) <= 1e-5
+    # the same bits in any batch
+    one, _ = pace.pace_apc_density_tokens(bf16_tensor(bits[cu[-2]:cu[-1]]), [0, lens[-1]], [252], [252])
+    np.testing.assert_array_equal(one.cpu().numpy(), d[cu[-2]:cu[-1]])
+
+
+def test_tokens_with_non_finite_rows(pace):
+    """A NaN or infinite token spoils its own distance and leaves the others finite."""
+    rng = np.random.default_rng(2)
+    T = rng.normal(size=(64, 256)).astype(np.float32)
+    bits = synth.f32_to_bf16_bits(T)
+    bits[20, 3], bits[41, 7] = 0x7FC0, 0x7F80
+    d, _ = pace.pace_apc_density_tokens(bf16_tensor(bits), [0, 64], [252], [252])
+    bad = ~np.isfinite(d.cpu().numpy())
+    assert bad[20] and bad.sum() <= 2 and not bad[:20].any()
