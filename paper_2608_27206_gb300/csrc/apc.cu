@@ -37,7 +37,6 @@ constexpr int kPatch = 14;
 constexpr int kPatchBytes = kPatch * kPatch * 3;     // 588
 constexpr int kTokDim = kPatchBytes + 1;             // 589: pixels + constant coordinate
 constexpr int kStrip = 32;                           // patches per strip
-constexpr int kStripRowBytes = kStrip * kPatch * 3;  // 1344 bytes of one image row per strip
 constexpr int kApcThreads = 256;
 constexpr int kApcMaxB = 64;
 // Column sums are 2^-32 fixed point in 64-bit integers.  The conversions below use only 32-bit
@@ -93,57 +92,10 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait_group() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// Stages the 14 rows x (np * 42) bytes of one strip into s (row pitch kStripRowBytes).  WIDE:
-// asynchronous copies that the caller commits and waits for; otherwise plain loads and stores.
-// Either way the caller synchronises the block before reading s.
-template <bool WIDE>
-__device__ __forceinline__ void load_strip(const uint8_t* __restrict__ img, int W, int py, int px0, int np,
-                                           uint8_t* s) {
-  const int seg = np * kPatch * 3;  // bytes per row (even; a multiple of 4 when WIDE)
-  const int64_t pitch = static_cast<int64_t>(W) * 3;
-  const uint8_t* base = img + static_cast<int64_t>(py) * kPatch * pitch + static_cast<int64_t>(px0) * kPatch * 3;
-  // a warp per image row (rows warp, warp + 8), lanes along the row: no per-element division
-  const int lane = threadIdx.x & 31;
-  for (int y = threadIdx.x >> 5; y < kPatch; y += kApcThreads / 32) {
-    const uint8_t* src = base + y * pitch;
-    uint8_t* dst = s + y * kStripRowBytes;
-    if (WIDE) {
-      const int words = seg >> 2;
-      for (int w = lane; w < words; w += 32)
-        cp_async4(dst + 4 * w, reinterpret_cast<const uint32_t*>(src) + w);
-    } else {
-      const int halves = seg >> 1;
-      for (int w = lane; w < halves; w += 32)
-        *reinterpret_cast<uint16_t*>(dst + 2 * w) = __ldg(reinterpret_cast<const uint16_t*>(src) + w);
-    }
-  }
-}
-
 __device__ __forceinline__ float warp_sum_f(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
-}
-
-struct Strip {
-  int b, u, py, px0, np;
-};
-
-__device__ __forceinline__ Strip strip_of(const ApcTable& t, int unit) {
-  Strip q;
-  q.b = find_image(t, unit);
-  q.u = unit - t.unit_prefix[q.b];
-  q.py = q.u / t.chunks[q.b];
-  q.px0 = (q.u - q.py * t.chunks[q.b]) * kStrip;
-  q.np = min(kStrip, t.gw[q.b] - q.px0);
-  return q;
-}
-
-template <bool WIDE>
-__device__ __forceinline__ void issue_strip(const uint8_t* __restrict__ img, const ApcTable& t, int unit, uint8_t* s) {
-  const Strip q = strip_of(t, unit);
-  load_strip<WIDE>(img + t.off[q.b], t.W[q.b], q.py, q.px0, q.np, s);
-  cp_async_commit();
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -536,6 +488,19 @@ struct Pass2Group {
   uint64_t bars[2];
   StripRef ref[2];
 };
+// The same for a warp whose lanes often hold equal distances (a preview with few values): one
+// addition per different value.
+__device__ __forceinline__ void tail_count_warp(TailWork* w, float d, bool live) {
+  const unsigned act = __ballot_sync(0xffffffffu, live);
+  if (!live) return;
+  const unsigned peers = __match_any_sync(act, __float_as_uint(d));
+  if ((threadIdx.x & 31) != static_cast<unsigned>(__ffs(peers) - 1)) return;
+  const unsigned n = static_cast<unsigned>(__popc(peers));
+  const int b = tail_bucket(d);
+  atomicAdd(&w->hist[b], n);
+  atomicAdd(&w->sum[b], fix32(d) * n);
+}
+
 struct Pass2Smem {
   Pass2Group g[kDGroups];
   // the four bytes of c_hat (2^-32 fixed point) of a pair's words, the two patches one after the
@@ -1448,16 +1413,19 @@ __device__ __forceinline__ long long warp_sum_ll(long long v) {
   return v;
 }
 
-// One warp computes the feature token of the patch at `px` (staged strip, row pitch
-// kStripRowBytes): out[0 .. kPixDim).  `luma` (196 ints) and `hist` (48 ints) are the warp's
-// scratch in shared memory.
-__device__ __forceinline__ void patch_feature(const uint8_t* px, int feature, int* luma, int* hist, float* out) {
+// One warp computes the feature token of the patch whose pixel (y, x) is staged at px(y, x), the same
+// in every lane.  `luma` (196 ints) is the warp's scratch in shared memory (the entropy's 48 counts
+// take its start).
+template <typename Pixel>
+__device__ __forceinline__ void patch_feature(Pixel px, int feature, int* luma, float (&tok)[kPixDim]) {
   const int lane = threadIdx.x & 31;
-  float tok[kPixDim] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  int* hist = luma;
+#pragma unroll
+  for (int k = 0; k < kPixDim; ++k) tok[k] = 0.f;
   if (feature == kFeatRgb) {
     uint32_t s[3] = {0u, 0u, 0u}, q[3] = {0u, 0u, 0u};
     for (int i = lane; i < kPatch * kPatch; i += 32) {
-      const uint8_t* p = px + (i / kPatch) * kStripRowBytes + (i % kPatch) * 3;
+      const uint8_t* p = px(i / kPatch, i % kPatch);
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         const uint32_t v = p[c];
@@ -1478,7 +1446,7 @@ __device__ __forceinline__ void patch_feature(const uint8_t* px, int feature, in
     for (int i = lane; i < 48; i += 32) hist[i] = 0;
     __syncwarp();
     for (int i = lane; i < kPatch * kPatch; i += 32) {
-      const uint8_t* p = px + (i / kPatch) * kStripRowBytes + (i % kPatch) * 3;
+      const uint8_t* p = px(i / kPatch, i % kPatch);
 #pragma unroll
       for (int c = 0; c < 3; ++c) atomicAdd(&hist[c * 16 + (p[c] >> 4)], 1);
     }
@@ -1500,7 +1468,7 @@ __device__ __forceinline__ void patch_feature(const uint8_t* px, int feature, in
     __syncwarp();   // hist is rewritten by the warp's next patch
   } else {
     for (int i = lane; i < kPatch * kPatch; i += 32) {
-      const uint8_t* p = px + (i / kPatch) * kStripRowBytes + (i % kPatch) * 3;
+      const uint8_t* p = px(i / kPatch, i % kPatch);
       luma[i] = kLumaR * p[0] + kLumaG * p[1] + kLumaB * p[2];
     }
     __syncwarp();
@@ -1531,48 +1499,92 @@ __device__ __forceinline__ void patch_feature(const uint8_t* px, int feature, in
     tok[1] = 1.f;
     __syncwarp();   // luma is rewritten by the warp's next patch
   }
-  if (lane < kPixDim) {
-    float v = tok[0];
-#pragma unroll
-    for (int k = 1; k < kPixDim; ++k)
-      if (lane == k) v = tok[k];
-    out[lane] = v;
-  }
 }
 
 // Feature tokens of every patch: a resident grid over the strips (as the density passes),
-// a warp per patch.
-template <bool WIDE>
-__global__ void __launch_bounds__(kApcThreads) apc_pix_features(const uint8_t* __restrict__ img,
-                                                                const __grid_constant__ ApcTable t, int units,
-                                                                int feature, float* __restrict__ tokens) {
-  __shared__ __align__(16) uint8_t s2[2][kPatch * kStripRowBytes];
-  __shared__ int luma[kApcThreads / 32][kPatch * kPatch];
-  __shared__ int hist[kApcThreads / 32][48];
-  int unit = blockIdx.x;
-  if (unit >= units) return;
-  const int warp = threadIdx.x >> 5;
-  issue_strip<WIDE>(img, t, unit, s2[0]);
-  for (int i = 0; unit < units; ++i, unit += gridDim.x) {
-    const int next = unit + static_cast<int>(gridDim.x);
-    if (next < units) {
-      issue_strip<WIDE>(img, t, next, s2[(i + 1) & 1]);
-      cp_async_wait_group<1>();
-    } else {
-      cp_async_wait_group<0>();
+// a warp per patch.  DENSITY: the tokens are stored l2-normalised and their column sums added to
+// `sums` in 2^-32 fixed point (each token exactly rounded, so the order does not matter): one atomic
+// per coordinate and CTA into one of kPixSlots copies, which keeps the CTAs off each other's words.
+constexpr int kPixSlots = 16;
+constexpr int kPixCtasPerSm = 4;
+template <bool DENSITY>
+__global__ void __launch_bounds__(kApcThreads, kPixCtasPerSm) apc_pix_features(const uint8_t* __restrict__ img,
+                                                                               const __grid_constant__ ApcTable t,
+                                                                               int units, int feature,
+                                                                               float* __restrict__ tokens,
+                                                                               unsigned long long* __restrict__ sums,
+                                                                               int* status) {
+  constexpr int kWarps = kApcThreads / 32;
+  __shared__ __align__(16) uint8_t s2[2][kStageBytes];
+  __shared__ int luma[kWarps][kPatch * kPatch];
+  __shared__ unsigned long long part[kWarps][kPixDim];
+  __shared__ uint64_t bars[2];
+  __shared__ StripRef ref[2];
+  ptx::launch_dependents();
+  const int2 range = unit_range(units);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  unsigned long long acc = 0ull;   // lane k < kPixDim: coordinate k
+  if (threadIdx.x == 0) {
+    ptx::mbar_init(ptx::smem_u32(&bars[0]), 1);
+    ptx::mbar_init(ptx::smem_u32(&bars[1]), 1);
+    ptx::fence_mbar_init();
+  }
+  __syncthreads();
+  StripPipe<1> pipe{s2, bars, ref, 0u};
+  int first = range.x;
+  for (int b = first < range.y ? find_image(t, first) : 0; first < range.y; ++b) {   // the CTA's strips of image b
+    const int end = min(range.y, t.unit_prefix[b + 1]);
+    if (warp == 0) pipe.begin(img, t, first, end);
+    for (int unit = first; unit < end; ++unit, ++pipe.used) {
+      if (!pipe.wait()) record_error(status, PACE_ERR_TIMEOUT, K_APC_PASS1);
+      const StripRef cur = pipe.place();
+      const uint8_t* s = pipe.data();
+      if (unit > first && unit + 1 < end) {
+        __syncthreads();   // everyone is done with the other buffer
+        if (warp == 0) pipe.next(img, t, cur);
+      }
+      const int64_t p0 = static_cast<int64_t>(t.patch0[b]) + cur.py * t.gw[b] + cur.px0;
+      for (int p = warp; p < cur.np; p += kWarps) {
+        float tok[kPixDim];
+        patch_feature([&](int y, int x) { return s + y * kStageRow + row_phase(cur, y) + (p * kPatch + x) * 3; }, feature,
+                      luma[warp], tok);
+        if (DENSITY) {
+          float n2 = 0.f;
+#pragma unroll
+          for (int k = 0; k < kPixDim; ++k) n2 = fmaf(tok[k], tok[k], n2);
+          const float iv = n2 > 0.f ? 1.0f / sqrtf(n2) : 0.f;
+#pragma unroll
+          for (int k = 0; k < kPixDim; ++k) tok[k] *= iv;
+        }
+        float v = tok[0];
+#pragma unroll
+        for (int k = 1; k < kPixDim; ++k)
+          if (lane == k) v = tok[k];
+        if (lane < kPixDim) {
+          tokens[(p0 + p) * kPixDim + lane] = v;
+          if (DENSITY) acc += fix32_signed(v);
+        }
+      }
+    }
+    if (DENSITY) {   // the image's sums
+      if (lane < kPixDim) part[warp][lane] = acc;
+      acc = 0ull;
+      ptx::grid_dependency_wait();   // the zeroed sums
     }
     __syncthreads();
-    const Strip q = strip_of(t, unit);
-    const uint8_t* s = s2[i & 1];
-    for (int p = warp; p < q.np; p += kApcThreads / 32)
-      patch_feature(s + p * 42, feature, luma[warp], hist[warp],
-                    tokens + (static_cast<int64_t>(t.patch0[q.b]) + q.py * t.gw[q.b] + q.px0 + p) * kPixDim);
-    __syncthreads();   // this buffer is refilled two strips on
+    if (DENSITY && threadIdx.x < kPixDim) {
+      unsigned long long x = 0ull;
+#pragma unroll
+      for (int w = 0; w < kWarps; ++w) x += part[w][threadIdx.x];
+      atomicAdd(sums + (static_cast<int64_t>(t.b_base + b) * kPixSlots + blockIdx.x % kPixSlots) * kPixDim + threadIdx.x, x);
+    }
+    first = end;
+    if (DENSITY && first < range.y) __syncthreads();   // `part` is rewritten
   }
 }
 
-// Density of kPixDim-float tokens, pass 1: t_hat in place and the chunk's column sums (2^-32
-// fixed point, deterministic).  A CTA takes kApcThreads tokens of one image, a thread per token.
+// The density of the normalised tokens: a CTA takes kApcThreads tokens of one image, a thread per
+// token.
 struct PixTable {
   int tok0[kApcMaxB];
   int n[kApcMaxB];
@@ -1588,42 +1600,6 @@ __device__ __forceinline__ int find_pix_image(const PixTable& t, int unit) {
   return b;
 }
 
-__global__ void __launch_bounds__(kApcThreads) apc_pix_pass1(const __grid_constant__ PixTable t,
-                                                             float* __restrict__ tokens,
-                                                             unsigned long long* __restrict__ sums) {
-  __shared__ float part[kApcThreads / 32][kPixDim];
-  const int b = find_pix_image(t, blockIdx.x);
-  const int i = (blockIdx.x - t.unit_prefix[b]) * kApcThreads + threadIdx.x;
-  const bool live = i < t.n[b];
-  float v[kPixDim] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  float4* row = reinterpret_cast<float4*>(tokens + (static_cast<int64_t>(t.tok0[b]) + (live ? i : 0)) * kPixDim);
-  if (live) {
-    const float4 a = row[0], c = row[1];
-    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = c.x; v[5] = c.y; v[6] = c.z; v[7] = c.w;
-    float n2 = 0.f;
-#pragma unroll
-    for (int k = 0; k < kPixDim; ++k) n2 = fmaf(v[k], v[k], n2);
-    const float iv = n2 > 0.f ? 1.0f / sqrtf(n2) : 0.f;
-#pragma unroll
-    for (int k = 0; k < kPixDim; ++k) v[k] *= iv;
-    row[0] = make_float4(v[0], v[1], v[2], v[3]);
-    row[1] = make_float4(v[4], v[5], v[6], v[7]);
-  }
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-  for (int k = 0; k < kPixDim; ++k) {
-    const float w = warp_sum_f(v[k]);
-    if (lane == 0) part[warp][k] = w;
-  }
-  __syncthreads();
-  if (threadIdx.x < kPixDim) {
-    float a = 0.f;
-#pragma unroll
-    for (int w = 0; w < kApcThreads / 32; ++w) a += part[w][threadIdx.x];
-    atomicAdd(sums + static_cast<int64_t>(t.b_base + b) * kPixDim + threadIdx.x, fix32_signed(a));
-  }
-}
-
 // Pass 2: c = sums / N, phi = |c|^2, c_hat = c / |c|, d_i = |t_hat_i - c_hat| (thread per token).
 __global__ void __launch_bounds__(kApcThreads) apc_pix_pass2(const __grid_constant__ PixTable t,
                                                              const float* __restrict__ tokens,
@@ -1631,16 +1607,30 @@ __global__ void __launch_bounds__(kApcThreads) apc_pix_pass2(const __grid_consta
                                                              float* __restrict__ d_out,
                                                              pace_apc_stats* __restrict__ stats,
                                                              TailWork* __restrict__ work) {
+  __shared__ unsigned long long csum[kPixDim];
+  ptx::launch_dependents();
+  ptx::grid_dependency_wait();
   const int b = find_pix_image(t, blockIdx.x);
   const int u = blockIdx.x - t.unit_prefix[b];
   const int i = u * kApcThreads + threadIdx.x;
   const int N = t.n[b];
+  const bool live = i < N;
+  const float4* row = reinterpret_cast<const float4*>(tokens + (static_cast<int64_t>(t.tok0[b]) + (live ? i : 0)) * kPixDim);
+  const float4 a = __ldcg(row), e = __ldcg(row + 1);
+  if (threadIdx.x < kPixDim) {
+    const unsigned long long* sb = sums + static_cast<int64_t>(t.b_base + b) * kPixSlots * kPixDim + threadIdx.x;
+    unsigned long long x = 0ull;
+#pragma unroll
+    for (int k = 0; k < kPixSlots; ++k) x += __ldcg(sb + k * kPixDim);
+    csum[threadIdx.x] = x;
+  }
+  __syncthreads();
   const float inv_n = 1.0f / static_cast<float>(N);
   float c[kPixDim];
   float phi = 0.f;
 #pragma unroll
   for (int k = 0; k < kPixDim; ++k) {
-    c[k] = unfix32<true>(sums[static_cast<int64_t>(t.b_base + b) * kPixDim + k], inv_n);
+    c[k] = unfix32<true>(csum[k], inv_n);
     phi = fmaf(c[k], c[k], phi);
   }
   const float inv_c = phi > 0.f ? 1.0f / sqrtf(phi) : 0.f;
@@ -1650,9 +1640,6 @@ __global__ void __launch_bounds__(kApcThreads) apc_pix_pass2(const __grid_consta
     stats[t.b_base + b].n_patches = N;
     stats[t.b_base + b].k_tail = t.ktail[b];
   }
-  if (i >= N) return;
-  const float4* row = reinterpret_cast<const float4*>(tokens + (static_cast<int64_t>(t.tok0[b]) + i) * kPixDim);
-  const float4 a = row[0], e = row[1];
   const float v[kPixDim] = {a.x, a.y, a.z, a.w, e.x, e.y, e.z, e.w};
   float acc = 0.f;
 #pragma unroll
@@ -1661,8 +1648,8 @@ __global__ void __launch_bounds__(kApcThreads) apc_pix_pass2(const __grid_consta
     acc = fmaf(x, x, acc);
   }
   const float dv = sqrtf(acc);
-  d_out[t.tok0[b] + i] = dv;
-  tail_count(work + t.b_base + b, dv);
+  if (live) d_out[t.tok0[b] + i] = dv;
+  tail_count_warp(work + t.b_base + b, dv, live);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -2008,22 +1995,6 @@ DensityLayout density_layout(int B, const int32_t* H, const int32_t* W) {
   L.d_off = L.sumsq_off + align_up(static_cast<size_t>(n) * sizeof(float), 256);
   L.total = L.d_off + align_up(static_cast<size_t>(n) * sizeof(float), 256);
   return L;
-}
-
-// Grid of the strip walks: the CTAs that are resident at once (capped by the strips).
-unsigned strip_grid(int units) {
-  static std::atomic<int> cap[64];
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) dev = 0;
-  int c = cap[dev & 63].load(std::memory_order_relaxed);
-  if (c == 0) {
-    int nsm = 0, per = 0;
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, apc_pix_features<true>, kApcThreads, 0);
-    c = std::max(1, nsm * std::max(per, 1));
-    cap[dev & 63].store(c, std::memory_order_relaxed);
-  }
-  return static_cast<unsigned>(std::max(1, std::min(units, c)));
 }
 
 // Launches apc_tail on one ApcTable: a cluster of CTAs per image, one CTA when every image's
@@ -2473,12 +2444,20 @@ extern "C" pace_status_t pace_apc_density_tokens(const void* T, const int32_t* c
 namespace pace {
 namespace {
 
-pace_status_t launch_pix_features(const uint8_t* img, const ApcTable& t, int feature, float* tokens,
-                                  cudaStream_t stream) {
-  const int units = t.unit_prefix[t.nb];
-  const bool wide = rows_aligned(t);
-  if (wide) apc_pix_features<true><<<strip_grid(units), kApcThreads, 0, stream>>>(img, t, units, feature, tokens);
-  else apc_pix_features<false><<<strip_grid(units), kApcThreads, 0, stream>>>(img, t, units, feature, tokens);
+// Fills t for images c0 .. c0 + nb - 1 and launches the feature kernel on them (sums: null for the
+// tokens alone).
+pace_status_t launch_pix_features(const uint8_t* img, ApcTable& t, int c0, int nb, const int64_t* img_off, const int32_t* H,
+                                  const int32_t* W, float tail_frac, int& patch0, int feature, float* tokens,
+                                  unsigned long long* sums, cudaStream_t stream) {
+  int sms = 0;
+  PACE_CHECK(sm_count(&sms));
+  fill_strip_table(t, c0, nb, img_off, H, W, tail_frac, kPixCtasPerSm * sms, patch0);
+  const int units = t.unit_prefix[nb];
+  const unsigned grid = static_cast<unsigned>(std::min(units, kPixCtasPerSm * sms));
+  int* status = device_status_word();
+  if (sums != nullptr)
+    return launch_dependent(apc_pix_features<true>, grid, kApcThreads, 0, 1, stream, img, t, units, feature, tokens, sums, status);
+  apc_pix_features<false><<<grid, kApcThreads, 0, stream>>>(img, t, units, feature, tokens, sums, status);
   return check_launch();
 }
 
@@ -2502,8 +2481,8 @@ extern "C" pace_status_t pace_apc_pixel_features(const uint8_t* img, const int64
   int patch0 = 0;
   for (int c0 = 0; c0 < B; c0 += kApcMaxB) {
     ApcTable t;
-    fill_strip_table(t, c0, std::min(kApcMaxB, B - c0), img_off, H, W, 0.1f, 0, patch0);
-    PACE_CHECK(launch_pix_features(img, t, feature, tokens, stream));
+    PACE_CHECK(launch_pix_features(img, t, c0, std::min(kApcMaxB, B - c0), img_off, H, W, 0.1f, patch0, feature, tokens,
+                                   nullptr, stream));
   }
   return PACE_OK;
 }
@@ -2513,7 +2492,7 @@ extern "C" size_t pace_apc_density_pixel_workspace_size(int B, const int32_t* H,
   for (int b = 0; b < B; ++b)
     if (H[b] < kPatch || W[b] < kPatch) return 0;
   return align_up(static_cast<size_t>(total_patches(B, H, W)) * kPixDim * sizeof(float), 256) +
-         align_up(static_cast<size_t>(B) * kPixDim * sizeof(unsigned long long), 256) +
+         align_up(static_cast<size_t>(B) * kPixSlots * kPixDim * sizeof(unsigned long long), 256) +
          static_cast<size_t>(B) * sizeof(TailWork);
 }
 
@@ -2534,15 +2513,14 @@ extern "C" pace_status_t pace_apc_density_pixel(const uint8_t* img, const int64_
   PACE_CHECK(check_device());
   auto* tokens = static_cast<float*>(ws);
   auto* sums = reinterpret_cast<unsigned long long*>(static_cast<uint8_t*>(ws) + tok_bytes);
-  const size_t sums_bytes = align_up(static_cast<size_t>(B) * kPixDim * sizeof(unsigned long long), 256);
+  const size_t sums_bytes = align_up(static_cast<size_t>(B) * kPixSlots * kPixDim * sizeof(unsigned long long), 256);
   auto* work = reinterpret_cast<TailWork*>(reinterpret_cast<uint8_t*>(sums) + sums_bytes);
-  PACE_CUDA(cudaMemsetAsync(sums, 0, sums_bytes + static_cast<size_t>(B) * sizeof(TailWork), stream));   // sums, tail scratch
+  PACE_CHECK(launch_zero(sums, sums_bytes, work, static_cast<size_t>(B) * sizeof(TailWork), stream));
   int patch0 = 0;
   for (int c0 = 0; c0 < B; c0 += kApcMaxB) {
     const int nb = std::min(kApcMaxB, B - c0);
     ApcTable at;
-    fill_strip_table(at, c0, nb, img_off, H, W, p.tail_frac, 0, patch0);
-    PACE_CHECK(launch_pix_features(img, at, feature, tokens, stream));
+    PACE_CHECK(launch_pix_features(img, at, c0, nb, img_off, H, W, p.tail_frac, patch0, feature, tokens, sums, stream));
     PixTable pt{};
     pt.nb = nb;
     pt.b_base = c0;
@@ -2554,10 +2532,9 @@ extern "C" pace_status_t pace_apc_density_pixel(const uint8_t* img, const int64_
       pt.unit_prefix[i + 1] = pt.unit_prefix[i] + (at.n[i] + kApcThreads - 1) / kApcThreads;
     }
     const int units = pt.unit_prefix[nb];
-    apc_pix_pass1<<<units, kApcThreads, 0, stream>>>(pt, tokens, sums);
-    PACE_CHECK(check_launch());
-    apc_pix_pass2<<<units, kApcThreads, 0, stream>>>(pt, tokens, sums, d_out, stats, work);
-    PACE_CHECK(check_launch());
+    PACE_CHECK(launch_dependent(apc_pix_pass2, static_cast<unsigned>(units), kApcThreads, 0, 1, stream, pt,
+                                static_cast<const float*>(tokens), static_cast<const unsigned long long*>(sums), d_out,
+                                stats, work));
     TailParams tp{p.alpha, p.gamma, p.r_min, p.r_max, p.align};
     PACE_CHECK(launch_tail(at, d_out, tp, stats, work, stream));
   }
