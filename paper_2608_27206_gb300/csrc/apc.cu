@@ -12,9 +12,9 @@
 //   apc_tail   the k_tail-th largest's bucket from the counts, its members from the distances, the
 //              tail mean, rho_d, rho, r and the target size.  The token and pixel-statistic
 //              densities share it (their pass 2 fills the buckets the same way).
-// Resize: apc_resample, four CTAs per SM walking the 16 x 32 output tiles of the batch; for
-// downscales up to 2.75x per side the input window is staged in shared memory and filtered
-// there with precomputed weights, steeper downscales take a generic path with per-tap weights.
+// Resize: apc_resample, four CTAs per SM walking the output tiles of the batch; downscales of up to 8x
+// per side are filtered vertically in registers, then horizontally from shared memory, steeper ones
+// take a generic path with per-tap weights.
 #include <algorithm>
 #include <atomic>
 #include <cfloat>
@@ -87,7 +87,6 @@ __device__ __forceinline__ void cp_async4(void* dst, const void* src) {
                "l"(src)
                : "memory");
 }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait_group() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
@@ -1655,8 +1654,8 @@ __global__ void __launch_bounds__(kApcThreads) apc_pix_pass2(const __grid_consta
 // ------------------------------------------------------------------------------------------------
 // resample
 // ------------------------------------------------------------------------------------------------
-constexpr int kRsThreads = 256;  // threads of a resample CTA
-constexpr int kRsTH = 8;         // output rows of a generic tile (kRsTH x kRsTW = kRsThreads)
+constexpr int kRsThreads = 128;  // threads of a resample CTA
+constexpr int kRsTH = 4;         // output rows of a generic tile (kRsTH x kRsTW = kRsThreads)
 constexpr int kRsTW = 32;        // output columns of a generic tile
 constexpr int kRsChunk = 8;      // input rows filtered per step of the generic path
 
@@ -1680,7 +1679,6 @@ __device__ __forceinline__ float cubic_w(float t) {
 }
 
 __device__ __forceinline__ int64_t floor_div(int64_t x, int64_t d) { return x >= 0 ? x / d : -((-x + d - 1) / d); }
-__device__ __forceinline__ int64_t ceil_div(int64_t x, int64_t d) { return x >= 0 ? (x + d - 1) / d : -((-x) / d); }
 
 // Window of output index o (reading R5) in exact integer arithmetic.  With s = n_in / n_out
 // and fs = max(s, 1), the centre is c = (2o + 1) n_in / (2 n_out), the taps are
@@ -1696,8 +1694,14 @@ __device__ __forceinline__ Win exact_window(int o, int n_in, int n_out) {
   const int64_t cn = (2 * static_cast<int64_t>(o) + 1) * n_in;                   // c * 2 n_out
   const int64_t sup = 4 * static_cast<int64_t>(down ? n_in : n_out);           // 2 fs * 2 n_out
   const int64_t d = 2 * static_cast<int64_t>(n_out);
-  int64_t a = floor_div(cn - sup, d), e = ceil_div(cn + sup, d);
-  if (a < 0) a = 0;
+  int64_t a = max(cn - sup, static_cast<int64_t>(0)), e = cn + sup + d - 1;
+  if (e < (int64_t{1} << 32)) {   // a 32-bit division is several times cheaper
+    a = static_cast<uint32_t>(a) / static_cast<uint32_t>(d);
+    e = static_cast<uint32_t>(e) / static_cast<uint32_t>(d);
+  } else {
+    a /= d;
+    e /= d;
+  }
   if (e > n_in) e = n_in;
   Win w;
   w.lo = static_cast<int>(a);
@@ -1721,14 +1725,21 @@ __device__ __forceinline__ void window_1d(int o, int n_in, int n_out, int& lo, i
   inorm = 1.0f / s;
 }
 
-// Any downscale: one 4 x 32 output tile, weights evaluated per tap, input read through L1.
-__device__ void resample_tile_generic(const uint8_t* __restrict__ img, int H, int W, int Ho, int Wo, int ox0,
+// Steep downscales: one 4 x 32 output tile, weights evaluated per tap, input read through L1.
+struct GenericSmem {
+  int xlo[kRsTW], xn[kRsTW];
+  float xoff[kRsTW], xifs[kRsTW], xnorm[kRsTW];
+  int ylo[kRsTH], yn[kRsTH];
+  float yoff[kRsTH], yifs[kRsTH], ynorm[kRsTH];
+  float hbuf[kRsChunk][kRsTW][3];
+};
+__device__ void resample_tile_generic(GenericSmem& sh, const uint8_t* __restrict__ img, int H, int W, int Ho, int Wo, int ox0,
                                       int oy0, uint8_t* __restrict__ out) {
-  __shared__ int xlo[kRsTW], xn[kRsTW];
-  __shared__ float xoff[kRsTW], xifs[kRsTW], xnorm[kRsTW];
-  __shared__ int ylo[kRsTH], yn[kRsTH];
-  __shared__ float yoff[kRsTH], yifs[kRsTH], ynorm[kRsTH];
-  __shared__ float hbuf[kRsChunk][kRsTW][3];
+  auto &xlo = sh.xlo, &xn = sh.xn;
+  auto &xoff = sh.xoff, &xifs = sh.xifs, &xnorm = sh.xnorm;
+  auto &ylo = sh.ylo, &yn = sh.yn;
+  auto &yoff = sh.yoff, &yifs = sh.yifs, &ynorm = sh.ynorm;
+  auto& hbuf = sh.hbuf;
   if (ox0 >= Wo || oy0 >= Ho) return;
   const int tid = threadIdx.x;
   if (tid < kRsTW) {
@@ -1791,166 +1802,323 @@ __device__ void resample_tile_generic(const uint8_t* __restrict__ img, int H, in
   __syncthreads();   // shared tile buffers are reused by the next call
 }
 
-// Downscale of at most 2.75 per side: one 16 x 32 output tile.  The CTA stages its whole
-// input window in shared memory with 4-byte loads (every image starts 16-byte aligned and
-// holds a multiple of 4 bytes, so the rounded loads stay inside it) and precomputes the
-// normalised tap weights of its rows and columns; thread (column, channel) keeps its column's
-// weights in registers, filters every staged row horizontally into a shared fp32 buffer and
-// then its output column vertically.
-constexpr int kFTH = 16, kFTW = 32, kFMaxTaps = 14;
-// the fast path takes downscales of at most 2.75 = 11 / 4 per side (tested as 4 n_in <= 11 n_out)
-constexpr int kFRows = 58;                   // >= 16 * 2.75 + 14 staged input rows
-constexpr int kFCols = 118;                  // >= 32 * 2.75 + 14 window pixels + 14 read past it (weight 0)
-constexpr int kFPitch = 368;                 // bytes per staged row: 3 * kFCols + 3 alignment slack, rounded
-constexpr int kFLine = kFTW * 3;             // floats per row of the horizontal result
-static_assert(kFPitch >= 3 * kFCols + 6 && kFPitch % 16 == 0, "staged row pitch");
-static_assert(kFRows >= kFTH * 2.75 + 14 && kFCols >= kFTW * 2.75 + 14 + kFMaxTaps, "staged window");
-static_assert(3 * kFTW <= kRsThreads / 2 && 64 + kFTH <= kRsThreads, "thread roles of the fast tile");
-constexpr size_t kFSmem = static_cast<size_t>(kFRows) * kFPitch + static_cast<size_t>(kFRows) * kFLine * 4 +
-                          (kFTW + kFTH) * kFMaxTaps * 4 + (2 * kFTW + 2 * kFTH + kFRows + 4) * 4;
-constexpr int kRsCtasPerSm = 4;
+// Downscales of up to 8 per side: a tile of up to kVPx input columns, filtered vertically first.
+//
+// Bound by instruction issue, so every input byte is turned into a float once per tile and used from
+// registers: a thread owns four pixels (12 bytes) of a column strip and walks down the input rows,
+// adding each to the (at most) four output rows whose windows hold it; a finished pair of rows goes
+// to shared memory as float2 (row, row + 1), and after four rows the CTA filters them horizontally,
+// a thread per column, one packed FMA per tap, channel and two rows.  Input rows come through a
+// per-thread ring of asynchronous copies (no barrier: a thread reads only what it
+// copied itself).  At most four windows hold an input row because they are
+// 4 fs wide and fs apart (fs = n_in / n_out >= 1), so four accumulators, reused in turn, are enough
+// and the row loop needs no rotation once it is unrolled over four output rows.
+// Byte-wise taps in the horizontal pass first (the reverse order) cost a shared load and a
+// conversion for every tap of every input row: 4K at r = 0.248 took 57 us.
+constexpr int kVThreads = 128;
+constexpr int kVPx = 4 * kVThreads;          // input columns of a tile
+constexpr int kVHalf = kVPx / 2 + 4;         // even (odd) columns of a plane, and slack for the last taps
+constexpr int kVPlane = 2 * kVHalf;
+constexpr int kVGroup = 4;                   // output rows per horizontal pass: two pairs
+constexpr int kVMaxTH = 32;                  // output rows of a tile, at most
+constexpr int kVMaxRows = 96;                // and input rows
+constexpr int kVMaxScale = 8;
+constexpr int kVWeights = 2560;              // horizontal weights of a tile
+constexpr int kVMaxCols = kVPx;
+constexpr int kVCtasPerSm = 4;
+// The input ring, taken two rows at a time: aligned rows are three words per thread, others four.
+template <bool ALIGNED>
+struct Ring {
+  static constexpr int kWords = ALIGNED ? 3 : 4;
+  static constexpr int kSlots = ALIGNED ? 8 : 4;
+  static constexpr int kAhead = kSlots - 2;   // rows in flight
+};
+constexpr int kVRingWords = 24;              // words per thread of the larger ring
+static_assert(Ring<true>::kWords * Ring<true>::kSlots <= kVRingWords && Ring<false>::kWords * Ring<false>::kSlots <= kVRingWords,
+              "ring size");
+struct ResampleSmem {
+  float2 v[kVGroup / 2][3][kVPlane];         // filtered row pairs: channel planes, even columns then odd
+  float2 wy[kVMaxRows][4];                   // (w, w) of input row y for output rows r .. r + 3, r the first unfinished
+  uint32_t raw[kVRingWords][kVThreads];      // [row, word][thread] of the input ring
+  float wx[kVWeights];                       // [tap][column]
+  int y0;                                    // first input row of the tile
+  int xlo[kVMaxCols];
+  int last[kVMaxTH];                         // last input row of output row r
+  float ynorm[kVMaxTH];
+};
 
-// Normalised weights of the window of output index o (reading R5); returns the tap count.
-__device__ __forceinline__ int window_weights(int o, int n_in, int n_out, int& lo, float* w) {
-  const Win win = exact_window(o, n_in, n_out);
-  if (win.n > kFMaxTaps) return win.n;
-  float sum = 0.f;
-  for (int i = 0; i < win.n; ++i) {
-    w[i] = cubic_w(static_cast<float>(win.num0 + i * win.step) * win.inv_den);
-    sum += w[i];
-  }
-  const float inv = 1.0f / sum;
-  for (int i = 0; i < win.n; ++i) w[i] *= inv;
-  lo = win.lo;
-  return win.n;
+// Four bytes as floats, exactly (2^23 + b by byte permutes, one packed subtract per pair).
+__device__ __forceinline__ void word_to_floats(uint32_t v, float2& lo, float2& hi) {
+  const float2 m = make_float2(-8388608.0f, -8388608.0f);
+  lo = ptx::fadd2(make_float2(__uint_as_float(__byte_perm(v, 0x4B000000u, 0x7540)),
+                              __uint_as_float(__byte_perm(v, 0x4B000000u, 0x7541))),
+                  m);
+  hi = ptx::fadd2(make_float2(__uint_as_float(__byte_perm(v, 0x4B000000u, 0x7542)),
+                              __uint_as_float(__byte_perm(v, 0x4B000000u, 0x7543))),
+                  m);
 }
 
-template <int MAXT>
-__device__ __forceinline__ void resample_tile_fast(const uint8_t* __restrict__ img, int H, int W, int Ho, int Wo,
-                                                   int ox0, int oy0, uint8_t* __restrict__ out) {
-  extern __shared__ __align__(16) unsigned char rs_smem[];
-  unsigned char* sin = rs_smem;                                           // [kFRows][kFPitch] bytes
-  float* sh = reinterpret_cast<float*>(sin + kFRows * kFPitch);            // [kFRows][kFTW * 3]
-  float* wx = sh + kFRows * kFLine;                                        // [kFTW][kFMaxTaps]
-  float* wy = wx + kFTW * kFMaxTaps;                                       // [kFTH][kFMaxTaps]
-  int* xlo = reinterpret_cast<int*>(wy + kFTH * kFMaxTaps);
-  int* xn = xlo + kFTW;
-  int* ylo = xn + kFTW;
-  int* yn = ylo + kFTH;
-  int* shift = yn + kFTH;                                                  // [kFRows]
+// Taps of every window of a downscale by s (a window has at most floor(4 s) + 2), made even.
+__device__ __forceinline__ int tap_count(float s) { return (static_cast<int>(4.0f * s) + 3) & ~1; }
+
+static_assert(sizeof(GenericSmem) <= sizeof(ResampleSmem), "one buffer for both kinds of tile");
+
+// Tiles of a Ho x Wo output: columns per tile (its window, starting up to 3 pixels early, fits kVPx
+// and its taps kVWeights), spread evenly.
+__device__ __forceinline__ int cols_per_tile(int W, int Wo) {
+  const float s = static_cast<float>(W) / static_cast<float>(Wo);
+  const int taps = tap_count(s);
+  const int most = max(1, min(static_cast<int>((static_cast<float>(kVPx - 8) - 4.0f * s) / s), kVWeights / taps));
+  const int tiles = (Wo + most - 1) / most;
+  return (Wo + tiles - 1) / tiles;
+}
+
+// Starts the copy of four pixels (12 bytes) at byte `off` of the image into a slot of the thread's
+// ring; nothing past the image's last word is read (what lies there is never used).
+template <bool ALIGNED>
+__device__ __forceinline__ void fetch_px4(const uint8_t* __restrict__ img, uint32_t off, uint32_t last, uint32_t* slot) {
+  const uint32_t a = ALIGNED ? off : off & ~3u;
+#pragma unroll
+  for (int k = 0; k < (ALIGNED ? 3 : 4); ++k) cp_async4(slot + k * kVThreads, img + min(a + 4u * k, last));
+}
+
+template <bool ALIGNED>
+__device__ __forceinline__ void resample_tile(ResampleSmem& sh, const uint8_t* __restrict__ img, int H, int W, int Ho,
+                                              int Wo, int ox0, int ncol, int oy0, int nrow, uint8_t* __restrict__ out) {
   const int tid = threadIdx.x;
-  const int ncol = min(kFTW, Wo - ox0), nrow = min(kFTH, Ho - oy0);
-  // with both scales <= 2.75 every window has <= 4 * 2.75 + 2 = 13 taps (min() is a guard)
-  if (tid < ncol) xn[tid] = min(kFMaxTaps, window_weights(ox0 + tid, W, Wo, xlo[tid], wx + tid * kFMaxTaps));
-  if (tid >= 64 && tid < 64 + nrow)
-    yn[tid - 64] =
-        min(kFMaxTaps, window_weights(oy0 + tid - 64, H, Ho, ylo[tid - 64], wy + (tid - 64) * kFMaxTaps));
-  __syncthreads();
-  const int x0 = xlo[0], x1 = xlo[ncol - 1] + xn[ncol - 1];
-  const int y0 = ylo[0], y1 = ylo[nrow - 1] + yn[nrow - 1];
-  const int nin_c = x1 - x0, nin_r = y1 - y0;
-  // stage the input window (4-byte words covering each row segment), asynchronously: a warp per
-  // row, every copy in flight at once
-  const int64_t pitch = static_cast<int64_t>(W) * 3;
-  const int64_t img_bytes = static_cast<int64_t>(H) * pitch;
-  const int words = (nin_c * 3 + 3 + 3) >> 2;
-  for (int r = tid >> 5; r < nin_r; r += kRsThreads / 32) {
-    const int64_t start = (static_cast<int64_t>(y0 + r) * pitch + static_cast<int64_t>(x0) * 3);
-    const int64_t a = start & ~int64_t{3};
-    if ((tid & 31) == 0) shift[r] = static_cast<int>(start - a);
-    for (int w = tid & 31; w < words; w += 32)
-      if (a + 4 * w < img_bytes) cp_async4(sin + r * kFPitch + 4 * w, img + a + 4 * w);
+  // horizontal windows and normalised weights (reading R5), padded to an even number of taps
+  const float sx = static_cast<float>(W) / static_cast<float>(Wo);
+  const int taps = tap_count(sx);
+  for (int c = tid; c < ncol; c += kVThreads) {
+    const Win w = exact_window(ox0 + c, W, Wo);
+    sh.xlo[c] = w.lo;
+    float sum = 0.f;
+    for (int i = 0; i < taps; ++i) {
+      const float x = i < w.n ? cubic_w(static_cast<float>(w.num0 + i * w.step) * w.inv_den) : 0.f;
+      sh.wx[i * ncol + c] = x;
+      sum += x;
+    }
+    const float inv = 1.0f / sum;
+    for (int i = 0; i < taps; ++i) sh.wx[i * ncol + c] *= inv;
   }
-  cp_async_wait_all();
-  __syncthreads();
-  // the two halves of the CTA take the two halves of the rows; thread tt = (column, channel)
-  const int half = tid / (kRsThreads / 2), tt = tid - half * (kRsThreads / 2);
-  if (tt < 3 * ncol) {
-    // horizontal pass: this half's staged rows, this thread's (column, channel)
-    // (taps past the window have weight 0 and read staged bytes that exist: the staged row
-    // holds kFCols >= the window of the last column + MAXT pixels)
-    const int c = tt / 3, ch = tt - 3 * c;
-    const int n = xn[c];
-    // A byte b enters as the float 1 + b / 256 (b in the top 8 mantissa bits of 1.0, one integer
-    // multiply-add), so sum_k w_k (1 + b_k / 256) = W + (sum_k w_k b_k) / 256 with W = sum_k w_k;
-    // the accumulators stay in [1, 2) (fp32 steps of 2^-23, i.e. 3e-5 in pixel units after the
-    // final 256 (acc - W)), and two rows share each packed FMA.
-    float w[MAXT];
-    float wsum = 0.f;
-#pragma unroll
-    for (int k = 0; k < MAXT; ++k) {
-      w[k] = k < n ? wx[c * kFMaxTaps + k] : 0.f;
-      wsum += w[k];
-    }
-    const float2 post = make_float2(-256.0f * wsum, -256.0f * wsum);
-    const float2 k256 = make_float2(256.0f, 256.0f);
-    auto unit = [](unsigned b) { return __uint_as_float(b * 32768u + 0x3F800000u); };
-    const int base = (xlo[c] - x0) * 3 + ch;
-    const int r_end = half ? nin_r : (nin_r + 1) / 2;
-    int r = half ? (nin_r + 1) / 2 : 0;
-    for (; r + 1 < r_end; r += 2) {   // two rows at a time: twice the independent work in flight
-      const unsigned char* px0 = sin + r * kFPitch + shift[r] + base;
-      const unsigned char* px1 = sin + (r + 1) * kFPitch + shift[r + 1] + base;
-      float2 acc = make_float2(0.f, 0.f);
-#pragma unroll
-      for (int k = 0; k < MAXT; ++k)
-        acc = ptx::ffma2(make_float2(w[k], w[k]), make_float2(unit(px0[3 * k]), unit(px1[3 * k])), acc);
-      const float2 h = ptx::ffma2(acc, k256, post);
-      sh[r * kFLine + tt] = h.x;
-      sh[(r + 1) * kFLine + tt] = h.y;
-    }
-    if (r < r_end) {
-      const unsigned char* px = sin + r * kFPitch + shift[r] + base;
-      float acc = 0.f;
-#pragma unroll
-      for (int k = 0; k < MAXT; ++k) acc = fmaf(w[k], unit(px[3 * k]), acc);
-      sh[r * kFLine + tt] = fmaf(acc, 256.0f, post.x);
-    }
+  // vertical windows: the last input row whose centre lies inside, 1 / sum of the weights
+  if (tid < nrow) {
+    const int o = oy0 + tid;
+    const Win w = exact_window(o, H, Ho);
+    float sum = 0.f;
+    for (int i = 0; i < w.n; ++i) sum += cubic_w(static_cast<float>(w.num0 + i * w.step) * w.inv_den);
+    sh.ynorm[tid] = 1.0f / sum;
+    const int64_t reach = (2 * static_cast<int64_t>(o) + 1) * H + 4 * static_cast<int64_t>(max(H, Ho)) - 1 - Ho;   // centre + 2 fs
+    const int64_t d = 2 * static_cast<int64_t>(Ho);
+    const int64_t i = reach < (int64_t{1} << 32) ? static_cast<int64_t>(static_cast<uint32_t>(reach) / static_cast<uint32_t>(d))
+                                                 : reach / d;
+    sh.last[tid] = static_cast<int>(min(static_cast<int64_t>(H - 1), i));
+    if (tid == 0) sh.y0 = w.lo;
   }
   __syncthreads();
-  // vertical pass and the uint8 store (a row of the tile is 3 * ncol consecutive bytes): thread
-  // (g, p) of 4 x 48 filters line entries 2p and 2p + 1 of output rows g, g + 4, .. with one
-  // 8-byte load and one packed FMA per tap (entry 3 * ncol, past the line when it is odd, holds
-  // whatever the buffer held and is not stored)
-  constexpr int kVPairs = kFLine / 2;
-  static_assert(4 * kVPairs <= kRsThreads, "thread roles of the vertical pass");
-  const int vg = tid / kVPairs, t0 = 2 * (tid - vg * kVPairs);
-  if (vg < 4 && t0 < 3 * ncol) {
-    const bool two = t0 + 1 < 3 * ncol;
-    uint8_t* o = out + (static_cast<int64_t>(oy0) * Wo + ox0) * 3 + t0;
-    for (int r = vg; r < nrow; r += 4) {
-      const float* w = wy + r * kFMaxTaps;
-      const float2* col = reinterpret_cast<const float2*>(sh + (ylo[r] - y0) * kFLine + t0);
-      const int n = yn[r];
-      float2 acc = make_float2(0.f, 0.f);
-#pragma unroll 4
-      for (int k = 0; k < n; ++k) acc = ptx::ffma2(make_float2(w[k], w[k]), col[k * kVPairs], acc);
-      uint8_t* orow = o + static_cast<int64_t>(r) * Wo * 3;
-      orow[0] = static_cast<uint8_t>(min(255, max(0, __float2int_rn(acc.x))));
-      if (two) orow[1] = static_cast<uint8_t>(min(255, max(0, __float2int_rn(acc.y))));
+  const int x0 = sh.xlo[0] & ~3;
+  const int y0 = sh.y0, y1 = sh.last[nrow - 1] + 1;
+  const float inv_den = 1.0f / static_cast<float>(2 * max(H, Ho));
+  for (int i = tid; i < (y1 - y0) * 4; i += kVThreads) {
+    const int y = y0 + (i >> 2);
+    int r = 0;
+    for (int half = kVMaxTH / 2; half > 0; half >>= 1)   // first row that ends at y or later
+      if (r + half <= nrow && sh.last[r + half - 1] < y) r += half;
+    if (r < nrow && sh.last[r] < y) ++r;
+    const int rr = r + (i & 3);
+    float w = 0.f;
+    if (rr < nrow) {
+      const int64_t num = (2 * static_cast<int64_t>(y) + 1) * Ho - (2 * static_cast<int64_t>(oy0 + rr) + 1) * H;
+      w = cubic_w(static_cast<float>(num) * inv_den) * sh.ynorm[rr];
     }
+    sh.wy[y - y0][i & 3] = make_float2(w, w);
   }
-  __syncthreads();   // the shared buffers are reused by the next tile
+  __syncthreads();
+  const uint32_t pitch = static_cast<uint32_t>(W) * 3u;
+  const uint32_t last_word = static_cast<uint32_t>(static_cast<int64_t>(H) * pitch - 4);
+  const int px = x0 + 4 * tid;                     // this thread's four columns
+  const bool works = px < sh.xlo[ncol - 1] + taps; // some window may reach them
+  float2 acc[4][6];                                // four output rows x 12 bytes
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int e = 0; e < 6; ++e) acc[j][e] = make_float2(0.f, 0.f);
+  uint32_t off = static_cast<uint32_t>(y0) * pitch + static_cast<uint32_t>(px) * 3u;   // of the next row to fetch
+  const uint32_t shr = (off & 2u) * 8u, flip = ALIGNED ? 0u : (pitch & 2u) * 8u;        // alignment of a row, of the next
+  uint32_t sft = ALIGNED ? 0u : shr;
+  using R = Ring<ALIGNED>;
+  uint32_t* ring = &sh.raw[0][tid];
+  constexpr int kRow = R::kWords * kVThreads;   // words from slot to slot
+  int y = y0, head = 0;   // the next row to filter, and its slot
+  auto fetch_next = [&](int row, int slot) {    // one group of copies per row, empty past the tile's last
+    if (works && row < y1) fetch_px4<ALIGNED>(img, off, last_word, ring + slot * kRow);
+    cp_async_commit();
+    off += pitch;
+  };
+#pragma unroll
+  for (int k = 0; k < R::kAhead; ++k) fetch_next(y0 + k, k);
+  // filters the next NR input rows; acc[(PH + j) & 3] is output row r + j of the phase's row r
+  auto rows = [&](auto phase, auto count) {
+    constexpr int PH = decltype(phase)::value, NR = decltype(count)::value;
+    cp_async_wait_group<R::kAhead - NR>();
+    uint32_t w[NR][3];
+    float4 wy[NR][2];
+#pragma unroll
+    for (int i = 0; i < NR; ++i) {
+      const uint32_t* slot = ring + ((head + i) & (R::kSlots - 1)) * kRow;
+      uint32_t x[R::kWords];
+#pragma unroll
+      for (int k = 0; k < R::kWords; ++k) x[k] = slot[k * kVThreads];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        if constexpr (ALIGNED) w[i][k] = x[k];
+        else w[i][k] = __funnelshift_r(x[k], x[k + 1], sft);
+      }
+      sft ^= flip;
+      const float4* wp = reinterpret_cast<const float4*>(sh.wy[y + i - y0]);
+      wy[i][0] = wp[0];
+      wy[i][1] = wp[1];
+    }
+#pragma unroll
+    for (int i = 0; i < NR; ++i) fetch_next(y + R::kAhead + i, (head + R::kAhead + i) & (R::kSlots - 1));
+    y += NR;
+    head = (head + NR) & (R::kSlots - 1);
+#pragma unroll
+    for (int i = 0; i < NR; ++i) {
+      float2 f[6];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) word_to_floats(w[i][k], f[2 * k], f[2 * k + 1]);
+      const float2 wj[4] = {make_float2(wy[i][0].x, wy[i][0].y), make_float2(wy[i][0].z, wy[i][0].w),
+                            make_float2(wy[i][1].x, wy[i][1].y), make_float2(wy[i][1].z, wy[i][1].w)};
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int e = 0; e < 6; ++e) acc[(PH + j) & 3][e] = ptx::ffma2(wj[j], f[e], acc[(PH + j) & 3][e]);
+    }
+  };
+  // the input rows up to the last one of the phase's output row, two at a time
+  auto advance = [&](auto phase, int upto) {
+    while (y < upto) rows(phase, std::integral_constant<int, 2>{});
+    if (y == upto) rows(phase, std::integral_constant<int, 1>{});
+  };
+  // byte 3 i + ch of the thread's 12 is channel ch of its pixel i
+  auto byte_of = [](const float2 (&v)[6], int b) { return (b & 1) ? v[b >> 1].y : v[b >> 1].x; };
+  for (int g = 0; g < nrow; g += kVGroup) {
+    float2 held[6];
+    auto finish = [&](auto phase) {
+      constexpr int PH = decltype(phase)::value;
+      advance(phase, g + PH < nrow ? sh.last[g + PH] : -1);
+      if constexpr ((PH & 1) == 0) {
+#pragma unroll
+        for (int e = 0; e < 6; ++e) held[e] = acc[PH][e];
+      } else if (works) {
+#pragma unroll
+        for (int ch = 0; ch < 3; ++ch) {
+          float2* plane = sh.v[PH >> 1][ch];
+#pragma unroll
+          for (int odd = 0; odd < 2; ++odd)   // pixels odd and odd + 2
+            *reinterpret_cast<float4*>(plane + odd * kVHalf + 2 * tid) =
+                make_float4(byte_of(held, 3 * odd + ch), byte_of(acc[PH], 3 * odd + ch), byte_of(held, 3 * odd + 6 + ch),
+                            byte_of(acc[PH], 3 * odd + 6 + ch));
+        }
+      }
+#pragma unroll
+      for (int e = 0; e < 6; ++e) acc[PH][e] = make_float2(0.f, 0.f);
+    };
+    finish(std::integral_constant<int, 0>{});
+    finish(std::integral_constant<int, 1>{});
+    finish(std::integral_constant<int, 2>{});
+    finish(std::integral_constant<int, 3>{});
+    __syncthreads();
+    // horizontal pass of these four rows: a thread per column, all three channels
+    for (int c = tid; c < ncol; c += kVThreads) {
+      const int x = sh.xlo[c] - x0;
+      const float2* even = sh.v[0][0] + (x & 1) * kVHalf + (x >> 1);           // taps 0, 2, ..
+      const float2* odd = sh.v[0][0] + ((x + 1) & 1) * kVHalf + ((x + 1) >> 1);   // taps 1, 3, ..
+      const float* w = sh.wx + c;
+      float2 a[2][3];
+#pragma unroll
+      for (int p = 0; p < 2; ++p)
+#pragma unroll
+        for (int ch = 0; ch < 3; ++ch) a[p][ch] = make_float2(0.f, 0.f);
+#pragma unroll 2
+      for (int k = 0; k < taps; k += 2, w += 2 * ncol, ++even, ++odd) {
+        const float2 w0 = make_float2(w[0], w[0]), w1 = make_float2(w[ncol], w[ncol]);
+#pragma unroll
+        for (int p = 0; p < 2; ++p)
+#pragma unroll
+          for (int ch = 0; ch < 3; ++ch) {
+            a[p][ch] = ptx::ffma2(w0, even[(3 * p + ch) * kVPlane], a[p][ch]);
+            a[p][ch] = ptx::ffma2(w1, odd[(3 * p + ch) * kVPlane], a[p][ch]);
+          }
+      }
+      uint8_t* o = out + (static_cast<int64_t>(oy0 + g) * Wo + ox0 + c) * 3;
+      auto put = [&](uint8_t* q, float v) { *q = static_cast<uint8_t>(ptx::round_u8(v)); };
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        if (g + r >= nrow) break;
+#pragma unroll
+        for (int ch = 0; ch < 3; ++ch) put(o + ch, (r & 1) ? a[r >> 1][ch].y : a[r >> 1][ch].x);
+        o += static_cast<int64_t>(Wo) * 3;
+      }
+    }
+    __syncthreads();   // the row pairs are rewritten
+  }
 }
 
-// Every CTA walks the output tiles of the whole batch (16 x 32 tiles; target sizes read from
-// the density statistics on the device, or given), so the grid never holds empty CTAs.
-__global__ void __launch_bounds__(kRsThreads) apc_resample(const uint8_t* __restrict__ src,
-                                                           const __grid_constant__ ResampleTable t,
-                                                           const pace_apc_stats* __restrict__ stats,
-                                                           uint8_t* __restrict__ dst) {
+// Every CTA walks the output tiles of the whole batch (target sizes read from the density statistics
+// on the device, or given), so the grid never holds empty CTAs.
+__global__ void __launch_bounds__(kVThreads, kVCtasPerSm) apc_resample(const uint8_t* __restrict__ src,
+                                                                       const __grid_constant__ ResampleTable t,
+                                                                       const pace_apc_stats* __restrict__ stats,
+                                                                       uint8_t* __restrict__ dst) {
+  extern __shared__ __align__(16) unsigned char rs_smem[];
+  ResampleSmem& sh = *reinterpret_cast<ResampleSmem*>(rs_smem);
   __shared__ int tile_prefix[kApcMaxB + 1];
-  __shared__ int sho[kApcMaxB], swo[kApcMaxB];
-  if (threadIdx.x == 0) {
+  __shared__ int sho[kApcMaxB], swo[kApcMaxB], stw[kApcMaxB];   // target size, columns per tile (0: generic tiles)
+  __shared__ int s_th;
+  const int tid = threadIdx.x;
+  for (int b = tid; b < t.nb; b += kVThreads) {
+    int Ho = stats ? stats[t.b_base + b].h_out : t.Ho[b];
+    int Wo = stats ? stats[t.b_base + b].w_out : t.Wo[b];
+    if (Ho < 1 || Wo < 1 || Ho > t.H[b] || Wo > t.W[b]) Ho = Wo = 0;   // nothing to write
+    sho[b] = Ho;
+    swo[b] = Wo;
+    stw[b] = Ho > 0 && t.H[b] <= kVMaxScale * Ho && t.W[b] <= kVMaxScale * Wo ? cols_per_tile(t.W[b], Wo) : 0;
+  }
+  __syncthreads();
+  // Rows per tile, a multiple of four: a tile reads (rows + 4) fs input rows, so tall tiles filter
+  // least twice, but the tiles should also fill the SMs.  Lane l of warp 0 rates 4 (l + 1) rows: a
+  // tile's time is about rows + 4 + 3 (the set-up) when it has an SM to itself, and n tiles on an SM
+  // take about max(1, 0.4 n) times that.
+  if (tid < 32) {
+    const int th = 4 * (tid + 1);
+    unsigned cost = 0xFFFFFFFFu;
+    if (th <= kVMaxTH) {
+      int64_t tiles = 0;
+      for (int b = 0; b < t.nb; ++b)
+        if (stw[b] > 0) {
+          // no more rows than the input rows that a tile can hold
+          const int rows = min(th, max(4, static_cast<int>(static_cast<float>(kVMaxRows - 4) * sho[b] / t.H[b] - 3.0f) & ~3));
+          tiles += static_cast<int64_t>((swo[b] + stw[b] - 1) / stw[b]) * ((sho[b] + rows - 1) / rows);
+        }
+      const int64_t sms = gridDim.x / kVCtasPerSm, per_sm = (tiles + sms - 1) / sms;
+      cost = static_cast<unsigned>(max(static_cast<int64_t>(5), 2 * min(static_cast<int64_t>(1 << 24), per_sm))) * (th + 7);
+    }
+    const unsigned best = __reduce_min_sync(0xffffffffu, cost);
+    const unsigned who = __ballot_sync(0xffffffffu, cost == best);
+    if (tid == 0) s_th = 4 * __ffs(who);
+  }
+  __syncthreads();
+  auto rows_of = [&](int b) {
+    return min(s_th, max(4, static_cast<int>(static_cast<float>(kVMaxRows - 4) * sho[b] / t.H[b] - 3.0f) & ~3));
+  };
+  if (tid == 0) {
     int acc = 0;
     for (int b = 0; b < t.nb; ++b) {
-      int Ho = stats ? stats[t.b_base + b].h_out : t.Ho[b];
-      int Wo = stats ? stats[t.b_base + b].w_out : t.Wo[b];
-      if (Ho < 1 || Wo < 1 || Ho > t.H[b] || Wo > t.W[b]) Ho = Wo = 0;   // nothing to write
-      sho[b] = Ho;
-      swo[b] = Wo;
       tile_prefix[b] = acc;
-      acc += ((Ho + kFTH - 1) / kFTH) * ((Wo + kFTW - 1) / kFTW);
+      const int th = stw[b] > 0 ? rows_of(b) : kRsTH, tw = stw[b] > 0 ? stw[b] : kRsTW;
+      acc += ((sho[b] + th - 1) / th) * ((swo[b] + tw - 1) / tw);
     }
     tile_prefix[t.nb] = acc;
   }
@@ -1960,17 +2128,18 @@ __global__ void __launch_bounds__(kRsThreads) apc_resample(const uint8_t* __rest
     int b = 0;
     while (b + 1 < t.nb && tile_prefix[b + 1] <= g) ++b;
     const int Ho = sho[b], Wo = swo[b], H = t.H[b], W = t.W[b];
-    const int tw = (Wo + kFTW - 1) / kFTW;
+    const int th = stw[b] > 0 ? rows_of(b) : kRsTH, tw = stw[b] > 0 ? stw[b] : kRsTW;
+    const int nx = (Wo + tw - 1) / tw;
     const int l = g - tile_prefix[b];
-    const int oy0 = (l / tw) * kFTH, ox0 = (l - (l / tw) * tw) * kFTW;
+    const int oy0 = (l / nx) * th, ox0 = (l - (l / nx) * nx) * tw;
     const uint8_t* img = src + t.src_off[b];
     uint8_t* out = dst + t.dst_off[b];
-    if (4 * W <= 11 * Wo && 4 * H <= 11 * Ho) {   // both scales <= 2.75 = 11 / 4
-      if (4 * W <= 9 * Wo && 4 * H <= 9 * Ho) resample_tile_fast<10>(img, H, W, Ho, Wo, ox0, oy0, out);   // <= 10 taps
-      else resample_tile_fast<kFMaxTaps>(img, H, W, Ho, Wo, ox0, oy0, out);
+    if (stw[b] > 0) {
+      const int ncol = min(tw, Wo - ox0), nrow = min(th, Ho - oy0);
+      if (W % 4 == 0) resample_tile<true>(sh, img, H, W, Ho, Wo, ox0, ncol, oy0, nrow, out);
+      else resample_tile<false>(sh, img, H, W, Ho, Wo, ox0, ncol, oy0, nrow, out);
     } else {
-        for (int sy = 0; sy < kFTH; sy += kRsTH)
-        for (int sx = 0; sx < kFTW; sx += kRsTW) resample_tile_generic(img, H, W, Ho, Wo, ox0 + sx, oy0 + sy, out);
+      resample_tile_generic(*reinterpret_cast<GenericSmem*>(rs_smem), img, H, W, Ho, Wo, ox0, oy0, out);
     }
   }
 }
@@ -2157,29 +2326,19 @@ static pace_status_t resample_impl(const uint8_t* src, const int64_t* src_off, c
   for (int b = 0; b < B; ++b)
     if (dst_off[b] < 0) return PACE_ERR_INVALID_ARG;
   PACE_CHECK(check_device());
-  int sms = 1;
-  {
-    // opt in to the fast path's shared memory and read the SM count, once per device
-    static DeviceOnce once;
-    static std::atomic<int> sm_count[64];
-    int dev = 0;
-    PACE_CUDA(cudaGetDevice(&dev));
-    if (!once.done(dev)) {
-      int n = 0;
-      PACE_CUDA(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
-      sm_count[dev & 63].store(n, std::memory_order_relaxed);
-      PACE_CUDA(cudaFuncSetAttribute(apc_resample, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     static_cast<int>(kFSmem)));
-      once.mark(dev);
-    }
-    sms = std::max(sm_count[dev & 63].load(std::memory_order_relaxed), 1);
+  int sms = 0, dev = 0;
+  PACE_CHECK(sm_count(&sms));
+  PACE_CUDA(cudaGetDevice(&dev));
+  static DeviceOnce once;   // opt in to the tiles' shared memory
+  if (!once.done(dev)) {
+    PACE_CUDA(cudaFuncSetAttribute(apc_resample, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(ResampleSmem)));
+    once.mark(dev);
   }
   for (int c0 = 0; c0 < B; c0 += kApcMaxB) {
     const int nb = (B - c0) < kApcMaxB ? (B - c0) : kApcMaxB;
     ResampleTable t{};
     t.nb = nb;
     t.b_base = c0;
-    int hmax = 1, wmax = 1;
     for (int i = 0; i < nb; ++i) {
       const int b = c0 + i;
       t.src_off[i] = src_off[b];
@@ -2188,12 +2347,8 @@ static pace_status_t resample_impl(const uint8_t* src, const int64_t* src_off, c
       t.W[i] = W[b];
       t.Ho[i] = stats ? H[b] : Ho[b];
       t.Wo[i] = stats ? W[b] : Wo[b];
-      if (t.Ho[i] > hmax) hmax = t.Ho[i];
-      if (t.Wo[i] > wmax) wmax = t.Wo[i];
     }
-    const int64_t tiles = static_cast<int64_t>((wmax + kFTW - 1) / kFTW) * ((hmax + kFTH - 1) / kFTH) * nb;
-    const int grid = static_cast<int>(std::min<int64_t>(tiles, static_cast<int64_t>(kRsCtasPerSm) * sms));
-    apc_resample<<<grid, kRsThreads, kFSmem, stream>>>(src, t, stats, dst);
+    apc_resample<<<kVCtasPerSm * sms, kVThreads, sizeof(ResampleSmem), stream>>>(src, t, stats, dst);
     PACE_CHECK(check_launch());
   }
   return PACE_OK;

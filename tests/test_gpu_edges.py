@@ -164,3 +164,23 @@ def test_tokens_with_non_finite_rows(pace):
     d, _ = pace.pace_apc_density_tokens(bf16_tensor(bits), [0, 64], [252], [252])
     bad = ~np.isfinite(d.cpu().numpy())
     assert bad[20] and bad.sum() <= 2 and not bad[:20].any()
+
+
+# scales 1 to 8 per side (filtered vertically first) and just above (generic), widths on 2-byte
+# boundaries, one and several column strips, heights below a group of four rows, odd sizes
+@pytest.mark.parametrize("shape,size", [((14, 14), (14, 14)), ((14, 14), (1, 1)), ((28, 14), (3, 2)), ((98, 42), (97, 41)),
+                                        ((70, 1302), (35, 1301)), ((42, 2030), (30, 600)), ((560, 70), (70, 9)),
+                                        ((560, 70), (69, 9)), ((126, 1036), (125, 130)), ((126, 1036), (45, 129)),
+                                        ((700, 700), (501, 88))])
+def test_resample_scales(pace, shape, size):
+    rng = np.random.default_rng(shape[0] + size[1])
+    img = synth.make_image(rng, *shape, 3, 3, 0.5)
+    dst = torch.zeros(shape[0] * shape[1] * 3, dtype=torch.uint8, device="cuda")
+    pace.pace_apc_resample_to(torch.from_numpy(img.reshape(-1)).cuda(), [0], [shape[0]], [shape[1]], [size[0]], [size[1]], dst, [0])
+    n = size[0] * size[1] * 3
+    out, ref = dst.cpu().numpy()[:n].reshape(*size, 3), O.apc_resample(img, *size)
+    assert np.abs(out.astype(int) - ref.astype(int)).max() <= 1
+    # bytes off by one are those whose exact value is within rounding of a half
+    x = O.resample_float(img, *size)
+    assert np.all(np.abs(x - np.floor(x) - 0.5)[out != ref] <= 2e-4)
+    assert not dst[n:].any()
