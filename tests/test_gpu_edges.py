@@ -133,6 +133,41 @@ def test_density_tail_cluster(pace, kind):
     assert abs(pace.stats_dict(st)[0]["d_top"] - top) <= 4e-7 * top + 1e-9
 
 
+# distances counted per warp (pictures: the first and the last live lane's bucket at once, the rest one
+# by one) and per run of equal buckets (tokens): all equal, two values in turn, background with few or
+# many others among it, partial warps
+@pytest.mark.parametrize("kind", ["all", "two", "few", "half", "most", "none"])
+@pytest.mark.parametrize("rows,cols", [(1, 3), (3, 33), (40, 60)])
+def test_tail_counts_of_backgrounds(pace, kind, rows, cols):
+    rng = np.random.default_rng(rows * cols)
+    n, h, w = rows * cols, rows * 14, cols * 14
+    share = {"all": 0.0, "two": 0.0, "few": 0.1, "half": 0.5, "most": 0.9, "none": 1.0}[kind]
+    noise = rng.uniform(size=n) < share
+    img = np.full((h, w, 3), 40, np.uint8)
+    for q in range(n):
+        y, x = divmod(q, cols)
+        p = img[14 * y:14 * y + 14, 14 * x:14 * x + 14]
+        if noise[q]:
+            p[:] = rng.integers(0, 256, p.shape, dtype=np.uint8)
+        elif kind == "two" and q % 2:
+            p[:, :7] = 200
+
+    def check(d, st):
+        d = d.cpu().numpy().astype(np.float64)
+        s = pace.stats_dict(st)[0]
+        top = np.sort(d)[::-1][:s["k_tail"]].mean()
+        assert abs(s["d_top"] - top) <= 4e-7 * top + 1e-9   # fp32 rounding of the mean
+        return d
+
+    src = torch.from_numpy(img.reshape(-1)).cuda()
+    assert_distances_close(check(*pace.pace_apc_density(src, [0], [h], [w])), O.apc_density(img)["d"])
+    check(*pace.pace_apc_density_pixel(src, [0], [h], [w], "rgb_stats"))
+    T = np.where(noise[:, None], rng.normal(size=(n, 64)), 1.0 + (kind == "two") * (np.arange(n)[:, None] % 2) * np.arange(64))
+    bits = synth.f32_to_bf16_bits(T.astype(np.float32))
+    d = check(*pace.pace_apc_density_tokens(bf16_tensor(bits), [0, n], [h], [w]))
+    assert_distances_close(d, O.apc_density_preview(f64(bits), w, h)["d"])
+
+
 # register kernels (whole 16-byte vectors, up to 1536) and the staged ones (other widths), runs of 8
 # tokens with remainders, several images per CTA
 @pytest.mark.parametrize("D", [8, 248, 256, 264, 1152, 1536, 1544, 1284, 6])
