@@ -145,7 +145,7 @@ __device__ __forceinline__ int2 unit_range(int units) {
 // starts beside it and waits for it before its first atomic.  A memset in its place is a full stop in
 // the stream: 2.3 us.
 __global__ void __launch_bounds__(256) apc_zero(uint4* __restrict__ a, unsigned na, uint4* __restrict__ b, unsigned nb) {
-  ptx::launch_dependents();
+  ptx::begin_call();
   for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < na + nb; i += gridDim.x * blockDim.x)
     *(i < na ? a + i : b + (i - na)) = make_uint4(0u, 0u, 0u, 0u);
 }
@@ -1256,8 +1256,7 @@ __global__ void __launch_bounds__(1024) apc_tail(const __grid_constant__ ApcTabl
     key_max = 0u;
   }
   if (ncta > 1) ptx::cluster_arrive();   // the first CTA's list is ready: waited for before the first append
-  ptx::launch_dependents();
-  ptx::grid_dependency_wait();
+  ptx::begin_call();   // (nothing of this call follows: the next call's first kernel)
   const int b = blockIdx.y;
   const int N = t.n[b];
   const TailWork* w = work + (t.b_base + b);
@@ -2133,10 +2132,11 @@ __global__ void __launch_bounds__(kVThreads, kVCtasPerSm) apc_resample(const uin
   __shared__ int tile_prefix[kApcMaxB + 1];
   __shared__ int sho[kApcMaxB], swo[kApcMaxB], stw[kApcMaxB];   // target size, columns per tile (0: generic tiles)
   __shared__ int s_th;
+  ptx::begin_call();
   const int tid = threadIdx.x;
   for (int b = tid; b < t.nb; b += kVThreads) {
-    int Ho = stats ? stats[t.b_base + b].h_out : t.Ho[b];
-    int Wo = stats ? stats[t.b_base + b].w_out : t.Wo[b];
+    int Ho = stats ? __ldcg(&stats[t.b_base + b].h_out) : t.Ho[b];
+    int Wo = stats ? __ldcg(&stats[t.b_base + b].w_out) : t.Wo[b];
     if (Ho < 1 || Wo < 1 || Ho > t.H[b] || Wo > t.W[b]) Ho = Wo = 0;   // nothing to write
     sho[b] = Ho;
     swo[b] = Wo;
@@ -2235,9 +2235,8 @@ pace_status_t launch_tail(const ApcTable& t, const float* d, TailParams tp, pace
 
 pace_status_t launch_zero(void* a, size_t a_bytes, void* b, size_t b_bytes, cudaStream_t stream) {
   const size_t na = a_bytes / 16, nb = b_bytes / 16;
-  apc_zero<<<static_cast<unsigned>(std::min<size_t>((na + nb + 1023) / 1024, 2048)), 256, 0, stream>>>(
-      static_cast<uint4*>(a), static_cast<unsigned>(na), static_cast<uint4*>(b), static_cast<unsigned>(nb));
-  return check_launch();
+  return launch_dependent(apc_zero, static_cast<unsigned>(std::min<size_t>((na + nb + 1023) / 1024, 2048)), 256, 0, 1, stream,
+                          static_cast<uint4*>(a), static_cast<unsigned>(na), static_cast<uint4*>(b), static_cast<unsigned>(nb));
 }
 
 // Strip table of images c0 .. c0 + nb - 1; patch0 runs on over the calls.  Each image has the widest
@@ -2404,8 +2403,8 @@ static pace_status_t resample_impl(const uint8_t* src, const int64_t* src_off, c
       t.Ho[i] = stats ? H[b] : Ho[b];
       t.Wo[i] = stats ? W[b] : Wo[b];
     }
-    apc_resample<<<kVCtasPerSm * sms, kVThreads, sizeof(ResampleSmem), stream>>>(src, t, stats, dst);
-    PACE_CHECK(check_launch());
+    PACE_CHECK(launch_dependent(apc_resample, static_cast<unsigned>(kVCtasPerSm * sms), kVThreads, sizeof(ResampleSmem), 1,
+                                stream, src, t, stats, dst));
   }
   return PACE_OK;
 }

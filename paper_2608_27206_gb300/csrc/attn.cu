@@ -412,7 +412,6 @@ __global__ void __launch_bounds__(kThreads, 1) attn_row_lse(const __grid_constan
   uint8_t* sQ = smem;                                // this CTA's resident query tile
   uint8_t* sK = sQ + C::A::BYTES;                    // ST stages of a key tile
   SmemCtl* ctl = reinterpret_cast<SmemCtl*>(sK + ST * C::B::BYTES);
-  launch_dependents();   // the next kernel's blocks take the SMs that the last wave leaves idle
   const uint32_t b_qfull = smem_u32(&ctl->bars[0]);     // query tile landed
   const uint32_t b_done = smem_u32(&ctl->bars[1]);      // all MMAs of a round finished
   auto b_kfull = [&](int s) { return smem_u32(&ctl->bars[2 + s]); };
@@ -467,6 +466,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_row_lse(const __grid_constan
       prefetch_tensormap(&tmq32);
       prefetch_tensormap(&tmk32);
     }
+    begin_call();   // (the next kernel's blocks take the SMs that the last wave leaves idle)
     mbar_arrive_expect_tx(b_qfull, C::A::BYTES);
     load_tile<D, kTile>(sQ, &tmq, &tmq32, h * D, t.q0[b] + qrow0, b_qfull);
     for (int j = 0; j < pre; ++j) {
@@ -646,10 +646,10 @@ __global__ void __launch_bounds__(128) attn_lse_combine(const __grid_constant__ 
     return;
   }
   float M = -INFINITY;
-  for (int s = 0; s < t.splits; ++s) M = fmaxf(M, ml[static_cast<int64_t>(s) * t.H * t.prows + prow].x);
+  for (int s = 0; s < t.splits; ++s) M = fmaxf(M, __ldcg(&ml[static_cast<int64_t>(s) * t.H * t.prows + prow]).x);
   float l = 0.f;
   for (int s = 0; s < t.splits; ++s) {
-    const float2 p = ml[static_cast<int64_t>(s) * t.H * t.prows + prow];
+    const float2 p = __ldcg(&ml[static_cast<int64_t>(s) * t.H * t.prows + prow]);
     if (p.y > 0.f) l += p.y * ex2_approx(p.x - M);
   }
   store_shift_row(shift_out + prow * kShiftCols, -(M + log2f(l)) / c);
@@ -951,7 +951,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_colsum(const __grid_constant
 constexpr int kReduceLanes = 4;
 __global__ void __launch_bounds__(256) attn_reduce(const float* __restrict__ part, int groups, int ktot, int merge,
                                                    float* __restrict__ out) {
-  grid_dependency_wait();
+  begin_call();   // (nothing of this call follows: the next call's first kernel)
   const int tid = blockIdx.x * blockDim.x + threadIdx.x;
   const int m = tid / kReduceLanes, j = tid % kReduceLanes;
   const int nout = ktot / merge;
@@ -965,7 +965,7 @@ __global__ void __launch_bounds__(256) attn_reduce(const float* __restrict__ par
         gs = (v.x + v.y) + (v.z + v.w);
       } else {
         gs = 0.f;
-        for (int q = 0; q < merge; ++q) gs += p[q];
+        for (int q = 0; q < merge; ++q) gs += __ldcg(p + q);
       }
       s += gs;
     }
@@ -1254,9 +1254,9 @@ pace_status_t run_importance(const void* Q, const void* K, int64_t qrows, int64_
       }
       if (chunks.n > 0) PACE_CUDA(cudaStreamWaitEvent(stream, chunks.ready[pc], 0));
       if (items_pc > 0) {   // two CTAs per work item
-        attn_row_lse<D, CAUSAL><<<2 * static_cast<unsigned>(items_pc), kThreads, s1, stream>>>(mq, mq32, mk, mk32, t, c, Lw,
-                                                                                               ml, status);
-        PACE_CHECK(check_launch());
+        // (a piece that waits for an event is launched plainly)
+        PACE_CHECK(launch_ex(chunks.n == 0, attn_row_lse<D, CAUSAL>, 2 * static_cast<unsigned>(items_pc), kThreads, s1, 1,
+                             stream, mq, mq32, mk, mk32, t, c, Lw, ml, status));
       }
     }
     if (Lay.splits > 1 && ctiles > 0) {

@@ -14,6 +14,7 @@
 #include <cmath>
 
 #include "pace_common.cuh"
+#include "pace_ptx.cuh"
 #include "pace_select.cuh"
 
 namespace pace {
@@ -158,6 +159,7 @@ __global__ void __launch_bounds__(kSelThreads) ddae_select_kernel(const float* _
                                                                   float* __restrict__ weights,
                                                                   int32_t* __restrict__ kept, int b_base, int* status) {
   __shared__ SelShared sh;
+  ptx::begin_call();
   const int b = blockIdx.x;
   const int nv = tab.nv[b], v0 = tab.v0[b];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -171,7 +173,7 @@ __global__ void __launch_bounds__(kSelThreads) ddae_select_kernel(const float* _
 
   // 1. min / max and shifted moments (and the finiteness check); the first round's bins are
   // cleared on the way
-  const float ca = __ldg(pa), cv = __ldg(pv);
+  const float ca = __ldcg(pa), cv = __ldcg(pv);
   for (int q = tid; q < kSelBins; q += kSelThreads) sh.bins[q] = 0u;
   if (tid == 0) sh.ncand = 0u;
   float amin = FLT_MAX, amax = -FLT_MAX, vmin = FLT_MAX, vmax = -FLT_MAX;
@@ -189,15 +191,15 @@ __global__ void __launch_bounds__(kSelThreads) ddae_select_kernel(const float* _
 #pragma unroll
     for (int k = 0; k < RM; ++k)
       if (has(k)) {
-        ra[k] = __ldg(pa + idx(k));
-        rv[k] = __ldg(pv + idx(k));
+        ra[k] = __ldcg(pa + idx(k));
+        rv[k] = __ldcg(pv + idx(k));
       }
 #pragma unroll
     for (int k = 0; k < RM; ++k)
       if (has(k)) take(ra[k], rv[k]);
   } else {
     for (int k = 0; k < R; ++k)
-      if (has(k)) take(__ldg(pa + idx(k)), __ldg(pv + idx(k)));
+      if (has(k)) take(__ldcg(pa + idx(k)), __ldcg(pv + idx(k)));
   }
   amin = warp_min(amin); amax = warp_max(amax);
   vmin = warp_min(vmin); vmax = warp_max(vmax);
@@ -259,7 +261,7 @@ __global__ void __launch_bounds__(kSelThreads) ddae_select_kernel(const float* _
       if (has(k)) ra[k] = fused(ra[k], rv[k]);
   } else if (s_final != nullptr) {
     for (int k = 0; k < R; ++k)
-      if (has(k)) s_final[v0 + idx(k)] = fused(__ldg(pa + idx(k)), __ldg(pv + idx(k)));
+      if (has(k)) s_final[v0 + idx(k)] = fused(__ldcg(pa + idx(k)), __ldcg(pv + idx(k)));
   }
   auto store_final = [&](int k) {
     if constexpr (RM > 0)
@@ -269,7 +271,7 @@ __global__ void __launch_bounds__(kSelThreads) ddae_select_kernel(const float* _
   auto key_of = [&](int k) -> unsigned {
     if (!has(k)) return 0u;
     if constexpr (RM > 0) return sel_key(ra[k]);
-    else return sel_key(fused(__ldg(pa + idx(k)), __ldg(pv + idx(k))));
+    else return sel_key(fused(__ldcg(pa + idx(k)), __ldcg(pv + idx(k))));
   };
   // calls f(k) for k = kb .. ke - 1 (the same k for every thread at each call)
   auto for_rows = [&](int kb, int ke, auto&& f) {
@@ -471,6 +473,7 @@ constexpr int kGatherPiece = 32 * kGatherU;   // vectors per warp-piece
 __global__ void __launch_bounds__(256) gather_rows_v16(const uint4* __restrict__ src, int64_t n_src,
                                                        int64_t row_vec, const int32_t* __restrict__ idx,
                                                        int64_t n_idx, uint4* __restrict__ dst, int* status) {
+  ptx::begin_call();
   const int lane = threadIdx.x & 31;
   const int64_t warp0 = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
@@ -478,7 +481,7 @@ __global__ void __launch_bounds__(256) gather_rows_v16(const uint4* __restrict__
   for (int64_t w = warp0; w < n_idx * pieces; w += nwarps) {
     const int64_t r = w / pieces;
     const int64_t c0 = (w - r * pieces) * kGatherPiece;
-    const int64_t s = idx[r];
+    const int64_t s = __ldcg(idx + r);
     uint4* dp = dst + r * row_vec;
     if (s < 0 || s >= n_src) {
       for (int64_t c = c0 + lane; c < min(row_vec, c0 + kGatherPiece); c += 32) dp[c] = make_uint4(0u, 0u, 0u, 0u);
@@ -507,13 +510,14 @@ template <int U>
 __global__ void __launch_bounds__(128) gather_rows_warp(const uint4* __restrict__ src, int64_t n_src, int row_vec,
                                                         const int32_t* __restrict__ idx, int64_t n_idx,
                                                         uint4* __restrict__ dst, int* status) {
+  ptx::begin_call();
   const int lane = threadIdx.x & 31;
   const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
   int64_t r = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-  int64_t s_next = r < n_idx ? __ldg(idx + r) : 0;
+  int64_t s_next = r < n_idx ? __ldcg(idx + r) : 0;
   for (; r < n_idx; r += nwarps) {
     const int64_t s = s_next;
-    if (r + nwarps < n_idx) s_next = __ldg(idx + r + nwarps);
+    if (r + nwarps < n_idx) s_next = __ldcg(idx + r + nwarps);
     uint4* dp = dst + r * row_vec;
     if (s < 0 || s >= n_src) {
       for (int c = lane; c < row_vec; c += 32) dp[c] = make_uint4(0u, 0u, 0u, 0u);
@@ -535,11 +539,12 @@ __global__ void __launch_bounds__(128) gather_rows_warp(const uint4* __restrict_
 __global__ void __launch_bounds__(256) gather_rows_bytes(const uint8_t* __restrict__ src, int64_t n_src,
                                                          int64_t row_bytes, const int32_t* __restrict__ idx,
                                                          int64_t n_idx, uint8_t* __restrict__ dst, int* status) {
+  ptx::begin_call();
   const int lane = threadIdx.x & 31;
   const int64_t warp0 = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
   for (int64_t r = warp0; r < n_idx; r += nwarps) {
-    const int64_t s = idx[r];
+    const int64_t s = __ldcg(idx + r);
     uint8_t* dp = dst + r * row_bytes;
     if (s < 0 || s >= n_src) {
       for (int64_t c = lane; c < row_bytes; c += 32) dp[c] = 0;
@@ -570,6 +575,7 @@ struct PruneTable {
 __global__ void __launch_bounds__(256) prune_index_kernel(const __grid_constant__ PruneTable t,
                                                           const int32_t* __restrict__ kept,
                                                           int32_t* __restrict__ out, int* status) {
+  ptx::begin_call();
   const int b = blockIdx.y;
   const int n_post = t.n_pre[b] - t.nv[b] + t.nk[b];
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_post; i += gridDim.x * blockDim.x) {
@@ -577,7 +583,7 @@ __global__ void __launch_bounds__(256) prune_index_kernel(const __grid_constant_
     if (i < t.vis[b]) {
       row = i;                                                    // before the visual span
     } else if (i < t.vis[b] + t.nk[b]) {
-      const int k = kept[t.k0[b] + i - t.vis[b]] - t.v0[b];       // kept visual token (local)
+      const int k = __ldcg(kept + t.k0[b] + i - t.vis[b]) - t.v0[b];       // kept visual token (local)
       if (k < 0 || k >= t.nv[b]) {
         record_error(status, PACE_ERR_INVALID_ARG, K_PRUNE_INDEX);
         row = -1;
@@ -622,7 +628,7 @@ __device__ __forceinline__ void gather_block(const pace_gather_tensor& g, INDEX 
     col[u] = e - r * cols;
     slab[u] = r / n_idx;
     row[u] = r - slab[u] * n_idx;
-    src[u] = e < total ? __ldg(idx + row[u]) : -1;
+    src[u] = e < total ? __ldcg(idx + row[u]) : -1;
   }
 #pragma unroll
   for (int u = 0; u < kGmU; ++u) {
@@ -655,6 +661,7 @@ __device__ __forceinline__ void gather_block_of(const pace_gather_tensor& g, int
 __global__ void __launch_bounds__(kGmThreads) gather_multi_kernel(const __grid_constant__ GatherMultiTable t,
                                                                   const int32_t* __restrict__ idx, int64_t n_idx,
                                                                   int* status) {
+  ptx::begin_call();
   for (int64_t w = blockIdx.x; w < t.block_prefix[t.n]; w += gridDim.x) {
     int k = 0;
     while (k + 1 < t.n && t.block_prefix[k + 1] <= w) ++k;
@@ -702,17 +709,13 @@ extern "C" pace_status_t pace_ddae_select(const float* s_llm_raw, const float* s
       t.nk[i] = cu_keep[b + 1] - cu_keep[b];
       per_thread = std::max(per_thread, (t.nv[i] + kSelThreads - 1) / kSelThreads);
     }
-    // scores per thread in registers: 4 or 12, else (maps above 12288 tokens) read again per pass
-    if (per_thread <= 4)
-      ddae_select_kernel<4><<<nb, kSelThreads, 0, stream>>>(s_llm_raw, s_vis_raw, t, tau, fusion, s_final, weights,
-                                                             kept, c0, status);
-    else if (per_thread <= kSelRegMax)
-      ddae_select_kernel<kSelRegMax><<<nb, kSelThreads, 0, stream>>>(s_llm_raw, s_vis_raw, t, tau, fusion, s_final,
-                                                                      weights, kept, c0, status);
-    else
-      ddae_select_kernel<0><<<nb, kSelThreads, 0, stream>>>(s_llm_raw, s_vis_raw, t, tau, fusion, s_final, weights,
-                                                             kept, c0, status);
-    PACE_CHECK(check_launch());
+    // scores per thread in registers: 4, 8 or 12, else (maps above 12288 tokens) read again per pass
+    auto* kernel = per_thread <= 4            ? ddae_select_kernel<4>
+                   : per_thread <= 8          ? ddae_select_kernel<8>
+                   : per_thread <= kSelRegMax ? ddae_select_kernel<kSelRegMax>
+                                              : ddae_select_kernel<0>;
+    PACE_CHECK(launch_dependent(kernel, static_cast<unsigned>(nb), kSelThreads, 0, 1, stream, s_llm_raw, s_vis_raw, t, tau,
+                                fusion, s_final, weights, kept, c0, status));
   }
   return PACE_OK;
 }
@@ -743,19 +746,17 @@ extern "C" pace_status_t pace_gather(const void* src, int64_t n_src_rows, int64_
     const int rv = static_cast<int>(row_vec);
     const uint4* s4 = static_cast<const uint4*>(src);
     uint4* d4 = static_cast<uint4*>(dst);
-    if (row_vec <= 32 * 4) gather_rows_warp<4><<<g, 128, 0, stream>>>(s4, n_src_rows, rv, idx, n_idx, d4, status);
-    else if (row_vec <= 32 * 8) gather_rows_warp<8><<<g, 128, 0, stream>>>(s4, n_src_rows, rv, idx, n_idx, d4, status);
-    else gather_rows_warp<16><<<g, 128, 0, stream>>>(s4, n_src_rows, rv, idx, n_idx, d4, status);
-  } else if (vec) {
+    auto* kernel = row_vec <= 32 * 4 ? gather_rows_warp<4> : row_vec <= 32 * 8 ? gather_rows_warp<8> : gather_rows_warp<16>;
+    return launch_dependent(kernel, g, 128, 0, 1, stream, s4, n_src_rows, rv, idx, n_idx, d4, status);
+  }
+  if (vec) {
     const int64_t pieces = (row_bytes / 16 + kGatherPiece - 1) / kGatherPiece;
     blocks = std::min<int64_t>((n_idx * pieces + warps_per_block - 1) / warps_per_block, static_cast<int64_t>(sms) * 8);
-    gather_rows_v16<<<static_cast<unsigned>(blocks), 256, 0, stream>>>(
-        static_cast<const uint4*>(src), n_src_rows, row_bytes / 16, idx, n_idx, static_cast<uint4*>(dst), status);
-  } else {
-    gather_rows_bytes<<<static_cast<unsigned>(blocks), 256, 0, stream>>>(
-        static_cast<const uint8_t*>(src), n_src_rows, row_bytes, idx, n_idx, static_cast<uint8_t*>(dst), status);
+    return launch_dependent(gather_rows_v16, static_cast<unsigned>(blocks), 256, 0, 1, stream, static_cast<const uint4*>(src),
+                            n_src_rows, row_bytes / 16, idx, n_idx, static_cast<uint4*>(dst), status);
   }
-  return check_launch();
+  return launch_dependent(gather_rows_bytes, static_cast<unsigned>(blocks), 256, 0, 1, stream, static_cast<const uint8_t*>(src),
+                          n_src_rows, row_bytes, idx, n_idx, static_cast<uint8_t*>(dst), status);
 }
 
 extern "C" pace_status_t pace_prune_index(int B, const int32_t* cu_seq, const int32_t* vis_start,
@@ -797,8 +798,7 @@ extern "C" pace_status_t pace_prune_index(int B, const int32_t* cu_seq, const in
       if (np > max_post) max_post = np;
     }
     const dim3 grid(static_cast<unsigned>(std::min((max_post + 255) / 256, 64)), static_cast<unsigned>(nb));
-    prune_index_kernel<<<grid, 256, 0, stream>>>(t, kept, out_idx, status);
-    PACE_CHECK(check_launch());
+    PACE_CHECK(launch_dependent(prune_index_kernel, grid, 256, 0, 1, stream, t, kept, out_idx, status));
   }
   return PACE_OK;
 }
@@ -829,6 +829,5 @@ extern "C" pace_status_t pace_gather_multi(const pace_gather_tensor* tensors, in
   PACE_CHECK(check_device());
   int* status = device_status_word();
   const unsigned grid = static_cast<unsigned>(std::min<int64_t>(t.block_prefix[n_tensors], 1 << 20));
-  gather_multi_kernel<<<grid, kGmThreads, 0, stream>>>(t, idx, n_idx, status);
-  return check_launch();
+  return launch_dependent(gather_multi_kernel, grid, kGmThreads, 0, 1, stream, t, idx, n_idx, status);
 }

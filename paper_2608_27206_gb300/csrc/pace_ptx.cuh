@@ -30,6 +30,14 @@ __device__ __forceinline__ uint64_t globaltimer_ns() {
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// The start of a call's first kernel, itself launched dependent: whatever ran before in the stream is
+// complete, and only then may the call's next kernel (or the next call) be started.  The order matters:
+// a kernel started earlier could run beside work of the previous call that still uses its scratch.
+__device__ __forceinline__ void begin_call() {
+  grid_dependency_wait();
+  launch_dependents();
+}
+
 // Cluster barrier in two halves (release / acquire); every thread of the cluster calls both.
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }

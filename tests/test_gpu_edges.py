@@ -219,3 +219,42 @@ def test_resample_scales(pace, shape, size):
     x = O.resample_float(img, *size)
     assert np.all(np.abs(x - np.floor(x) - 0.5)[out != ref] <= 2e-4)
     assert not dst[n:].any()
+
+
+# every call's first kernel may be launched while the stream's previous work runs: inputs written right
+# before a call, scratch and outputs used again right after one, in a stream and in a captured graph
+@pytest.mark.parametrize("captured", [False, True])
+def test_calls_back_to_back(pace, captured):
+    from paper_2608_27206_gb300.hotpath import HotPath
+    hp = HotPath(synth.make_workload("img448", seed=3), "cuda")
+    names = ("stats", "dist", "resized", "s_vis", "s_llm", "s_final", "weights", "kept", "rows")
+    inputs = {k: v.clone() for k, v in hp.d.items()}
+    other = {k: (255 - v if k == "img" else -v.flip(0)) for k, v in inputs.items()}
+
+    def run(src, sync):
+        for _, call in hp.parts:
+            for k, v in src.items():   # written just before each call
+                hp.d[k].copy_(v)
+            call()
+            if sync:
+                torch.cuda.synchronize()
+        return {k: getattr(hp, k).clone() for k in names}
+
+    want = [run(s, True) for s in (inputs, other)]
+    torch.cuda.synchronize()
+    stream, rounds = torch.cuda.Stream(), 5
+    with torch.cuda.stream(stream):
+        if captured:
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=stream):
+                out = [run(s, False) for s in (inputs, other)]
+            got = []
+            for _ in range(rounds):
+                g.replay()
+                got += [{k: v.clone() for k, v in o.items()} for o in out]
+        else:
+            got = [run(s, False) for _ in range(rounds) for s in (inputs, other)]
+    torch.cuda.synchronize()
+    for i, o in enumerate(got):
+        for k in names:
+            assert torch.equal(o[k].view(torch.uint8), want[i % 2][k].view(torch.uint8)), (i, k)
