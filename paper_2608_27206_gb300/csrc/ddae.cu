@@ -37,6 +37,7 @@ struct SelectTable {
 };
 
 struct SelShared {
+  float4 coef;                  // the maps' minima, then their weights over their ranges
   float red[8][kSelWarps];      // warp partials of the block reduction (min, max and two moments per map)
   unsigned bins[kSelBins];      // histogram of the current selection round
   unsigned wtot[kSelWarps];     // per-warp totals (bin prefix)
@@ -210,51 +211,55 @@ __global__ void __launch_bounds__(kSelThreads) ddae_select_kernel(const float* _
     sh.red[4][warp] = s1a; sh.red[5][warp] = s2a; sh.red[6][warp] = s1v; sh.red[7][warp] = s2v;
   }
   if (__syncthreads_or(bad) && tid == 0) record_error(status, PACE_ERR_INVALID_ARG, K_DDAE_SELECT);
-  // lane l takes warp l's partials; the butterflies leave the block's values in every lane
-  const float mna = warp_min(sh.red[0][lane]), mxa = warp_max(sh.red[1][lane]);
-  const float mnv = warp_min(sh.red[2][lane]), mxv = warp_max(sh.red[3][lane]);
-  const float t1a = warp_sum(sh.red[4][lane]), t2a = warp_sum(sh.red[5][lane]);
-  const float t1v = warp_sum(sh.red[6][lane]), t2v = warp_sum(sh.red[7][lane]);
-  const float ar = mxa - mna, vr = mxv - mnv;
-  // (x - min) / range as a product with the range's reciprocal: within an ulp of the quotient,
-  // and exact when the range is a power of two (a map spanning [0, 1] keeps its values)
-  const float ia = ar > 0.f ? 1.0f / ar : 0.f, iv = vr > 0.f ? 1.0f / vr : 0.f;
-
-  // 2-3. the normalised maps' population variances: (x - min) / range has the variance of x
-  // divided by range^2, and var x = E[(x - c)^2] - (E[x - c])^2
-  const float inv_n = 1.0f / static_cast<float>(nv);
-  const float m1a = t1a * inv_n, m1v = t1v * inv_n;
-  const float var_a = fmaxf(fmaf(-m1a, m1a, t2a * inv_n), 0.f) * ia * ia;
-  const float var_v = fmaxf(fmaf(-m1v, m1v, t2v * inv_n), 0.f) * iv * iv;
-  const float sig_a = sqrtf(var_a), sig_v = sqrtf(var_v);
-  float wa, wv;
-  if (fusion == PACE_DDAE_ONLY_LLM) {
-    wa = 1.f;
-    wv = 0.f;
-  } else if (fusion == PACE_DDAE_ONLY_VIT) {
-    wa = 0.f;
-    wv = 1.f;
-  } else if (fusion == PACE_DDAE_FIXED) {
-    wa = wv = 0.5f;
-  } else {   // Eq. 7
-    // (every thread evaluates these; the fast intrinsics are within a few ulp)
-    const float za = __fdividef(sig_a, tau), zv = __fdividef(sig_v, tau), zm = fmaxf(za, zv);
-    const float ea = __expf(za - zm), ev = __expf(zv - zm);
-    const float inv = __fdividef(1.0f, ea + ev);
-    wa = ea * inv;
-    wv = ev * inv;
+  // 2-3. by the first warp alone, lane l taking warp l's partials (32 warps at it, each for itself, took
+  // 0.7 us of a 9.5 us map): the normalised maps' population variances ((x - min) / range has the
+  // variance of x divided by range^2, and var x = E[(x - c)^2] - (E[x - c])^2), then the weights
+  if (warp == 0) {
+    const float mna = warp_min(sh.red[0][lane]), mxa = warp_max(sh.red[1][lane]);
+    const float mnv = warp_min(sh.red[2][lane]), mxv = warp_max(sh.red[3][lane]);
+    const float t1a = warp_sum(sh.red[4][lane]), t2a = warp_sum(sh.red[5][lane]);
+    const float t1v = warp_sum(sh.red[6][lane]), t2v = warp_sum(sh.red[7][lane]);
+    const float ar = mxa - mna, vr = mxv - mnv;
+    // (x - min) / range as a product with the range's reciprocal: within an ulp of the quotient,
+    // and exact when the range is a power of two (a map spanning [0, 1] keeps its values)
+    const float ia = ar > 0.f ? 1.0f / ar : 0.f, iv = vr > 0.f ? 1.0f / vr : 0.f;
+    const float inv_n = 1.0f / static_cast<float>(nv);
+    const float m1a = t1a * inv_n, m1v = t1v * inv_n;
+    const float var_a = fmaxf(fmaf(-m1a, m1a, t2a * inv_n), 0.f) * ia * ia;
+    const float var_v = fmaxf(fmaf(-m1v, m1v, t2v * inv_n), 0.f) * iv * iv;
+    const float sig_a = sqrtf(var_a), sig_v = sqrtf(var_v);
+    float wa, wv;
+    if (fusion == PACE_DDAE_ONLY_LLM) {
+      wa = 1.f;
+      wv = 0.f;
+    } else if (fusion == PACE_DDAE_ONLY_VIT) {
+      wa = 0.f;
+      wv = 1.f;
+    } else if (fusion == PACE_DDAE_FIXED) {
+      wa = wv = 0.5f;
+    } else {   // Eq. 7 (the fast intrinsics are within a few ulp)
+      const float za = __fdividef(sig_a, tau), zv = __fdividef(sig_v, tau), zm = fmaxf(za, zv);
+      const float ea = __expf(za - zm), ev = __expf(zv - zm);
+      const float inv = __fdividef(1.0f, ea + ev);
+      wa = ea * inv;
+      wv = ev * inv;
+    }
+    if (lane == 0) {
+      if (weights != nullptr) {
+        weights[2 * (b_base + b)] = wa;
+        weights[2 * (b_base + b) + 1] = wv;
+      }
+      sh.coef = make_float4(mna, mnv, wa * ia, wv * iv);
+    }
   }
-  if (tid == 0 && weights != nullptr) {
-    weights[2 * (b_base + b)] = wa;
-    weights[2 * (b_base + b) + 1] = wv;
-  }
+  __syncthreads();
+  const float4 coef = sh.coef;
 
   // 4. S_final (in registers, ra reused, when RM > 0: written out by the first counting pass
   // below, or before an early return; otherwise written here)
   // alpha_w (a - min_a) / range_a + beta_w (v - min_v) / range_v with each map's weight and
   // reciprocal range folded into one coefficient
-  const float cfa = wa * ia, cfv = wv * iv;
-  auto fused = [&](float a, float v) { return fmaf(cfa, a - mna, cfv * (v - mnv)); };
+  auto fused = [&](float a, float v) { return fmaf(coef.z, a - coef.x, coef.w * (v - coef.y)); };
   if constexpr (RM > 0) {
 #pragma unroll
     for (int k = 0; k < RM; ++k)

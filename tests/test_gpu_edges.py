@@ -258,3 +258,19 @@ def test_calls_back_to_back(pace, captured):
     for i, o in enumerate(got):
         for k in names:
             assert torch.equal(o[k].view(torch.uint8), want[i % 2][k].view(torch.uint8)), (i, k)
+
+
+# scores held in registers for 4, 8 and 12 per thread of a block of 1024, and read again per pass above
+@pytest.mark.parametrize("n", [4096, 4097, 8192, 8193, 12288, 12289])
+def test_select_registers(pace, n):
+    rng = np.random.default_rng(n)
+    # one map for both: S_final is the map itself when it spans [0, 1] and the weights are 1/2
+    x = (rng.permutation(n).astype(np.float32) / np.float32(1 << 14)).astype(np.float32)
+    x[rng.integers(1, n - 1)] = 1.0
+    x[0] = 0.0
+    K = O.budget(n, 0.1)
+    s = torch.from_numpy(x).cuda()
+    s_final, w, kept = pace.pace_ddae_select(s, s, [0, n], [0, K])
+    np.testing.assert_array_equal(s_final.cpu().numpy(), x)
+    assert w.cpu().numpy().tolist() == [[0.5, 0.5]]
+    np.testing.assert_array_equal(kept.cpu().numpy(), O.top_k_ascending(x.astype(np.float64), K))
