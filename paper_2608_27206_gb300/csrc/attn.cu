@@ -424,21 +424,30 @@ __global__ void __launch_bounds__(kThreads, 1) attn_row_lse(const __grid_constan
   const int item = blockIdx.x >> 1;
   const int b = find_image(t, item);
   int r = item - t.item_prefix[b];
-  const int split = r % t.splits;
-  r /= t.splits;
+  // (the set-up before the barriers is on every CTA's critical path: no divisions that are not needed,
+  // none in 64 bits)
+  int split = 0;
+  if (t.splits > 1) {
+    split = r % t.splits;
+    r /= t.splits;
+  }
   const int npair = t.pair_n[b];
   const int diag = t.diag[b];
   // causal images: the last query rows see the most keys, so those of every head are scheduled
   // first; otherwise the query tiles of a head follow one another (they stream the same keys)
-  const int h = CAUSAL ? r % t.H : r / npair;
-  const int pair = t.pair_lo[b] + (CAUSAL ? npair - 1 - r / t.H : r % npair);
-  const int g = h / t.G;
+  const int rq = CAUSAL ? r / t.H : r / npair, rr0 = r - rq * (CAUSAL ? t.H : npair);
+  const int h = CAUSAL ? rr0 : rq;
+  const int pair = t.pair_lo[b] + (CAUSAL ? npair - 1 - rq : rr0);
+  const int g = t.G > 1 ? h / t.G : h;
   const int qrow0 = pair * kPair + kTile * static_cast<int>(rank);     // this CTA's first local query row
   if (qrow0 >= t.nq[b]) return;   // the item's second half lies past the image: pass 2 does not read its shift rows
   const int nkt_all = (t.nk[b] + kStream - 1) / kStream;
-  const int kt0 = static_cast<int>((static_cast<int64_t>(split) * nkt_all) / t.splits);
+  int kt0 = 0, kt1_all = nkt_all;
+  if (t.splits > 1) {   // at most 32 splits of fewer than 2^23 tiles
+    kt0 = static_cast<unsigned>(split * nkt_all) / static_cast<unsigned>(t.splits);
+    kt1_all = static_cast<unsigned>((split + 1) * nkt_all) / static_cast<unsigned>(t.splits);
+  }
   // causal: key tiles past the one holding key qrow0 + 127 + diag are masked for every row (diag >= 0)
-  const int kt1_all = static_cast<int>((static_cast<int64_t>(split + 1) * nkt_all) / t.splits);
   const int kt1 = CAUSAL ? min(kt1_all, (diag + qrow0 + kTile - 1) / kStream + 1) : kt1_all;
   const int nj = max(kt1 - kt0, 0);
   const int pre = min(nj, ST);   // key stages issued in the prologue (round 0, first use of each stage)
@@ -692,14 +701,18 @@ __global__ void __launch_bounds__(kThreads, 1) attn_colsum(const __grid_constant
   const int item = blockIdx.x >> 1;
   const int b = find_image(t, item);
   int r = item - t.item_prefix[b];
-  const int sp = r % t.splits2;
-  r /= t.splits2;
+  int sp = 0;
+  if (t.splits2 > 1) {
+    sp = r % t.splits2;
+    r /= t.splits2;
+  }
   const int nkp = (t.nk[b] + kPair - 1) / kPair;
   // causal images: the first keys are seen by the most queries, so those of every KV head are
   // scheduled first; otherwise the key tiles of a head follow one another
-  const int nkv = t.H / t.G;
-  const int g = CAUSAL ? r % nkv : r / nkp;
-  const int kp = CAUSAL ? r / nkv : r % nkp;
+  const int per = CAUSAL ? t.H / t.G : nkp;
+  const int rq = r / per, rr0 = r - rq * per;
+  const int g = CAUSAL ? rr0 : rq;
+  const int kp = CAUSAL ? rq : rr0;
   const int krow0 = kp * kPair + kTile * static_cast<int>(rank);     // this CTA's first local key row
   if (krow0 >= t.nk[b]) return;   // the item's second half lies past the image
   const int diag = t.diag[b];
@@ -709,9 +722,12 @@ __global__ void __launch_bounds__(kThreads, 1) attn_colsum(const __grid_constant
   const int nspan = max(nqt - qt_min, 0);
   // the stream: (head in group, query tile), of which this CTA takes items j0 .. j0 + nj - 1
   const int nj_all = t.G * nspan;
-  const int each = nj_all / t.splits2, extra = nj_all - each * t.splits2;
-  const int j0 = sp * each + min(sp, extra);
-  const int nj = each + (sp < extra ? 1 : 0);
+  int j0 = 0, nj = nj_all;
+  if (t.splits2 > 1) {
+    const int each = nj_all / t.splits2, extra = nj_all - each * t.splits2;
+    j0 = sp * each + min(sp, extra);
+    nj = each + (sp < extra ? 1 : 0);
+  }
   // A last query tile that ends inside the stream tile:
   //  - its rows past the image are zeros when the image is the last of Q (they lie outside the
   //    tensor), else the next image's rows, which warp 0 overwrites with zeros (`fix`).  It then
@@ -726,17 +742,17 @@ __global__ void __launch_bounds__(kThreads, 1) attn_colsum(const __grid_constant
   // first local stream item that is such a tile (the next ones follow every nspan items)
   auto first_special = [&]() {
     if (!(fix || half) || nj <= 0) return INT_MAX;
-    const int d = special - j0 % nspan;
+    const int d = special - (j0 == 0 ? 0 : j0 % nspan);
     return d < 0 ? d + nspan : d;
   };
   struct Pos {   // a stream item: head in group hq, position i in its query tiles
     int hq, i;
   };
   auto pos_at = [&](int j) {
-    Pos q{0, 0};
-    if (nj > 0) {
-      q.hq = (j0 + j) / nspan;
-      q.i = j0 + j - q.hq * nspan;
+    Pos q{0, j0 + j};
+    if (nj > 0 && q.i >= nspan) {
+      q.hq = q.i / nspan;
+      q.i -= q.hq * nspan;
     }
     return q;
   };
