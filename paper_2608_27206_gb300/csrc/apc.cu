@@ -459,7 +459,6 @@ struct TailParams {
 };
 
 constexpr int kTailBins = 4096;            // level-1 buckets of the tail select
-constexpr int kTailBins2 = 1024;           // level-2 offset bins over a listed bucket
 
 // Bucket of a distance d >= 0: floor(2048 d), capped at the top bucket (monotone in d; NaN goes to
 // bucket 0).  Full-rate arithmetic only (no float-to-integer conversion): once clamped to
@@ -1195,10 +1194,10 @@ __device__ __forceinline__ void select_from_top(const unsigned* bins, unsigned r
   static_assert(PER >= 1 && PER * 1024 == NBINS, "bins");
   __shared__ unsigned count;
   const int top = NBINS - 1 - PER * static_cast<int>(threadIdx.x);
-  unsigned c[PER];
-#pragma unroll
-  for (int q = 0; q < PER; ++q) c[q] = bins[top - q];
-  select_from_counts<PER>(c, top, r, sel, wsum, &count);
+  static_assert(PER == 4, "one 16-byte read per thread");
+  const uint4 v = *reinterpret_cast<const uint4*>(bins + top - 3);
+  const unsigned c[4] = {v.w, v.z, v.y, v.x};
+  select_from_counts<4>(c, top, r, sel, wsum, &count);
 }
 
 // Eq. 5-6 and R3-R4 from the tail mean d_top of image b: rho_d, rho, r and the target size.
@@ -1229,12 +1228,16 @@ __device__ __forceinline__ void tail_finish(const ApcTable& t, int b, const Tail
 // counts alone, and only that bucket's members are looked for in the distances.  A cluster of
 // CTAs per image: every CTA selects the bucket for itself, scans its share of the distances
 // (loaded before the selection, so that the two latencies overlap) and appends the members to the
-// first CTA's shared list; after one cluster barrier the first CTA narrows the members to the k-th
-// largest distance T (members all equal: at once; at most 1024: each ranked against the others;
-// else rounds of 1024 bins over the key offsets from the bucket's first fp32 key) and writes the
-// statistics.  A bucket with too many different members for the list is narrowed over the whole
-// array by rounds of 4096 bins.  Everything is latency: a chain of L2 reads and block barriers.
+// first CTA's shared list, with one reservation per warp (a remote atomic and its answer take about
+// half a microsecond, and one per distance row made eight in a row); after one cluster barrier the
+// first CTA narrows the members to the k-th largest distance T (at most kTailRank: each ranked
+// against the others; else rounds of 4096 bins over the key offsets from the smallest member) and
+// writes the statistics.  A bucket with too many different members for the list is narrowed over the
+// whole array by such rounds.  Everything is latency: a chain of L2 reads and block barriers.
 constexpr int kTailList = 4096;    // members listed
+// Members ranked directly: c^2 comparisons over 1024 threads take 1 us at 256 members, 16 us at 1024,
+// a round of bins about 1 us whatever their number.
+constexpr int kTailRank = 256;
 constexpr int kTailAhead = 8;      // distances per thread loaded ahead of the selection
 constexpr int kTailCluster = 8;    // CTAs per image above kTailAhead * 1024 distances
 
@@ -1242,7 +1245,7 @@ __global__ void __launch_bounds__(1024) apc_tail(const __grid_constant__ ApcTabl
                                                  TailParams prm, pace_apc_stats* __restrict__ stats,
                                                  const TailWork* __restrict__ work) {
   __shared__ unsigned list[kTailList];
-  __shared__ unsigned bins[kTailBins];   // bins of the narrowing rounds
+  __shared__ __align__(16) unsigned bins[kTailBins];   // bins of the narrowing rounds
   __shared__ unsigned sel[2], selb[2];
   __shared__ unsigned cred[32];
   __shared__ unsigned long long fred[32];
@@ -1292,7 +1295,7 @@ __global__ void __launch_bounds__(1024) apc_tail(const __grid_constant__ ApcTabl
     if (top - 2 > tb) s_fix += s23.y;
     if (top - 3 > tb) s_fix += s23.x;
   }
-  const bool listed = cb <= kTailList, spread = cb > 1024u;
+  const bool listed = cb <= kTailList;
   unsigned* list0 = list;
   unsigned *n0 = &list_n, *min0 = &key_min, *max0 = &key_max;
   if (ncta > 1) {
@@ -1302,30 +1305,51 @@ __global__ void __launch_bounds__(1024) apc_tail(const __grid_constant__ ApcTabl
     min0 = cluster.map_shared_rank(&key_min, 0);
     max0 = cluster.map_shared_rank(&key_max, 0);
   }
-  // this CTA's members of the bucket
+  // this CTA's members of the bucket: the keys lo .. lo + span - 1 (bucket 0 also takes NaN, whose key
+  // lies elsewhere)
+  unsigned lo = __float_as_uint(static_cast<float>(tb) * (1.0f / 2048.0f));
+  unsigned span = (tb == kTailBins - 1 ? 0x7F800001u : __float_as_uint(static_cast<float>(tb + 1) * (1.0f / 2048.0f))) - lo;
+  const unsigned bucket_lo = lo, bucket_span = span;
   unsigned kmin = 0xFFFFFFFFu, kmax = 0u;
-  auto scan = [&](float v, bool live) {
-    const bool member = live && tail_bucket(v) == tb;
-    const unsigned ball = __ballot_sync(0xffffffffu, member);
-    if (ball == 0u) return;
-    const unsigned key = __float_as_uint(v);
-    if (member) {
-      kmin = min(kmin, key);
-      kmax = max(kmax, key);
-    }
-    if (!listed) return;
-    unsigned slot = 0u;   // one slot reservation per warp
-    if (lane == 0) slot = atomicAdd(n0, static_cast<unsigned>(__popc(ball)));
-    slot = __shfl_sync(0xffffffffu, slot, 0) + __popc(ball & ((1u << lane) - 1u));
-    if (member) list0[slot] = key;
-  };
+  for (int base = rank * 1024; base < N; base += kTailAhead * step) {   // uniform trip count per CTA
+    unsigned members = 0u;   // bit q: ahead[q] is one
 #pragma unroll
-  for (int q = 0; q < kTailAhead; ++q) scan(ahead[q], i0 + q * step < N);
-  for (int base = rank * 1024 + kTailAhead * step; base < N; base += step) {   // uniform trip count per CTA
-    const int i = base + tid;
-    scan(i < N ? __ldcg(db + i) : 0.f, i < N);
+    for (int q = 0; q < kTailAhead; ++q) {
+      const bool in = tb != 0 ? __float_as_uint(ahead[q]) - bucket_lo < bucket_span   // (0 past the end: no member)
+                              : base + tid + q * step < N && tail_bucket(ahead[q]) == 0;
+      members |= in ? 1u << q : 0u;
+    }
+    const unsigned mine = static_cast<unsigned>(__popc(members)), all = __reduce_add_sync(0xffffffffu, mine);
+    if (all != 0u) {   // warp-uniform
+      unsigned slot = 0u;
+      if (listed) {
+        unsigned incl = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const unsigned n = __shfl_up_sync(0xffffffffu, incl, o);
+          if (lane >= o) incl += n;
+        }
+        if (lane == 0) slot = atomicAdd(n0, all);
+        slot = __shfl_sync(0xffffffffu, slot, 0) + incl - mine;
+      }
+#pragma unroll
+      for (int q = 0; q < kTailAhead; ++q) {
+        if (!((members >> q) & 1u)) continue;
+        const unsigned key = __float_as_uint(ahead[q]);
+        kmin = min(kmin, key);
+        kmax = max(kmax, key);
+        if (listed) list0[slot++] = key;
+      }
+    }
+    if (base + kTailAhead * step < N) {
+#pragma unroll
+      for (int q = 0; q < kTailAhead; ++q) {
+        const int i = base + tid + (kTailAhead + q) * step;
+        ahead[q] = i < N ? __ldcg(db + i) : 0.f;
+      }
+    }
   }
-  if (spread) {
+  if (!listed) {
     kmin = __reduce_min_sync(0xffffffffu, kmin);
     kmax = __reduce_max_sync(0xffffffffu, kmax);
     if (lane == 0 && kmax >= kmin) {
@@ -1339,11 +1363,8 @@ __global__ void __launch_bounds__(1024) apc_tail(const __grid_constant__ ApcTabl
   // level 2: T = the k-th largest distance; the members of the bucket above T are summed in fixed
   // point (c counts every distance above T)
   unsigned remaining = k - above_n, cnt = 0u;
-  unsigned lo = __float_as_uint(static_cast<float>(tb) * (1.0f / 2048.0f));
-  unsigned span = (tb == kTailBins - 1 ? 0x7F800001u : __float_as_uint(static_cast<float>(tb + 1) * (1.0f / 2048.0f))) - lo;
-  const unsigned bucket_lo = lo, bucket_span = span;
   unsigned prefix;
-  if (!spread) {
+  if (cb <= kTailRank) {
     // one member per thread, ranked against the whole list: a member with fewer than `remaining`
     // members at or above it lies above the k-th largest (and is summed); with fewer than
     // `remaining` above it but at least that many at or above it, it is the k-th largest
@@ -1360,25 +1381,45 @@ __global__ void __launch_bounds__(1024) apc_tail(const __grid_constant__ ApcTabl
     }
     __syncthreads();
     prefix = selb[1];
-  } else if (key_min == key_max) {   // every member is the same distance
-    prefix = key_min;
   } else if (listed) {
-    while (true) {
+    unsigned mn = 0xFFFFFFFFu, mx = 0u;
+    for (int i = tid; i < static_cast<int>(cb); i += blockDim.x) {
+      mn = min(mn, list[i]);
+      mx = max(mx, list[i]);
+    }
+    mn = __reduce_min_sync(0xffffffffu, mn);
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if (lane == 0) {
+      atomicMin(&key_min, mn);
+      atomicMax(&key_max, mx);
+    }
+    static_assert(kTailBins == 4 * 1024, "one 16-byte store per thread clears the bins");
+    reinterpret_cast<uint4*>(bins)[tid] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+    lo = key_min;
+    span = key_max - lo + 1u;
+    while (span > 1u) {   // (one key: every member is the same distance)
       const int bits = 32 - __clz(span - 1u);
-      const int shift = bits > 10 ? bits - 10 : 0;
-      for (int i = tid; i < kTailBins2; i += blockDim.x) bins[i] = 0u;
-      __syncthreads();
-      for (int i = tid; i < static_cast<int>(cb); i += blockDim.x) {
-        const unsigned off = list[i] - lo;   // wraps for keys below lo
-        if (off < span) atomicAdd(&bins[off >> shift], 1u);
+      const int shift = bits > 12 ? bits - 12 : 0;
+      for (int base = 0; base < static_cast<int>(cb); base += blockDim.x) {
+        const unsigned off = base + tid < static_cast<int>(cb) ? list[base + tid] - lo : span;   // wraps for keys below lo
+        const unsigned bin = off < span ? off >> shift : kTailBins;
+        const unsigned first = __shfl_sync(0xffffffffu, bin, 0);
+        if (__all_sync(0xffffffffu, bin == first)) {   // equal distances: one addition
+          if (lane == 0 && first < kTailBins) atomicAdd(&bins[first], 32u);
+        } else if (bin < kTailBins) {
+          atomicAdd(&bins[bin], 1u);
+        }
       }
       __syncthreads();
-      select_from_top<kTailBins2>(bins, remaining, sel, cred);
+      select_from_top<kTailBins>(bins, remaining, sel, cred);
       lo += sel[0] << shift;
       remaining -= sel[1];
       if (shift == 0) break;
       span = min(span - (sel[0] << shift), 1u << shift);
       __syncthreads();   // everyone has read sel and the bins
+      reinterpret_cast<uint4*>(bins)[tid] = make_uint4(0u, 0u, 0u, 0u);
+      __syncthreads();
     }
     prefix = lo;
     for (int i = tid; i < static_cast<int>(cb); i += blockDim.x) {
@@ -1388,6 +1429,8 @@ __global__ void __launch_bounds__(1024) apc_tail(const __grid_constant__ ApcTabl
         ++cnt;
       }
     }
+  } else if (key_min == key_max) {   // every member is the same distance
+    prefix = key_min;
   } else {
     // a crowded bucket: its members by key offset from its first key over the whole array,
     // 4096 offsets (2^shift keys each) at a time, until one key is left
@@ -1399,7 +1442,7 @@ __global__ void __launch_bounds__(1024) apc_tail(const __grid_constant__ ApcTabl
       __syncthreads();
       for (int base = 0; base < N; base += blockDim.x) {   // uniform trip count: __match_any_sync below
         const int i = base + tid;
-        const unsigned off = i < N ? __float_as_uint(db[i]) - lo : span;   // wraps for keys below lo
+        const unsigned off = i < N ? __float_as_uint(__ldcg(db + i)) - lo : span;   // wraps for keys below lo
         const bool in = off < span;
         const unsigned digit = in ? off >> shift : kTailBins;
         const unsigned members = __ballot_sync(0xffffffffu, in);
@@ -1419,7 +1462,7 @@ __global__ void __launch_bounds__(1024) apc_tail(const __grid_constant__ ApcTabl
     }
     prefix = lo;
     for (int i = tid; i < N; i += blockDim.x) {   // the bucket's members above T
-      const unsigned key = __float_as_uint(db[i]);
+      const unsigned key = __float_as_uint(__ldcg(db + i));
       if (key > prefix && key - bucket_lo < bucket_span) {
         s_fix += fix32(__uint_as_float(key));
         ++cnt;

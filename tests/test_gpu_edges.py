@@ -133,6 +133,26 @@ def test_density_tail_cluster(pace, kind):
     assert abs(pace.stats_dict(st)[0]["d_top"] - top) <= 4e-7 * top + 1e-9
 
 
+# the tail's bucket: ranked directly (up to 256 members), by rounds over the list (up to 4096), over the
+# whole array, in one CTA (up to 8192 distances) and a cluster; in the first bucket and in another, a few
+# and many different distances
+@pytest.mark.parametrize("n", [256, 257, 600, 4096, 4300, 9000, 70000])
+@pytest.mark.parametrize("offset,values", [(0.0, 3), (0.0, 128), (0.5, 2), (0.5, 128)])
+def test_tail_members(pace, n, offset, values):
+    rng = np.random.default_rng(n)
+    # unit-ish tokens (1, +-offset, y): y moves the distance to the mean by less than a bucket (2^-11)
+    T = np.zeros((n, 8))
+    T[:, 0], T[:, 1] = 1.0, offset * np.where(np.arange(n) % 2, 1, -1)
+    T[:, 2] = rng.integers(0, values, n) * ((2.0 ** -12 if offset == 0.0 else 2.0 ** -6) / values)
+    bits = synth.f32_to_bf16_bits(T.astype(np.float32))
+    d, st = pace.pace_apc_density_tokens(bf16_tensor(bits), [0, n], [252], [252])
+    d, s = d.cpu().numpy(), pace.stats_dict(st)[0]
+    assert_distances_close(d, O.apc_density_preview(f64(bits), 252, 252)["d"])
+    top = np.sort(d.astype(np.float64))[::-1][:s["k_tail"]].mean()
+    # fixed point of 2^-32 per distance, fp32 rounding of the mean
+    assert abs(s["d_top"] - top) <= 4e-7 * top + 2.0 ** -32
+
+
 # distances counted per warp (pictures: the first and the last live lane's bucket at once, the rest one
 # by one) and per run of equal buckets (tokens): all equal, two values in turn, background with few or
 # many others among it, partial warps
