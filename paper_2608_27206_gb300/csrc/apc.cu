@@ -1065,7 +1065,7 @@ __global__ void __launch_bounds__(kApcThreads, 2) apc_tok_vec2(const uint4* __re
   __shared__ __align__(16) float chat[kTokVecMax * 256];
   __shared__ float red[kApcThreads / 32];
   ptx::launch_dependents();
-  ptx::grid_dependency_wait();
+  bool waited = false;
   constexpr int kWarps = kApcThreads / 32;
   const int D = t.D, vecs = D >> 3;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1079,6 +1079,11 @@ __global__ void __launch_bounds__(kApcThreads, 2) apc_tok_vec2(const uint4* __re
 #pragma unroll
     for (int r = 0; r < 2; ++r)
       if (tok - r * kWarps >= lo) tok_load<V>(buf[r], T, tok - r * kWarps, vecs);
+    if (!waited) ptx::grid_dependency_wait();   // (the tokens do not depend on pass 1)
+    waited = true;
+    float inv[2];   // the rows' inverse norms, loaded with them
+#pragma unroll
+    for (int r = 0; r < 2; ++r) inv[r] = tok - r * kWarps >= lo ? __ldcg(inv_norm + tok - r * kWarps) : 0.f;
     const int N = t.n[b];
     const float inv_n = 1.0f / static_cast<float>(N);
     const unsigned long long* sb = sums + static_cast<int64_t>(t.b_base + b) * kSumSlots * D;
@@ -1120,8 +1125,7 @@ __global__ void __launch_bounds__(kApcThreads, 2) apc_tok_vec2(const uint4* __re
 #pragma unroll
       for (int r = 0; r < 2; ++r, tok -= kWarps) {
         if (tok < lo) break;
-        const float iv = __ldcg(inv_norm + tok);
-        const float2 iv2 = make_float2(iv, iv);
+        const float2 iv2 = make_float2(inv[r], inv[r]);
         float2 acc = make_float2(0.f, 0.f), acc1 = acc;
 #pragma unroll
         for (int i = 0; i < V; ++i)
@@ -1131,7 +1135,10 @@ __global__ void __launch_bounds__(kApcThreads, 2) apc_tok_vec2(const uint4* __re
             if (q & 1) acc1 = ptx::ffma2(e, e, acc1);
             else acc = ptx::ffma2(e, e, acc);
           }
-        if (tok - 2 * kWarps >= lo) tok_load<V>(buf[r], T, tok - 2 * kWarps, vecs);
+        if (tok - 2 * kWarps >= lo) {
+          tok_load<V>(buf[r], T, tok - 2 * kWarps, vecs);
+          inv[r] = __ldcg(inv_norm + tok - 2 * kWarps);
+        }
         acc = ptx::fadd2(acc, acc1);
         const float d2 = warp_sum_f(acc.x + acc.y);
         if (lane == 0) {
