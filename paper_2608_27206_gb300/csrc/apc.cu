@@ -1194,9 +1194,9 @@ __device__ __forceinline__ void select_from_counts(const unsigned (&c)[PER], int
   __syncthreads();
 }
 
-// The same for NBINS counts in shared memory.
+// The same for NBINS counts in shared memory; returns the entries in the bin.
 template <int NBINS>
-__device__ __forceinline__ void select_from_top(const unsigned* bins, unsigned r, unsigned* sel, unsigned* wsum) {
+__device__ __forceinline__ unsigned select_from_top(const unsigned* bins, unsigned r, unsigned* sel, unsigned* wsum) {
   constexpr int PER = NBINS / 1024;   // bins per thread
   static_assert(PER >= 1 && PER * 1024 == NBINS, "bins");
   __shared__ unsigned count;
@@ -1205,6 +1205,7 @@ __device__ __forceinline__ void select_from_top(const unsigned* bins, unsigned r
   const uint4 v = *reinterpret_cast<const uint4*>(bins + top - 3);
   const unsigned c[4] = {v.w, v.z, v.y, v.x};
   select_from_counts<4>(c, top, r, sel, wsum, &count);
+  return count;
 }
 
 // Eq. 5-6 and R3-R4 from the tail mean d_top of image b: rho_d, rho, r and the target size.
@@ -1242,9 +1243,10 @@ __device__ __forceinline__ void tail_finish(const ApcTable& t, int b, const Tail
 // writes the statistics.  A bucket with too many different members for the list is narrowed over the
 // whole array by such rounds.  Everything is latency: a chain of L2 reads and block barriers.
 constexpr int kTailList = 4096;    // members listed
-// Members ranked directly: c^2 comparisons over 1024 threads take 1 us at 256 members, 16 us at 1024,
-// a round of bins about 1 us whatever their number.
-constexpr int kTailRank = 256;
+// Members ranked directly: c^2 comparisons over 1024 threads take 1.0 us at 68 members, 4.6 at 229, 16
+// at 1024; a round of bins about 1 us whatever their number.  The line lies where rank_in_list goes from
+// eight threads per member to four.
+constexpr int kTailRank = 128;
 constexpr int kTailAhead = 8;      // distances per thread loaded ahead of the selection
 constexpr int kTailCluster = 8;    // CTAs per image above kTailAhead * 1024 distances
 
@@ -1405,6 +1407,7 @@ __global__ void __launch_bounds__(1024) apc_tail(const __grid_constant__ ApcTabl
     __syncthreads();
     lo = key_min;
     span = key_max - lo + 1u;
+    unsigned only = 0u;   // the k-th largest is the one member among this many keys from lo on
     while (span > 1u) {   // (one key: every member is the same distance)
       const int bits = 32 - __clz(span - 1u);
       const int shift = bits > 12 ? bits - 12 : 0;
@@ -1419,16 +1422,26 @@ __global__ void __launch_bounds__(1024) apc_tail(const __grid_constant__ ApcTabl
         }
       }
       __syncthreads();
-      select_from_top<kTailBins>(bins, remaining, sel, cred);
+      const unsigned in_bin = select_from_top<kTailBins>(bins, remaining, sel, cred);
       lo += sel[0] << shift;
       remaining -= sel[1];
       if (shift == 0) break;
+      if (in_bin == 1u) {
+        only = 1u << shift;
+        break;
+      }
       span = min(span - (sel[0] << shift), 1u << shift);
       __syncthreads();   // everyone has read sel and the bins
       reinterpret_cast<uint4*>(bins)[tid] = make_uint4(0u, 0u, 0u, 0u);
       __syncthreads();
     }
     prefix = lo;
+    if (only != 0u) {
+      for (int i = tid; i < static_cast<int>(cb); i += blockDim.x)
+        if (list[i] - lo < only) selb[1] = list[i];
+      __syncthreads();
+      prefix = selb[1];
+    }
     for (int i = tid; i < static_cast<int>(cb); i += blockDim.x) {
       const unsigned key = list[i];
       if (key > prefix) {

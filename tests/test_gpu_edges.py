@@ -133,10 +133,10 @@ def test_density_tail_cluster(pace, kind):
     assert abs(pace.stats_dict(st)[0]["d_top"] - top) <= 4e-7 * top + 1e-9
 
 
-# the tail's bucket: ranked directly (up to 256 members), by rounds over the list (up to 4096), over the
+# the tail's bucket: ranked directly (up to 128 members), by rounds over the list (up to 4096), over the
 # whole array, in one CTA (up to 8192 distances) and a cluster; in the first bucket and in another, a few
 # and many different distances
-@pytest.mark.parametrize("n", [256, 257, 600, 4096, 4300, 9000, 70000])
+@pytest.mark.parametrize("n", [128, 129, 256, 257, 600, 4096, 4300, 9000, 70000])
 @pytest.mark.parametrize("offset,values", [(0.0, 3), (0.0, 128), (0.5, 2), (0.5, 128)])
 def test_tail_members(pace, n, offset, values):
     rng = np.random.default_rng(n)
