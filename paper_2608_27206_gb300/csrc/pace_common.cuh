@@ -98,11 +98,6 @@ pace_status_t launch_dependent(void (*kernel)(Params...), dim3 grid, dim3 thread
                                cudaStream_t stream, Args... args) {
   return launch_ex(true, kernel, grid, threads, smem, cluster, stream, args...);
 }
-template <typename... Params, typename... Args>
-pace_status_t launch_cluster(void (*kernel)(Params...), dim3 grid, dim3 threads, size_t smem, unsigned cluster,
-                             cudaStream_t stream, Args... args) {
-  return launch_ex(false, kernel, grid, threads, smem, cluster, stream, args...);
-}
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
