@@ -73,6 +73,7 @@ struct ApcTable {
   int nb;
   int b_base;               // global index of image 0 of this table
   int strip_log2[kApcMaxB]; // log2 of the patches per strip of image b
+  float col_scale[kApcMaxB]; // 2 / (255 n): the mean of a column of image b from its sum in units of 2^-31 / 255
 };
 
 __device__ __forceinline__ int find_image(const ApcTable& t, int unit) {
@@ -591,15 +592,15 @@ __global__ void __launch_bounds__(kDAll, 1) apc_pass2(const uint8_t* __restrict_
     ptx::grid_dependency_wait();
     // c = sums / N, |c|^2 (fixed summation order), c_hat = c / |c|
     const int N = t.n[b];
-    const float inv_n = 1.0f / static_cast<float>(N);
     const unsigned long long* sb = sums + static_cast<int64_t>(t.b_base + b) * (kSumSlots * kTokDim);
     float c = 0.f;
     if (ct < kTokDim) {   // a thread per coordinate
       unsigned long long x = 0ull;
 #pragma unroll
       for (int r = 0; r < kSumSlots; ++r) x += __ldcg(sb + r * kTokDim + ct);
-      // sums are multiples of 2^-31 (and, but for the constant coordinate, of 1/255)
-      c = unfix32<false>(x, inv_n) * (ct < kPatchBytes ? 2.0f / 255.0f : 2.0f);
+      // sums are multiples of 2^-31 (and, but for the constant coordinate, of 1/255): one factor, rounded
+      // once, for all coordinates of the image (1/n and 1/255 rounded apart shift phi, and 1 - phi more)
+      c = unfix32<false>(x, t.col_scale[b]) * (ct < kPatchBytes ? 1.0f : 255.0f);
       if (ct == kPatchBytes) sh.craw[0] = c;
     }
     const float p2 = warp_sum_f(c * c);
@@ -2351,6 +2352,7 @@ void fill_strip_table(ApcTable& t, int c0, int nb, const int64_t* img_off, const
     t.patch0[i] = patch0;
     const int N = (H[b] / kPatch) * t.gw[i];
     t.n[i] = N;
+    t.col_scale[i] = static_cast<float>(2.0 / (255.0 * N));
     double kt = std::floor(static_cast<double>(tail_frac) * N + 0.5);
     if (kt < 1) kt = 1;
     if (kt > N) kt = N;

@@ -210,6 +210,22 @@ def test_token_widths(pace, D, lens):
     np.testing.assert_array_equal(one.cpu().numpy(), d[cu[-2]:cu[-1]])
 
 
+# tokens that start on a 4-byte, not a 16-byte boundary take the staged kernels: the same statistics
+def test_tokens_unaligned_start(pace):
+    rng = np.random.default_rng(8)
+    bits = synth.f32_to_bf16_bits(rng.normal(0.4, 1.0, size=(700, 256)).astype(np.float32))
+    flat = torch.empty(bits.size + 2, dtype=torch.bfloat16, device="cuda")
+    flat[2:].copy_(bf16_tensor(bits).reshape(-1))
+    shifted = flat[2:].view(700, 256)
+    assert shifted.data_ptr() % 16 == 4
+    ref = O.apc_density_preview(f64(bits), 252, 252)
+    for T in (shifted, bf16_tensor(bits)):
+        d, st = pace.pace_apc_density_tokens(T, [0, 700], [252], [252])
+        s = pace.stats_dict(st)[0]
+        assert_distances_close(d.cpu().numpy(), ref["d"])
+        assert abs(s["phi"] - ref["phi"]) <= 1e-5 and abs(s["d_top"] - ref["d_top"]) <= 1e-5
+
+
 def test_tokens_with_non_finite_rows(pace):
     """A NaN or infinite token spoils its own distance and leaves the others finite."""
     rng = np.random.default_rng(2)
