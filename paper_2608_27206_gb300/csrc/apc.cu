@@ -73,7 +73,8 @@ struct ApcTable {
   int nb;
   int b_base;               // global index of image 0 of this table
   int strip_log2[kApcMaxB]; // log2 of the patches per strip of image b
-  float col_scale[kApcMaxB]; // 2 / (255 n): the mean of a column of image b from its sum in units of 2^-31 / 255
+  float2 col_scale[kApcMaxB]; // 2 / (255 n) as a sum of two floats: the mean of a column of image b from its sum
+                              // in units of 2^-31 / 255
 };
 
 __device__ __forceinline__ int find_image(const ApcTable& t, int unit) {
@@ -98,6 +99,14 @@ __device__ __forceinline__ float warp_sum_f(float v) {
   return v;
 }
 
+// Sum over the warp, in every lane (below 2^64).
+__device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v) {
+  const unsigned p0 = __reduce_add_sync(0xffffffffu, static_cast<unsigned>(v) & 0xFFFFu);
+  const unsigned p1 = __reduce_add_sync(0xffffffffu, static_cast<unsigned>(v) >> 16);
+  const unsigned p2 = __reduce_add_sync(0xffffffffu, static_cast<unsigned>(v >> 32));
+  return (static_cast<unsigned long long>(p2) << 32) + (static_cast<unsigned long long>(p1) << 16) + p0;
+}
+
 // ------------------------------------------------------------------------------------------------
 // density on raw pixels
 // ------------------------------------------------------------------------------------------------
@@ -118,7 +127,8 @@ __device__ __forceinline__ float warp_sum_f(float v) {
 // Everything works on the 84 bytes of a patch pair's image row as 21 words: one 4-byte shared load
 // brings four coordinates.  Word 10 holds the last two coordinates of the first patch and the first
 // two of the second; a single last patch has an absent partner with weight 0.  On a 4K image the two
-// passes took 19.9 + 15.8 us with a byte-to-float conversion and a packed fp32 FMA per coordinate.
+// passes took 19.9 + 15.8 us with a byte-to-float conversion and a packed fp32 FMA per coordinate, now
+// 11.4 + 12.4 (three to four strips per group, each two group barriers and a wait for its rows).
 constexpr int kDThreads = 320;                       // threads of a group
 constexpr int kDGroups = 3;                          // groups of a CTA
 constexpr int kDAll = kDThreads * kDGroups;
@@ -558,8 +568,7 @@ struct Pass2Smem {
   // other: [image row][word][byte][coordinate of the word]
   uint8_t cdig[kPatch][kPairWords][4][4];
   float craw[kTokDim + 3];
-  float red[kDAll / 32];
-  unsigned long long redq[kDAll / 32];
+  unsigned long long redq[kDAll / 32], redc[kDAll / 32];
 };
 static_assert(sizeof(Pass2Group) % 16 == 0 && offsetof(Pass2Smem, cdig) % 16 == 0, "shared layout");
 
@@ -598,17 +607,21 @@ __global__ void __launch_bounds__(kDAll, 1) apc_pass2(const uint8_t* __restrict_
       unsigned long long x = 0ull;
 #pragma unroll
       for (int r = 0; r < kSumSlots; ++r) x += __ldcg(sb + r * kTokDim + ct);
-      // sums are multiples of 2^-31 (and, but for the constant coordinate, of 1/255): one factor, rounded
-      // once, for all coordinates of the image (1/n and 1/255 rounded apart shift phi, and 1 - phi more)
-      c = unfix32<false>(x, t.col_scale[b]) * (ct < kPatchBytes ? 1.0f : 255.0f);
+      // sums are multiples of 2^-31 (and, but for the constant coordinate, of 1/255); the factor of all
+      // coordinates in two floats, since its rounding would move phi, and 1 - phi more
+      const float v = unfix32<false>(x, 1.0f);
+      c = fmaf(v, t.col_scale[b].y, v * t.col_scale[b].x) * (ct < kPatchBytes ? 1.0f : 255.0f);
       if (ct == kPatchBytes) sh.craw[0] = c;
     }
-    const float p2 = warp_sum_f(c * c);
-    if (lane == 0) sh.red[ct >> 5] = p2;
+    // |c|^2 in 2^-62 fixed point (c <= 1), so that 1 - phi is exact too
+    const uint32_t cu = __float2uint_rn(c * 2147483648.0f);
+    const unsigned long long p2 = warp_sum_u64(static_cast<unsigned long long>(cu) * cu);
+    if (lane == 0) sh.redq[ct >> 5] = p2;
     __syncthreads();
-    float phi = 0.f;
+    unsigned long long phi62 = 0ull;
 #pragma unroll
-    for (int w = 0; w < (kTokDim + 31) / 32; ++w) phi += sh.red[w];
+    for (int w = 0; w < (kTokDim + 31) / 32; ++w) phi62 += sh.redq[w];
+    const float phi = static_cast<float>(phi62) * 0x1p-62f;
     const float inv_c = 1.0f / sqrtf(phi);
     unsigned long long sq = 0ull;   // square, 2^-56 fixed point
     if (ct < kPatchBytes) {
@@ -622,21 +635,20 @@ __global__ void __launch_bounds__(kDAll, 1) apc_pass2(const uint8_t* __restrict_
         sh.cdig[y][(x + 42) >> 2][d][(x + 42) & 3] = byte;
       }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-    if (lane == 0) sh.redq[ct >> 5] = sq;
+    sq = warp_sum_u64(sq);
+    if (lane == 0) sh.redc[ct >> 5] = sq;
     __syncthreads();
     double cc = 0.0, c1 = 0.0;   // a group's warp 0: |c_hat|^2 and the constant coordinate of c_hat
     if (warp == 0) {             // (fp64 is slow on this GPU: one warp's worth per group and strip)
       sq = 0ull;
 #pragma unroll
-      for (int w = 0; w < (kPatchBytes + 31) / 32; ++w) sq += sh.redq[w];
+      for (int w = 0; w < (kPatchBytes + 31) / 32; ++w) sq += sh.redc[w];
       c1 = static_cast<double>(sh.craw[0] * inv_c);
       cc = fma(static_cast<double>(sq), 0x1p-56, c1 * c1);
     }
     if (first == t.unit_prefix[b] && ct == 0) {
       stats[t.b_base + b].phi = phi;
-      stats[t.b_base + b].rho_g = 1.0f - phi;
+      stats[t.b_base + b].rho_g = static_cast<float>(static_cast<long long>((1ull << 62) - phi62)) * 0x1p-62f;
       stats[t.b_base + b].n_patches = N;
       stats[t.b_base + b].k_tail = t.ktail[b];
     }
@@ -898,8 +910,11 @@ __global__ void __launch_bounds__(kApcThreads) apc_tok_pass2(const uint32_t* __r
 
 // Token widths of up to 1536 in whole 16-byte vectors (the ViT widths): a warp per token, lane l
 // holding vectors l, l + 32, .. in registers, so a token is read once per pass straight into the
-// norm, the column sums and the distance, with no staging and no block barrier (bound by HBM in
-// pass 1).  Other widths take the staged kernels below.
+// norm, the column sums and the distance, with no staging and no block barrier.  Pass 1 is bound by a
+// warp's chain per token (load, sum of squares over the lanes, square root and division, column sums),
+// pass 2 by L2 and HBM.  42196 tokens of 1280: 84.5 us for the call staged, 55.5 in registers (passes
+// 38.8 + 31.9, now 25.3 + 28).  Other widths, and tokens off a 16-byte boundary, take the staged kernels
+// above.
 constexpr int kTokVecMax = 6;            // 16-byte vectors per lane
 constexpr int kTokThreads = 384;         // of pass 1: one CTA per SM, since each ends an image with D atomics
 constexpr int kTokAhead = 2;             // tokens a warp of pass 1 has in flight
@@ -1953,7 +1968,7 @@ __device__ void resample_tile_generic(GenericSmem& sh, const uint8_t* __restrict
 // 4 fs wide and fs apart (fs = n_in / n_out >= 1), so four accumulators, reused in turn, are enough
 // and the row loop needs no rotation once it is unrolled over four output rows.
 // Byte-wise taps in the horizontal pass first (the reverse order) cost a shared load and a
-// conversion for every tap of every input row: 4K at r = 0.248 took 57 us.
+// conversion for every tap of every input row: 4K at r = 0.248 took 57 us, now 35.5.
 constexpr int kVThreads = 128;
 constexpr int kVPx = 4 * kVThreads;          // input columns of a tile
 constexpr int kVHalf = kVPx / 2 + 4;         // even (odd) columns of a plane, and slack for the last taps
@@ -2352,7 +2367,9 @@ void fill_strip_table(ApcTable& t, int c0, int nb, const int64_t* img_off, const
     t.patch0[i] = patch0;
     const int N = (H[b] / kPatch) * t.gw[i];
     t.n[i] = N;
-    t.col_scale[i] = static_cast<float>(2.0 / (255.0 * N));
+    const double scale = 2.0 / (255.0 * N);
+    t.col_scale[i].x = static_cast<float>(scale);
+    t.col_scale[i].y = static_cast<float>(scale - static_cast<double>(t.col_scale[i].x));
     double kt = std::floor(static_cast<double>(tail_frac) * N + 0.5);
     if (kt < 1) kt = 1;
     if (kt > N) kt = N;

