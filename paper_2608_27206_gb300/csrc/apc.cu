@@ -1828,11 +1828,9 @@ struct ResampleTable {
 __device__ __forceinline__ float cubic_w(float t) {
   // Keys' cubic convolution, a = -0.5
   t = fabsf(t);
-  if (t < 1.0f) return (1.5f * t - 2.5f) * t * t + 1.0f;
-  if (t < 2.0f) return ((-0.5f * t + 2.5f) * t - 4.0f) * t + 2.0f;
-  return 0.0f;
+  const float inner = (1.5f * t - 2.5f) * t * t + 1.0f, outer = ((-0.5f * t + 2.5f) * t - 4.0f) * t + 2.0f;
+  return t < 1.0f ? inner : t < 2.0f ? outer : 0.0f;
 }
-
 
 // Window of output index o (reading R5) in exact integer arithmetic.  With s = n_in / n_out
 // and fs = max(s, 1), the centre is c = (2o + 1) n_in / (2 n_out), the taps are
@@ -1980,6 +1978,8 @@ constexpr int kVMaxScale = 8;
 constexpr int kVWeights = 2560;              // horizontal weights of a tile
 constexpr int kVMaxCols = kVPx;
 constexpr int kVCtasPerSm = 4;
+constexpr int kVWidths = 2;                  // tile widths: up to kVPx columns, or up to kVThreads
+static_assert(kVPx >> 2 == kVThreads, "the narrow width");
 // The input ring, taken two rows at a time: aligned rows are three words per thread, others four.
 template <bool ALIGNED>
 struct Ring {
@@ -1995,7 +1995,6 @@ struct ResampleSmem {
   float2 wy[kVMaxRows][4];                   // (w, w) of input row y for output rows r .. r + 3, r the first unfinished
   uint32_t raw[kVRingWords][kVThreads];      // [row, word][thread] of the input ring
   float wx[kVWeights];                       // [tap][column]
-  int y0;                                    // first input row of the tile
   int xlo[kVMaxCols];
   int last[kVMaxTH];                         // last input row of output row r
   float ynorm[kVMaxTH];
@@ -2018,11 +2017,11 @@ __device__ __forceinline__ int tap_count(float s) { return (static_cast<int>(4.0
 static_assert(sizeof(GenericSmem) <= sizeof(ResampleSmem), "one buffer for both kinds of tile");
 
 // Tiles of a Ho x Wo output: columns per tile (its window, starting up to 3 pixels early, fits kVPx
-// and its taps kVWeights), spread evenly.
-__device__ __forceinline__ int cols_per_tile(int W, int Wo) {
+// and its taps kVWeights; `limit` at most), spread evenly.
+__device__ __forceinline__ int cols_per_tile(int W, int Wo, int limit) {
   const float s = static_cast<float>(W) / static_cast<float>(Wo);
   const int taps = tap_count(s);
-  const int most = max(1, min(static_cast<int>((static_cast<float>(kVPx - 8) - 4.0f * s) / s), kVWeights / taps));
+  const int most = max(1, min(min(static_cast<int>((static_cast<float>(kVPx - 8) - 4.0f * s) / s), kVWeights / taps), limit));
   const int tiles = (Wo + most - 1) / most;
   return (Wo + tiles - 1) / tiles;
 }
@@ -2036,42 +2035,70 @@ __device__ __forceinline__ void fetch_px4(const uint8_t* __restrict__ img, uint3
   for (int k = 0; k < (ALIGNED ? 3 : 4); ++k) cp_async4(slot + k * kVThreads, img + min(a + 4u * k, last));
 }
 
+// The last of n_in inputs whose centre lies in the window of output index o.
+__device__ __forceinline__ int last_input(int o, int n_in, int n_out) {
+  const int64_t reach = (2 * static_cast<int64_t>(o) + 1) * n_in + 4 * static_cast<int64_t>(max(n_in, n_out)) - 1 - n_out;   // centre + 2 fs
+  const int64_t d = 2 * static_cast<int64_t>(n_out);
+  const int64_t i = reach < (int64_t{1} << 32) ? static_cast<int64_t>(static_cast<uint32_t>(reach) / static_cast<uint32_t>(d))
+                                               : reach / d;
+  return static_cast<int>(min(static_cast<int64_t>(n_in - 1), i));
+}
+
 template <bool ALIGNED>
 __device__ __forceinline__ void resample_tile(ResampleSmem& sh, const uint8_t* __restrict__ img, int H, int W, int Ho,
                                               int Wo, int ox0, int ncol, int oy0, int nrow, uint8_t* __restrict__ out) {
   const int tid = threadIdx.x;
-  // horizontal windows and normalised weights (reading R5), padded to an even number of taps
   const float sx = static_cast<float>(W) / static_cast<float>(Wo);
   const int taps = tap_count(sx);
+  // the first input rows are requested before the weights are worked out
+  const int x0 = exact_window(ox0, W, Wo).lo & ~3;
+  const int y0 = exact_window(oy0, H, Ho).lo, y1 = last_input(oy0 + nrow - 1, H, Ho) + 1;
+  const uint32_t pitch = static_cast<uint32_t>(W) * 3u;
+  const uint32_t last_word = static_cast<uint32_t>(static_cast<int64_t>(H) * pitch - 4);
+  const int px = x0 + 4 * tid;                     // this thread's four columns
+  const bool works = px < exact_window(ox0 + ncol - 1, W, Wo).lo + taps; // some window may reach them
+  uint32_t off = static_cast<uint32_t>(y0) * pitch + static_cast<uint32_t>(px) * 3u;   // of the next row to fetch
+  const uint32_t shr = (off & 2u) * 8u, flip = ALIGNED ? 0u : (pitch & 2u) * 8u;        // alignment of a row, of the next
+  uint32_t sft = ALIGNED ? 0u : shr;
+  using R = Ring<ALIGNED>;
+  uint32_t* ring = &sh.raw[0][tid];
+  constexpr int kRow = R::kWords * kVThreads;   // words from slot to slot
+  int y = y0, head = 0;   // the next row to filter, and its slot
+  auto fetch_next = [&](int row, int slot) {    // one group of copies per row, empty past the tile's last
+    if (works && row < y1) fetch_px4<ALIGNED>(img, off, last_word, ring + slot * kRow);
+    cp_async_commit();
+    off += pitch;
+  };
+#pragma unroll
+  for (int k = 0; k < R::kAhead; ++k) fetch_next(y0 + k, k);
+  // horizontal windows and normalised weights (reading R5), padded to an even number of taps
   for (int c = tid; c < ncol; c += kVThreads) {
     const Win w = exact_window(ox0 + c, W, Wo);
     sh.xlo[c] = w.lo;
     float sum = 0.f;
+#pragma unroll 4
     for (int i = 0; i < taps; ++i) {
       const float x = i < w.n ? cubic_w(static_cast<float>(w.num0 + i * w.step) * w.inv_den) : 0.f;
       sh.wx[i * ncol + c] = x;
       sum += x;
     }
     const float inv = 1.0f / sum;
+#pragma unroll 4
     for (int i = 0; i < taps; ++i) sh.wx[i * ncol + c] *= inv;
   }
-  // vertical windows: the last input row whose centre lies inside, 1 / sum of the weights
-  if (tid < nrow) {
-    const int o = oy0 + tid;
+  // vertical windows (by the threads that have fewest columns): the last input row whose centre lies
+  // inside, 1 / sum of the weights
+  const int vt = kVThreads - 1 - tid;
+  if (vt < nrow) {
+    const int o = oy0 + vt;
     const Win w = exact_window(o, H, Ho);
     float sum = 0.f;
+#pragma unroll 4
     for (int i = 0; i < w.n; ++i) sum += cubic_w(static_cast<float>(w.num0 + i * w.step) * w.inv_den);
-    sh.ynorm[tid] = 1.0f / sum;
-    const int64_t reach = (2 * static_cast<int64_t>(o) + 1) * H + 4 * static_cast<int64_t>(max(H, Ho)) - 1 - Ho;   // centre + 2 fs
-    const int64_t d = 2 * static_cast<int64_t>(Ho);
-    const int64_t i = reach < (int64_t{1} << 32) ? static_cast<int64_t>(static_cast<uint32_t>(reach) / static_cast<uint32_t>(d))
-                                                 : reach / d;
-    sh.last[tid] = static_cast<int>(min(static_cast<int64_t>(H - 1), i));
-    if (tid == 0) sh.y0 = w.lo;
+    sh.ynorm[vt] = 1.0f / sum;
+    sh.last[vt] = last_input(o, H, Ho);
   }
   __syncthreads();
-  const int x0 = sh.xlo[0] & ~3;
-  const int y0 = sh.y0, y1 = sh.last[nrow - 1] + 1;
   const float inv_den = 1.0f / static_cast<float>(2 * max(H, Ho));
   for (int i = tid; i < (y1 - y0) * 4; i += kVThreads) {
     const int y = y0 + (i >> 2);
@@ -2088,29 +2115,11 @@ __device__ __forceinline__ void resample_tile(ResampleSmem& sh, const uint8_t* _
     sh.wy[y - y0][i & 3] = make_float2(w, w);
   }
   __syncthreads();
-  const uint32_t pitch = static_cast<uint32_t>(W) * 3u;
-  const uint32_t last_word = static_cast<uint32_t>(static_cast<int64_t>(H) * pitch - 4);
-  const int px = x0 + 4 * tid;                     // this thread's four columns
-  const bool works = px < sh.xlo[ncol - 1] + taps; // some window may reach them
   float2 acc[4][6];                                // four output rows x 12 bytes
 #pragma unroll
   for (int j = 0; j < 4; ++j)
 #pragma unroll
     for (int e = 0; e < 6; ++e) acc[j][e] = make_float2(0.f, 0.f);
-  uint32_t off = static_cast<uint32_t>(y0) * pitch + static_cast<uint32_t>(px) * 3u;   // of the next row to fetch
-  const uint32_t shr = (off & 2u) * 8u, flip = ALIGNED ? 0u : (pitch & 2u) * 8u;        // alignment of a row, of the next
-  uint32_t sft = ALIGNED ? 0u : shr;
-  using R = Ring<ALIGNED>;
-  uint32_t* ring = &sh.raw[0][tid];
-  constexpr int kRow = R::kWords * kVThreads;   // words from slot to slot
-  int y = y0, head = 0;   // the next row to filter, and its slot
-  auto fetch_next = [&](int row, int slot) {    // one group of copies per row, empty past the tile's last
-    if (works && row < y1) fetch_px4<ALIGNED>(img, off, last_word, ring + slot * kRow);
-    cp_async_commit();
-    off += pitch;
-  };
-#pragma unroll
-  for (int k = 0; k < R::kAhead; ++k) fetch_next(y0 + k, k);
   // filters the next NR input rows; acc[(PH + j) & 3] is output row r + j of the phase's row r
   auto rows = [&](auto phase, auto count) {
     constexpr int PH = decltype(phase)::value, NR = decltype(count)::value;
@@ -2229,8 +2238,9 @@ __global__ void __launch_bounds__(kVThreads, kVCtasPerSm) apc_resample(const uin
   extern __shared__ __align__(16) unsigned char rs_smem[];
   ResampleSmem& sh = *reinterpret_cast<ResampleSmem*>(rs_smem);
   __shared__ int tile_prefix[kApcMaxB + 1];
-  __shared__ int sho[kApcMaxB], swo[kApcMaxB], stw[kApcMaxB];   // target size, columns per tile (0: generic tiles)
-  __shared__ int s_th;
+  __shared__ int sho[kApcMaxB], swo[kApcMaxB];
+  __shared__ int stw[kVWidths][kApcMaxB];   // columns per tile (0: generic tiles), for each limit
+  __shared__ int s_th, s_tw;                // the tiles' rows and which limit
   ptx::begin_call();
   const int tid = threadIdx.x;
   for (int b = tid; b < t.nb; b += kVThreads) {
@@ -2239,32 +2249,41 @@ __global__ void __launch_bounds__(kVThreads, kVCtasPerSm) apc_resample(const uin
     if (Ho < 1 || Wo < 1 || Ho > t.H[b] || Wo > t.W[b]) Ho = Wo = 0;   // nothing to write
     sho[b] = Ho;
     swo[b] = Wo;
-    stw[b] = Ho > 0 && t.H[b] <= kVMaxScale * Ho && t.W[b] <= kVMaxScale * Wo ? cols_per_tile(t.W[b], Wo) : 0;
+    const bool tiles = Ho > 0 && t.H[b] <= kVMaxScale * Ho && t.W[b] <= kVMaxScale * Wo;
+#pragma unroll
+    for (int k = 0; k < kVWidths; ++k) stw[k][b] = tiles ? cols_per_tile(t.W[b], Wo, kVPx >> (2 * k)) : 0;
   }
   __syncthreads();
-  // Rows per tile, a multiple of four: a tile reads (rows + 4) fs input rows, so tall tiles filter
-  // least twice, but the tiles should also fill the SMs.  Lane l of warp 0 rates 4 (l + 1) rows: a
-  // tile's time is about rows + 4 + 3 (the set-up) when it has an SM to itself, and n tiles on an SM
-  // take about max(1, 0.4 n) times that.
+  // Rows per tile, a multiple of four, and columns, as many as fit or at most a thread each: a tile reads
+  // (rows + 4) fs input rows, so tall tiles filter least twice and wide ones share the set-up, but the
+  // tiles should also fill the SMs.  Lane 8 k + l of warp 0 rates 4 (l + 1) rows in width k: a tile's time
+  // is about rows + 4 + 3 (the set-up) times 3 + the columns per thread when it has an SM to itself, and n
+  // tiles on an SM take about max(1, 0.4 n) times that; narrow tiles 1, 1.1 and 1.3 for one to three, and
+  // more of them are not considered (8 images of 1344 x 1008 at r = 0.25: 39.5 us in wide tiles, 52.5 in
+  // five narrow ones per SM; one of 448 x 448 at r = 0.8: 13.8 in wide ones, 9.7 in narrow ones).
   if (tid < 32) {
-    const int th = 4 * (tid + 1);
-    unsigned cost = 0xFFFFFFFFu;
-    if (th <= kVMaxTH) {
-      int64_t tiles = 0;
-      for (int b = 0; b < t.nb; ++b)
-        if (stw[b] > 0) {
-          // no more rows than the input rows that a tile can hold
-          const int rows = min(th, max(4, static_cast<int>(static_cast<float>(kVMaxRows - 4) * sho[b] / t.H[b] - 3.0f) & ~3));
-          tiles += static_cast<int64_t>((swo[b] + stw[b] - 1) / stw[b]) * ((sho[b] + rows - 1) / rows);
-        }
-      const int64_t sms = gridDim.x / kVCtasPerSm, per_sm = (tiles + sms - 1) / sms;
-      cost = static_cast<unsigned>(max(static_cast<int64_t>(5), 2 * min(static_cast<int64_t>(1 << 24), per_sm))) * (th + 7);
-    }
+    const int th = 4 * ((tid & 7) + 1), k = min(tid >> 3, kVWidths - 1);
+    static_assert(kVMaxTH == 32 && kVWidths == 2, "eight heights, two widths");
+    uint32_t tiles = 0u, turns = 1u;   // (an image has fewer than 2^30 pixels)
+    for (int b = 0; b < t.nb; ++b)
+      if (stw[k][b] > 0) {
+        // no more rows than the input rows that a tile can hold
+        const int rows = min(th, max(4, static_cast<int>(static_cast<float>(kVMaxRows - 4) * sho[b] / t.H[b] - 3.0f) & ~3));
+        tiles += static_cast<uint32_t>((swo[b] + stw[k][b] - 1) / stw[k][b]) * static_cast<uint32_t>((sho[b] + rows - 1) / rows);
+        turns = max(turns, static_cast<uint32_t>(stw[k][b] + kVThreads - 1) / kVThreads);
+      }
+    const uint32_t sms = gridDim.x / kVCtasPerSm, per_sm = min(1u << 16, (tiles + sms - 1u) / sms);
+    const uint32_t load = k == 0 ? max(10u, 4u * per_sm) : per_sm <= 1u ? 10u : per_sm == 2u ? 11u : 13u;
+    const uint32_t cost = k > 0 && per_sm > 3u ? 0xFFFFFFFFu : (3u + turns) * load * static_cast<uint32_t>(th + 7);
     const unsigned best = __reduce_min_sync(0xffffffffu, cost);
     const unsigned who = __ballot_sync(0xffffffffu, cost == best);
-    if (tid == 0) s_th = 4 * __ffs(who);
+    if (tid == 0) {
+      s_th = 4 * (((__ffs(who) - 1) & 7) + 1);
+      s_tw = min((__ffs(who) - 1) >> 3, kVWidths - 1);
+    }
   }
   __syncthreads();
+  const int* cols = stw[s_tw];
   auto rows_of = [&](int b) {
     return min(s_th, max(4, static_cast<int>(static_cast<float>(kVMaxRows - 4) * sho[b] / t.H[b] - 3.0f) & ~3));
   };
@@ -2272,7 +2291,7 @@ __global__ void __launch_bounds__(kVThreads, kVCtasPerSm) apc_resample(const uin
     int acc = 0;
     for (int b = 0; b < t.nb; ++b) {
       tile_prefix[b] = acc;
-      const int th = stw[b] > 0 ? rows_of(b) : kRsTH, tw = stw[b] > 0 ? stw[b] : kRsTW;
+      const int th = cols[b] > 0 ? rows_of(b) : kRsTH, tw = cols[b] > 0 ? cols[b] : kRsTW;
       acc += ((sho[b] + th - 1) / th) * ((swo[b] + tw - 1) / tw);
     }
     tile_prefix[t.nb] = acc;
@@ -2283,13 +2302,13 @@ __global__ void __launch_bounds__(kVThreads, kVCtasPerSm) apc_resample(const uin
     int b = 0;
     while (b + 1 < t.nb && tile_prefix[b + 1] <= g) ++b;
     const int Ho = sho[b], Wo = swo[b], H = t.H[b], W = t.W[b];
-    const int th = stw[b] > 0 ? rows_of(b) : kRsTH, tw = stw[b] > 0 ? stw[b] : kRsTW;
+    const int th = cols[b] > 0 ? rows_of(b) : kRsTH, tw = cols[b] > 0 ? cols[b] : kRsTW;
     const int nx = (Wo + tw - 1) / tw;
     const int l = g - tile_prefix[b];
     const int oy0 = (l / nx) * th, ox0 = (l - (l / nx) * nx) * tw;
     const uint8_t* img = src + t.src_off[b];
     uint8_t* out = dst + t.dst_off[b];
-    if (stw[b] > 0) {
+    if (cols[b] > 0) {
       const int ncol = min(tw, Wo - ox0), nrow = min(th, Ho - oy0);
       if (W % 4 == 0) resample_tile<true>(sh, img, H, W, Ho, Wo, ox0, ncol, oy0, nrow, out);
       else resample_tile<false>(sh, img, H, W, Ho, Wo, ox0, ncol, oy0, nrow, out);
