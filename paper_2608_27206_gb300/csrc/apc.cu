@@ -1966,7 +1966,7 @@ __device__ void resample_tile_generic(GenericSmem& sh, const uint8_t* __restrict
 // 4 fs wide and fs apart (fs = n_in / n_out >= 1), so four accumulators, reused in turn, are enough
 // and the row loop needs no rotation once it is unrolled over four output rows.
 // Byte-wise taps in the horizontal pass first (the reverse order) cost a shared load and a
-// conversion for every tap of every input row: 4K at r = 0.248 took 57 us, now 35.5.
+// conversion for every tap of every input row: 4K at r = 0.248 took 57 us, now 34.8.
 constexpr int kVThreads = 128;
 constexpr int kVPx = 4 * kVThreads;          // input columns of a tile
 constexpr int kVHalf = kVPx / 2 + 4;         // even (odd) columns of a plane, and slack for the last taps
