@@ -257,6 +257,27 @@ def test_resample_scales(pace, shape, size):
     assert not dst[n:].any()
 
 
+# an image alone (tiles of at most a column per thread) and the same one in a batch (wide tiles, other
+# heights): the same bytes, whatever the tiles; aligned rows and rows on 2-byte boundaries
+@pytest.mark.parametrize("shape,size", [((448, 448), (190, 190)), ((448, 448), (448, 401)), ((434, 462), (300, 257)),
+                                        ((336, 322), (41, 129))])
+def test_resample_tile_widths(pace, shape, size):
+    rng = np.random.default_rng(size[1])
+    img = synth.make_image(rng, *shape, 3, 3, 0.5)
+    ref = O.apc_resample(img, *size).astype(int)
+    n, pad = size[0] * size[1] * 3, (img.size + 255) // 256 * 256
+    outs = []
+    for B in (1, 24):
+        src = torch.zeros(B, pad, dtype=torch.uint8, device="cuda")
+        src[:, :img.size] = torch.from_numpy(img.reshape(-1)).cuda()
+        dst, off = torch.zeros_like(src), [pad * b for b in range(B)]
+        pace.pace_apc_resample_to(src.view(-1), off, [shape[0]] * B, [shape[1]] * B, [size[0]] * B, [size[1]] * B, dst.view(-1), off)
+        outs.append(dst[:, :n])
+        assert not dst[:, n:].any()
+    assert np.abs(outs[0][0].cpu().numpy().reshape(*size, 3).astype(int) - ref).max() <= 1
+    assert (outs[1] == outs[0]).all()
+
+
 # every call's first kernel may be launched while the stream's previous work runs: inputs written right
 # before a call, scratch and outputs used again right after one, in a stream and in a captured graph
 @pytest.mark.parametrize("captured", [False, True])
