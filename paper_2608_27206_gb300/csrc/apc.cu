@@ -2257,10 +2257,12 @@ __global__ void __launch_bounds__(kVThreads, kVCtasPerSm) apc_resample(const uin
   // Rows per tile, a multiple of four, and columns, as many as fit or at most a thread each: a tile reads
   // (rows + 4) fs input rows, so tall tiles filter least twice and wide ones share the set-up, but the
   // tiles should also fill the SMs.  Lane 8 k + l of warp 0 rates 4 (l + 1) rows in width k: a tile's time
-  // is about rows + 4 + 3 (the set-up) times 3 + the columns per thread when it has an SM to itself, and n
-  // tiles on an SM take about max(1, 0.4 n) times that; narrow tiles 1, 1.1 and 1.3 for one to three, and
-  // more of them are not considered (8 images of 1344 x 1008 at r = 0.25: 39.5 us in wide tiles, 52.5 in
-  // five narrow ones per SM; one of 448 x 448 at r = 0.8: 13.8 in wide ones, 9.7 in narrow ones).
+  // is about rows + 4 + 3 (the set-up) times 3 + the columns per thread when it has an SM to itself, and
+  // hardly more beside others as long as the SM holds them all: n tiles on an SM take about max(1, n / 4)
+  // times that (rated at 0.4 n, one of 4K at r = 0.25 took three tall tiles per SM and 34.8 us, now four and
+  // 30.0; rated at 0.2 n 33.5, with 8 images of 1344 x 1008 at r = 0.18 57.7 against 44.0).  More than four
+  // narrow tiles are not considered (8 such images at r = 0.25: 39.5 us in wide tiles, 52.5 in five
+  // narrow ones per SM; one of 448 x 448 at r = 0.8: 13.8 in wide ones, 9.7 in narrow ones).
   if (tid < 32) {
     const int th = 4 * ((tid & 7) + 1), k = min(tid >> 3, kVWidths - 1);
     static_assert(kVMaxTH == 32 && kVWidths == 2, "eight heights, two widths");
@@ -2273,8 +2275,8 @@ __global__ void __launch_bounds__(kVThreads, kVCtasPerSm) apc_resample(const uin
         turns = max(turns, static_cast<uint32_t>(stw[k][b] + kVThreads - 1) / kVThreads);
       }
     const uint32_t sms = gridDim.x / kVCtasPerSm, per_sm = min(1u << 16, (tiles + sms - 1u) / sms);
-    const uint32_t load = k == 0 ? max(10u, 4u * per_sm) : per_sm <= 1u ? 10u : per_sm == 2u ? 11u : 13u;
-    const uint32_t cost = k > 0 && per_sm > 3u ? 0xFFFFFFFFu : (3u + turns) * load * static_cast<uint32_t>(th + 7);
+    const uint32_t load = k == 0 ? max(10u, (5u * per_sm + 1u) / 2u) : per_sm <= 3u ? 10u : 11u;
+    const uint32_t cost = k > 0 && per_sm > 4u ? 0xFFFFFFFFu : (3u + turns) * load * static_cast<uint32_t>(th + 7);
     const unsigned best = __reduce_min_sync(0xffffffffu, cost);
     const unsigned who = __ballot_sync(0xffffffffu, cost == best);
     if (tid == 0) {
