@@ -1956,8 +1956,8 @@ __device__ void resample_tile_generic(GenericSmem& sh, const uint8_t* __restrict
 
 // Downscales of up to 8 per side: a tile of up to kVPx input columns, filtered vertically first.
 //
-// Bound by instruction issue, so every input byte is turned into a float once per tile and used from
-// registers: a thread owns four pixels (12 bytes) of a column strip and walks down the input rows,
+// Bound by instructions and their latency, so every input byte is turned into a float once per tile and
+// used from registers: a thread owns four pixels (12 bytes) of a column strip and walks down the input rows,
 // adding each to the (at most) four output rows whose windows hold it; a finished pair of rows goes
 // to shared memory as float2 (row, row + 1), and after four rows the CTA filters them horizontally,
 // a thread per column, one packed FMA per tap, channel and two rows.  Input rows come through a
@@ -1966,7 +1966,7 @@ __device__ void resample_tile_generic(GenericSmem& sh, const uint8_t* __restrict
 // 4 fs wide and fs apart (fs = n_in / n_out >= 1), so four accumulators, reused in turn, are enough
 // and the row loop needs no rotation once it is unrolled over four output rows.
 // Byte-wise taps in the horizontal pass first (the reverse order) cost a shared load and a
-// conversion for every tap of every input row: 4K at r = 0.248 took 57 us, now 34.8.
+// conversion for every tap of every input row: 4K at r = 0.248 took 57 us, now 30.0.
 constexpr int kVThreads = 128;
 constexpr int kVPx = 4 * kVThreads;          // input columns of a tile
 constexpr int kVHalf = kVPx / 2 + 4;         // even (odd) columns of a plane, and slack for the last taps
