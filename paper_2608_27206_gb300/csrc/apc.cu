@@ -1832,6 +1832,8 @@ __device__ __forceinline__ float cubic_w(float t) {
   return t < 1.0f ? inner : t < 2.0f ? outer : 0.0f;
 }
 
+__device__ __forceinline__ int div_up(int a, int b) { return (a + b - 1) / b; }
+
 // Window of output index o (reading R5) in exact integer arithmetic.  With s = n_in / n_out
 // and fs = max(s, 1), the centre is c = (2o + 1) n_in / (2 n_out), the taps are
 // lo .. lo + n - 1 with lo = max(0, floor(c - 2 fs)) and lo + n = min(n_in, ceil(c + 2 fs)),
@@ -2022,8 +2024,7 @@ __device__ __forceinline__ int cols_per_tile(int W, int Wo, int limit) {
   const float s = static_cast<float>(W) / static_cast<float>(Wo);
   const int taps = tap_count(s);
   const int most = max(1, min(min(static_cast<int>((static_cast<float>(kVPx - 8) - 4.0f * s) / s), kVWeights / taps), limit));
-  const int tiles = (Wo + most - 1) / most;
-  return (Wo + tiles - 1) / tiles;
+  return div_up(Wo, div_up(Wo, most));
 }
 
 // Starts the copy of four pixels (12 bytes) at byte `off` of the image into a slot of the thread's
@@ -2240,7 +2241,8 @@ __global__ void __launch_bounds__(kVThreads, kVCtasPerSm) apc_resample(const uin
   __shared__ int tile_prefix[kApcMaxB + 1];
   __shared__ int sho[kApcMaxB], swo[kApcMaxB];
   __shared__ int stw[kVWidths][kApcMaxB];   // columns per tile (0: generic tiles), for each limit
-  __shared__ int s_th, s_tw;                // the tiles' rows and which limit
+  __shared__ int s_tw;                      // which limit
+  __shared__ int srows[kApcMaxB], snx[kApcMaxB];   // rows per tile, tiles per row of tiles
   ptx::begin_call();
   const int tid = threadIdx.x;
   for (int b = tid; b < t.nb; b += kVThreads) {
@@ -2266,48 +2268,68 @@ __global__ void __launch_bounds__(kVThreads, kVCtasPerSm) apc_resample(const uin
   if (tid < 32) {
     const int th = 4 * ((tid & 7) + 1), k = min(tid >> 3, kVWidths - 1);
     static_assert(kVMaxTH == 32 && kVWidths == 2, "eight heights, two widths");
+    // no more rows than the input rows that a tile can hold
+    auto rows_of = [&](int b, int rows) {
+      return min(rows, max(4, static_cast<int>(static_cast<float>(kVMaxRows - 4) * sho[b] / t.H[b] - 3.0f) & ~3));
+    };
     uint32_t tiles = 0u, turns = 1u;   // (an image has fewer than 2^30 pixels)
     for (int b = 0; b < t.nb; ++b)
       if (stw[k][b] > 0) {
-        // no more rows than the input rows that a tile can hold
-        const int rows = min(th, max(4, static_cast<int>(static_cast<float>(kVMaxRows - 4) * sho[b] / t.H[b] - 3.0f) & ~3));
-        tiles += static_cast<uint32_t>((swo[b] + stw[k][b] - 1) / stw[k][b]) * static_cast<uint32_t>((sho[b] + rows - 1) / rows);
+        tiles += static_cast<uint32_t>(div_up(swo[b], stw[k][b])) * static_cast<uint32_t>(div_up(sho[b], rows_of(b, th)));
         turns = max(turns, static_cast<uint32_t>(stw[k][b] + kVThreads - 1) / kVThreads);
       }
     const uint32_t sms = gridDim.x / kVCtasPerSm, per_sm = min(1u << 16, (tiles + sms - 1u) / sms);
     const uint32_t load = k == 0 ? max(10u, (5u * per_sm + 1u) / 2u) : per_sm <= 3u ? 10u : 11u;
     const uint32_t cost = k > 0 && per_sm > 4u ? 0xFFFFFFFFu : (3u + turns) * load * static_cast<uint32_t>(th + 7);
     const unsigned best = __reduce_min_sync(0xffffffffu, cost);
-    const unsigned who = __ballot_sync(0xffffffffu, cost == best);
-    if (tid == 0) {
-      s_th = 4 * (((__ffs(who) - 1) & 7) + 1);
-      s_tw = min((__ffs(who) - 1) >> 3, kVWidths - 1);
+    const int who = __ffs(__ballot_sync(0xffffffffu, cost == best)) - 1;
+    const int best_th = 4 * ((who & 7) + 1), best_k = min(who >> 3, kVWidths - 1);
+    if (tid == 0) s_tw = best_k;
+    // the images' first tiles, lane l taking images l and l + 32 (one thread after the other took 2 us of a
+    // batch of 16)
+    static_assert(kApcMaxB == 64, "two images per lane");
+    int n[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int b = tid + 32 * h;
+      n[h] = 0;
+      if (b < t.nb) {
+        const int tw = stw[best_k][b];
+        srows[b] = tw > 0 ? rows_of(b, best_th) : kRsTH;
+        snx[b] = div_up(swo[b], tw > 0 ? tw : kRsTW);
+        n[h] = div_up(sho[b], srows[b]) * snx[b];
+      }
     }
+    int incl[2] = {n[0], n[1]};
+    if (t.nb > 1) {
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int up = __shfl_up_sync(0xffffffffu, incl[h], o);
+          if (tid >= o) incl[h] += up;
+        }
+    } else {
+      incl[0] = __shfl_sync(0xffffffffu, n[0], 0);
+    }
+    const int half = __shfl_sync(0xffffffffu, incl[0], 31);
+    tile_prefix[tid] = incl[0] - n[0];
+    tile_prefix[tid + 32] = half + incl[1] - n[1];
+    if (tid == 31) tile_prefix[kApcMaxB] = half + incl[1];
   }
   __syncthreads();
   const int* cols = stw[s_tw];
-  auto rows_of = [&](int b) {
-    return min(s_th, max(4, static_cast<int>(static_cast<float>(kVMaxRows - 4) * sho[b] / t.H[b] - 3.0f) & ~3));
-  };
-  if (tid == 0) {
-    int acc = 0;
-    for (int b = 0; b < t.nb; ++b) {
-      tile_prefix[b] = acc;
-      const int th = cols[b] > 0 ? rows_of(b) : kRsTH, tw = cols[b] > 0 ? cols[b] : kRsTW;
-      acc += ((sho[b] + th - 1) / th) * ((swo[b] + tw - 1) / tw);
-    }
-    tile_prefix[t.nb] = acc;
-  }
-  __syncthreads();
   const int total = tile_prefix[t.nb];
   for (int g = blockIdx.x; g < total; g += gridDim.x) {
-    int b = 0;
-    while (b + 1 < t.nb && tile_prefix[b + 1] <= g) ++b;
+    int b = 0;   // the last image whose first tile is g or before
+#pragma unroll
+    for (int step = kApcMaxB / 2; step > 0; step >>= 1)
+      if (b + step < t.nb && tile_prefix[b + step] <= g) b += step;
     const int Ho = sho[b], Wo = swo[b], H = t.H[b], W = t.W[b];
-    const int th = cols[b] > 0 ? rows_of(b) : kRsTH, tw = cols[b] > 0 ? cols[b] : kRsTW;
-    const int nx = (Wo + tw - 1) / tw;
+    const int th = srows[b], tw = cols[b] > 0 ? cols[b] : kRsTW, nx = snx[b];
     const int l = g - tile_prefix[b];
-    const int oy0 = (l / nx) * th, ox0 = (l - (l / nx) * nx) * tw;
+    const int row = l / nx;
+    const int oy0 = row * th, ox0 = (l - row * nx) * tw;
     const uint8_t* img = src + t.src_off[b];
     uint8_t* out = dst + t.dst_off[b];
     if (cols[b] > 0) {
