@@ -318,11 +318,11 @@ def test_calls_back_to_back(pace, captured):
 
 
 # scores held in registers for 4, 8 and 12 per thread of a block of 1024, and read again per pass above
-@pytest.mark.parametrize("n", [4096, 4097, 8192, 8193, 12288, 12289])
+@pytest.mark.parametrize("n", [4096, 4097, 8192, 8193, 12288, 12289, 16384, 20481])
 def test_select_registers(pace, n):
     rng = np.random.default_rng(n)
     # one map for both: S_final is the map itself when it spans [0, 1] and the weights are 1/2
-    x = (rng.permutation(n).astype(np.float32) / np.float32(1 << 14)).astype(np.float32)
+    x = (rng.permutation(n).astype(np.float32) / np.float32(1 << (14 if n <= 16384 else 15))).astype(np.float32)
     x[rng.integers(1, n - 1)] = 1.0
     x[0] = 0.0
     K = O.budget(n, 0.1)
