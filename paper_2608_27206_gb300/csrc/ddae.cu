@@ -626,31 +626,51 @@ __global__ void __launch_bounds__(256) prune_index_kernel(const __grid_constant_
 // column) order, cut into blocks of kGmBlock elements; a thread takes kGmU of them a block apart,
 // with all its loads in flight, so that rows of any length (7 KB hidden states, 256-byte K and V
 // heads, 4-byte position ids) fill the warps alike (a 4K prompt's prune step, 1331 rows and 35.5 MB:
-// 13 us with a warp per row, now 8.3; bound by memory latency and HBM).
-constexpr int kGmThreads = 256, kGmU = 4, kGmBlock = kGmThreads * kGmU;
+// 13 us with a warp per row, now 7.9; bound by memory latency and HBM).  Finding an element's row
+// weighs little on 16 bytes but sets the time of narrower elements, so rows of at least kGmRow of those
+// take a warp each (20000 rows of 7170 bytes: 635 us by elements, 147 by rows; of 1000 bytes, in words,
+// 20 and 9; of 50 bytes 6.2 and 7.2), and so do shorter ones down to kGmShort when the SMs hold a warp for
+// every row at once (1331 rows of 50 bytes: 4.1 us by elements, 3.1 by rows).
+constexpr int kGmThreads = 256, kGmU = 4, kGmBlock = kGmThreads * kGmU, kGmRow = 64, kGmShort = 4, kGmFew = 8192;
+// Division of n < 2^31 by d >= 1 as a multiplication (Granlund and Montgomery): with 2^(l-1) < d <= 2^l and
+// m = floor(2^(31+l) / d) + 1, m d exceeds 2^(31+l) by at most 2^l, so floor(n m / 2^(31+l)) is the quotient.
+struct FastDiv {
+  uint32_t m, shift;
+};
+FastDiv fast_div(uint32_t d) {
+  uint32_t l = 0;
+  while ((uint64_t{1} << l) < d) ++l;
+  return {static_cast<uint32_t>((uint64_t{1} << (31 + l)) / d + 1), 31 + l};
+}
 struct GatherMultiTable {
   pace_gather_tensor g[PACE_GATHER_MAX_TENSORS];
-  int64_t block_prefix[PACE_GATHER_MAX_TENSORS + 1];   // blocks of kGmBlock elements
+  int64_t block_prefix[PACE_GATHER_MAX_TENSORS + 1];   // blocks of kGmBlock elements, or of a row per warp
   int width[PACE_GATHER_MAX_TENSORS];                  // element width in bytes: 16, 4 or 1
+  bool rows[PACE_GATHER_MAX_TENSORS];                  // a warp per row
+  FastDiv by_cols[PACE_GATHER_MAX_TENSORS];            // by the elements of a row, below 2^31 elements
+  FastDiv by_rows;                                     // by the rows gathered, below 2^31
   int n;
 };
 
-// INDEX: unsigned when the tensor has fewer than 2^31 elements (a 64-bit division is several times
-// a 32-bit one), else the 64-bit type.
+// INDEX: unsigned when the tensor has fewer than 2^31 elements (no divisions), else the 64-bit type.
 template <typename V, typename INDEX>
 __device__ __forceinline__ void gather_block(const pace_gather_tensor& g, INDEX first, const int32_t* __restrict__ idx,
-                                             INDEX n_idx, int* status) {
+                                             INDEX n_idx, FastDiv by_cols, FastDiv by_rows, int* status) {
   const INDEX cols = static_cast<INDEX>(g.row_bytes / static_cast<int64_t>(sizeof(V)));
   const INDEX total = static_cast<INDEX>(g.n_slabs) * n_idx * cols;
+  auto divide = [](INDEX n, INDEX d, FastDiv by) {
+    if constexpr (sizeof(INDEX) == 4) return static_cast<INDEX>(static_cast<uint64_t>(n) * by.m >> by.shift);
+    else return n / d;
+  };
   INDEX slab[kGmU], row[kGmU], col[kGmU];
   int32_t src[kGmU];
   V v[kGmU];
 #pragma unroll
   for (int u = 0; u < kGmU; ++u) {
-    const INDEX e = first + static_cast<INDEX>(u * kGmThreads + threadIdx.x);
-    const INDEX r = e / cols;
+    const INDEX e = first + static_cast<INDEX>(u * kGmThreads + threadIdx.x);   // (past 2^31 only beyond total)
+    const INDEX r = divide(e, cols, by_cols);
     col[u] = e - r * cols;
-    slab[u] = r / n_idx;
+    slab[u] = divide(r, n_idx, by_rows);
     row[u] = r - slab[u] * n_idx;
     src[u] = e < total ? __ldcg(idx + row[u]) : -1;
   }
@@ -671,15 +691,41 @@ __device__ __forceinline__ void gather_block(const pace_gather_tensor& g, INDEX 
   }
 }
 
+// Rows 8 block .. 8 block + 7 of the tensor's slabs, a warp each.
 template <typename V>
-__device__ __forceinline__ void gather_block_of(const pace_gather_tensor& g, int64_t block, const int32_t* __restrict__ idx,
+__device__ __forceinline__ void gather_rows_of(const pace_gather_tensor& g, int64_t block, const int32_t* __restrict__ idx,
+                                               int64_t n_idx, int* status) {
+  const int lane = threadIdx.x & 31;
+  const int64_t item = block * (kGmThreads / 32) + (threadIdx.x >> 5);   // (slab, row)
+  if (item >= g.n_slabs * n_idx) return;
+  const int64_t slab = (item | n_idx) >> 32 == 0 ? static_cast<uint32_t>(item) / static_cast<uint32_t>(n_idx) : item / n_idx;
+  const int64_t row = item - slab * n_idx, cols = g.row_bytes / static_cast<int64_t>(sizeof(V));
+  const int32_t s = __ldcg(idx + row);
+  const bool in = s >= 0 && s < g.n_src_rows;
+  if (!in && lane == 0) record_error(status, PACE_ERR_INVALID_ARG, K_GATHER_MULTI);
+  const V* sp = reinterpret_cast<const V*>(static_cast<const uint8_t*>(g.src) + slab * g.src_slab_stride + (in ? s * g.src_row_stride : 0));
+  V* dp = reinterpret_cast<V*>(static_cast<uint8_t*>(g.dst) + slab * g.dst_slab_stride + row * g.dst_row_stride);
+  for (int64_t c = lane; c < cols; c += 32 * kGmU) {
+    V v[kGmU];
+#pragma unroll
+    for (int u = 0; u < kGmU; ++u) v[u] = in && c + 32 * u < cols ? __ldcs(sp + c + 32 * u) : V{};
+#pragma unroll
+    for (int u = 0; u < kGmU; ++u)
+      if (c + 32 * u < cols) __stcs(dp + c + 32 * u, v[u]);
+  }
+}
+
+template <typename V>
+__device__ __forceinline__ void gather_block_of(const GatherMultiTable& t, int k, int64_t block, const int32_t* __restrict__ idx,
                                                 int64_t n_idx, int* status) {
+  const pace_gather_tensor& g = t.g[k];
   const int64_t total = g.n_slabs * n_idx * (g.row_bytes / static_cast<int64_t>(sizeof(V)));
   if (total < (int64_t{1} << 31))
-    gather_block<V, unsigned>(g, static_cast<unsigned>(block * kGmBlock), idx, static_cast<unsigned>(n_idx), status);
+    gather_block<V, unsigned>(g, static_cast<unsigned>(block * kGmBlock), idx, static_cast<unsigned>(n_idx), t.by_cols[k],
+                              t.by_rows, status);
   else
     gather_block<V, unsigned long long>(g, static_cast<unsigned long long>(block * kGmBlock), idx,
-                                        static_cast<unsigned long long>(n_idx), status);
+                                        static_cast<unsigned long long>(n_idx), t.by_cols[k], t.by_rows, status);
 }
 
 __global__ void __launch_bounds__(kGmThreads) gather_multi_kernel(const __grid_constant__ GatherMultiTable t,
@@ -690,9 +736,12 @@ __global__ void __launch_bounds__(kGmThreads) gather_multi_kernel(const __grid_c
     int k = 0;
     while (k + 1 < t.n && t.block_prefix[k + 1] <= w) ++k;
     const int64_t block = w - t.block_prefix[k];
-    if (t.width[k] == 16) gather_block_of<uint4>(t.g[k], block, idx, n_idx, status);
-    else if (t.width[k] == 4) gather_block_of<uint32_t>(t.g[k], block, idx, n_idx, status);
-    else gather_block_of<uint8_t>(t.g[k], block, idx, n_idx, status);
+    if (t.rows[k]) {
+      if (t.width[k] == 4) gather_rows_of<uint32_t>(t.g[k], block, idx, n_idx, status);
+      else gather_rows_of<uint8_t>(t.g[k], block, idx, n_idx, status);
+    } else if (t.width[k] == 16) gather_block_of<uint4>(t, k, block, idx, n_idx, status);
+    else if (t.width[k] == 4) gather_block_of<uint32_t>(t, k, block, idx, n_idx, status);
+    else gather_block_of<uint8_t>(t, k, block, idx, n_idx, status);
   }
 }
 
@@ -835,6 +884,7 @@ extern "C" pace_status_t pace_gather_multi(const pace_gather_tensor* tensors, in
   GatherMultiTable t{};
   t.n = n_tensors;
   t.block_prefix[0] = 0;
+  if (n_idx < (int64_t{1} << 31)) t.by_rows = fast_div(static_cast<uint32_t>(n_idx));
   for (int k = 0; k < n_tensors; ++k) {
     const pace_gather_tensor& g = tensors[k];
     if (g.src == nullptr || g.dst == nullptr || g.row_bytes <= 0 || g.n_slabs < 0 || g.n_src_rows < 0 ||
@@ -846,8 +896,11 @@ extern "C" pace_status_t pace_gather_multi(const pace_gather_tensor* tensors, in
                         static_cast<uintptr_t>(g.dst_row_stride) | static_cast<uintptr_t>(g.src_slab_stride) |
                         static_cast<uintptr_t>(g.dst_slab_stride);
     t.width[k] = (a % 16 == 0) ? 16 : (a % 4 == 0) ? 4 : 1;
-    t.block_prefix[k + 1] =
-        t.block_prefix[k] + (g.n_slabs * n_idx * (g.row_bytes / t.width[k]) + kGmBlock - 1) / kGmBlock;
+    const int64_t cols = g.row_bytes / t.width[k];
+    t.rows[k] = t.width[k] < 16 && (cols >= kGmRow || (cols >= kGmShort && g.n_slabs * n_idx <= kGmFew));
+    if (cols < (int64_t{1} << 31)) t.by_cols[k] = fast_div(static_cast<uint32_t>(cols));
+    const int64_t items = g.n_slabs * n_idx * (t.rows[k] ? 1 : cols), per = t.rows[k] ? kGmThreads / 32 : kGmBlock;
+    t.block_prefix[k + 1] = t.block_prefix[k] + (items + per - 1) / per;
   }
   if (t.block_prefix[n_tensors] == 0) return PACE_OK;
   PACE_CHECK(check_device());

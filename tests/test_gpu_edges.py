@@ -60,7 +60,7 @@ def test_sequence_stream_splits(pace, before, nv, after, query_set):
 
 # element widths 16, 4 and 1, blocks of 1024 elements with remainders, several tensors and slabs,
 # rows out of range
-@pytest.mark.parametrize("n_idx", [1, 63, 64, 65, 341])
+@pytest.mark.parametrize("n_idx", [1, 63, 64, 65, 341, 8193])
 def test_gather_multi_blocks(pace, n_idx):
     rng = np.random.default_rng(n_idx)
     idx = rng.integers(0, 50, n_idx).astype(np.int32)
@@ -77,6 +77,25 @@ def test_gather_multi_blocks(pace, n_idx):
     assert pace.pace_device_status(clear=True) == (pace.PACE_ERR_INVALID_ARG, 13)
     for b, (_, d) in zip(dst, shapes):
         assert not b.select(d, 0).any()
+
+
+# rows of 1- and 4-byte elements: a warp per row (64 elements and more, 4 and more where the rows are few) and by
+# elements, several steps of a warp with remainders, slabs, rows out of range
+@pytest.mark.parametrize("n_idx,slabs", [(7, 1), (4096, 2), (4097, 2)])
+@pytest.mark.parametrize("nbytes,strided", [(3, False), (4, False), (63, False), (64, False), (65, True), (127, False), (129, True),
+                                            (252, False), (256 + 4, True), (1022, False)])
+def test_gather_multi_narrow_rows(pace, n_idx, slabs, nbytes, strided):
+    rng = np.random.default_rng(nbytes + n_idx)
+    idx = torch.from_numpy(rng.integers(0, 30, n_idx).astype(np.int32)).cuda()
+    wide = torch.from_numpy(rng.integers(0, 255, (slabs, 30, nbytes + (4 if strided else 0)), dtype=np.uint8)).cuda()
+    src, dst = wide[:, :, :nbytes], torch.full((slabs, n_idx, nbytes), 7, dtype=torch.uint8, device="cuda")
+    g = pace.GatherTensor(src.data_ptr(), dst.data_ptr(), nbytes, src.stride(1), nbytes, slabs, src.stride(0), dst.stride(0), 30)
+    pace.pace_gather_multi([g], idx)
+    assert torch.equal(dst, src.index_select(1, idx.long()))
+    idx[n_idx - 1] = -1
+    pace.pace_gather_multi([g], idx)
+    assert pace.pace_device_status(clear=True) == (pace.PACE_ERR_INVALID_ARG, 13)
+    assert not dst[:, n_idx - 1].any() and torch.equal(dst[:, :n_idx - 1], src.index_select(1, idx[:-1].long()))
 
 
 # strips of 8, 16 and 32 patches, full and partial, single last patches (odd widths: image rows on
