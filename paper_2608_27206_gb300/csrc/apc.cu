@@ -1811,6 +1811,7 @@ __global__ void __launch_bounds__(kApcThreads) apc_pix_pass2(const __grid_consta
 // ------------------------------------------------------------------------------------------------
 constexpr int kRsThreads = 128;  // threads of a resample CTA
 constexpr int kRsTH = 4;         // output rows of a generic tile (kRsTH x kRsTW = kRsThreads)
+constexpr int kRsTall = 8;       // and of a tall one
 constexpr int kRsTW = 32;        // output columns of a generic tile
 constexpr int kRsChunk = 8;      // input rows filtered per step of the generic path
 
@@ -1879,16 +1880,23 @@ __device__ __forceinline__ void window_1d(int o, int n_in, int n_out, int& lo, i
   inorm = 1.0f / s;
 }
 
-// Steep downscales: one 4 x 32 output tile, weights evaluated per tap, input read through L1.
+// Steep downscales: one 4 x 32 or 8 x 32 output tile, weights evaluated per tap, input read through L1.
+// It is bound by the horizontal pass, which works on (rows + 3) fs input rows per tile, so a call with
+// tall tiles for three quarters of the grid takes those (8 images of 4K at 8.5 per side, 3840 tall tiles:
+// 1000 us, in tiles of four rows 1214; one such image, 480: 150 and 165) and others have twice the tiles
+// (one at 15 per side, 144: 224 us, in tall ones 326).  Not inlined: it needs none of the caller's values.
 struct GenericSmem {
   int xlo[kRsTW], xn[kRsTW];
   float xoff[kRsTW], xifs[kRsTW], xnorm[kRsTW];
-  int ylo[kRsTH], yn[kRsTH];
-  float yoff[kRsTH], yifs[kRsTH], ynorm[kRsTH];
+  int ylo[kRsTall], yn[kRsTall];
+  float yoff[kRsTall], yifs[kRsTall], ynorm[kRsTall];
   float hbuf[kRsChunk][kRsTW][3];
 };
-__device__ void resample_tile_generic(GenericSmem& sh, const uint8_t* __restrict__ img, int H, int W, int Ho, int Wo, int ox0,
-                                      int oy0, uint8_t* __restrict__ out) {
+template <int ROWS>
+__device__ __noinline__ void resample_tile_generic(const uint8_t* __restrict__ img, int H, int W, int Ho, int Wo, int ox0,
+                                                   int oy0, int nrows, uint8_t* __restrict__ out) {
+  extern __shared__ __align__(16) unsigned char rs_smem[];
+  GenericSmem& sh = *reinterpret_cast<GenericSmem*>(rs_smem);
   auto &xlo = sh.xlo, &xn = sh.xn;
   auto &xoff = sh.xoff, &xifs = sh.xifs, &xnorm = sh.xnorm;
   auto &ylo = sh.ylo, &yn = sh.yn;
@@ -1899,19 +1907,18 @@ __device__ void resample_tile_generic(GenericSmem& sh, const uint8_t* __restrict
   if (tid < kRsTW) {
     const int ox = min(ox0 + tid, Wo - 1);
     window_1d(ox, W, Wo, xlo[tid], xn[tid], xoff[tid], xifs[tid], xnorm[tid]);
-  } else if (tid >= 32 && tid < 32 + kRsTH) {
+  } else if (tid >= 32 && tid < 32 + nrows) {
     const int i = tid - 32;
-    const int oy = min(oy0 + i, Ho - 1);
+    const int oy = oy0 + i;
     window_1d(oy, H, Ho, ylo[i], yn[i], yoff[i], yifs[i], ynorm[i]);
   }
   __syncthreads();
-  const int nrows = min(kRsTH, Ho - oy0);
   const int iy_lo = ylo[0];
   const int iy_hi = ylo[nrows - 1] + yn[nrows - 1];  // exclusive
   const int64_t pitch = static_cast<int64_t>(W) * 3;
-  // this thread's output pixel
+  // this thread's output pixels: rows my_r and, of a tall tile, my_r + 4
   const int my_r = tid / kRsTW, my_c = tid % kRsTW;
-  float acc0 = 0.f, acc1 = 0.f, acc2 = 0.f;
+  float acc[ROWS / kRsTH][3] = {};
   for (int r0 = iy_lo; r0 < iy_hi; r0 += kRsChunk) {
     // horizontal pass: kRsChunk rows x 32 columns x 3 channels
     for (int v = tid; v < kRsChunk * kRsTW * 3; v += kRsThreads) {
@@ -1930,28 +1937,32 @@ __device__ void resample_tile_generic(GenericSmem& sh, const uint8_t* __restrict
       hbuf[rr][cc][ch] = h;
     }
     __syncthreads();
-    if (my_r < nrows) {
-      const int lo = ylo[my_r], n = yn[my_r];
-      const float off = yoff[my_r], ifs = yifs[my_r];
+#pragma unroll
+    for (int q = 0; q < ROWS / kRsTH; ++q) {
+      const int r = my_r + q * kRsTH;
+      if (r >= nrows) break;
+      const int lo = ylo[r], n = yn[r];
+      const float off = yoff[r], ifs = yifs[r];
       for (int rr = 0; rr < kRsChunk; ++rr) {
         const int i = r0 + rr - lo;
         if (i >= 0 && i < n) {
           const float w = cubic_w(fmaf(static_cast<float>(i), ifs, off));
-          acc0 = fmaf(w, hbuf[rr][my_c][0], acc0);
-          acc1 = fmaf(w, hbuf[rr][my_c][1], acc1);
-          acc2 = fmaf(w, hbuf[rr][my_c][2], acc2);
+#pragma unroll
+          for (int ch = 0; ch < 3; ++ch) acc[q][ch] = fmaf(w, hbuf[rr][my_c][ch], acc[q][ch]);
         }
       }
     }
     __syncthreads();
   }
-  const int oy = oy0 + my_r, ox = ox0 + my_c;
-  if (my_r < nrows && ox < Wo) {
-    const float nrm = ynorm[my_r];
-    uint8_t* o = out + (static_cast<int64_t>(oy) * Wo + ox) * 3;
-    o[0] = static_cast<uint8_t>(min(255, max(0, __float2int_rn(acc0 * nrm))));
-    o[1] = static_cast<uint8_t>(min(255, max(0, __float2int_rn(acc1 * nrm))));
-    o[2] = static_cast<uint8_t>(min(255, max(0, __float2int_rn(acc2 * nrm))));
+#pragma unroll
+  for (int q = 0; q < ROWS / kRsTH; ++q) {
+    const int r = my_r + q * kRsTH, oy = oy0 + r, ox = ox0 + my_c;
+    if (r < nrows && ox < Wo) {
+      const float nrm = ynorm[r];
+      uint8_t* o = out + (static_cast<int64_t>(oy) * Wo + ox) * 3;
+#pragma unroll
+      for (int ch = 0; ch < 3; ++ch) o[ch] = static_cast<uint8_t>(min(255, max(0, __float2int_rn(acc[q][ch] * nrm))));
+    }
   }
   __syncthreads();   // shared tile buffers are reused by the next call
 }
@@ -2285,6 +2296,13 @@ __global__ void __launch_bounds__(kVThreads, kVCtasPerSm) apc_resample(const uin
     const int who = __ffs(__ballot_sync(0xffffffffu, cost == best)) - 1;
     const int best_th = 4 * ((who & 7) + 1), best_k = min(who >> 3, kVWidths - 1);
     if (tid == 0) s_tw = best_k;
+    // images in generic tiles: rows by the tall tiles that the call has
+    uint32_t tall = 0u;
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (const int b = tid + 32 * h; b < t.nb && stw[0][b] == 0)
+        tall += min(1u << 20, static_cast<uint32_t>(swo[b] + kRsTW - 1) / kRsTW * (static_cast<uint32_t>(sho[b] + kRsTall - 1) / kRsTall));
+    const int generic_rows = __reduce_add_sync(0xffffffffu, tall) >= gridDim.x / 4u * 3u ? kRsTall : kRsTH;
     // the images' first tiles, lane l taking images l and l + 32 (one thread after the other took 2 us of a
     // batch of 16)
     static_assert(kApcMaxB == 64, "two images per lane");
@@ -2295,7 +2313,7 @@ __global__ void __launch_bounds__(kVThreads, kVCtasPerSm) apc_resample(const uin
       n[h] = 0;
       if (b < t.nb) {
         const int tw = stw[best_k][b];
-        srows[b] = tw > 0 ? rows_of(b, best_th) : kRsTH;
+        srows[b] = tw > 0 ? rows_of(b, best_th) : generic_rows;
         snx[b] = div_up(swo[b], tw > 0 ? tw : kRsTW);
         n[h] = div_up(sho[b], srows[b]) * snx[b];
       }
@@ -2337,7 +2355,9 @@ __global__ void __launch_bounds__(kVThreads, kVCtasPerSm) apc_resample(const uin
       if (W % 4 == 0) resample_tile<true>(sh, img, H, W, Ho, Wo, ox0, ncol, oy0, nrow, out);
       else resample_tile<false>(sh, img, H, W, Ho, Wo, ox0, ncol, oy0, nrow, out);
     } else {
-      resample_tile_generic(*reinterpret_cast<GenericSmem*>(rs_smem), img, H, W, Ho, Wo, ox0, oy0, out);
+      const int nrow = min(th, Ho - oy0);
+      if (th == kRsTall) resample_tile_generic<kRsTall>(img, H, W, Ho, Wo, ox0, oy0, nrow, out);
+      else resample_tile_generic<kRsTH>(img, H, W, Ho, Wo, ox0, oy0, nrow, out);
     }
   }
 }

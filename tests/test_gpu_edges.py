@@ -297,6 +297,24 @@ def test_resample_tile_widths(pace, shape, size):
     assert (outs[1] == outs[0]).all()
 
 
+# steep downscales: tiles of eight rows where a call has many, else of four, remainders of both: the same bytes
+@pytest.mark.parametrize("size", [(124, 124), (121, 97)])
+def test_resample_generic_heights(pace, size):
+    rng = np.random.default_rng(size[0])
+    H = W = 1036
+    img = synth.make_image(rng, H, W, 9, 9, 0.5)
+    n, outs = size[0] * size[1] * 3, []
+    pad = (img.size + 255) // 256 * 256
+    for B in (1, 8):
+        src = torch.zeros(B, pad, dtype=torch.uint8, device="cuda")
+        src[:, :img.size] = torch.from_numpy(img.reshape(-1)).cuda()
+        dst, off = torch.zeros_like(src), [pad * b for b in range(B)]
+        pace.pace_apc_resample_to(src.view(-1), off, [H] * B, [W] * B, [size[0]] * B, [size[1]] * B, dst.view(-1), off)
+        outs.append(dst)
+    assert (outs[1][:, :n] == outs[0][0, :n]).all() and not outs[1][:, n:].any()
+    assert np.abs(outs[0][0, :n].cpu().numpy().reshape(*size, 3).astype(int) - O.apc_resample(img, *size).astype(int)).max() <= 1
+
+
 # every call's first kernel may be launched while the stream's previous work runs: inputs written right
 # before a call, scratch and outputs used again right after one, in a stream and in a captured graph
 @pytest.mark.parametrize("captured", [False, True])
