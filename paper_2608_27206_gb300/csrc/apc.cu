@@ -89,6 +89,12 @@ __device__ __forceinline__ void cp_async4(void* dst, const void* src) {
                "l"(src)
                : "memory");
 }
+// 16 bytes, of which the first `bytes` are read and the others become zeros.
+__device__ __forceinline__ void cp_async16(void* dst, const void* src, uint32_t bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
+               "l"(src), "r"(bytes)
+               : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait_group() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
@@ -2241,14 +2247,162 @@ __device__ __forceinline__ void resample_tile(ResampleSmem& sh, const uint8_t* _
   }
 }
 
-// Every CTA walks the output tiles of the whole batch (target sizes read from the density statistics
-// on the device, or given), so the grid never holds empty CTAs.
-__global__ void __launch_bounds__(kVThreads, kVCtasPerSm) apc_resample(const uint8_t* __restrict__ src,
-                                                                       const __grid_constant__ ResampleTable t,
-                                                                       const pace_apc_stats* __restrict__ stats,
-                                                                       uint8_t* __restrict__ dst) {
-  extern __shared__ __align__(16) unsigned char rs_smem[];
-  ResampleSmem& sh = *reinterpret_cast<ResampleSmem*>(rs_smem);
+// Small outputs, downscaled by up to 2.75 per side: an 8 x 32 tile whose input window is staged in shared
+// memory, warp w filtering rows 2 w and 2 w + 1 vertically (a lane per four bytes) and then horizontally
+// (a lane per column).  Such a call is all latency: the wide tiles above spend 9000 to 10000 cycles on a
+// rating, windows and weights before their first row, these on four window edges at once and on one
+// window per lane (one image of 448 x 448 at r = 0.25: 5.9 us, in wide tiles 10.2; at r = 0.8 7.2 and
+// 10.3).  Every sum is taken in the same order with the same weights as there, so the bytes do not
+// depend on which tiles a call gets.
+constexpr int kSTH = 8, kSTW = 32;           // output rows and columns
+constexpr int kSTaps = 14;                   // a window has at most floor(4 * 2.75) + 2 taps
+constexpr int kSRows = 36;                   // 7 * 2.75 + 4 * 2.75 + 2 input rows, and two read with weight 0
+constexpr int kSPx = 102;                    // 31 * 2.75 + 4 * 2.75 + 2 input columns, starting up to 3 early
+constexpr int kSPitch = 336;                 // 15 bytes of alignment, 3 kSPx, in 16-byte pieces
+constexpr int kSLine = 308;                  // 3 kSPx in fours
+static_assert(4 * kSRows >= 4 * 2 + 11 * 7 + 11 * 4 + 8 && 4 * kSPx >= 11 * 31 + 11 * 4 + 8 + 12, "staged window");
+static_assert(kSPitch >= (15 + 3 * kSPx + 3 + 15) / 16 * 16 && kSPitch % 16 == 0 && kSPitch <= 32 * 16 && kSLine >= 3 * kSPx,
+              "staged row");
+struct SmallSmem {
+  uint8_t raw[kSRows][kSPitch];              // input rows, from the 16-byte boundary before the window
+  float v[kSTH][kSLine];                     // vertically filtered rows
+  float wx[kSTaps][kSTW];
+  float wy[kSTH][kSTaps];
+  int xlo[kSTW], xn[kSTW], ylo[kSTH], yn[kSTH];
+};
+static_assert(sizeof(SmallSmem) <= sizeof(ResampleSmem), "one buffer for every kind of tile");
+__device__ __forceinline__ bool small_scale(int H, int W, int Ho, int Wo) { return 4 * H <= 11 * Ho && 4 * W <= 11 * Wo; }
+
+template <bool ALIGNED>
+__device__ __forceinline__ void resample_tile_small(SmallSmem& sh, const uint8_t* __restrict__ img, int H, int W, int Ho,
+                                                    int Wo, int ox0, int oy0, uint8_t* __restrict__ out) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int ncol = min(kSTW, Wo - ox0), nrow = min(kSTH, Ho - oy0);
+  // the input window: lane 0 works out its left edge, lanes 1 to 3 the top, the right and the bottom one
+  const bool rows = lane & 1, far = lane & 2;
+  const Win e = exact_window(rows ? oy0 + (far ? nrow - 1 : 0) : ox0 + (far ? ncol - 1 : 0), rows ? H : W, rows ? Ho : Wo);
+  const int edge = far ? e.lo + e.n : e.lo;
+  const int x0 = __shfl_sync(0xffffffffu, edge, 0) & ~3, y0 = __shfl_sync(0xffffffffu, edge, 1);
+  const int x1 = __shfl_sync(0xffffffffu, edge, 2), y1 = __shfl_sync(0xffffffffu, edge, 3);
+  const uint32_t pitch = static_cast<uint32_t>(W) * 3u, bytes = static_cast<uint32_t>(H) * pitch;   // below 2^32
+  const uint32_t first = static_cast<uint32_t>(y0) * pitch + static_cast<uint32_t>(x0) * 3u;
+  const uint32_t span = static_cast<uint32_t>(x1 - x0) * 3u;
+  for (int r = warp; r < y1 - y0; r += kVThreads / 32) {   // a warp per row, a lane per 16 bytes
+    const uint32_t b = first + static_cast<uint32_t>(r) * pitch, a = (b & ~15u) + 16u * lane;
+    if (a < b + span && a < bytes) cp_async16(sh.raw[r] + 16 * lane, img + a, min(16u, bytes - a));
+  }
+  cp_async_commit();
+  // the windows' weights: columns by the first warp, rows by the second
+  if (warp < 2 && lane < (warp == 0 ? ncol : nrow)) {
+    const int o = warp == 0 ? ox0 + lane : oy0 + lane, n_in = warp == 0 ? W : H, n_out = warp == 0 ? Wo : Ho;
+    const Win w = exact_window(o, n_in, n_out);
+    float* to = warp == 0 ? &sh.wx[0][lane] : &sh.wy[lane][0];
+    const int step = warp == 0 ? kSTW : 1, n = min(w.n, kSTaps);
+    float sum = 0.f;
+#pragma unroll 4
+    for (int i = 0; i < n; ++i) {
+      const float x = cubic_w(static_cast<float>(w.num0 + i * w.step) * w.inv_den);
+      to[i * step] = x;
+      sum += x;
+    }
+    const float inv = 1.0f / sum;
+#pragma unroll 4
+    for (int i = 0; i < n; ++i) to[i * step] *= inv;
+    (warp == 0 ? sh.xlo : sh.ylo)[lane] = w.lo;
+    (warp == 0 ? sh.xn : sh.yn)[lane] = warp == 0 ? n : min(n, last_input(o, n_in, n_out) - w.lo + 1);
+  }
+  cp_async_wait_group<0>();
+  __syncthreads();
+  const int ra = 2 * warp, rb = min(ra + 1, nrow - 1);
+  if (ra < nrow) {
+    const int la = sh.ylo[ra], na = sh.yn[ra], lb = sh.ylo[rb], nb = sh.yn[rb];
+    for (int j = lane; 4 * j < static_cast<int>(span); j += 32) {
+      float2 acc[2][2] = {};
+      auto take = [&](int row, float w, float2 (&a)[2]) {   // one staged row into an output row
+        const uint32_t ph = (first + static_cast<uint32_t>(row) * pitch) & 15u;
+        const uint32_t* p = reinterpret_cast<const uint32_t*>(sh.raw[row] + (ph & 12u)) + j;
+        const uint32_t word = ALIGNED ? p[0] : __funnelshift_r(p[0], p[1], (ph & 2u) * 8u);
+        float2 lo, hi;
+        word_to_floats(word, lo, hi);
+        const float2 w2 = make_float2(w, w);
+        a[0] = ptx::ffma2(w2, lo, a[0]);
+        a[1] = ptx::ffma2(w2, hi, a[1]);
+      };
+#pragma unroll 4
+      for (int i = 0; i < max(na, nb); ++i) {
+        take(la - y0 + i, i < na ? sh.wy[ra][i] : 0.f, acc[0]);
+        take(lb - y0 + i, i < nb ? sh.wy[rb][i] : 0.f, acc[1]);
+      }
+#pragma unroll
+      for (int q = 0; q < 2; ++q)
+        *reinterpret_cast<float4*>(&sh.v[ra + q][4 * j]) = make_float4(acc[q][0].x, acc[q][0].y, acc[q][1].x, acc[q][1].y);
+    }
+    __syncwarp();
+    if (lane < ncol) {
+      const float* va = &sh.v[ra][(sh.xlo[lane] - x0) * 3];
+      const int n = sh.xn[lane];
+      float acc[2][3] = {};
+#pragma unroll 4
+      for (int k = 0; k < n; ++k) {
+        const float w = sh.wx[k][lane];
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+#pragma unroll
+          for (int ch = 0; ch < 3; ++ch) acc[q][ch] = fmaf(w, va[q * kSLine + 3 * k + ch], acc[q][ch]);
+      }
+      uint8_t* o = out + (static_cast<int64_t>(oy0 + ra) * Wo + ox0 + lane) * 3;
+#pragma unroll
+      for (int q = 0; q < 2; ++q, o += static_cast<int64_t>(Wo) * 3) {
+        if (ra + q >= nrow) break;
+#pragma unroll
+        for (int ch = 0; ch < 3; ++ch) o[ch] = static_cast<uint8_t>(ptx::round_u8(acc[q][ch]));
+      }
+    }
+  }
+  __syncthreads();   // the shared buffers are reused by the next tile
+}
+// The small tiles of a batch: lane l of every warp holds images l and l + 32, their sizes and numbers of tiles.
+__device__ __forceinline__ void resample_small(SmallSmem& sh, const uint8_t* __restrict__ src, const ResampleTable& t,
+                                               uint8_t* __restrict__ dst, const int (&ho)[2], const int (&wo)[2],
+                                               const uint32_t (&n)[2]) {
+  const int lane = threadIdx.x & 31;
+  uint32_t end0 = n[0], end1 = n[1];   // tiles up to the image's last one
+  if (t.nb > 1) {
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t up0 = __shfl_up_sync(0xffffffffu, end0, o), up1 = __shfl_up_sync(0xffffffffu, end1, o);
+      if (lane >= o) {
+        end0 += up0;
+        end1 += up1;
+      }
+    }
+    end1 += __shfl_sync(0xffffffffu, end0, 31);
+  }
+  const uint32_t total = t.nb > 1 ? __shfl_sync(0xffffffffu, end1, 31) : __shfl_sync(0xffffffffu, n[0], 0);
+  for (uint32_t g = blockIdx.x; g < total; g += gridDim.x) {
+    int b = 0;
+    if (t.nb > 1) {
+      b = __popc(__ballot_sync(0xffffffffu, end0 <= g));
+      if (b == 32) b += __popc(__ballot_sync(0xffffffffu, end1 <= g));
+    }
+    const int Ho = __shfl_sync(0xffffffffu, b < 32 ? ho[0] : ho[1], b & 31);
+    const int Wo = __shfl_sync(0xffffffffu, b < 32 ? wo[0] : wo[1], b & 31);
+    const int l = static_cast<int>(g - __shfl_sync(0xffffffffu, b < 32 ? end0 - n[0] : end1 - n[1], b & 31));
+    const int nx = (Wo + kSTW - 1) / kSTW, row = l / nx;
+    const int H = t.H[b], W = t.W[b], ox0 = (l - row * nx) * kSTW, oy0 = row * kSTH;
+    if (W % 4 == 0) resample_tile_small<true>(sh, src + t.src_off[b], H, W, Ho, Wo, ox0, oy0, dst + t.dst_off[b]);
+    else resample_tile_small<false>(sh, src + t.src_off[b], H, W, Ho, Wo, ox0, oy0, dst + t.dst_off[b]);
+  }
+}
+// Tiles x scale per CTA of the grid (a quarter more where rows start on 2-byte boundaries, which costs a
+// second word per read) up to which a call takes small tiles.  Both kinds, in us: 2.3 rounds at 2.3
+// (8 images of 448 x 448, 5.3) 15.5 and 18.5, 2.4 at 2.4 (1064 x 1904, 5.7) 15.4 and 17.4, 5.2 at 1 (896 x 896)
+// 15.0 and 15.4, 2.9 at 2 (1344 x 1344, 5.8) 14.4 and 14.3, 4.7 at 1.6 (7.5) 20.5 and 18.5.
+constexpr float kSmallWork = 5.7f;
+
+// Wide and generic tiles of the batch, ho and wo as in resample_small.
+__device__ __forceinline__ void resample_large(ResampleSmem& sh, const uint8_t* __restrict__ src, const ResampleTable& t,
+                                               uint8_t* __restrict__ dst, const int (&ho)[2], const int (&wo)[2]) {
   __shared__ int tile_prefix[kApcMaxB + 1];
   __shared__ int sho[kApcMaxB], swo[kApcMaxB];
   __shared__ int stw[kVWidths][kApcMaxB];   // columns per tile (0: generic tiles), for each limit
@@ -2257,15 +2411,11 @@ __global__ void __launch_bounds__(kVThreads, kVCtasPerSm) apc_resample(const uin
   __shared__ int smost[kApcMaxB];           // rows per tile, at most
   __shared__ uint32_t srcp[kApcMaxB];       // the reciprocal of a quarter of that
   __shared__ int srows[kApcMaxB], snx[kApcMaxB];   // rows per tile, tiles per row of tiles
-  ptx::begin_call();
   const int tid = threadIdx.x;
   auto rcp = [](uint32_t m) { return 0xFFFFFFFFu / m + 1u; };   // 2^32 / m, rounded up (m > 1)
   static_assert(kVThreads == kVWidths * kApcMaxB, "a thread per image and width");
   if (const int b = tid & (kApcMaxB - 1), k = tid / kApcMaxB; b < t.nb) {
-    const int H = t.H[b], W = t.W[b];
-    int Ho = stats ? __ldcg(&stats[t.b_base + b].h_out) : t.Ho[b];
-    int Wo = stats ? __ldcg(&stats[t.b_base + b].w_out) : t.Wo[b];
-    if (Ho < 1 || Wo < 1 || Ho > H || Wo > W) Ho = Wo = 0;   // nothing to write
+    const int Ho = b < 32 ? ho[0] : ho[1], Wo = b < 32 ? wo[0] : wo[1], H = t.H[b], W = t.W[b];
     const bool tiles = Ho > 0 && H <= kVMaxScale * Ho && W <= kVMaxScale * Wo;
     const int tw = tiles ? cols_per_tile(W, Wo, kVPx >> (2 * k)) : 0;
     stw[k][b] = tw;
@@ -2321,7 +2471,6 @@ __global__ void __launch_bounds__(kVThreads, kVCtasPerSm) apc_resample(const uin
     const int generic_rows = __reduce_add_sync(0xffffffffu, tall) >= gridDim.x / 4u * 3u ? kRsTall : kRsTH;
     // the images' first tiles, lane l taking images l and l + 32 (one thread after the other took 2 us of a
     // batch of 16)
-    static_assert(kApcMaxB == 64, "two images per lane");
     int n[2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
@@ -2376,6 +2525,73 @@ __global__ void __launch_bounds__(kVThreads, kVCtasPerSm) apc_resample(const uin
       else resample_tile_generic<kRsTH>(img, H, W, Ho, Wo, ox0, oy0, nrow, out);
     }
   }
+}
+
+// Every CTA walks the output tiles of the whole batch (target sizes read from the density statistics
+// on the device, or given), so the grid never holds empty CTAs.
+__global__ void __launch_bounds__(kVThreads, kVCtasPerSm) apc_resample(const uint8_t* __restrict__ src,
+                                                                       const __grid_constant__ ResampleTable t,
+                                                                       const pace_apc_stats* __restrict__ stats,
+                                                                       uint8_t* __restrict__ dst) {
+  extern __shared__ __align__(16) unsigned char rs_smem[];
+  ptx::begin_call();
+  const int lane = threadIdx.x & 31;
+  auto size_of = [&](int b, int& Ho, int& Wo) {
+    Ho = stats ? __ldcg(&stats[t.b_base + b].h_out) : t.Ho[b];
+    Wo = stats ? __ldcg(&stats[t.b_base + b].w_out) : t.Wo[b];
+    if (Ho < 1 || Wo < 1 || Ho > t.H[b] || Wo > t.W[b]) Ho = Wo = 0;   // nothing to write
+  };
+  // every warp: lane l holds images l and l + 32, their sizes and their small tiles (and the work of these,
+  // too much to count where an image can't have them); of a batch the first warp works them out, since the
+  // lanes read the table one after the other (64 images of 224 x 224: by every warp 3 us more)
+  static_assert(kApcMaxB == 64, "two images per lane");
+  constexpr float kNoSmall = static_cast<float>(1 << 20);
+  __shared__ int s_ho[kApcMaxB], s_wo[kApcMaxB];
+  __shared__ uint32_t s_small[kApcMaxB], s_work;
+  int ho[2] = {}, wo[2] = {};
+  uint32_t small_n[2] = {}, total_work = 0u;
+  if (t.nb == 1 || threadIdx.x < 32) {
+    float work = 0.f;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int b = lane + 32 * h;
+      if (b >= t.nb) continue;
+      size_of(b, ho[h], wo[h]);
+      if (ho[h] == 0) continue;
+      const int H = t.H[b], W = t.W[b];
+      small_n[h] = static_cast<uint32_t>(wo[h] + kSTW - 1) / kSTW * (static_cast<uint32_t>(ho[h] + kSTH - 1) / kSTH);
+      const float scale = fmaxf(__fdividef(static_cast<float>(W), static_cast<float>(wo[h])),
+                                __fdividef(static_cast<float>(H), static_cast<float>(ho[h])));
+      work += small_scale(H, W, ho[h], wo[h])
+                  ? fminf(kNoSmall, static_cast<float>(small_n[h]) * scale * (W % 4 == 0 ? 1.0f : 1.25f)) : kNoSmall;
+    }
+    total_work = __reduce_add_sync(0xffffffffu, static_cast<uint32_t>(work));
+  }
+  if (t.nb > 1) {
+    if (threadIdx.x < 32) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        s_ho[lane + 32 * h] = ho[h];
+        s_wo[lane + 32 * h] = wo[h];
+        s_small[lane + 32 * h] = small_n[h];
+      }
+      if (lane == 0) s_work = total_work;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      ho[h] = s_ho[lane + 32 * h];
+      wo[h] = s_wo[lane + 32 * h];
+      small_n[h] = s_small[lane + 32 * h];
+    }
+    total_work = s_work;
+  }
+  // (the small tiles' code last: in front of the other, it made the first launch of a call in wide tiles, which
+  // fetches its instructions from memory, 6 us longer)
+  if (static_cast<float>(total_work) > kSmallWork * static_cast<float>(gridDim.x))
+    resample_large(*reinterpret_cast<ResampleSmem*>(rs_smem), src, t, dst, ho, wo);
+  else
+    resample_small(*reinterpret_cast<SmallSmem*>(rs_smem), src, t, dst, ho, wo, small_n);
 }
 
 // ------------------------------------------------------------------------------------------------

@@ -297,6 +297,46 @@ def test_resample_tile_widths(pace, shape, size):
     assert (outs[1] == outs[0]).all()
 
 
+# small outputs (8 x 32 tiles) and the same image beside a large one (wide tiles): the same bytes; 2.75 per side and
+# just above, tiles with remainders and below one tile, the image's last bytes, rows on 2-byte boundaries
+@pytest.mark.parametrize("shape,size", [((14, 14), (14, 14)), ((14, 14), (6, 6)), ((28, 14), (11, 6)), ((308, 308), (112, 112)),
+                                        ((308, 434), (112, 158)), ((308, 308), (111, 112)), ((42, 2030), (33, 740)),
+                                        ((700, 28), (257, 27)), ((434, 462), (300, 257)), ((98, 896), (65, 544))])
+def test_resample_small_tiles(pace, shape, size):
+    rng = np.random.default_rng(shape[1] + size[1])
+    img = rng.integers(0, 256, (*shape, 3), dtype=np.uint8)
+    img[-1, -1] = 255
+    n, big = size[0] * size[1] * 3, (1344, 1344)
+    pad = (img.size + 255) // 256 * 256
+    src = torch.zeros(pad + big[0] * big[1] * 3, dtype=torch.uint8, device="cuda")
+    src[:img.size] = torch.from_numpy(img.reshape(-1)).cuda()
+    one, two = torch.full_like(src, 7), torch.full_like(src, 7)
+    pace.pace_apc_resample_to(src, [0], shape[:1], shape[1:], size[:1], size[1:], one, [0])
+    pace.pace_apc_resample_to(src, [0, pad], [shape[0], big[0]], [shape[1], big[1]], [size[0], big[0]], [size[1], big[1]], two, [0, pad])
+    assert torch.equal(one[:n], two[:n]) and bool((one[n:] == 7).all()) and bool((two[n:pad] == 7).all())
+    assert np.abs(one[:n].cpu().numpy().reshape(*size, 3).astype(int) - O.apc_resample(img, *size).astype(int)).max() <= 1
+
+
+# a batch in small tiles, more images than a warp has lanes, among them one with nothing to write
+def test_resample_small_batch(pace):
+    rng = np.random.default_rng(5)
+    shapes = [(14 * int(a), 14 * int(b)) for a, b in rng.integers(1, 5, (40, 2))]
+    sizes = [tuple(int(rng.integers(-(-4 * x // 11), x + 1)) for x in s) for s in shapes]
+    off = np.concatenate([[0], np.cumsum([(h * w * 3 + 255) // 256 * 256 for h, w in shapes])])
+    src = torch.from_numpy(rng.integers(0, 256, int(off[-1]), dtype=np.uint8)).cuda()
+    # sizes read on the device; image 33's is out of range
+    stats = torch.zeros((40, 10), dtype=torch.int32, device="cuda")
+    stats[:, 8:10] = torch.tensor(sizes, dtype=torch.int32)
+    stats[33, 8] = 0
+    got = torch.full_like(src, 7)
+    pace.pace_apc_resample(src, off[:-1].tolist(), [s[0] for s in shapes], [s[1] for s in shapes], stats, got, off[:-1].tolist())
+    want = torch.full_like(src, 7)
+    for b in range(40):
+        if b != 33:
+            pace.pace_apc_resample_to(src, [int(off[b])], shapes[b][:1], shapes[b][1:], sizes[b][:1], sizes[b][1:], want, [int(off[b])])
+    assert torch.equal(got, want)
+
+
 # steep downscales: tiles of eight rows where a call has many, else of four, remainders of both: the same bytes
 @pytest.mark.parametrize("size", [(124, 124), (121, 97)])
 def test_resample_generic_heights(pace, size):
