@@ -128,6 +128,19 @@ def test_density_extreme_values(pace, value):
     assert_distances_close(d.cpu().numpy(), O.apc_density(img)["d"])
 
 
+# column sums whose high word passes 2^24 (from about 186000 patches on) are rounded once, as smaller ones: four times the same patches have exactly four times the sums, so the same means, bit for bit
+@pytest.mark.parametrize("rows,cols,first,value", [(700, 520, 1, 241), (700, 520, 1, 201), (700, 520, 3, 201), (748, 498, 6, 201)])
+def test_density_large_sums(pace, rows, cols, first, value):
+    got = []
+    for r, c in ((rows, cols), (rows // 2, cols // 2)):
+        img = torch.zeros((r, 14, c, 14 * 3), dtype=torch.uint8, device="cuda")
+        img[:, 0, :, :first] = value   # the first bytes of every patch
+        d, st = pace.pace_apc_density(img.view(-1), [0], [14 * r], [14 * c])
+        assert bool((d == d[0]).all())
+        got.append((st[0, :2].tolist(), d[0].item()))
+    assert got[0] == got[1]
+
+
 # the tail over a cluster (more than 8192 distances): a bucket of equal distances too many for the
 # list, a list ranked in rounds (quantised values: many equal, several different), a direct ranking
 @pytest.mark.parametrize("kind", ["equal", "steps", "natural"])
