@@ -937,6 +937,10 @@ constexpr int kTokAhead = 2;             // tokens a warp of pass 1 has in fligh
 constexpr int kTokRun = 8;               // tokens (from a multiple of it on) whose column sums stay in fp32
                                          // before they are rounded, whatever the batch and the grid
 static_assert(kTokRun % kTokAhead == 0, "a run's tokens keep to their buffers");
+// A finite sum over a run is at most this: a coordinate of a normalised token is at most 1, or sqrt(3/2)
+// when |T|^2 is so small that it is rounded to a multiple of 2^-149.
+constexpr float kTokMost = 2.0f * kTokRun;
+static_assert(kTokMost < 512.0f, "the range of fix_add");
 
 // 2^-32 fixed point without conversions: v + 1.5 2^11 leaves v rounded to 2^-12 in the low mantissa
 // bits, the exact remainder times 2^32 plus 1.5 2^23 the rest, so acc collects
@@ -1072,8 +1076,8 @@ __global__ void __launch_bounds__(kTokThreads, 1) apc_tok_vec1(const uint4* __re
           for (int e = 0; e < 4; ++e) {
             ulonglong2* p = reinterpret_cast<ulonglong2*>(own) + 32 * (4 * i + e) + lane;
             ulonglong2 x = *p;
-            fix_add(x.x, fabsf(col[i][e].x) <= kTokRun ? col[i][e].x : 0.f);   // (a NaN counts as 0)
-            fix_add(x.y, fabsf(col[i][e].y) <= kTokRun ? col[i][e].y : 0.f);
+            fix_add(x.x, fabsf(col[i][e].x) <= kTokMost ? col[i][e].x : 0.f);   // (a NaN counts as 0)
+            fix_add(x.y, fabsf(col[i][e].y) <= kTokMost ? col[i][e].y : 0.f);
             *p = x;
           }
         }

@@ -269,6 +269,18 @@ def test_tokens_with_non_finite_rows(pace):
     assert bad[20] and bad.sum() <= 2 and not bad[:20].any()
 
 
+# |T|^2 of 1.125 and 1.477 units of the smallest subnormal is rounded to one: normalised, such tokens are a little
+# longer than 1, by either kind of kernel, and must not count as nothing
+@pytest.mark.parametrize("D", [256, 250])
+@pytest.mark.parametrize("mantissa", [1.5, 1.71875])
+def test_tokens_with_subnormal_squares(pace, D, mantissa):
+    T = np.zeros((40, D), np.float32)
+    T[:, 5] = mantissa * 2.0 ** -75
+    d, st = pace.pace_apc_density_tokens(bf16_tensor(synth.f32_to_bf16_bits(T)), [0, 40], [252], [252])
+    s, sq = pace.stats_dict(st)[0], mantissa * mantissa / 2   # |T|^2 over its rounded value
+    assert abs(s["phi"] - sq) <= 1e-6 and bool((d <= 1e-6 + sq ** 0.5 - 1).all())
+
+
 # scales 1 to 8 per side (filtered vertically first) and just above (generic), widths on 2-byte
 # boundaries, one and several column strips, heights below a group of four rows, odd sizes
 @pytest.mark.parametrize("shape,size", [((14, 14), (14, 14)), ((14, 14), (1, 1)), ((28, 14), (3, 2)), ((98, 42), (97, 41)),
