@@ -74,7 +74,9 @@ PACE_API pace_status_t pace_device_status(int* code, int* where, int clear);
 /* Exercises the bounded-wait path: launches one CTA that waits on a barrier nothing ever
  * arrives at.  After limit_us microseconds (1 .. 1000000) the wait gives up, the kernel
  * records PACE_ERR_TIMEOUT (kernel id 11) in the device status word and returns; the CUDA
- * context stays usable.  For failure-detection tests of callers. */
+ * context stays usable.  For failure-detection tests of callers.  Before it, a CTA waits 3 ms for
+ * image rows that never land, as the density passes do, and records PACE_ERR_INVALID_ARG
+ * (kernel id 11) if it went on to work on them. */
 PACE_API pace_status_t pace_selftest_wait_timeout(uint32_t limit_us, pace_stream_t stream);
 
 /* Number of CUDA kernels this library has launched in the calling process (all threads,

@@ -181,10 +181,12 @@ struct alignas(16) StripRef {
   int pairs_log2;   // log2 of the pairs of a full strip
   uint32_t first;   // byte of the image at which the strip's first row starts (an image is below 2^32 bytes)
   uint32_t pitch;   // bytes per image row
+  int patch;        // the first patch's number in the call
 };
 __device__ __forceinline__ void strip_place(const ApcTable& t, StripRef& q) {
   q.np = min(2 << q.pairs_log2, t.gw[q.b] - q.px0);
   q.first = static_cast<uint32_t>(q.py) * kPatch * q.pitch + static_cast<uint32_t>(q.px0) * (kPatch * 3);
+  q.patch = t.patch0[q.b] + q.py * t.gw[q.b] + q.px0;
 }
 __device__ __forceinline__ void strip_image(const ApcTable& t, StripRef& q) {
   q.pairs_log2 = t.strip_log2[q.b] - 1;
@@ -282,20 +284,52 @@ __device__ __forceinline__ float inv_norm_of(uint32_t ss) {
   return 1.0f / sqrtf(static_cast<float>(ss) * (1.0f / 65025.0f) + 1.0f);
 }
 
+// Waits for use `use` of a group's buffers (two, used in turn).  After a wait that runs out the group's waits
+// end at once, *gave_up holding 2; before that (1) both buffers get one more limit, so that no copy lands
+// after the CTA has ended.
+template <uint64_t LIMIT_NS>
+__device__ __noinline__ void strip_wait(uint64_t* bars, volatile int* gave_up, unsigned use, int* status, int kernel) {
+  auto wait = [&](unsigned u) { return ptx::mbar_wait(ptx::smem_u32(&bars[u & 1]), (u >> 1) & 1u, LIMIT_NS); };
+  if (*gave_up == 0) {
+    if (wait(use)) return;
+    record_error(status, PACE_ERR_TIMEOUT, kernel);
+    *gave_up = 1;
+  }
+  if (*gave_up == 1) {
+    wait(use);
+    wait(use + 1);
+    *gave_up = 2;
+  }
+}
+
 // A group's strips of one image (first, first + STEP, .. below end), which one of its warps copies into
 // its two buffers.  `used` counts the strips that the group has worked on, i.e. the uses of its buffers.
-template <int STEP>
+// A group that has given up copies nothing any more and works on what its buffers hold, from the places that
+// the copying warp last gave them (empty ones at the start), so within the call's images.
+template <int STEP, uint64_t LIMIT_NS = kWaitLimitNs>
 struct StripPipe {
   uint8_t (*s2)[kStageBytes];
   uint64_t* bars;
   StripRef* ref;
+  volatile int* gave_up;
   unsigned used;
+  // by one thread of the group, before the others come past a barrier
+  __device__ __forceinline__ void init() {
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      ptx::mbar_init(ptx::smem_u32(&bars[k]), 1);
+      ref[k] = StripRef{};
+    }
+    *gave_up = 0;
+    ptx::fence_mbar_init();
+  }
   __device__ __forceinline__ void copy(const uint8_t* img, const ApcTable& t, const StripRef& q, unsigned use) {
     copy_strip(img, t, q, s2[use & 1], ptx::smem_u32(&bars[use & 1]), &ref[use & 1]);
   }
+  __device__ __forceinline__ bool stopped() const { return __any_sync(0xffffffffu, *gave_up != 0); }
   // the image's first two strips (called by the copying warp of a group that is done with its buffers)
   __device__ __forceinline__ void begin(const uint8_t* img, const ApcTable& t, int first, int end) {
-    if (first >= end) return;
+    if (first >= end || stopped()) return;
     StripRef q = strip_ref(t, first);
     copy(img, t, q, used);
     if (first + STEP < end) {
@@ -303,16 +337,40 @@ struct StripPipe {
       copy(img, t, q, used + 1);
     }
   }
-  __device__ __forceinline__ bool wait() { return ptx::mbar_wait(ptx::smem_u32(&bars[used & 1]), (used >> 1) & 1u, kWaitLimitNs); }
+  __device__ __forceinline__ void wait(int* status, int kernel) {
+    if (!ptx::mbar_try_wait(ptx::smem_u32(&bars[used & 1]), (used >> 1) & 1u))
+      strip_wait<LIMIT_NS>(bars, gave_up, used, status, kernel);
+  }
   __device__ __forceinline__ const uint8_t* data() const { return s2[used & 1]; }
   __device__ __forceinline__ const StripRef& place() const { return ref[used & 1]; }
   // the strip after `cur`, once the group is done with the strip before it (called by the copying warp)
   __device__ __forceinline__ void next(const uint8_t* img, const ApcTable& t, const StripRef& cur) {
+    if (stopped()) return;
     StripRef q = cur;
     strip_advance(t, q, STEP);
     copy(img, t, q, used + 1);
   }
 };
+
+// Strips whose rows never land: the first wait runs out after a millisecond, the ones after it end at once, and
+// the strips are empty.
+__global__ void __launch_bounds__(64) strip_selftest(int* status) {
+  __shared__ __align__(16) uint8_t s2[2][kStageBytes];
+  __shared__ uint64_t bars[2];
+  __shared__ StripRef ref[2];
+  __shared__ int gave_up;
+  StripPipe<1, 1000000ull> pipe{s2, bars, ref, &gave_up, 0u};
+  if (threadIdx.x == 0) pipe.init();
+  __syncthreads();
+  const uint64_t start = ptx::globaltimer_ns();
+  for (int i = 0; i < 1000; ++i, ++pipe.used) {
+    pipe.wait(nullptr, K_SELFTEST);
+    const StripRef cur = pipe.place();
+    if (gave_up == 0 || cur.np != 0 || cur.first != 0u || cur.pitch != 0u || cur.patch != 0)
+      record_error(status, PACE_ERR_INVALID_ARG, K_SELFTEST);
+  }
+  if (!pipe.stopped() || ptx::globaltimer_ns() - start > 500000000ull) record_error(status, PACE_ERR_INVALID_ARG, K_SELFTEST);
+}
 
 struct Pass1Group {
   uint8_t s2[2][kStageBytes];
@@ -322,6 +380,7 @@ struct Pass1Group {
   unsigned long long col[kTokDim + 1];
   uint64_t bars[2];
   StripRef ref[2];
+  int gave_up[4];
 };
 static_assert(kStageBytes % 16 == 0 && offsetof(Pass1Group, wdig) % 16 == 0 && sizeof(Pass1Group) % 16 == 0, "shared layout");
 
@@ -337,13 +396,9 @@ __global__ void __launch_bounds__(kDAll, 1) apc_pass1(const uint8_t* __restrict_
   auto group_sync = [&]() { ptx::named_barrier_sync(1 + grp, kDThreads); };
   const int2 range = unit_range(units);
   constexpr int kCopyWarp = kDThreads / 32 - 1;
-  if (tid == 0) {
-    ptx::mbar_init(ptx::smem_u32(&sh.bars[0]), 1);
-    ptx::mbar_init(ptx::smem_u32(&sh.bars[1]), 1);
-    ptx::fence_mbar_init();
-  }
+  StripPipe<kDGroups> pipe{sh.s2, sh.bars, sh.ref, sh.gave_up, 0u};
+  if (tid == 0) pipe.init();
   group_sync();
-  StripPipe<kDGroups> pipe{sh.s2, sh.bars, sh.ref, 0u};
   // thread j < 294 owns the four columns of word position j (row j / 21): their digit sums; lane 0 of
   // warp 0 the constant coordinate
   uint32_t acc[4][4] = {};
@@ -386,7 +441,7 @@ __global__ void __launch_bounds__(kDAll, 1) apc_pass1(const uint8_t* __restrict_
     if (warp == kCopyWarp) pipe.begin(img, t, first + grp, end);
     bool folded = false;
     for (int unit = first + grp; unit < end; unit += kDGroups, ++pipe.used) {
-      if (!pipe.wait()) record_error(status, PACE_ERR_TIMEOUT, K_APC_PASS1);
+      pipe.wait(status, K_APC_PASS1);
       const StripRef cur = pipe.place();
       const uint8_t* s = pipe.data();
       if (strips == kFoldStrips) {
@@ -420,7 +475,7 @@ __global__ void __launch_bounds__(kDAll, 1) apc_pass1(const uint8_t* __restrict_
           uint32_t ss = 0u;
 #pragma unroll
           for (int y = 0; y < kPatch; ++y) ss += sh.ssq[y][tid];
-          sumsq[t.patch0[b] + cur.py * t.gw[b] + cur.px0 + tid] = ss;
+          sumsq[cur.patch + tid] = ss;
           weight = __float2uint_rn(inv_norm_of(ss) * 2147483648.0f);   // exact
         }
 #pragma unroll
@@ -576,6 +631,7 @@ struct Pass2Group {
   unsigned long long part[2][kPatch][kStrip];   // x . c_hat of one image row of a patch
   uint64_t bars[2];
   StripRef ref[2];
+  int gave_up[4];
 };
 struct Pass2Smem {
   Pass2Group g[kDGroups];
@@ -602,13 +658,9 @@ __global__ void __launch_bounds__(kDAll, 1) apc_pass2(const uint8_t* __restrict_
   auto group_sync = [&]() { ptx::named_barrier_sync(1 + grp, kDThreads); };
   constexpr int kCopyWarp = kDThreads / 32 - 1;
   const int2 range = unit_range(units);
-  if (tid == 0) {
-    ptx::mbar_init(ptx::smem_u32(&my.bars[0]), 1);
-    ptx::mbar_init(ptx::smem_u32(&my.bars[1]), 1);
-    ptx::fence_mbar_init();
-  }
+  StripPipe<kDGroups> pipe{my.s2, my.bars, my.ref, my.gave_up, 0u};
+  if (tid == 0) pipe.init();
   group_sync();
-  StripPipe<kDGroups> pipe{my.s2, my.bars, my.ref, 0u};
   int first = range.x;
   for (int b = first < range.y ? find_image(t, first) : 0; first < range.y; ++b) {   // the CTA's strips of image b
     const int end = min(range.y, t.unit_prefix[b + 1]);
@@ -669,11 +721,11 @@ __global__ void __launch_bounds__(kDAll, 1) apc_pass2(const uint8_t* __restrict_
       stats[t.b_base + b].k_tail = t.ktail[b];
     }
     for (int unit = first + grp; unit < end; unit += kDGroups, ++pipe.used) {
-      if (!pipe.wait()) record_error(status, PACE_ERR_TIMEOUT, K_APC_PASS2);
+      pipe.wait(status, K_APC_PASS2);
       const StripRef cur = pipe.place();
       const uint8_t* s = pipe.data();
       auto& part = my.part[pipe.used & 1];
-      const int p0 = t.patch0[b] + cur.py * t.gw[b] + cur.px0;   // the strip's first patch
+      const int p0 = cur.patch;
       const int npair = (cur.np + 1) >> 1;
       const int iy = tid >> cur.pairs_log2, ip = tid & ((1 << cur.pairs_log2) - 1);   // this thread's (row, pair)
       uint32_t ss = 0u;
@@ -1694,30 +1746,27 @@ __global__ void __launch_bounds__(kApcThreads, kPixCtasPerSm) apc_pix_features(c
   __shared__ unsigned long long part[kWarps][kPixDim];
   __shared__ uint64_t bars[2];
   __shared__ StripRef ref[2];
+  __shared__ int gave_up;
   ptx::launch_dependents();
   const int2 range = unit_range(units);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   unsigned long long acc = 0ull;   // lane k < kPixDim: coordinate k
-  if (threadIdx.x == 0) {
-    ptx::mbar_init(ptx::smem_u32(&bars[0]), 1);
-    ptx::mbar_init(ptx::smem_u32(&bars[1]), 1);
-    ptx::fence_mbar_init();
-  }
+  StripPipe<1> pipe{s2, bars, ref, &gave_up, 0u};
+  if (threadIdx.x == 0) pipe.init();
   __syncthreads();
-  StripPipe<1> pipe{s2, bars, ref, 0u};
   int first = range.x;
   for (int b = first < range.y ? find_image(t, first) : 0; first < range.y; ++b) {   // the CTA's strips of image b
     const int end = min(range.y, t.unit_prefix[b + 1]);
     if (warp == 0) pipe.begin(img, t, first, end);
     for (int unit = first; unit < end; ++unit, ++pipe.used) {
-      if (!pipe.wait()) record_error(status, PACE_ERR_TIMEOUT, K_APC_PASS1);
+      pipe.wait(status, K_APC_PASS1);
       const StripRef cur = pipe.place();
       const uint8_t* s = pipe.data();
       if (unit > first && unit + 1 < end) {
         __syncthreads();   // everyone is done with the other buffer
         if (warp == 0) pipe.next(img, t, cur);
       }
-      const int64_t p0 = static_cast<int64_t>(t.patch0[b]) + cur.py * t.gw[b] + cur.px0;
+      const int64_t p0 = cur.patch;
       for (int p = warp; p < cur.np; p += kWarps) {
         float tok[kPixDim];
         patch_feature([&](int y, int x) { return s + y * kStageRow + row_phase(cur, y) + (p * kPatch + x) * 3; }, feature,
@@ -2753,6 +2802,11 @@ pace_status_t check_images(const uint8_t* img, const int64_t* off, const int32_t
 }
 
 }  // namespace
+
+pace_status_t launch_strip_selftest(int* status, cudaStream_t stream) {
+  strip_selftest<<<1, 64, 0, stream>>>(status);
+  return check_launch();
+}
 }  // namespace pace
 
 using namespace pace;

@@ -152,6 +152,7 @@ pace_status_t pace_device_status(int* code, int* where, int clear) {
 pace_status_t pace_selftest_wait_timeout(uint32_t limit_us, pace_stream_t stream) {
   if (limit_us == 0 || limit_us > 1000000u) return PACE_ERR_INVALID_ARG;
   PACE_CHECK(pace::check_device());
+  PACE_CHECK(pace::launch_strip_selftest(pace::device_status_word(), stream));
   pace::selftest_wait_kernel<<<1, 32, 0, stream>>>(static_cast<uint64_t>(limit_us) * 1000ull,
                                                    pace::device_status_word());
   return pace::check_launch();

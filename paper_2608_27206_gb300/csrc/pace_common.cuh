@@ -42,6 +42,7 @@ pace_status_t check_device();              // current device is sm_103 and initi
 int* device_status_word();                 // status word of the current device
 pace_status_t check_launch();              // cudaGetLastError -> status
 pace_status_t sm_count(int* sms);          // SMs of the current device
+pace_status_t launch_strip_selftest(int* status, cudaStream_t stream);   // apc.cu: a wait for image rows that runs out
 
 // Generation of the library's per-device set-up.  pace_init(dev) advances it, so every cache
 // built on DeviceOnce below (function attributes, symbol addresses) is filled again on the next
