@@ -448,7 +448,7 @@ def pace_vit_attn_importance(Q: torch.Tensor, K: torch.Tensor, cu_seqlens, scale
     cu, cp, B = _i32(cu_seqlens)
     B -= 1
     total, Hh, D = Q.shape
-    n = int(cu[-1]) // merge
+    n = int(cu[-1]) // merge if merge else 0   # (refused by the library)
     if scale is None:
         scale = float(D) ** -0.5
     if out is None:
@@ -486,7 +486,7 @@ def pace_vit_attn_importance_chunked(Q: torch.Tensor, K: torch.Tensor, cu_seqlen
     cu, cp, B = _i32(cu_seqlens)
     B -= 1
     total, Hh, D = Q.shape
-    n = int(cu[-1]) // merge
+    n = int(cu[-1]) // merge if merge else 0   # (refused by the library)
     if scale is None:
         scale = float(D) ** -0.5
     if out is None:

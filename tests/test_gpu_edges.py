@@ -38,6 +38,20 @@ def test_vit_last_tile(pace, lens):
     assert_scores_close(got, O.vit_attn_importance(f64(q), f64(k), cu, 80 ** -0.5, 4))
 
 
+# a merge of 0 is refused by the library, whatever the caller brings
+@pytest.mark.parametrize("given", [False, True])
+def test_vit_merge_of_zero(pace, given):
+    q = bf16_tensor(synth.random_small_qk(1, 8, 3, 80))
+    out = torch.empty(8, device="cuda") if given else None
+    ev = torch.cuda.Event()
+    ev.record()
+    for call in (lambda: pace.pace_vit_attn_importance(q, q, [0, 8], merge=0, out=out),
+                 lambda: pace.pace_vit_attn_importance_chunked(q, q, [0, 8], [8], [ev], merge=0, out=out)):
+        with pytest.raises(pace.PaceError) as e:
+            call()
+        assert e.value.status == pace.PACE_ERR_INVALID_ARG
+
+
 # few keys and several heads per KV head: pass 2 splits a group's heads over CTAs (7 heads; 1 and 2
 # query tiles), down to one stream item per CTA
 @pytest.mark.parametrize("tq,nv", [((1,), (1,)), ((128,), (300,)), ((129,), (128,)), ((257, 5), (40, 513))])
