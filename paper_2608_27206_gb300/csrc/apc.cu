@@ -1747,7 +1747,9 @@ __global__ void __launch_bounds__(kApcThreads, kPixCtasPerSm) apc_pix_features(c
   __shared__ uint64_t bars[2];
   __shared__ StripRef ref[2];
   __shared__ int gave_up;
-  ptx::launch_dependents();
+  // (for the tokens alone this is the call's first kernel, and its last)
+  if (DENSITY) ptx::launch_dependents();
+  else ptx::begin_call();
   const int2 range = unit_range(units);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   unsigned long long acc = 0ull;   // lane k < kPixDim: coordinate k
@@ -3137,8 +3139,7 @@ pace_status_t launch_pix_features(const uint8_t* img, ApcTable& t, int c0, int n
   int* status = device_status_word();
   if (sums != nullptr)
     return launch_dependent(apc_pix_features<true>, grid, kApcThreads, 0, 1, stream, img, t, units, feature, tokens, sums, status);
-  apc_pix_features<false><<<grid, kApcThreads, 0, stream>>>(img, t, units, feature, tokens, sums, status);
-  return check_launch();
+  return launch_dependent(apc_pix_features<false>, grid, kApcThreads, 0, 1, stream, img, t, units, feature, tokens, sums, status);
 }
 
 int64_t total_patches(int B, const int32_t* H, const int32_t* W) {

@@ -433,6 +433,82 @@ def test_calls_back_to_back(pace, captured):
             assert torch.equal(o[k].view(torch.uint8), want[i % 2][k].view(torch.uint8)), (i, k)
 
 
+# the calls that the path above leaves out, each twice on one scratch with other inputs and never synchronised:
+# their first kernels write scratch before they wait for earlier work, and the next call's may start early
+@pytest.mark.parametrize("captured", [False, True])
+def test_other_calls_back_to_back(pace, captured):
+    rng = np.random.default_rng(4)
+    H, W = [448, 224, 154], [448, 308, 14 * 40]
+    n = sum(h * w for h, w in zip(H, W)) // 196
+    buf, off = synth.pack_images([rng.integers(0, 256, (h, w, 3), dtype=np.uint8) for h, w in zip(H, W)])
+    cu = _cu([h * w // 196 for h, w in zip(H, W)])
+    seq, vis, nv, hq, hk = [0, 300, 700], [10, 0], [200, 333], 14, 2
+    img, kept = torch.from_numpy(buf).cuda(), torch.arange(0, 533, 5, dtype=torch.int32, device="cuda")
+    keep = _cu([40, 67])
+    T = {D: bf16_tensor(synth.f32_to_bf16_bits(rng.normal(size=(n, D)).astype(np.float32))) for D in (256, 250)}
+    q, k = (bf16_tensor(synth.random_small_qk(i, 700, h, 128)) for i, h in ((1, hq), (2, hk)))
+    hid = torch.from_numpy(rng.integers(0, 255, (700, 1024), dtype=np.uint8)).cuda()
+    pos = torch.arange(3 * 700, dtype=torch.int32, device="cuda").view(3, 700)
+    inputs = [img, *T.values(), q, k, hid, pos]
+    first = [x.clone() for x in inputs]
+    other = [x.flip(0).contiguous() if i else 255 - x for i, x in enumerate(first)]
+    d, st = torch.empty(n, device="cuda"), torch.zeros((3, 10), dtype=torch.int32, device="cuda")
+    ws = torch.empty(max(pace.pace_apc_density_workspace_size(H, W), pace.pace_apc_density_pixel_workspace_size(H, W),
+                         *(pace.pace_apc_density_tokens_workspace_size(cu, D) for D in T),
+                         pace.pace_llm_sequence_importance_workspace_size(seq, vis, nv, hq, hk)), dtype=torch.uint8, device="cuda")
+    tok, s_llm = torch.empty((n, 8), device="cuda"), torch.empty(533, device="cuda")
+    idx = torch.empty(700 - 533 + 107, dtype=torch.int32, device="cuda")
+    dst = torch.empty((idx.numel(), 1024), dtype=torch.uint8, device="cuda")
+    dpos, small = torch.empty((3, idx.numel()), dtype=torch.int32, device="cuda"), torch.zeros_like(img)
+
+    def gather():
+        pace.pace_prune_index(seq, vis, [0, 200, 533], keep, kept, out=idx)
+        pace.pace_gather_multi([pace.gather_spec(hid, dst, 0), pace.gather_spec(pos, dpos, 1)], idx)
+
+    def chain():   # a resized image is the next call's picture, a gathered row list the next gather's
+        pace.pace_apc_resample_to(img, off, H, W, [h // 2 // 14 * 14 for h in H], [w // 2 // 14 * 14 for w in W], small, off)
+        pace.pace_apc_density(small, off, [h // 2 // 14 * 14 for h in H], [w // 2 // 14 * 14 for w in W], d_out=d, stats=st, ws=ws)
+
+    calls = [(lambda D=D: pace.pace_apc_density_tokens(T[D], cu, H, W, d_out=d, stats=st, ws=ws), (d, st)) for D in T]
+    calls += [(lambda f=f: pace.pace_apc_density_pixel(img, off, H, W, f, d_out=d, stats=st, ws=ws), (d, st))
+              for f in ("edge_density", "rgb_stats")]
+    calls += [(lambda: pace.pace_apc_pixel_features(img, off, H, W, "laplacian", out=tok), (tok,)),
+              (lambda: pace.pace_apc_density_static(img, off, H, W, d_out=d, stats=st), (d, st)),
+              (lambda: pace.pace_llm_sequence_importance(q, k, seq, vis, nv, out=s_llm, ws=ws), (s_llm,)),
+              (gather, (idx, dst, dpos)), (chain, (small, d, st))]
+
+    def run(sync):
+        out = []
+        for call, results in calls:
+            for src in (first, other):
+                for x, y in zip(inputs, src):
+                    x.copy_(y)
+                call()
+                call()
+                out += [r.clone() for r in results]
+                if sync:
+                    torch.cuda.synchronize()
+        return out
+
+    pace.pace_apc_density_static(img, off, H, W, d_out=d, stats=st)   # (its first call looks its scratch up)
+    want = run(True)
+    stream = torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(stream):
+        if captured:
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=stream):
+                out = run(False)
+            g.replay()
+            g.replay()
+        else:
+            run(False)
+            out = run(False)
+    torch.cuda.synchronize()
+    for i, (a, b) in enumerate(zip(out, want)):
+        assert torch.equal(a.view(torch.uint8), b.view(torch.uint8)), i
+
+
 # scores held in registers for 4, 8 and 12 per thread of a block of 1024, and read again per pass above
 @pytest.mark.parametrize("n", [4096, 4097, 8192, 8193, 12288, 12289, 16384, 20481])
 def test_select_registers(pace, n):
