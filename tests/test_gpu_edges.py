@@ -234,6 +234,20 @@ def test_tail_counts_of_backgrounds(pace, kind, rows, cols):
     assert_distances_close(d, O.apc_density_preview(f64(bits), w, h)["d"])
 
 
+# more images than one table holds: the second table's feature kernel follows the first one's tail
+def test_pixel_density_two_tables(pace):
+    rng = np.random.default_rng(7)
+    shapes = [(14 * int(a), 14 * int(b)) for a, b in rng.integers(1, 9, (70, 2))]
+    buf, off = synth.pack_images([rng.integers(0, 256, (*s, 3), dtype=np.uint8) for s in shapes])
+    H, W, src = [s[0] for s in shapes], [s[1] for s in shapes], torch.from_numpy(buf).cuda()
+    n = [h * w // 196 for h, w in shapes]
+    for f in ("rgb_stats", "color_entropy", "edge_density", "laplacian"):
+        d, st = pace.pace_apc_density_pixel(src, off, H, W, f)
+        for b in (0, 1, 62, 63, 64, 65, 69):   # each alone gives the same
+            one, s = pace.pace_apc_density_pixel(src, [int(off[b])], [H[b]], [W[b]], f)
+            assert torch.equal(one, d[sum(n[:b]):sum(n[:b + 1])]) and torch.equal(s[0], st[b])
+
+
 # register kernels (whole 16-byte vectors, up to 1536) and the staged ones (other widths), runs of 8
 # tokens with remainders, several images per CTA
 @pytest.mark.parametrize("D", [8, 248, 256, 264, 1152, 1536, 1544, 1284, 6])
