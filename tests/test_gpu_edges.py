@@ -155,6 +155,23 @@ def test_density_large_sums(pace, rows, cols, first, value):
     assert got[0] == got[1]
 
 
+# pictures so narrow that a group of threads meets more strips than its 32-bit sums are trusted with (2048, of one or
+# two patches): four times the same four patches give the same means and distances, bit for bit
+@pytest.mark.parametrize("cols", [1, 2])
+def test_density_many_strips(pace, cols):
+    pattern = torch.randint(0, 256, (4, 14, cols, 42), dtype=torch.uint8, device="cuda", generator=torch.Generator("cuda").manual_seed(1))
+    got = []
+    for rows in (1 << 20, 1 << 18):
+        img = pattern.repeat(rows // 4, 1, 1, 1)
+        d, st = pace.pace_apc_density(img.view(-1), [0], [14 * rows], [14 * cols])
+        d = d.view(rows // 4, -1)
+        assert bool((d == d[0]).all())
+        got.append((st[0, :2].tolist(), d[0].tolist()))
+    assert got[0] == got[1]
+    ref = O.apc_density(pattern.reshape(56, cols * 14, 3).cpu().numpy())
+    np.testing.assert_allclose(got[0][1], ref["d"], rtol=1e-6)
+
+
 # the tail over a cluster (more than 8192 distances): a bucket of equal distances too many for the
 # list, a list ranked in rounds (quantised values: many equal, several different), a direct ranking
 @pytest.mark.parametrize("kind", ["equal", "steps", "natural"])
