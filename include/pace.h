@@ -16,6 +16,12 @@
  *  - All work is enqueued on `stream` (a cudaStream_t; NULL = legacy default
  *    stream) and runs asynchronously.  Launch failures return PACE_ERR_CUDA
  *    and the CUDA error code is kept for pace_last_cuda_error().
+ *  - Kernels are launched with programmatic stream serialization, and the last one
+ *    of a call lets the next kernel of the stream start before it has ended.  Work
+ *    enqueued the usual way (launches, copies, events, graph nodes) sees a finished
+ *    call all the same; a kernel of the caller's that is itself launched with
+ *    programmatic stream serialization has to wait (cudaGridDependencySynchronize,
+ *    griddepcontrol.wait) before it touches what the call reads or writes.
  *  - Device-side waits are bounded.  A kernel whose wait runs out records
  *    PACE_ERR_TIMEOUT in the device status word (pace_device_status) and
  *    returns early; its outputs are then undefined.
