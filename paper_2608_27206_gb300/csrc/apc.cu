@@ -217,8 +217,8 @@ __device__ __forceinline__ uint32_t row_phase(const StripRef& q, int y) {
 }
 
 // Called by one whole warp: copies a strip's 14 rows to s (a lane per row), counted on the mbarrier
-// `bar`, and the strip's place to `slot`.  Nothing past the image is read: the last row's last few bytes, which do not fill a 16-byte
-// piece, are stored by the lane itself, before the warp's arrival on the barrier.
+// `bar`, and the strip's place to `slot`.  Nothing past the image is read: the last row's last few bytes,
+// which do not fill a 16-byte piece, are stored by the lane itself, before the warp's arrival on the barrier.
 __device__ __forceinline__ void copy_strip(const uint8_t* __restrict__ img, const ApcTable& t, const StripRef& q, uint8_t* s,
                                            uint32_t bar, StripRef* slot) {
   const int lane = threadIdx.x & 31;
@@ -982,7 +982,8 @@ __global__ void __launch_bounds__(kApcThreads) apc_tok_pass2(const uint32_t* __r
 // warp's chain per token (load, sum of squares over the lanes, square root and division, column sums),
 // pass 2 by L2 and HBM.  42196 tokens of 1280: 84.5 us for the call staged, 55.5 in registers (passes
 // 38.8 + 31.9, now 25.3 + 28).  Other widths, and tokens off a 16-byte boundary, take the staged kernels
-// above.
+// above: with six vectors a lane of pass 1 has its 168 registers full (two rows in flight, a row unpacked
+// and its column sums, 8 per vector each), and a seventh would spill in every token's chain.
 constexpr int kTokVecMax = 6;            // 16-byte vectors per lane
 constexpr int kTokThreads = 384;         // of pass 1: one CTA per SM, since each ends an image with D atomics
 constexpr int kTokAhead = 2;             // tokens a warp of pass 1 has in flight

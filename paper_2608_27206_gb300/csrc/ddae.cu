@@ -812,7 +812,6 @@ extern "C" pace_status_t pace_gather(const void* src, int64_t n_src_rows, int64_
   const int64_t row_vec = row_bytes / 16;
   if (vec && row_vec <= 32 * 16) {
     // a warp per row: enough resident warps for every SM (about 24 per SM at U = 16), no more
-    // than there are rows
     // than there are rows; blocks of 4 warps, so that a few thousand rows still reach every SM
     const int64_t b = std::min<int64_t>((n_idx + 3) / 4, static_cast<int64_t>(sms) * 8);
     const unsigned g = static_cast<unsigned>(b);
