@@ -627,11 +627,14 @@ __global__ void __launch_bounds__(256) prune_index_kernel(const __grid_constant_
 // with all its loads in flight, so that rows of any length (7 KB hidden states, 256-byte K and V
 // heads, 4-byte position ids) fill the warps alike (a 4K prompt's prune step, 1331 rows and 35.5 MB:
 // 13 us with a warp per row, now 7.9; bound by memory latency and HBM).  Finding an element's row
-// weighs little on 16 bytes but sets the time of narrower elements, so rows of at least kGmRow of those
-// take a warp each (20000 rows of 7170 bytes: 635 us by elements, 147 by rows; of 1000 bytes, in words,
-// 20 and 9; of 50 bytes 6.2 and 7.2), and so do shorter ones down to kGmShort when the SMs hold a warp for
-// every row at once (1331 rows of 50 bytes: 4.1 us by elements, 3.1 by rows).
-constexpr int kGmThreads = 256, kGmU = 4, kGmBlock = kGmThreads * kGmU, kGmRow = 64, kGmShort = 4, kGmFew = 8192;
+// weighs little on 16 bytes but much on narrower elements, so rows of those take a warp each (us by
+// elements and by rows: 20000 rows of 1000 bytes, in words, 18.4 and 9.2, of 255 bytes 18.3 and 9.2; 450 of
+// 7170 17.5 and 14.3), but for few rows above kGmLong elements, which a warp alone takes long over (300 of 7170 13.3
+// and 14.4; 100 of 1022 4.1 and 5.1), and for many below kGmRow (20000 of 13 4.1 and 8.2; 300 of 13 4.1 and 3.1).
+// Those rows are read and written through L1, since they need not start on a sector (20000 of 3001: 37 us, streamed 44).
+constexpr int kGmThreads = 256, kGmU = 4, kGmBlock = kGmThreads * kGmU;
+constexpr int kGmShort = 4, kGmRow = 64, kGmLong = 256;   // elements of a row
+constexpr int kGmMost = 2048, kGmLeast = 384;             // rows: at most for short ones, at least for long ones
 // Division of n < 2^31 by d >= 1 as a multiplication (Granlund and Montgomery): with 2^(l-1) < d <= 2^l and
 // m = floor(2^(31+l) / d) + 1, m d exceeds 2^(31+l) by at most 2^l, so floor(n m / 2^(31+l)) is the quotient.
 struct FastDiv {
@@ -708,10 +711,10 @@ __device__ __forceinline__ void gather_rows_of(const pace_gather_tensor& g, int6
   for (int64_t c = lane; c < cols; c += 32 * kGmU) {
     V v[kGmU];
 #pragma unroll
-    for (int u = 0; u < kGmU; ++u) v[u] = in && c + 32 * u < cols ? __ldcs(sp + c + 32 * u) : V{};
+    for (int u = 0; u < kGmU; ++u) v[u] = in && c + 32 * u < cols ? sp[c + 32 * u] : V{};
 #pragma unroll
     for (int u = 0; u < kGmU; ++u)
-      if (c + 32 * u < cols) __stcs(dp + c + 32 * u, v[u]);
+      if (c + 32 * u < cols) dp[c + 32 * u] = v[u];
   }
 }
 
@@ -896,9 +899,10 @@ extern "C" pace_status_t pace_gather_multi(const pace_gather_tensor* tensors, in
                         static_cast<uintptr_t>(g.dst_slab_stride);
     t.width[k] = (a % 16 == 0) ? 16 : (a % 4 == 0) ? 4 : 1;
     const int64_t cols = g.row_bytes / t.width[k];
-    t.rows[k] = t.width[k] < 16 && (cols >= kGmRow || (cols >= kGmShort && g.n_slabs * n_idx <= kGmFew));
+    const int64_t n_rows = g.n_slabs * n_idx;
+    t.rows[k] = t.width[k] < 16 && (cols > kGmLong ? n_rows >= kGmLeast : cols >= kGmRow || (cols >= kGmShort && n_rows <= kGmMost));
     if (cols < (int64_t{1} << 31)) t.by_cols[k] = fast_div(static_cast<uint32_t>(cols));
-    const int64_t items = g.n_slabs * n_idx * (t.rows[k] ? 1 : cols), per = t.rows[k] ? kGmThreads / 32 : kGmBlock;
+    const int64_t items = n_rows * (t.rows[k] ? 1 : cols), per = t.rows[k] ? kGmThreads / 32 : kGmBlock;
     t.block_prefix[k + 1] = t.block_prefix[k] + (items + per - 1) / per;
   }
   if (t.block_prefix[n_tensors] == 0) return PACE_OK;

@@ -103,11 +103,11 @@ def test_gather_multi_blocks(pace, n_idx):
         assert not b.select(d, 0).any()
 
 
-# rows of 1- and 4-byte elements: a warp per row (64 elements and more, 4 and more where the rows are few) and by
-# elements, several steps of a warp with remainders, slabs, rows out of range
-@pytest.mark.parametrize("n_idx,slabs", [(7, 1), (4096, 2), (4097, 2)])
+# rows of 1- and 4-byte elements: a warp per row (64 elements and more, 4 and more where the rows are few, more than 256
+# where they are many) and by elements, several steps of a warp with remainders, slabs, rows out of range
+@pytest.mark.parametrize("n_idx,slabs", [(7, 1), (191, 2), (192, 2), (1024, 2), (1025, 2)])
 @pytest.mark.parametrize("nbytes,strided", [(3, False), (4, False), (63, False), (64, False), (65, True), (127, False), (129, True),
-                                            (252, False), (256 + 4, True), (1022, False)])
+                                            (255, False), (257, False), (252, True), (1024, False), (1028, True), (1022, False)])
 def test_gather_multi_narrow_rows(pace, n_idx, slabs, nbytes, strided):
     rng = np.random.default_rng(nbytes + n_idx)
     idx = torch.from_numpy(rng.integers(0, 30, n_idx).astype(np.int32)).cuda()
