@@ -2319,7 +2319,10 @@ __device__ __forceinline__ void resample_tile(ResampleSmem& sh, const uint8_t* _
 // rating, windows and weights before their first row, these on four window edges at once and on one
 // window per lane (one image of 448 x 448 at r = 0.25: 5.9 us, in wide tiles 10.2; at r = 0.8 7.2 and
 // 10.3).  Every sum is taken in the same order with the same weights as there, so the bytes do not
-// depend on which tiles a call gets.
+// depend on which tiles a call gets.  A launch after other work fetches its instructions from memory, so
+// this code comes first in the kernel and its loops are not unrolled: such a call on 448 x 448 takes 8.7 us,
+// 14.8 with the code behind that of the wide tiles and unrolled by four, 12.8 in wide tiles; a first call in
+// wide tiles of 4K 55 us, as without this code (61 with it in front and unrolled).
 constexpr int kSTH = 8, kSTW = 32;           // output rows and columns
 constexpr int kSTaps = 14;                   // a window has at most floor(4 * 2.75) + 2 taps
 constexpr int kSRows = 36;                   // 7 * 2.75 + 4 * 2.75 + 2 input rows, and two read with weight 0
@@ -2365,14 +2368,14 @@ __device__ __forceinline__ void resample_tile_small(SmallSmem& sh, const uint8_t
     float* to = warp == 0 ? &sh.wx[0][lane] : &sh.wy[lane][0];
     const int step = warp == 0 ? kSTW : 1, n = min(w.n, kSTaps);
     float sum = 0.f;
-#pragma unroll 4
+#pragma unroll 1
     for (int i = 0; i < n; ++i) {
       const float x = cubic_w(static_cast<float>(w.num0 + i * w.step) * w.inv_den);
       to[i * step] = x;
       sum += x;
     }
     const float inv = 1.0f / sum;
-#pragma unroll 4
+#pragma unroll 1
     for (int i = 0; i < n; ++i) to[i * step] *= inv;
     (warp == 0 ? sh.xlo : sh.ylo)[lane] = w.lo;
     (warp == 0 ? sh.xn : sh.yn)[lane] = warp == 0 ? n : min(n, last_input(o, n_in, n_out) - w.lo + 1);
@@ -2394,7 +2397,7 @@ __device__ __forceinline__ void resample_tile_small(SmallSmem& sh, const uint8_t
         a[0] = ptx::ffma2(w2, lo, a[0]);
         a[1] = ptx::ffma2(w2, hi, a[1]);
       };
-#pragma unroll 4
+#pragma unroll 1
       for (int i = 0; i < max(na, nb); ++i) {
         take(la - y0 + i, i < na ? sh.wy[ra][i] : 0.f, acc[0]);
         take(lb - y0 + i, i < nb ? sh.wy[rb][i] : 0.f, acc[1]);
@@ -2408,7 +2411,7 @@ __device__ __forceinline__ void resample_tile_small(SmallSmem& sh, const uint8_t
       const float* va = &sh.v[ra][(sh.xlo[lane] - x0) * 3];
       const int n = sh.xn[lane];
       float acc[2][3] = {};
-#pragma unroll 4
+#pragma unroll 1
       for (int k = 0; k < n; ++k) {
         const float w = sh.wx[k][lane];
 #pragma unroll
@@ -2461,10 +2464,10 @@ __device__ __forceinline__ void resample_small(SmallSmem& sh, const uint8_t* __r
   }
 }
 // Tiles x scale per CTA of the grid (a quarter more where rows start on 2-byte boundaries, which costs a
-// second word per read) up to which a call takes small tiles.  Both kinds, in us: 2.3 rounds at 2.3
-// (8 images of 448 x 448, 5.3) 15.5 and 18.5, 2.4 at 2.4 (1064 x 1904, 5.7) 15.4 and 17.4, 5.2 at 1 (896 x 896)
-// 15.0 and 15.4, 2.9 at 2 (1344 x 1344, 5.8) 14.4 and 14.3, 4.7 at 1.6 (7.5) 20.5 and 18.5.
-constexpr float kSmallWork = 5.7f;
+// second word per read) up to which a call takes small tiles.  Both kinds, in us: 2.9 rounds at 1 (672 x 672)
+// 9.2 and 12.3, 2.1 at 1.6 (896 x 896, 3.3) 13.3 and 14.3, 3.2 at 1.3 (896 x 896, 4.1) 15.4 and 14.3, 2.1 at 2.4
+// (1344 x 1344, 5.0) 18.1 and 16.4.
+constexpr float kSmallWork = 3.8f;
 
 // Wide and generic tiles of the batch, ho and wo as in resample_small.
 __device__ __forceinline__ void resample_large(ResampleSmem& sh, const uint8_t* __restrict__ src, const ResampleTable& t,
@@ -2652,12 +2655,11 @@ __global__ void __launch_bounds__(kVThreads, kVCtasPerSm) apc_resample(const uin
     }
     total_work = s_work;
   }
-  // (the small tiles' code last: in front of the other, it made the first launch of a call in wide tiles, which
-  // fetches its instructions from memory, 6 us longer)
-  if (static_cast<float>(total_work) > kSmallWork * static_cast<float>(gridDim.x))
-    resample_large(*reinterpret_cast<ResampleSmem*>(rs_smem), src, t, dst, ho, wo);
-  else
+  if (static_cast<float>(total_work) <= kSmallWork * static_cast<float>(gridDim.x)) {   // (this code first: see there)
     resample_small(*reinterpret_cast<SmallSmem*>(rs_smem), src, t, dst, ho, wo, small_n);
+    return;
+  }
+  resample_large(*reinterpret_cast<ResampleSmem*>(rs_smem), src, t, dst, ho, wo);
 }
 
 // ------------------------------------------------------------------------------------------------
