@@ -2317,12 +2317,13 @@ __device__ __forceinline__ void resample_tile(ResampleSmem& sh, const uint8_t* _
 // memory, warp w filtering rows 2 w and 2 w + 1 vertically (a lane per four bytes) and then horizontally
 // (a lane per column).  Such a call is all latency: the wide tiles above spend 9000 to 10000 cycles on a
 // rating, windows and weights before their first row, these on four window edges at once and on one
-// window per lane (one image of 448 x 448 at r = 0.25: 5.9 us, in wide tiles 10.2; at r = 0.8 7.2 and
+// window per lane (one image of 448 x 448 at r = 0.25: 6.2 us, in wide tiles 10.2; at r = 0.8 7.2 and
 // 10.3).  Every sum is taken in the same order with the same weights as there, so the bytes do not
 // depend on which tiles a call gets.  A launch after other work fetches its instructions from memory, so
-// this code comes first in the kernel and its loops are not unrolled: such a call on 448 x 448 takes 8.7 us,
-// 14.8 with the code behind that of the wide tiles and unrolled by four, 12.8 in wide tiles; a first call in
-// wide tiles of 4K 55 us, as without this code (61 with it in front and unrolled).
+// this code comes first in the kernel, once for rows on any boundary, and its loops are not unrolled: behind a
+// flush and other kernels such a call on 448 x 448 takes 10.3 us, 15.2 with the code behind that of the wide tiles,
+// twice and unrolled by four, 14.1 in wide tiles; a call in wide tiles of 4K 34.7, as without this code (36.0
+// with it twice).
 constexpr int kSTH = 8, kSTW = 32;           // output rows and columns
 constexpr int kSTaps = 14;                   // a window has at most floor(4 * 2.75) + 2 taps
 constexpr int kSRows = 36;                   // 7 * 2.75 + 4 * 2.75 + 2 input rows, and two read with weight 0
@@ -2342,7 +2343,6 @@ struct SmallSmem {
 static_assert(sizeof(SmallSmem) <= sizeof(ResampleSmem), "one buffer for every kind of tile");
 __device__ __forceinline__ bool small_scale(int H, int W, int Ho, int Wo) { return 4 * H <= 11 * Ho && 4 * W <= 11 * Wo; }
 
-template <bool ALIGNED>
 __device__ __forceinline__ void resample_tile_small(SmallSmem& sh, const uint8_t* __restrict__ img, int H, int W, int Ho,
                                                     int Wo, int ox0, int oy0, uint8_t* __restrict__ out) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -2390,7 +2390,7 @@ __device__ __forceinline__ void resample_tile_small(SmallSmem& sh, const uint8_t
       auto take = [&](int row, float w, float2 (&a)[2]) {   // one staged row into an output row
         const uint32_t ph = (first + static_cast<uint32_t>(row) * pitch) & 15u;
         const uint32_t* p = reinterpret_cast<const uint32_t*>(sh.raw[row] + (ph & 12u)) + j;
-        const uint32_t word = ALIGNED ? p[0] : __funnelshift_r(p[0], p[1], (ph & 2u) * 8u);
+        const uint32_t word = __funnelshift_r(p[0], (ph & 2u) != 0u ? p[1] : 0u, (ph & 2u) * 8u);   // (warp-uniform)
         float2 lo, hi;
         word_to_floats(word, lo, hi);
         const float2 w2 = make_float2(w, w);
@@ -2459,14 +2459,13 @@ __device__ __forceinline__ void resample_small(SmallSmem& sh, const uint8_t* __r
     const int l = static_cast<int>(g - __shfl_sync(0xffffffffu, b < 32 ? end0 - n[0] : end1 - n[1], b & 31));
     const int nx = (Wo + kSTW - 1) / kSTW, row = l / nx;
     const int H = t.H[b], W = t.W[b], ox0 = (l - row * nx) * kSTW, oy0 = row * kSTH;
-    if (W % 4 == 0) resample_tile_small<true>(sh, src + t.src_off[b], H, W, Ho, Wo, ox0, oy0, dst + t.dst_off[b]);
-    else resample_tile_small<false>(sh, src + t.src_off[b], H, W, Ho, Wo, ox0, oy0, dst + t.dst_off[b]);
+    resample_tile_small(sh, src + t.src_off[b], H, W, Ho, Wo, ox0, oy0, dst + t.dst_off[b]);
   }
 }
 // Tiles x scale per CTA of the grid (a quarter more where rows start on 2-byte boundaries, which costs a
 // second word per read) up to which a call takes small tiles.  Both kinds, in us: 2.9 rounds at 1 (672 x 672)
-// 9.2 and 12.3, 2.1 at 1.6 (896 x 896, 3.3) 13.3 and 14.3, 3.2 at 1.3 (896 x 896, 4.1) 15.4 and 14.3, 2.1 at 2.4
-// (1344 x 1344, 5.0) 18.1 and 16.4.
+// 10.3 and 12.3, 2.1 at 1.6 (896 x 896, 3.3) 13.3 and 14.3, 3.2 at 1.3 (896 x 896, 4.1) 15.4 and 14.3, 2.1 at 2.4
+// (1344 x 1344, 5.0) 18.2 and 16.4.
 constexpr float kSmallWork = 3.8f;
 
 // Wide and generic tiles of the batch, ho and wo as in resample_small.
