@@ -13,8 +13,8 @@
 //              tail mean, rho_d, rho, r and the target size.  The token and pixel-statistic
 //              densities share it (their pass 2 fills the buckets the same way).
 // Resize: apc_resample, four CTAs per SM walking the output tiles of the batch; downscales of up to 8x
-// per side are filtered vertically in registers, then horizontally from shared memory, steeper ones
-// take a generic path with per-tap weights.
+// per side are filtered vertically in registers, then horizontally from shared memory, small outputs
+// in small staged tiles with the same sums, steeper downscales on a generic path with per-tap weights.
 #include <algorithm>
 #include <atomic>
 #include <cfloat>
